@@ -206,6 +206,8 @@ int glide::plan_context(const glide_config *cfg, glide_ctx *ctx, std::vector<Wor
     off = align_up(off + 2 * halves * size_t(L) * units_per_layer * ctx->prefill_chunk * d, 256);
     ctx->off_s16 = off;
     off = align_up(off + 2 * halves * size_t(L) * units_per_layer * d * d, 256);
+    ctx->off_zsnap = off;
+    off = align_up(off + sizeof(float) * size_t(L) * units_per_layer * dp, 256);
     if (halves == 2) {
       ctx->off_phiq16 = off;
       off = align_up(off + 2 * halves * size_t(L) * units_per_layer * ctx->prefill_chunk * ctx->G * d, 256);

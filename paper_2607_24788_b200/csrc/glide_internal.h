@@ -155,11 +155,12 @@ struct PrefillParams {
   const LayerDev *layers;
   const int32_t *heads_of;
   Control *ctl;
-  float *phik;               // chunk scratch: [layer_count][B][Hkv][C][d] fp32, phi of the delayed keys
+  float *phik;               // scratch: [layer_count][B][Hkv][nsub * SC][dp] fp32, phi of the delayed keys
   void *phik16;              // tcgen05 kernel: the same rows as bf16 (read by TMA), [dp / d halves][units_cap * Cmax][d];
                              // nullptr when that kernel is not in use
-  void *s16;                 // tcgen05 kernel: bf16 copy of every unit's S as it is at the start of the chunk,
-                             // [dp / d halves][units_cap][d][d]
+  void *s16;                 // tcgen05 kernel: bf16 copy of every unit's S as it is at the start of every chunk of the pass,
+                             // [dp / d halves][units_cap][d][d], index (unit of the pass * nsub + chunk)
+  float *zsnap;              // tcgen05 kernel: z at the start of every chunk of the pass, [units_cap][dp], the same index
   void *phiq16;              // tcgen05 kernel, learned map: phi(q) of the chunk's query rows as bf16,
                              // [2 halves][units_cap * Cmax * G][d], row = (unit * Cmax + token) * G + head of the group
   int64_t units_cap;         // L * B * H_kv of the context: what separates the halves in the three arrays above
@@ -169,9 +170,13 @@ struct PrefillParams {
   void *out;
   int64_t n0;                // tokens absorbed before this call (all layers of the call)
   int64_t T;                 // tokens of this call
-  int64_t c0;                // first token (call-relative) of the current chunk
-  int32_t C;                 // tokens in the current chunk
-  int32_t Cmax;              // scratch stride (prefill_chunk)
+  // A pass takes C tokens from call-relative token c0 on, in nsub chunks of SC tokens (the last one may be shorter).  The
+  // CUDA-core and mma.sync attention kernels work on passes of one chunk.
+  int64_t c0;
+  int32_t C;
+  int32_t SC;                // tokens of a chunk (prefill_chunk)
+  int32_t nsub;              // chunks of the pass
+  int32_t Cmax;              // scratch rows per unit: nsub * SC
   int32_t layer_begin, layer_count;
   int32_t L, B, H, Hkv;      // B: sequences of the call's tensors
   int32_t b0;                // sequence slot of the context that the call's sequence 0 is (0 unless one sequence is prefilled)
@@ -214,7 +219,7 @@ struct glide_ctx {
   int G = 0;
   int dp = 0;                       // feature dimension of the linear part: d, or 2d for the learned map
   size_t off_phit = 0, off_gcum = 0;
-  size_t off_phik16 = 0, off_s16 = 0, off_phiq16 = 0;   // bf16 scratch of the tcgen05 prefill kernel (0: not laid out)
+  size_t off_phik16 = 0, off_s16 = 0, off_zsnap = 0, off_phiq16 = 0;   // bf16 scratch of the tcgen05 prefill kernel (0: not laid out)
   int device = 0;
   int sm_count = 0;
   int decode_grid = 0;

@@ -457,24 +457,25 @@ __global__ void __launch_bounds__(kPrefillThreads) prefill_state_kernel(const Pr
 
 // 1b. (sum-of-terms merges on the tcgen05 kernel) running sums of phi(K') over the chunk: zcum[i] = sum over the valid
 // delayed indices ii <= i of phi(k'_ii); a row's linear normaliser is then phi(q) . (z + zcum[own index]).
-// One thread per (unit, feature), sequential over the chunk (C <= 1024).
+// One thread per (unit, chunk, feature), sequential over the chunk.
 template <int D>
 __global__ void __launch_bounds__(kPrefillThreads) prefill_zcum_kernel(const PrefillParams p) {
   const int64_t idx = int64_t(blockIdx.x) * kPrefillThreads + threadIdx.x;
   const int64_t units = int64_t(p.layer_count) * p.B * p.Hkv;
   const int dp = p.dp;
-  if (idx >= units * dp) return;
+  if (idx >= units * p.nsub * dp) return;
   const int r = int(idx % dp);
-  const int64_t u = idx / dp;
+  const int64_t uc = idx / dp, u = uc / p.nsub;
+  const int chunk_c0 = int(uc - u * p.nsub) * p.SC, chunk_n = min(p.SC, p.C - chunk_c0);
   const int lrel = int(u / (int64_t(p.Hkv) * p.B));
   const LayerDev ld = p.layers[p.layer_begin + lrel];
   if (!ld.evicts) return;
-  const int64_t first = p.n0 + p.c0 - ld.wlin;
-  const int i_lo = first < 0 ? int(first < -int64_t(p.C) ? p.C : -first) : 0;
-  const float *pk = p.phik + size_t(u) * p.Cmax * dp + r;
-  float *zc = p.zcum + size_t(u) * p.Cmax * dp + r;
+  const int64_t first = p.n0 + p.c0 + chunk_c0 - ld.wlin;
+  const int i_lo = first < 0 ? int(first < -int64_t(chunk_n) ? chunk_n : -first) : 0;
+  const float *pk = p.phik + (size_t(u) * p.Cmax + chunk_c0) * dp + r;
+  float *zc = p.zcum + (size_t(u) * p.Cmax + chunk_c0) * dp + r;
   float run = 0.f;
-  for (int i = 0; i < p.C; ++i) {
+  for (int i = 0; i < chunk_n; ++i) {
     if (i >= i_lo) run += pk[size_t(i) * dp];
     zc[size_t(i) * dp] = run;
   }
@@ -533,30 +534,6 @@ __global__ void __launch_bounds__(kPrefillThreads) prefill_ring_kernel(const Pre
   }
 }
 
-// bf16 copy of the state of every unit of the call as it is before the chunk's state update: what the tcgen05 attention
-// kernel multiplies phi(Q) with (one 16-byte store per thread).  With the learned map S has 2 d rows: rows d .. 2d - 1
-// go to the second half of the array.
-__global__ void __launch_bounds__(kPrefillThreads) prefill_s16_kernel(const PrefillParams p) {
-  constexpr int D = 128;
-  const int64_t id = int64_t(blockIdx.x) * kPrefillThreads + threadIdx.x;   // 8 consecutive entries of one unit's S
-  const int64_t per_unit = int64_t(p.dp) * D / 8;
-  const int64_t u = id / per_unit;
-  if (u >= int64_t(p.layer_count) * p.B * p.Hkv) return;
-  const int g = int(u % p.Hkv);
-  const int b = int((u / p.Hkv) % p.B);
-  const int lrel = int(u / (int64_t(p.Hkv) * p.B));
-  const LayerDev ld = p.layers[p.layer_begin + lrel];
-  if (!ld.evicts) return;
-  const size_t e0 = size_t(id % per_unit) * 8;   // entry of S [dp][d]
-  const float *src = reinterpret_cast<const float *>(p.ws + ld.S) + (size_t(b + p.b0) * p.Hkv + g) * size_t(p.dp) * D + e0;
-  const float4 f0 = *reinterpret_cast<const float4 *>(src), f1 = *reinterpret_cast<const float4 *>(src + 4);
-  __nv_bfloat162 o[4] = {__floats2bfloat162_rn(f0.x, f0.y), __floats2bfloat162_rn(f0.z, f0.w),
-                         __floats2bfloat162_rn(f1.x, f1.y), __floats2bfloat162_rn(f1.z, f1.w)};
-  const size_t half = e0 / (size_t(D) * D);
-  *reinterpret_cast<uint4 *>(reinterpret_cast<__nv_bfloat16 *>(p.s16) + half * size_t(p.units_cap) * D * D + size_t(u) * D * D +
-                             (e0 - half * D * D)) = *reinterpret_cast<const uint4 *>(o);
-}
-
 }  // namespace
 
 int launch_prefill(glide_ctx *ctx, int layer_begin, int layer_count, int64_t T, const void *q, const void *k,
@@ -575,6 +552,8 @@ int launch_prefill(glide_ctx *ctx, int layer_begin, int layer_count, int64_t T, 
   p.out = out;
   p.n0 = n0;
   p.T = T;
+  p.SC = ctx->prefill_chunk;
+  p.nsub = 1;
   p.Cmax = ctx->prefill_chunk;
   p.layer_begin = layer_begin;
   p.layer_count = layer_count;
@@ -604,6 +583,7 @@ int launch_prefill(glide_ctx *ctx, int layer_begin, int layer_count, int64_t T, 
   const bool use_tc = impl == GLIDE_PREFILL_TCGEN05 && tc_kind && prefill_attn_tc_supported(ctx);
   p.phik16 = use_tc && out ? ctx->ws + ctx->off_phik16 : nullptr;
   p.s16 = use_tc && out ? ctx->ws + ctx->off_s16 : nullptr;
+  p.zsnap = reinterpret_cast<float *>(ctx->ws + ctx->off_zsnap);
   p.phiq16 = use_tc && out && ctx->off_phiq16 ? ctx->ws + ctx->off_phiq16 : nullptr;
   p.units_cap = int64_t(ctx->cfg.n_layers) * ctx->cfg.batch * ctx->cfg.n_kv_heads;
   // (the mma.sync kernel has the shared normaliser only: the other merges fall through to the CUDA-core kernel)
@@ -612,8 +592,65 @@ int launch_prefill(glide_ctx *ctx, int layer_begin, int layer_count, int64_t T, 
   // carry of the chunk scan: tensor cores with an error-free three-way bf16 split of phi(K') (bf16, d = 128), or the
   // CUDA-core kernel (fp32 I/O, d = 64, and whenever the CUDA-core prefill is asked for)
   const bool state_mma = !ctx->cfg.gated && prefill_state_mma_supported(ctx) && impl != GLIDE_PREFILL_FMA;   // (either feature map)
-  bool any_evicts = false;
-  for (int l = layer_begin; l < layer_begin + layer_count; ++l) any_evicts = any_evicts || ctx->layers[l].evicts;
+  auto evicts_in = [&](int first, int count) {
+    bool any = false;
+    for (int l = first; l < first + count; ++l) any = any || ctx->layers[l].evicts;
+    return any;
+  };
+  const bool any_evicts = evicts_in(layer_begin, layer_count);
+
+  // Tensor-core pipeline (outputs by the tcgen05 kernel, or no outputs and the tensor-core carry).  Nothing in a pass
+  // waits for the ring update of its own tokens, and the chunks of a pass depend on one another through S alone, which
+  // a scan over the chunk sums supplies: so a pass takes many chunks of few layers rather than one chunk of all
+  // layers, as many as the scratch holds (it is sized for one chunk of every unit).  Chunk by chunk, one layer of 8 KV
+  // heads left most of the chip idle: 32 CTAs of 40 us per chunk (32 layers, 8001 tokens, layer by layer: 76.2 ms).
+  auto run_passes = [&](auto tt, auto dd, auto pp) -> int {
+    using TT = typename decltype(tt)::type;
+    constexpr int D = decltype(dd)::value, DP = decltype(pp)::value;
+    constexpr bool kCanProject = DP == 2 * D && D == 128 && std::is_same<TT, __nv_bfloat16>::value;
+    const int64_t units_layer = int64_t(p.B) * p.Hkv;
+    const int64_t most = p.SC > 128 ? p.units_cap / units_layer : 1;   // (the chunk sums take 129 scratch rows of a chunk)
+    const int nsub_max = int(std::min<int64_t>(most, (T + p.SC - 1) / p.SC));
+    const int fit = int(std::min<int64_t>(layer_count, p.units_cap / (units_layer * nsub_max)));
+    const int n_groups = (layer_count + fit - 1) / fit;
+    const size_t elem = sizeof(TT);
+    for (int64_t c0 = 0; c0 < T; c0 += int64_t(nsub_max) * p.SC) {
+      for (int gi = 0; gi < n_groups; ++gi) {
+        const int l0 = int(int64_t(layer_count) * gi / n_groups), l1 = int(int64_t(layer_count) * (gi + 1) / n_groups);
+        PrefillParams s = p;
+        s.layer_begin = layer_begin + l0;
+        s.layer_count = l1 - l0;
+        const size_t seqs = size_t(l0) * p.B * size_t(T);   // tokens of the call's tensors before the group's first layer
+        s.k = static_cast<const unsigned char *>(k) + seqs * p.Hkv * D * elem;
+        s.v = static_cast<const unsigned char *>(v) + seqs * p.Hkv * D * elem;
+        if (q) s.q = static_cast<const unsigned char *>(q) + seqs * p.H * D * elem;
+        if (out) s.out = static_cast<unsigned char *>(out) + seqs * p.H * D * elem;
+        s.c0 = c0;
+        s.C = int(std::min<int64_t>(int64_t(nsub_max) * p.SC, T - c0));
+        s.nsub = (s.C + p.SC - 1) / p.SC;
+        s.Cmax = s.nsub * p.SC;
+        const int64_t units = int64_t(s.layer_count) * units_layer;
+        const int64_t warps4 = units * ((s.C + kTokPerWarp - 1) / kTokPerWarp);
+        const unsigned warp4_blocks = unsigned((warps4 * 32 + kPrefillThreads - 1) / kPrefillThreads);
+        if (evicts_in(s.layer_begin, s.layer_count)) {
+          if (kCanProject) {
+            if (launch_prefill_project(ctx, s, true, stream) != GLIDE_OK) return GLIDE_ERR_CUDA;
+          } else {
+            prefill_phi_kernel<TT, D, DP><<<warp4_blocks, kPrefillThreads, 0, stream>>>(s);
+          }
+          if (out && s.phiq16 && launch_prefill_project(ctx, s, false, stream) != GLIDE_OK) return GLIDE_ERR_CUDA;
+          if (out && p.merge != GLIDE_MERGE_SHARED)   // (before the carry: the chunk sums overwrite rows of phi(K'))
+            prefill_zcum_kernel<D><<<unsigned((units * s.nsub * D + kPrefillThreads - 1) / kPrefillThreads), kPrefillThreads, 0, stream>>>(s);
+          if (launch_prefill_state_mma(ctx, s, stream) != GLIDE_OK) return GLIDE_ERR_CUDA;
+        }
+        if (out && launch_prefill_attn_tc(ctx, s, stream) != GLIDE_OK) return GLIDE_ERR_CUDA;
+        prefill_ring_kernel<TT, D><<<warp4_blocks, kPrefillThreads, 0, stream>>>(s);
+        if (cudaGetLastError() != cudaSuccess) return GLIDE_ERR_CUDA;
+      }
+    }
+    return GLIDE_OK;
+  };
+  const bool passes = state_mma && (use_tc || !out);
 
   auto run_chunks = [&](auto tt, auto dd, auto gg, auto pp) -> int {
     using TT = typename decltype(tt)::type;
@@ -625,8 +662,6 @@ int launch_prefill(glide_ctx *ctx, int layer_begin, int layer_count, int64_t T, 
       const unsigned warp_blocks = unsigned((warps * 32 + kPrefillThreads - 1) / kPrefillThreads);
       const int64_t warps4 = units * ((p.C + kTokPerWarp - 1) / kTokPerWarp);
       const unsigned warp4_blocks = unsigned((warps4 * 32 + kPrefillThreads - 1) / kPrefillThreads);
-      // the learned map's projections of the delayed keys go to the tensor cores for bf16 / d = 128 unless the
-      // CUDA-core prefill was asked for
       constexpr bool kCanProject = DP == 2 * D && D == 128 && std::is_same<TT, __nv_bfloat16>::value;
       if (any_evicts && kCanProject && impl != GLIDE_PREFILL_FMA) {
         if (launch_prefill_project(ctx, p, true, stream) != GLIDE_OK) return GLIDE_ERR_CUDA;
@@ -636,14 +671,7 @@ int launch_prefill(glide_ctx *ctx, int layer_begin, int layer_count, int64_t T, 
       if (any_evicts && p.gated)
         prefill_gcum_kernel<TT, D><<<unsigned((units + kPrefillThreads - 1) / kPrefillThreads), kPrefillThreads, 0, stream>>>(p);
       if (out) {
-        if (use_tc) {
-          if (any_evicts)
-            prefill_s16_kernel<<<unsigned((units * (int64_t(p.dp) * 128 / 8) + kPrefillThreads - 1) / kPrefillThreads), kPrefillThreads, 0, stream>>>(p);
-          if (any_evicts && p.phiq16 && launch_prefill_project(ctx, p, false, stream) != GLIDE_OK) return GLIDE_ERR_CUDA;
-          if (any_evicts && p.merge != GLIDE_MERGE_SHARED)
-            prefill_zcum_kernel<D><<<unsigned((units * D + kPrefillThreads - 1) / kPrefillThreads), kPrefillThreads, 0, stream>>>(p);
-          if (launch_prefill_attn_tc(ctx, p, stream) != GLIDE_OK) return GLIDE_ERR_CUDA;
-        } else if (use_mma) {
+        if (use_mma) {
           if (launch_prefill_attn_mma(ctx, p, stream) != GLIDE_OK) return GLIDE_ERR_CUDA;
         } else {
           prefill_attn_kernel<TT, D, G, DP><<<warp_blocks, kPrefillThreads, 0, stream>>>(p);
@@ -663,6 +691,8 @@ int launch_prefill(glide_ctx *ctx, int layer_begin, int layer_count, int64_t T, 
   };
   int rc = dispatch_config(ctx->cfg.io_dtype, ctx->cfg.head_dim, ctx->G, [&](auto tt, auto dd, auto gg) -> int {
     constexpr int D = decltype(dd)::value;
+    if constexpr (D == 128 && std::is_same<typename decltype(tt)::type, __nv_bfloat16>::value)
+      if (passes) return ctx->dp == D ? run_passes(tt, dd, IntTag<D>{}) : run_passes(tt, dd, IntTag<2 * D>{});
     if (ctx->dp == D) return run_chunks(tt, dd, gg, IntTag<D>{});
     return run_chunks(tt, dd, gg, IntTag<2 * D>{});
   });

@@ -593,7 +593,7 @@ __global__ void __launch_bounds__(kThreads) prefill_project_mma_kernel(const Pre
     }
     bf16 *dst = KEYS ? reinterpret_cast<bf16 *>(p.phik16) + (size_t(u) * p.Cmax + i0 + tok) * kD + col
                      : reinterpret_cast<bf16 *>(p.phiq16) + ((size_t(u) * p.Cmax + i0 + tok) * G + hh) * kD + col;
-    const size_t half = KEYS ? size_t(p.units_cap) * p.Cmax * kD : size_t(p.units_cap) * p.Cmax * G * kD;
+    const size_t half = KEYS ? size_t(p.units_cap) * p.SC * kD : size_t(p.units_cap) * p.SC * G * kD;
     if (dst != nullptr && (!KEYS || p.phik16)) {
 #pragma unroll
       for (int nt = 0; nt < kD / 8; ++nt) {

@@ -55,20 +55,28 @@ __device__ __forceinline__ void split3(float x0, float x1, uint32_t &hi, uint32_
   lo = *reinterpret_cast<const uint32_t *>(&l);
 }
 
+// PARTIAL (passes of several chunks): the chunk's own sum goes to the scratch rows that the CTA has just consumed instead
+// of S (64 state rows x 128 values = 128 scratch rows x the CTA's 64 columns, z in row 128: chunks of more than 128
+// tokens), and prefill_scan_kernel adds the sums up in chunk order.  Otherwise S is updated in place, and its value
+// before the chunk is left as bf16 (z: fp32) for the attention kernel, which runs after this one.
+template <bool PARTIAL>
 __global__ void __launch_bounds__(kThreads) prefill_state_mma_kernel(const PrefillParams p) {
   using bf16 = __nv_bfloat16;
   __shared__ __align__(16) unsigned char stage[2][kPhiBytes + kVBytes];
   const int blocks_per_unit = p.dp / kRowsPerCta;   // rows of S: d, or 2 d with the learned feature map
-  const int64_t u = blockIdx.x / blocks_per_unit;
+  const int64_t uc = blockIdx.x / blocks_per_unit;   // (unit, chunk of the pass)
   const int rb = blockIdx.x % blocks_per_unit;
+  const int64_t u = PARTIAL ? uc / p.nsub : uc;
+  const int chunk_c0 = PARTIAL ? int(uc - u * p.nsub) * p.SC : 0;   // first token of the chunk, relative to the pass
+  const int chunk_n = min(p.SC, p.C - chunk_c0);
   const int g = int(u % p.Hkv);
   const int b = int((u / p.Hkv) % p.B);
   const int lrel = int(u / (int64_t(p.Hkv) * p.B));
   const LayerDev ld = p.layers[p.layer_begin + lrel];
   if (!ld.evicts) return;
-  const int64_t first = p.n0 + p.c0 - ld.wlin;    // delayed token of chunk index 0
-  const int i_lo = first < 0 ? int(first < -int64_t(p.C) ? p.C : -first) : 0;
-  if (i_lo >= p.C) return;
+  const int64_t first = p.n0 + p.c0 + chunk_c0 - ld.wlin;    // delayed token of chunk index 0
+  const int i_lo = first < 0 ? int(first < -int64_t(chunk_n) ? chunk_n : -first) : 0;
+  if (i_lo >= chunk_n) return;
   const int ub = (b + p.b0) * p.Hkv + g;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int gid = lane >> 2, tig = lane & 3;
@@ -77,7 +85,7 @@ __global__ void __launch_bounds__(kThreads) prefill_state_mma_kernel(const Prefi
   const bf16 *ringV = reinterpret_cast<const bf16 *>(p.ws + ld.ringV) + size_t(ub) * size_t(ld.cap) * kD;
   const bf16 *callV = reinterpret_cast<const bf16 *>(p.v) + ((size_t(lrel) * p.B + b) * size_t(p.T) * p.Hkv + g) * kD;
   const int64_t call_stride = int64_t(p.Hkv) * kD;
-  const float *pk = p.phik + size_t(u) * p.Cmax * p.dp + rb * kRowsPerCta;
+  float *pk = p.phik + (size_t(u) * p.Cmax + chunk_c0) * p.dp + rb * kRowsPerCta;
 
   float acc[kD / 8][4];
 #pragma unroll
@@ -86,7 +94,7 @@ __global__ void __launch_bounds__(kThreads) prefill_state_mma_kernel(const Prefi
 
   // tokens past the chunk's end are filled with zeros
   auto issue = [&](int buf, int i0) {
-    const int nt = min(kTok, p.C - i0);
+    const int nt = min(kTok, chunk_n - i0);
     const uint32_t sphi = smem_addr(stage[buf]), sv = sphi + kPhiBytes;
     for (int e = tid; e < kTok * (kRowsPerCta / 4); e += kThreads) {
       const int i = e / (kRowsPerCta / 4), c4 = e % (kRowsPerCta / 4);
@@ -102,8 +110,8 @@ __global__ void __launch_bounds__(kThreads) prefill_state_mma_kernel(const Prefi
   };
   issue(0, i_lo);
   int buf = 0;
-  for (int i0 = i_lo; i0 < p.C; i0 += kTok, buf ^= 1) {
-    if (i0 + kTok < p.C) {
+  for (int i0 = i_lo; i0 < chunk_n; i0 += kTok, buf ^= 1) {
+    if (i0 + kTok < chunk_n) {
       issue(buf ^ 1, i0 + kTok);
       asm volatile("cp.async.wait_group 1;" ::: "memory");
     } else {
@@ -143,22 +151,101 @@ __global__ void __launch_bounds__(kThreads) prefill_state_mma_kernel(const Prefi
     __syncthreads();   // the stage is refilled by the next iteration's issue
   }
   // accumulator fragment: c0, c1 -> (row gid, cols 2 tig + {0,1}); c2, c3 -> row gid + 8
-  float *Sb = reinterpret_cast<float *>(p.ws + ld.S) + size_t(ub) * p.dp * kD + size_t(rb * kRowsPerCta + warp * 16) * kD;
+  if (PARTIAL) {   // (every read of these scratch columns lies before the loop's last barrier)
 #pragma unroll
-  for (int n = 0; n < kD / 8; ++n) {
-    float2 *d0 = reinterpret_cast<float2 *>(Sb + size_t(gid) * kD + n * 8 + 2 * tig);
-    float2 *d1 = reinterpret_cast<float2 *>(Sb + size_t(gid + 8) * kD + n * 8 + 2 * tig);
-    float2 c0 = *d0, c1 = *d1;
-    c0.x += acc[n][0];
-    c0.y += acc[n][1];
-    c1.x += acc[n][2];
-    c1.y += acc[n][3];
-    *d0 = c0;
-    *d1 = c1;
+    for (int n = 0; n < kD / 8; ++n)
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int row = warp * 16 + gid + h * 8, col = n * 8 + 2 * tig;
+        *reinterpret_cast<float2 *>(pk + size_t(2 * row + (col >> 6)) * p.dp + (col & 63)) =
+            make_float2(acc[n][2 * h], acc[n][2 * h + 1]);
+      }
+    if (tid < kRowsPerCta) pk[size_t(kD) * p.dp + tid] = zacc;
+    return;
   }
+  float *Sb = reinterpret_cast<float *>(p.ws + ld.S) + size_t(ub) * p.dp * kD + size_t(rb * kRowsPerCta + warp * 16) * kD;
+  // the halves of a state with 2 d rows are units_cap units apart in the bf16 copy
+  bf16 *s16 = p.s16 ? reinterpret_cast<bf16 *>(p.s16) + (size_t(rb * kRowsPerCta / kD) * p.units_cap + u) * kD * kD +
+                          size_t(rb * kRowsPerCta % kD + warp * 16) * kD
+                    : nullptr;
+#pragma unroll
+  for (int n = 0; n < kD / 8; ++n)
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const size_t at = size_t(gid + h * 8) * kD + n * 8 + 2 * tig;
+      float2 *dst = reinterpret_cast<float2 *>(Sb + at);
+      float2 c = *dst;
+      if (s16) *reinterpret_cast<__nv_bfloat162 *>(s16 + at) = __floats2bfloat162_rn(c.x, c.y);
+      c.x += acc[n][2 * h];
+      c.y += acc[n][2 * h + 1];
+      *dst = c;
+    }
   if (tid < kRowsPerCta) {
     float *zb = reinterpret_cast<float *>(p.ws + ld.z) + size_t(ub) * p.dp + rb * kRowsPerCta;
-    zb[tid] += zacc;
+    const float z0 = zb[tid];
+    if (s16) p.zsnap[size_t(u) * p.dp + rb * kRowsPerCta + tid] = z0;
+    zb[tid] = z0 + zacc;
+  }
+}
+
+// The chunk sums of a pass added up in chunk order: S and z of the context move on by the whole pass, and their values at
+// the start of every chunk are left for the attention kernel (bf16 copy of S, fp32 z) when there are outputs.  One CTA per
+// (unit, 4 rows of S), a thread owns four columns of a row; the sums of four chunks are loaded together, so that the
+// chain over the chunks is one of additions and not of memory round trips.
+__global__ void __launch_bounds__(kThreads) prefill_scan_kernel(const PrefillParams p) {
+  using bf16 = __nv_bfloat16;
+  const int ctas_per_unit = p.dp / 4;
+  const int64_t u = blockIdx.x / ctas_per_unit;
+  const int j = int(blockIdx.x % ctas_per_unit), tid = threadIdx.x;
+  const int g = int(u % p.Hkv);
+  const int b = int((u / p.Hkv) % p.B);
+  const int lrel = int(u / (int64_t(p.Hkv) * p.B));
+  const LayerDev ld = p.layers[p.layer_begin + lrel];
+  if (!ld.evicts) return;
+  // chunks before the first delayed token add nothing (and have left no sum): k0 is the first that does
+  const int64_t first = p.n0 + p.c0 - ld.wlin;
+  if (first + p.C <= 0) return;
+  const int k0 = first < 0 ? int(-first / p.SC) : 0;
+  const int ub = (b + p.b0) * p.Hkv + g;
+  const int r = j * 4 + (tid >> 5), col = (tid & 31) * 4;
+  const float *part = p.phik + (size_t(u) * p.Cmax + 2 * (r & 63) + (col >> 6)) * p.dp + (r >> 6) * 64 + (col & 63);
+  const size_t step = size_t(p.SC) * p.dp;
+  float4 *Sp = reinterpret_cast<float4 *>(reinterpret_cast<float *>(p.ws + ld.S) + (size_t(ub) * p.dp + r) * kD + col);
+  const int half = r / kD;
+  bf16 *snap = p.s16 ? reinterpret_cast<bf16 *>(p.s16) + ((size_t(half) * p.units_cap + u * p.nsub) * kD + (r - half * kD)) * kD + col
+                     : nullptr;
+  float4 s = *Sp;
+  constexpr int kAhead = 4;
+  for (int k = k0; k < p.nsub; k += kAhead) {
+    float4 x[kAhead];
+#pragma unroll
+    for (int a = 0; a < kAhead; ++a)
+      if (k + a < p.nsub) x[a] = *reinterpret_cast<const float4 *>(part + size_t(k + a) * step);
+#pragma unroll
+    for (int a = 0; a < kAhead; ++a) {
+      if (k + a >= p.nsub) break;
+      if (snap) {
+        const __nv_bfloat162 lo = __floats2bfloat162_rn(s.x, s.y), hi = __floats2bfloat162_rn(s.z, s.w);
+        *reinterpret_cast<uint2 *>(snap + size_t(k + a) * kD * kD) =
+            make_uint2(*reinterpret_cast<const uint32_t *>(&lo), *reinterpret_cast<const uint32_t *>(&hi));
+      }
+      s.x += x[a].x;
+      s.y += x[a].y;
+      s.z += x[a].z;
+      s.w += x[a].w;
+    }
+  }
+  *Sp = s;
+  if (tid < 4) {   // z of the CTA's four rows
+    const int rz = j * 4 + tid;
+    const float *pz = p.phik + (size_t(u) * p.Cmax + kD) * p.dp + rz;
+    float *zp = reinterpret_cast<float *>(p.ws + ld.z) + size_t(ub) * p.dp + rz;
+    float z = *zp;
+    for (int k = k0; k < p.nsub; ++k) {
+      if (snap) p.zsnap[(size_t(u) * p.nsub + k) * p.dp + rz] = z;
+      z += pz[size_t(k) * step];
+    }
+    *zp = z;
   }
 }
 
@@ -171,7 +258,13 @@ bool prefill_state_mma_supported(const glide_ctx *ctx) {
 int launch_prefill_state_mma(glide_ctx *ctx, const PrefillParams &p, cudaStream_t stream) {
   (void)ctx;
   const int64_t units = int64_t(p.layer_count) * p.B * p.Hkv;
-  prefill_state_mma_kernel<<<unsigned(units * (p.dp / kRowsPerCta)), kThreads, 0, stream>>>(p);
+  const unsigned blocks = unsigned(units * p.nsub * (p.dp / kRowsPerCta));
+  if (p.nsub == 1) {
+    prefill_state_mma_kernel<false><<<blocks, kThreads, 0, stream>>>(p);
+  } else {
+    prefill_state_mma_kernel<true><<<blocks, kThreads, 0, stream>>>(p);
+    prefill_scan_kernel<<<unsigned(units * (p.dp / 4)), kThreads, 0, stream>>>(p);
+  }
   return cudaGetLastError() == cudaSuccess ? GLIDE_OK : GLIDE_ERR_CUDA;
 }
 

@@ -255,18 +255,25 @@ prefill_attn_tc_kernel(const PrefillParams p, const CUtensorMap *ring_maps, cons
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   Smem &sm = *reinterpret_cast<Smem *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int ctas_per_chunk = (p.C + TOKC - 1) / TOKC;
-  const int64_t u = blockIdx.x / ctas_per_chunk;
-  const int tok0 = int(blockIdx.x % ctas_per_chunk) * TOKC;
+  // CTAs of a unit: those of its full chunks, then those of the last one; from here on "the chunk" is the CTA's own
+  const int ctas_per_chunk = (p.SC + TOKC - 1) / TOKC;
+  const int ctas_per_unit = (p.nsub - 1) * ctas_per_chunk + (p.C - (p.nsub - 1) * p.SC + TOKC - 1) / TOKC;
+  const int64_t u = blockIdx.x / ctas_per_unit;
+  const int cta_u = int(blockIdx.x % ctas_per_unit);
+  const int sub = cta_u / ctas_per_chunk;
+  const int tok0 = (cta_u - sub * ctas_per_chunk) * TOKC;
+  const int chunk_c0 = int(p.c0) + sub * p.SC;                // first token of the chunk, relative to the call
+  const int chunk_n = min(p.SC, p.C - sub * p.SC);            // its tokens
+  const int64_t uc = u * p.nsub + sub;                        // (unit, chunk): index into the scratch arrays
   const int g = int(u % p.Hkv);
   const int b = int((u / p.Hkv) % p.B);
   const int lrel = int(u / (int64_t(p.Hkv) * p.B));
   const int layer = p.layer_begin + lrel;
   const LayerDev ld = p.layers[layer];
-  const int ntok = min(TOKC, p.C - tok0);
+  const int ntok = min(TOKC, chunk_n - tok0);
   const int ntokA = min(TOKT, ntok), ntokB = ntok - ntokA;
   const bool hasB = ntokB > 0;
-  const int64_t tq0 = p.n0 + p.c0 + tok0;
+  const int64_t tq0 = p.n0 + chunk_c0 + tok0;
   const int64_t tq_last = tq0 + ntok - 1;
   const int64_t w = ld.w;
   const int64_t wl = ld.wlin;                      // delay of the linear stream: w, or 0 when the state holds every token
@@ -332,7 +339,7 @@ prefill_attn_tc_kernel(const PrefillParams p, const CUtensorMap *ring_maps, cons
     const int Xq = (tid >> 7) & 1, rq = tid & 127;
     const int ntokXq = Xq ? ntokB : ntokA;
     if (tid < kSoftmaxThreads && ntokXq > 0) {
-      const bf16 *qbase = reinterpret_cast<const bf16 *>(p.q) + (seq + size_t(p.c0 + tok0 + Xq * TOKT)) * p.H * kD;
+      const bf16 *qbase = reinterpret_cast<const bf16 *>(p.q) + (seq + size_t(chunk_c0 + tok0 + Xq * TOKT)) * p.H * kD;
       const uint32_t sQx = smem_u32(sm.q[Xq]);
 #pragma unroll 4
       for (int i = 0; i < kRows * 16 / kRows; ++i) {
@@ -356,10 +363,10 @@ prefill_attn_tc_kernel(const PrefillParams p, const CUtensorMap *ring_maps, cons
   auto kv_addr = [&](int slot) { return sKV0 + uint32_t(slot) * kTileBytes; };
   // Linear part: what it needs is known now, so that the loader can fetch it behind the last key tiles.
   const bool linear = ld.evicts && tq_last >= wl;
-  const int64_t folded = p.n0 + p.c0 - wl;   // tokens below this index are in S, z at the start of the chunk
+  const int64_t folded = p.n0 + chunk_c0 - wl;   // tokens below this index are in S, z at the start of the chunk
   const bool need_state = linear && folded > 0;
   // intra-chunk steps: delayed tokens of this chunk up to the CTA's last token, 128 at a time
-  const int i_lo = folded < 0 ? int(-folded < int64_t(p.C) ? -folded : int64_t(p.C)) : 0;
+  const int i_lo = folded < 0 ? int(-folded < int64_t(chunk_n) ? -folded : int64_t(chunk_n)) : 0;
   const int i_hi = tok0 + ntok - 1;
   const int it0 = i_lo & ~(kKT - 1);
   const int n_itiles = (linear && it0 <= i_hi) ? (i_hi - it0) / kKT + 1 : 0;
@@ -376,7 +383,7 @@ prefill_attn_tc_kernel(const PrefillParams p, const CUtensorMap *ring_maps, cons
   auto load_pk = [&](int t) {   // one thread: the phi(K') rows of intra-chunk step t
     const uint32_t bar = smem_u32(&sm.bar_pk[t & 1]);
     const uint32_t dst = kv_addr(slotPk[t & 1]);
-    const int y = int(u * p.Cmax) + it0 + t * kKT;
+    const int y = int(uc * p.SC) + it0 + t * kKT;
     mbar_expect_tx(bar, kTileBytes);
     tma_load_2d(dst, map_pk, 0, y, bar);
     tma_load_2d(dst + kBoxBytes, map_pk, 64, y, bar);
@@ -389,7 +396,7 @@ prefill_attn_tc_kernel(const PrefillParams p, const CUtensorMap *ring_maps, cons
   const int ntokX = X ? ntokB : ntokA;
   const bool activeX = tid < kSoftmaxThreads && ntokX > 0;
   const int tl = tok0 + X * TOKT + tok_r;         // chunk-relative token of this row
-  const int64_t tok_abs = p.n0 + p.c0 + tl;
+  const int64_t tok_abs = p.n0 + chunk_c0 + tl;
   const uint32_t tS = tmem + (uint32_t((warp & 3) * 32) << 16) + uint32_t(X) * 128u;
   const uint32_t tO = tS + 256u;
   float m_ref = -CUDART_INF_F, l_sum = 0.f;
@@ -639,12 +646,11 @@ prefill_attn_tc_kernel(const PrefillParams p, const CUtensorMap *ring_maps, cons
         if (sq >= 0 && !mbar_wait(smem_u32(&sm.bar_free[sq % kStages]), uint32_t(sq / kStages) & 1u, failed)) break;
         if (k == 0) {
           if (!need_state) continue;
-          const int ub = (b + p.b0) * p.Hkv + g;
           const uint32_t bar = smem_u32(&sm.bar_state);
           mbar_expect_tx(bar, kTileBytes + uint32_t(kD * sizeof(float)));
-          tma_load_2d(kv_addr(slotSb), map_s16, 0, int(u * kD), bar);
-          tma_load_2d(kv_addr(slotSb) + kBoxBytes, map_s16, 64, int(u * kD), bar);
-          bulk_load(smem_u32(sm.z), p.ws + ld.z + size_t(ub) * kD * sizeof(float), uint32_t(kD * sizeof(float)), bar);
+          tma_load_2d(kv_addr(slotSb), map_s16, 0, int(uc * kD), bar);
+          tma_load_2d(kv_addr(slotSb) + kBoxBytes, map_s16, 64, int(uc * kD), bar);
+          bulk_load(smem_u32(sm.z), p.zsnap + size_t(uc) * kD, uint32_t(kD * sizeof(float)), bar);
         } else {
           load_pk(k - 1);
         }
@@ -775,7 +781,7 @@ prefill_attn_tc_kernel(const PrefillParams p, const CUtensorMap *ring_maps, cons
       // one pass of exponentials: kept as packed bf16, normalised by the sum of the unrounded values afterwards
       float sum0 = 0.f, sum1 = 0.f, dz0 = 0.f, dz1 = 0.f;
       const float mxl = mx * kLog2e;
-      const float4 *zrow = reinterpret_cast<const float4 *>(p.zcum + (size_t(u) * p.Cmax + size_t(tok_r < ntokX ? tl : tok0)) * kD);
+      const float4 *zrow = reinterpret_cast<const float4 *>(p.zcum + (size_t(uc) * p.SC + size_t(tok_r < ntokX ? tl : tok0)) * kD);
 #pragma unroll
       for (int i4 = 0; i4 < kD / 4; ++i4) {
         float zz[4] = {0.f, 0.f, 0.f, 0.f};
@@ -898,7 +904,7 @@ prefill_attn_tc_kernel(const PrefillParams p, const CUtensorMap *ring_maps, cons
       cp_async_commit();
     };
     const CUtensorMap *map_pq = map_pk + 2;
-    const int rows_q = int(p.units_cap) * p.Cmax * G, rows_s = int(p.units_cap) * kD, rows_k = int(p.units_cap) * p.Cmax;
+    const int rows_q = int(p.units_cap) * p.SC * G, rows_s = int(p.units_cap) * kD, rows_k = int(p.units_cap) * p.SC;
     auto tma_tile = [&](uint32_t dst, const CUtensorMap *m, int y, uint32_t bar) {
       tma_load_2d(dst, m, 0, y, bar);
       tma_load_2d(dst + kBoxBytes, m, 64, y, bar);
@@ -909,13 +915,12 @@ prefill_attn_tc_kernel(const PrefillParams p, const CUtensorMap *ring_maps, cons
       for (int hf = 0; hf < 2; ++hf)
         for (int x = 0; x < 2; ++x) {
           if (x == 1 && !hasB) break;
-          tma_tile(hf == 0 ? sQ[x] : kv_addr(x), map_pq, hf * rows_q + (int(u) * p.Cmax + tok0 + x * TOKT) * G, bar);
+          tma_tile(hf == 0 ? sQ[x] : kv_addr(x), map_pq, hf * rows_q + (int(uc) * p.SC + tok0 + x * TOKT) * G, bar);
         }
       if (need_state) {
-        const int ub = (b + p.b0) * p.Hkv + g;
-        tma_tile(kv_addr(2), map_s16, int(u) * kD, bar);
-        tma_tile(kv_addr(3), map_s16, rows_s + int(u) * kD, bar);
-        bulk_load(smem_u32(sm.z), p.ws + ld.z + size_t(ub) * 2 * kD * sizeof(float), uint32_t(2 * kD * sizeof(float)), bar);
+        tma_tile(kv_addr(2), map_s16, int(uc) * kD, bar);
+        tma_tile(kv_addr(3), map_s16, rows_s + int(uc) * kD, bar);
+        bulk_load(smem_u32(sm.z), p.zsnap + size_t(uc) * 2 * kD, uint32_t(2 * kD * sizeof(float)), bar);
       }
     }
     if (tid < kSoftmaxThreads && n_itiles > 0) load_vp(0);
@@ -971,8 +976,8 @@ prefill_attn_tc_kernel(const PrefillParams p, const CUtensorMap *ring_maps, cons
         // buffers 2 and 3 are free: the products that read them have completed
         const uint32_t bar = smem_u32(&sm.bar_pk[0]);
         mbar_expect_tx(bar, 2u * kTileBytes);
-        tma_tile(kv_addr(2), map_pk, int(u) * p.Cmax + i0, bar);
-        tma_tile(kv_addr(3), map_pk, rows_k + int(u) * p.Cmax + i0, bar);
+        tma_tile(kv_addr(2), map_pk, int(uc) * p.SC + i0, bar);
+        tma_tile(kv_addr(3), map_pk, rows_k + int(uc) * p.SC + i0, bar);
         mbar_wait(bar, uint32_t(t) & 1u, failed);
         tc_fence_after();
         for (int x = 0; x < 2; ++x) {
@@ -1008,7 +1013,7 @@ prefill_attn_tc_kernel(const PrefillParams p, const CUtensorMap *ring_maps, cons
     const bool store = tok_r < ntokX;   // the TMEM loads below are warp-collective: only the store is per row
     const float inv = store ? 1.0f / l_sum : 0.f;
     bf16 *op = reinterpret_cast<bf16 *>(p.out) +
-               ((seq + size_t(p.c0 + (store ? tl : tok0))) * p.H + p.heads_of[g * G + hh]) * kD;
+               ((seq + size_t(chunk_c0 + (store ? tl : tok0))) * p.H + p.heads_of[g * G + hh]) * kD;
     uint32_t ra[32], rb[32];
     tmem_ld32_nowait(tO, ra);
 #pragma unroll
@@ -1095,7 +1100,7 @@ int launch_prefill_attn_tc(glide_ctx *ctx, const PrefillParams &p, cudaStream_t 
     constexpr int G = decltype(gg)::value;
     constexpr int TOKC = 2 * kRows / G;
     const size_t smem = sizeof(Smem) + 1024;
-    const int64_t blocks = units * ((p.C + TOKC - 1) / TOKC);
+    const int64_t blocks = units * (int64_t(p.nsub - 1) * ((p.SC + TOKC - 1) / TOKC) + (p.C - (p.nsub - 1) * p.SC + TOKC - 1) / TOKC);
     auto run = [&](auto kern) -> int {
       if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)) != cudaSuccess) {
         cudaGetLastError();
