@@ -4,21 +4,23 @@
 // rows each, a row being (token, query head of the group), row = token * G + head.
 //   warps 0-3   softmax of tile A: thread r owns row r = TMEM lane r
 //   warps 4-7   softmax of tile B
-//   warp 8      one elected thread issues every tcgen05.mma
-//   warp 9      one elected thread issues the TMA loads of the K and V tiles
+//   warp 8      issues every tcgen05.mma (one elected lane)
+//   warp 9      loads every operand but Q (TMA; row by row where a 16-token group straddles two sources)
 // Window part, per 128-key tile t (keys are tokens j0 + 0..127, j0 a multiple of 16):
-//   loader    K_t and V_t as 16-token boxes (ring rows for tokens older than the call, the call's rows otherwise)
-//             into a ring of five 32 KiB buffers (kStages), 128-byte swizzle, completion on an mbarrier
+//   loader    K_t and V_t (ring rows for tokens older than the call, the call's rows otherwise) into a ring of five
+//             32 KiB buffers (kStages), 128-byte swizzle, completion on an mbarrier
 //   MMA       S_X = Q_X K_t^T into TMEM (8 x m128n128k16), committed to an mbarrier the softmax warps wait on
-//   softmax   tcgen05.ld of the own row, mask, row maximum without any shuffle, P = 2^(s - m_ref) as bf16 into
-//             the swizzled A-operand layout in shared memory; the reference m_ref is lazy: O is rescaled in
-//             TMEM only when the maximum grows by more than 2^8
+//   softmax   tcgen05.ld of the own row, mask, row maximum without any shuffle, P = 2^(s - m_ref) as bf16 over the
+//             consumed S columns; the reference m_ref is lazy: O is rescaled in TMEM only when the maximum grows by
+//             more than 2^8
 //   MMA       O_X += P_X V_t (V as the MN-major B operand), then S_X of the next tile: while one row tile is
 //             in its softmax the tensor core works for the other
 // TMEM columns: S_A [0,128) S_B [128,256) O_A [256,384) O_B [384,512).
-// Linear part (after the window tiles, the whole CTA in step): with a common reference M = max(m_ref, -64) per
-// row, phi(Q) 2^-M as bf16 times a bf16 copy of the state (inter-chunk), and C = phi(Q) phi(K')^T masked to
-// j' <= i, then C V' (intra-chunk), through the same MMAs; l accumulates the matching sums.  out = O / l.
+// Linear part (after the window tiles, by the same warps in the same way): with a common reference M = max(m_ref, -64)
+// per row, phi(Q) 2^-M as bf16 times a bf16 copy of the state (inter-chunk), and C = phi(Q) phi(K')^T masked to
+// j' <= i, then C V' (intra-chunk); l accumulates the matching sums.  out = O / l.
+// What bounds it: short windows, the fixed chain of a CTA (Q and K_0 from memory, one softmax, phi, two to three more
+// products, the store); long windows, the softmax threads' exponentials beside the tensor pipe.
 // Every mbarrier wait is bounded; on a time-out the CTA records kDevWaitTimeout, leaves its loops, frees its TMEM
 // columns and returns.
 #include <cuda.h>
@@ -70,52 +72,54 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
   asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
   return r;
 }
-// shared-memory matrix descriptor, 128-byte swizzle
-__device__ __forceinline__ uint64_t make_desc(uint32_t saddr, uint32_t lbo_bytes, uint32_t sbo_bytes) {
-  uint64_t d = 0;
-  d |= uint64_t((saddr & 0x3FFFF) >> 4);
-  d |= uint64_t((lbo_bytes >> 4) & 0x3FFF) << 16;
-  d |= uint64_t((sbo_bytes >> 4) & 0x3FFF) << 32;
-  d |= uint64_t(1) << 46;
-  d |= uint64_t(2) << 61;
-  return d;
-}
 // instruction descriptor: fp32 accumulate, bf16 A and B, M = N = 128; b_mn: B operand is MN-major
 __device__ __forceinline__ uint32_t make_idesc(bool b_mn) {
   return (1u << 4) | (1u << 7) | (1u << 10) | (b_mn ? (1u << 16) : 0u) | ((128u >> 3) << 17) | ((128u >> 4) << 24);
 }
-__device__ __forceinline__ void mma_f16(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem_d),
-      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-      : "memory");
+// Shared-memory matrix descriptor, 128-byte swizzle, as its two words: address and leading offset in the low one, the rest
+// constant.  The steps of a product differ by constants in the address field (16-byte units; no tile crosses its range).
+__device__ __forceinline__ uint32_t desc_lo(uint32_t saddr, uint32_t lbo_bytes) {
+  return ((saddr & 0x3FFFF) >> 4) | ((lbo_bytes >> 4) << 16);
 }
-// 8 MMAs of one 128 x 128 x 128 product; B K-major (D = A B^T) or MN-major (D (+)= A B)
-__device__ __forceinline__ void issue_mma(uint32_t tmem_d, uint32_t a_tile, uint32_t b_tile, bool b_mn, bool accumulate) {
+constexpr uint32_t kDescHi = (1024u >> 4) | (1u << 14) | (2u << 29);
+// 8 MMAs of one 128 x 128 x 128 product; B K-major (D = A B^T) or MN-major (D (+)= A B).  Called by the MMA warp as a
+// whole, with operands that are the same in all lanes: the instruction takes them from uniform registers, and in code of
+// one diverged lane every step moved them there anew (3400 cycles to issue the 32 MMAs of a key tile, which run in 2048).
+__device__ __forceinline__ void issue_mma(bool leader, uint32_t tmem_d, uint32_t a_tile, uint32_t b_tile, bool b_mn, bool accumulate) {
   const uint32_t idesc = make_idesc(b_mn);
+  const uint32_t a0 = desc_lo(a_tile, 16), b0 = desc_lo(b_tile, b_mn ? kBoxBytes : 16);
+  if (leader) {
 #pragma unroll
-  for (int ks = 0; ks < 8; ++ks) {
-    const uint64_t adesc = make_desc(a_tile + (ks >> 2) * kBoxBytes + (ks & 3) * 32, 16, 1024);
-    const uint64_t bdesc = b_mn ? make_desc(b_tile + ks * 2048, kBoxBytes, 1024)
-                                : make_desc(b_tile + (ks >> 2) * kBoxBytes + (ks & 3) * 32, 16, 1024);
-    mma_f16(tmem_d, adesc, bdesc, idesc, (accumulate || ks > 0) ? 1u : 0u);
+    for (int ks = 0; ks < 8; ++ks) {
+      const uint32_t step = uint32_t(((ks >> 2) * kBoxBytes + (ks & 3) * 32) >> 4);
+      asm volatile(
+          "{\n\t.reg .pred p;\n\t.reg .b64 a, b;\n\tsetp.ne.b32 p, %4, 0;\n\tmov.b64 a, {%1, %5};\n\tmov.b64 b, {%2, %5};\n\t"
+          "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, p;\n\t}" ::"r"(tmem_d),
+          "r"(a0 + step), "r"(b0 + (b_mn ? uint32_t(ks * 2048 >> 4) : step)), "r"(idesc),
+          "r"((accumulate || ks > 0) ? 1u : 0u), "r"(kDescHi)
+          : "memory");
+    }
   }
 }
 // the same product with the A operand in TMEM: lane = row, 32-bit column c = elements 2c (low half) and 2c+1 of
 // the row, 8 columns per k16 step; B MN-major in shared memory
-__device__ __forceinline__ void issue_mma_ts(uint32_t tmem_d, uint32_t tmem_a, uint32_t b_tile, bool accumulate) {
+__device__ __forceinline__ void issue_mma_ts(bool leader, uint32_t tmem_d, uint32_t tmem_a, uint32_t b_tile, bool accumulate) {
   const uint32_t idesc = make_idesc(true);
+  const uint32_t b0 = desc_lo(b_tile, kBoxBytes);
+  if (leader) {
 #pragma unroll
-  for (int ks = 0; ks < 8; ++ks) {
-    const uint64_t bdesc = make_desc(b_tile + ks * 2048, kBoxBytes, 1024);
-    const uint32_t acc = (accumulate || ks > 0) ? 1u : 0u;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}" ::"r"(tmem_d),
-        "r"(tmem_a + ks * 8), "l"(bdesc), "r"(idesc), "r"(acc)
-        : "memory");
+    for (int ks = 0; ks < 8; ++ks)
+      asm volatile(
+          "{\n\t.reg .pred p;\n\t.reg .b64 b;\n\tsetp.ne.b32 p, %4, 0;\n\tmov.b64 b, {%2, %5};\n\t"
+          "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], b, %3, p;\n\t}" ::"r"(tmem_d),
+          "r"(tmem_a + ks * 8), "r"(b0 + uint32_t(ks * 2048 >> 4)), "r"(idesc), "r"((accumulate || ks > 0) ? 1u : 0u), "r"(kDescHi)
+          : "memory");
   }
+}
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
+  return p != 0;
 }
 __device__ __forceinline__ void mma_commit(uint32_t bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
@@ -160,18 +164,7 @@ __device__ __forceinline__ void tma_load_4d(uint32_t dst, const void *tmap, int 
       "l"(tmap), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(bar)
       : "memory");
 }
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-      "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]),
-        "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]),
-        "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]),
-        "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-      : "r"(taddr));
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-}
-// the same load without the wait: the registers are valid only after tmem_wait_ld()
+// 32 columns of this thread's lane; the registers are valid only after tmem_wait_ld(r)
 __device__ __forceinline__ void tmem_ld32_nowait(uint32_t taddr, uint32_t (&r)[32]) {
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
@@ -182,7 +175,20 @@ __device__ __forceinline__ void tmem_ld32_nowait(uint32_t taddr, uint32_t (&r)[3
         "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
       : "r"(taddr));
 }
-__device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+// every load issued so far has landed; r (one of them) is an operand so that no use of it can move above the wait
+__device__ __forceinline__ void tmem_wait_ld(uint32_t (&r)[32]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
+                 "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15]),
+                 "+r"(r[16]), "+r"(r[17]), "+r"(r[18]), "+r"(r[19]), "+r"(r[20]), "+r"(r[21]), "+r"(r[22]), "+r"(r[23]),
+                 "+r"(r[24]), "+r"(r[25]), "+r"(r[26]), "+r"(r[27]), "+r"(r[28]), "+r"(r[29]), "+r"(r[30]), "+r"(r[31])
+               :
+               : "memory");
+}
+__device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
+  tmem_ld32_nowait(taddr, r);
+  tmem_wait_ld(r);
+}
 __device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&r)[32]) {
   asm volatile(
@@ -207,8 +213,9 @@ __device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&r)[16
 }
 
 #ifdef GLIDE_PF_CLOCKS
-// debug builds only: clock cycles per phase of thread 0 of every CTA, summed over the CTAs ([8] phases, [8] = CTAs)
-__device__ unsigned long long g_pf_clk[16];
+// debug builds only: clock cycles per phase of thread 0 of every CTA, summed over the CTAs ([8] = CTAs; [16] .. [20] the waits of
+// the MMA thread and of the loader)
+__device__ unsigned long long g_pf_clk[32];
 #define PF_CLK(i)                                                   \
   do {                                                              \
     if (threadIdx.x == 0) {                                         \
@@ -217,24 +224,33 @@ __device__ unsigned long long g_pf_clk[16];
       pf_t_ = now_;                                                 \
     }                                                               \
   } while (0)
+#define PF_LAP_INIT() long long pf_l_ = clock64()
+#define PF_LAP(i)                                                 \
+  do {                                                            \
+    const long long now_ = clock64();                             \
+    if ((threadIdx.x & 31) == 0) atomicAdd(&g_pf_clk[i], (unsigned long long)(now_ - pf_l_));  \
+    pf_l_ = now_;                                                 \
+  } while (0)
 #else
+#define PF_LAP_INIT() do { } while (0)
+#define PF_LAP(i) do { } while (0)
 #define PF_CLK(i) do { } while (0)
 #endif
 
 struct Smem {
-  unsigned char q[2][kTileBytes];        // Q_A, Q_B; later phi(Q) 2^-m*
-  unsigned char kv[kStages][kTileBytes]; // K and V tiles in turn; linear part: bf16 state, phi(K') tile, V' tile
+  unsigned char q[2][kTileBytes];        // Q_A, Q_B; then phi(Q) 2^-M; then the output rows on their way out
+  unsigned char kv[kStages][kTileBytes]; // K and V tiles in turn; linear part: state, phi(K') and V' tiles
   float z[2 * kD];                       // z of the unit (both halves with the learned map)
-  uint64_t bar_full[kStages];            // TMA bytes of the buffer have landed
+  uint64_t bar_full[kStages];            // the buffer's K or V tile has landed
   uint64_t bar_free[kStages];            // the MMAs that read the buffer have completed
   uint64_t bar_q[2];                     // Q_X staged (128 arrivals)
-  uint64_t bar_s[2];                     // S_X of the current tile is in TMEM
-  uint64_t bar_p[2];                     // P_X of the current tile is in TMEM (128 arrivals)
+  uint64_t bar_s[2];                     // MMA -> softmax threads of X: the products issued for X so far have completed
+  uint64_t bar_p[2];                     // softmax threads of X -> MMA: the A operand of X's next products is ready (128)
   uint64_t bar_done;                     // every window MMA has completed
-  uint64_t bar_lin;                      // linear part: the MMAs issued so far have completed
-  uint64_t bar_state;                    // the bf16 copy of S and z of the unit have landed
+  uint64_t bar_state;                    // the bf16 state and z of the unit have landed (learned map: phi(Q) as well)
   uint64_t bar_pk[2];                    // the phi(K') tile of an intra-chunk step has landed (even / odd steps)
-  uint64_t bar_vp[2];                    // the V' tile of the first / second intra-chunk step has landed (2 arrivals)
+  uint64_t bar_vp[2];                    // the V' tile of an intra-chunk step has landed (even / odd steps; 2 arrivals)
+  uint64_t bar_lfree[2];                 // the MMAs that read an intra-chunk step's buffers have completed
   uint32_t tmem_base;
   int failed;
 };
@@ -246,20 +262,48 @@ struct CallMaps {
   CUtensorMap k128, v128;   // boxes of a whole 128-key tile
 };
 
-template <int G, bool SUM, bool PHI2>
+enum : int { kModeShared = 0, kModeSum = 1, kModeLearned = 2 };
+
+// bit i: column c + i of a key tile is valid for a row whose valid columns are lo .. hi
+__device__ __forceinline__ uint32_t column_mask(int c, int lo, int hi) {
+  const int a = lo - c, b = hi - c;
+  const uint32_t ma = a <= 0 ? ~0u : (a >= 32 ? 0u : ~0u << a);
+  const uint32_t mb = b < 0 ? 0u : (b >= 31 ? ~0u : (2u << b) - 1u);
+  return ma & mb;
+}
+// two fp32 values at once (the packed instructions round like the scalar ones)
+__device__ __forceinline__ void fma2(float &a0, float &a1, float x0, float x1, float s, float c) {
+  asm("{\n\t.reg .b64 x, s, c, d;\n\tmov.b64 x, {%2, %3};\n\tmov.b64 s, {%4, %4};\n\tmov.b64 c, {%5, %5};\n\t"
+      "fma.rn.f32x2 d, x, s, c;\n\tmov.b64 {%0, %1}, d;\n\t}"
+      : "=f"(a0), "=f"(a1)
+      : "f"(x0), "f"(x1), "f"(s), "f"(c));
+}
+__device__ __forceinline__ void add2(float &a0, float &a1, float x0, float x1) {
+  asm("{\n\t.reg .b64 a, x;\n\tmov.b64 a, {%0, %1};\n\tmov.b64 x, {%2, %3};\n\tadd.rn.f32x2 a, a, x;\n\tmov.b64 {%0, %1}, a;\n\t}"
+      : "+f"(a0), "+f"(a1)
+      : "f"(x0), "f"(x1));
+}
+__device__ __forceinline__ void prefetch_map(const void *m) {
+  asm volatile("prefetch.tensormap [%0];" ::"l"(m) : "memory");
+}
+
+template <int G, int MODE>
 __global__ void __launch_bounds__(kThreads, 1)   // 10 warps = 3 on one scheduler: 168 registers per thread at most
 prefill_attn_tc_kernel(const PrefillParams p, const CUtensorMap *ring_maps, const __grid_constant__ CallMaps cm) {
   using bf16 = __nv_bfloat16;
+  constexpr bool SUM = MODE == kModeSum;          // sum of two normalised terms instead of the shared normaliser
+  constexpr bool PHI2 = MODE == kModeLearned;
   constexpr int TOKT = kRows / G;    // tokens per row tile
   constexpr int TOKC = 2 * TOKT;     // tokens per CTA
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   Smem &sm = *reinterpret_cast<Smem *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  // CTAs of a unit: those of its full chunks, then those of the last one; from here on "the chunk" is the CTA's own
+  // CTAs of a unit: those of its full chunks, then those of the last one, the last tokens first (their windows are the
+  // longest of a new prompt); from here on "the chunk" is the CTA's own
   const int ctas_per_chunk = (p.SC + TOKC - 1) / TOKC;
   const int ctas_per_unit = (p.nsub - 1) * ctas_per_chunk + (p.C - (p.nsub - 1) * p.SC + TOKC - 1) / TOKC;
   const int64_t u = blockIdx.x / ctas_per_unit;
-  const int cta_u = int(blockIdx.x % ctas_per_unit);
+  const int cta_u = ctas_per_unit - 1 - int(blockIdx.x % ctas_per_unit);
   const int sub = cta_u / ctas_per_chunk;
   const int tok0 = (cta_u - sub * ctas_per_chunk) * TOKC;
   const int chunk_c0 = int(p.c0) + sub * p.SC;                // first token of the chunk, relative to the call
@@ -277,7 +321,6 @@ prefill_attn_tc_kernel(const PrefillParams p, const CUtensorMap *ring_maps, cons
   const int64_t tq_last = tq0 + ntok - 1;
   const int64_t w = ld.w;
   const int64_t wl = ld.wlin;                      // delay of the linear stream: w, or 0 when the state holds every token
-  constexpr bool sum_terms = SUM;                  // sum of two normalised terms instead of the shared normaliser
   const uint32_t cap = ld.cap > 0 ? uint32_t(ld.cap) : 1u;
   const size_t unit_rows = (size_t(b + p.b0) * p.Hkv + g) * size_t(ld.cap);   // b + b0: the sequence's slot in the context
   const size_t seq = (size_t(lrel) * p.B + b) * size_t(p.T);
@@ -290,13 +333,18 @@ prefill_attn_tc_kernel(const PrefillParams p, const CUtensorMap *ring_maps, cons
   // a time-out recorded by an earlier CTA ends the launch quickly
   if (*reinterpret_cast<volatile int32_t *>(&p.ctl->status) == kDevWaitTimeout) return;
 
-  const bool has_window = w > 0;
   int64_t j_lo = tq0 - w + 1;
   if (j_lo < 0) j_lo = 0;
   j_lo &= ~int64_t(kGroup - 1);   // key tiles start at a multiple of the TMA box
-  const int n_tiles = has_window ? int((tq_last - j_lo) / kKT) + 1 : 0;
+  const int n_tiles = w > 0 ? int((tq_last - j_lo) / kKT) + 1 : 0;
+  // key tiles that row tile X has valid keys in: [t_first(X), t_end(X)) (A may end, B begin one tile off the CTA's range)
+  auto t_first = [&](int x) {
+    const int64_t lo = tq0 + x * TOKT - w + 1;
+    return lo <= j_lo ? 0 : int((lo - j_lo) / kKT);
+  };
+  auto t_end = [&](int x) { return n_tiles == 0 ? 0 : int((tq0 + x * TOKT + (x ? ntokB : ntokA) - 1 - j_lo) / kKT) + 1; };
 
-  if (tid == 0) {
+  if (tid == kSoftmaxThreads) {
     for (int s = 0; s < kStages; ++s) {
       mbar_init(smem_u32(&sm.bar_full[s]), 2);
       mbar_init(smem_u32(&sm.bar_free[s]), 1);
@@ -305,20 +353,24 @@ prefill_attn_tc_kernel(const PrefillParams p, const CUtensorMap *ring_maps, cons
       mbar_init(smem_u32(&sm.bar_q[x]), kRows);
       mbar_init(smem_u32(&sm.bar_s[x]), 1);
       mbar_init(smem_u32(&sm.bar_p[x]), kRows);
+      mbar_init(smem_u32(&sm.bar_pk[x]), 1);
+      mbar_init(smem_u32(&sm.bar_vp[x]), 2);
+      mbar_init(smem_u32(&sm.bar_lfree[x]), 1);
     }
     mbar_init(smem_u32(&sm.bar_done), 1);
-    mbar_init(smem_u32(&sm.bar_lin), 1);
     mbar_init(smem_u32(&sm.bar_state), 1);
-    mbar_init(smem_u32(&sm.bar_pk[0]), 1);
-    mbar_init(smem_u32(&sm.bar_pk[1]), 1);
-    mbar_init(smem_u32(&sm.bar_vp[0]), 2);
-    mbar_init(smem_u32(&sm.bar_vp[1]), 2);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     sm.failed = 0;
   }
-  if (warp == 0) {
+  if (warp == kLoadWarp) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(smem_u32(&sm.tmem_base)) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    if (lane == 0) {
+      prefetch_map(&cm.k128);
+      prefetch_map(&cm.v128);
+      prefetch_map(&cm.k);
+      prefetch_map(&cm.v);
+    }
   }
   // Token groups past the CTA's last token are never loaded (only the last tile has such groups), and what a
   // masked key's V row holds is multiplied by a zero weight, so it has to be finite: those rows of the buffer that
@@ -334,23 +386,24 @@ prefill_attn_tc_kernel(const PrefillParams p, const CUtensorMap *ring_maps, cons
     }
   }
   // Q_X: 128 rows x 16 chunks by the 128 threads of each row tile, asked for before the set-up's barrier so that the copy
-  // runs while the other warps finish setting up (it needs nothing of that; nothing else writes these tiles).
-  {
-    const int Xq = (tid >> 7) & 1, rq = tid & 127;
-    const int ntokXq = Xq ? ntokB : ntokA;
-    if (tid < kSoftmaxThreads && ntokXq > 0) {
-      const bf16 *qbase = reinterpret_cast<const bf16 *>(p.q) + (seq + size_t(chunk_c0 + tok0 + Xq * TOKT)) * p.H * kD;
-      const uint32_t sQx = smem_u32(sm.q[Xq]);
+  // runs while the other warps finish setting up (it needs nothing of that; nothing else writes these tiles).  A thread's
+  // rows are 8 apart, so all of them belong to one head of the group (G divides 8).
+  const int X = (tid >> 7) & 1;                   // row tile of this thread (softmax warps only)
+  const int row = tid & 127;
+  const int ntokX = X ? ntokB : ntokA;
+  const bool activeX = tid < kSoftmaxThreads && ntokX > 0;
+  if (activeX) {
+    const int c = row & 15, r0 = row >> 4, h2 = r0 % G;
+    const bf16 *src = reinterpret_cast<const bf16 *>(p.q) +
+                      ((seq + size_t(chunk_c0 + tok0 + X * TOKT)) * p.H + p.heads_of[g * G + h2]) * kD + c * 8;
+    const uint32_t dst = smem_u32(sm.q[X]) + sw128(r0, c);   // (r & 7 is the same for all rows of the thread)
 #pragma unroll 4
-      for (int i = 0; i < kRows * 16 / kRows; ++i) {
-        const int id = rq + kRows * i;
-        const int r = id >> 4, c = id & 15;
-        const int tk = r / G, h2 = r - tk * G;
-        const bool valid = tk < ntokXq;
-        cp_async16(sQx + sw128(r, c), qbase + (size_t(valid ? tk : 0) * p.H + p.heads_of[g * G + h2]) * kD + c * 8, valid);
-      }
-      cp_async_commit();
+    for (int i = 0; i < 16; ++i) {
+      const int tk = (r0 + 8 * i) / G;
+      const bool valid = tk < ntokX;
+      cp_async16(dst + uint32_t(i) * 8u * 128u, src + (valid ? size_t(tk) * p.H * kD : 0), valid);
     }
+    cp_async_commit();
   }
   fence_async_smem();
   tc_fence_before();
@@ -358,8 +411,9 @@ prefill_attn_tc_kernel(const PrefillParams p, const CUtensorMap *ring_maps, cons
   tc_fence_after();
   const uint32_t tmem = sm.tmem_base;
   PF_CLK(0);
-  const uint32_t sQ[2] = {smem_u32(sm.q[0]), smem_u32(sm.q[1])};
+  const uint32_t sQ0 = smem_u32(sm.q[0]);
   const uint32_t sKV0 = smem_u32(sm.kv[0]);
+  auto q_addr = [&](int x) { return sQ0 + uint32_t(x) * kTileBytes; };
   auto kv_addr = [&](int slot) { return sKV0 + uint32_t(slot) * kTileBytes; };
   // Linear part: what it needs is known now, so that the loader can fetch it behind the last key tiles.
   const bool linear = ld.evicts && tq_last >= wl;
@@ -369,176 +423,443 @@ prefill_attn_tc_kernel(const PrefillParams p, const CUtensorMap *ring_maps, cons
   const int i_lo = folded < 0 ? int(-folded < int64_t(chunk_n) ? -folded : int64_t(chunk_n)) : 0;
   const int i_hi = tok0 + ntok - 1;
   const int it0 = i_lo & ~(kKT - 1);
-  const int n_itiles = (linear && it0 <= i_hi) ? (i_hi - it0) / kKT + 1 : 0;
+  const int n_itiles = (linear && it0 <= i_hi) ? (i_hi - it0) / kKT + 1 : 0;   // (linear without a state: at least one)
   // Roles of the five buffers after the window loop, by the order in which the loop stops using them (load number
   // 2 n_tiles - 5 + k; a negative number is a buffer the loop never used): the first to come free receives the bf16
-  // copy of the unit's state, the next two the phi(K') tiles of the first two intra-chunk steps (all three by TMA
-  // while the last key tiles are still being processed), the last two the V' tiles of those steps.  Later steps
-  // take the buffers of the step before the previous one.
+  // copy of the unit's state, the next two the phi(K') tiles of the first two intra-chunk steps, the last two the V'
+  // tiles of those steps; all are on their way while the last key tiles are still being processed.  Later steps take the
+  // buffers of the step before the previous one.
+  // Learned map: twice the operands, so they come when every window product has completed: phi- of the two row tiles in
+  // buffers 0 and 1 (phi+ in the Q tiles), the state halves and then the phi(K') halves of each step in 2 and 3, V' in 4.
   auto late_seq = [&](int k) { return 2 * n_tiles - kStages + k; };
   auto late_slot = [&](int k) { const int sq = late_seq(k); return sq >= 0 ? sq % kStages : sq + kStages; };
-  const int slotSb = late_slot(0);
-  const int slotPk[2] = {late_slot(1), late_slot(2)}, slotVp[2] = {late_slot(3), late_slot(4)};
-  const CUtensorMap *map_pk = ring_maps + 5 * p.L, *map_s16 = map_pk + 1;
-  auto load_pk = [&](int t) {   // one thread: the phi(K') rows of intra-chunk step t
-    const uint32_t bar = smem_u32(&sm.bar_pk[t & 1]);
-    const uint32_t dst = kv_addr(slotPk[t & 1]);
-    const int y = int(uc * p.SC) + it0 + t * kKT;
-    mbar_expect_tx(bar, kTileBytes);
-    tma_load_2d(dst, map_pk, 0, y, bar);
-    tma_load_2d(dst + kBoxBytes, map_pk, 64, y, bar);
-  };
+  auto slot_state = [&]() { return PHI2 ? 2 : late_slot(0); };
+  auto slot_pk = [&](int t) { return PHI2 ? 2 : late_slot(1 + (t & 1)); };
+  auto slot_vp = [&](int t) { return PHI2 ? 4 : late_slot(3 + (t & 1)); };
 
-  // ---- softmax threads: per-row state that lives across the window and the linear part ----------------------
-  const int X = (tid >> 7) & 1;                   // row tile of this thread (softmax warps only)
-  const int row = tid & 127;
-  const int tok_r = row / G, hh = row - tok_r * G;
-  const int ntokX = X ? ntokB : ntokA;
-  const bool activeX = tid < kSoftmaxThreads && ntokX > 0;
-  const int tl = tok0 + X * TOKT + tok_r;         // chunk-relative token of this row
-  const int64_t tok_abs = p.n0 + chunk_c0 + tl;
-  const uint32_t tS = tmem + (uint32_t((warp & 3) * 32) << 16) + uint32_t(X) * 128u;
-  const uint32_t tO = tS + 256u;
-  float m_ref = -CUDART_INF_F, l_sum = 0.f;
-
-  // multiply this thread's O row by f (warp-collective TMEM read-modify-write)
-  auto scale_o = [&](float f) {
-#pragma unroll 1
-    for (int c0 = 0; c0 < kD; c0 += 32) {
-      uint32_t r[32];
-      tmem_ld32(tO + c0, r);
-#pragma unroll
-      for (int i = 0; i < 32; ++i) r[i] = __float_as_uint(__uint_as_float(r[i]) * f);
-      tmem_st32(tO + c0, r);
-    }
-  };
-  // weights of one S row against reference mr (log2 domain) -> bf16 P row in the swizzled A layout; returns their sum
-  auto write_p = [&](auto masked, int lo, int hi, float mr, float scale) -> float {
-    constexpr bool kMasked = decltype(masked)::value;
-    float sum0 = 0.f, sum1 = 0.f;
-    uint32_t ra[32], rb[32];
-    tmem_ld32_nowait(tS, ra);
-#pragma unroll
-    for (int c0 = 0; c0 < kKT; c0 += 32) {
-      uint32_t (&r)[32] = ((c0 >> 5) & 1) ? rb : ra;
-      uint32_t pk[16];
-      tmem_wait_ld();
-      // the next 32 columns are on their way while these are turned into weights; the store below touches
-      // columns [c0/2, c0/2+16), which lie below c0+32 only when they have been read already
-      if (c0 + 32 < kKT) tmem_ld32_nowait(tS + c0 + 32, ((c0 >> 5) & 1) ? ra : rb);
-#pragma unroll
-      for (int e = 0; e < 16; ++e) {
-        const int i = e * 2;
-        float a0 = ex2(fmaf(__uint_as_float(r[i]), scale, -mr));
-        float a1 = ex2(fmaf(__uint_as_float(r[i + 1]), scale, -mr));
-        if (kMasked) {
-          if (c0 + i < lo || c0 + i > hi) a0 = 0.f;
-          if (c0 + i + 1 < lo || c0 + i + 1 > hi) a1 = 0.f;
-        }
-        pk[e] = pack_bf16x2(a0, a1);
-        sum0 += __uint_as_float(pk[e] << 16);          // the sum uses the weights as the tensor core sees them
-        sum1 += __uint_as_float(pk[e] & 0xffff0000u);
-      }
-      // P overwrites the S columns this thread has already consumed: keys c0..c0+31 -> columns c0/2..c0/2+15
-      tmem_st16(tS + (c0 >> 1), pk);
-    }
-    tmem_wait_st();
-    return sum0 + sum1;
-  };
-  // =========================== window part: warp-specialised ===========================
   if (tid < kSoftmaxThreads) {
+    // =========================== softmax threads: one row each ===========================
+    // Every hand-over of row tile X is its own: the threads of A and of B meet only at the end of the CTA, so that one
+    // tile's arithmetic runs beside the other's products.  bar_s completes once per batch of products of X, bar_p once
+    // per operand that X's threads have written; both sides count in the same order.
+    const int tok_r = row / G;
+    const int tl = tok0 + X * TOKT + tok_r;         // chunk-relative token of this row
+    const int64_t tok_abs = p.n0 + chunk_c0 + tl;
+    const uint32_t tS = tmem + (uint32_t((warp & 3) * 32) << 16) + uint32_t(X) * 128u;
+    const uint32_t tO = tS + 256u;
+    float m_ref = -CUDART_INF_F, l_sum = 0.f;
+    uint32_t n_s = 0;                               // batches of products waited for
+    auto wait_s = [&]() {
+      const bool got = mbar_wait(smem_u32(&sm.bar_s[X]), n_s & 1u, failed);
+      ++n_s;
+      tc_fence_after();
+      return bool(__all_sync(0xffffffffu, got));    // warp-uniform: the TMEM accesses need every lane
+    };
+    // multiply this thread's O row by f (warp-collective TMEM read-modify-write)
+    auto scale_o = [&](float f) {
+#pragma unroll 1
+      for (int c0 = 0; c0 < kD; c0 += 32) {
+        uint32_t r[32];
+        tmem_ld32(tO + c0, r);
+#pragma unroll
+        for (int i = 0; i < 32; ++i) r[i] = __float_as_uint(__uint_as_float(r[i]) * f);
+        tmem_st32(tO + c0, r);
+      }
+    };
+    // One key tile: maximum, reference, weights.  Tiles without a masked key keep their loops unrolled; the others, one or
+    // two per row tile, keep them rolled: with everything unrolled the kernel was 210 KB of code that a CTA fetched once
+    // per phase (a CTA's first key tile took 12000 cycles, a later one 2500).
+    auto soft_tile = [&](auto masked, int lo, int hi, bool first) {
+      constexpr bool kMasked = decltype(masked)::value != 0;
+      constexpr int kUnroll = kMasked ? 1 : 2;
+      // pass 1: row maximum of the valid raw scores (the scale is positive: it is applied to the maximum)
+      float mx = -CUDART_INF_F;
+      uint32_t r[2][32];
+      tmem_ld32_nowait(tS, r[0]);
+#pragma unroll kUnroll
+      for (int c0 = 0; c0 < kKT; c0 += 64) {
+#pragma unroll
+        for (int hf = 0; hf < 2; ++hf) {
+          uint32_t (&x)[32] = r[hf];
+          const int c = c0 + hf * 32;
+          tmem_wait_ld(x);
+          if (hf == 0) tmem_ld32_nowait(tS + c + 32, r[1]);
+          else tmem_ld32_nowait(tS + ((c + 32) & (kKT - 1)), r[0]);   // (after the last columns: the first of pass 2)
+          if (kMasked) {
+            const uint32_t m = column_mask(c, lo, hi);
+#pragma unroll
+            for (int i = 0; i < 32; ++i) x[i] = (m >> i) & 1u ? x[i] : 0xff800000u;
+          }
+          float m4[4] = {mx, -CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F};
+#pragma unroll
+          for (int i = 0; i < 32; ++i) m4[i & 3] = fmaxf(m4[i & 3], __uint_as_float(x[i]));
+          mx = fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3]));
+        }
+      }
+      mx *= p.scale_log2;
+      // lazy reference: move it (and rescale O, l) only when the maximum grows by more than 2^kLazy
+      float f = 1.f;
+      if (mx > m_ref + kLazy || (m_ref == -CUDART_INF_F && mx > -CUDART_INF_F)) {
+        f = m_ref == -CUDART_INF_F ? 0.f : ex2(m_ref - mx);
+        m_ref = mx;
+      }
+      tmem_wait_ld(r[0]);
+      if (!first && __any_sync(0xffffffffu, f != 1.f)) scale_o(f);
+      l_sum *= f;
+      const float mr = m_ref == -CUDART_INF_F ? 0.f : m_ref;
+      // pass 2: weights against the reference -> bf16, over the S columns this thread has already consumed (keys
+      // c .. c + 31 -> columns c / 2 .. c / 2 + 15); the sum uses the weights as the tensor core sees them
+      float sum0 = 0.f, sum1 = 0.f;
+#pragma unroll kUnroll
+      for (int c0 = 0; c0 < kKT; c0 += 64) {
+#pragma unroll
+        for (int hf = 0; hf < 2; ++hf) {
+          uint32_t (&x)[32] = r[hf];
+          const int c = c0 + hf * 32;
+          uint32_t pk[16];
+          tmem_wait_ld(x);
+          // the next 32 columns are on their way while these are turned into weights
+          if (hf == 0) tmem_ld32_nowait(tS + c + 32, r[1]);
+          else if (c + 32 < kKT) tmem_ld32_nowait(tS + c + 32, r[0]);
+          if (kMasked) {
+            const uint32_t m = column_mask(c, lo, hi);
+#pragma unroll
+            for (int i = 0; i < 32; ++i) x[i] = (m >> i) & 1u ? x[i] : 0xff800000u;
+          }
+#pragma unroll
+          for (int e = 0; e < 16; ++e) {
+            float a0, a1;
+            fma2(a0, a1, __uint_as_float(x[e * 2]), __uint_as_float(x[e * 2 + 1]), p.scale_log2, -mr);
+            pk[e] = pack_bf16x2(ex2(a0), ex2(a1));
+            add2(sum0, sum1, __uint_as_float(pk[e] << 16), __uint_as_float(pk[e] & 0xffff0000u));
+          }
+          tmem_st16(tS + (c >> 1), pk);
+        }
+      }
+      tmem_wait_st();
+      l_sum += sum0 + sum1;
+    };
     if (activeX) {
       cp_async_wait_all();   // Q_X (asked for before the set-up's barrier) has landed
       fence_async_smem();
       mbar_arrive(smem_u32(&sm.bar_q[X]));
-
       const int64_t tqX0 = tq0 + X * TOKT, tqX_last = tqX0 + ntokX - 1;
-      bool o_written = false;   // a P V product has been accumulated into O_X (uniform over the row tile)
-      for (int t = 0; t < n_tiles; ++t) {
-        const bool got = mbar_wait(smem_u32(&sm.bar_s[X]), uint32_t(t) & 1u, failed);
-        if (!__all_sync(0xffffffffu, got)) break;   // warp-uniform: the collectives below need every lane
-        tc_fence_after();
+      const int tf = t_first(X), te = t_end(X);
+      bool ok = true;
+      for (int t = tf; t < te; ++t) {
+        ok = wait_s();
+        if (!ok) break;
+        if (t == tf) PF_CLK(11); else PF_CLK(12);
         const int64_t j0 = j_lo + int64_t(t) * kKT;
-        const bool interior = j0 + kKT - 1 <= tqX0 && j0 > tqX_last - w;
-        // valid columns of this row: lo <= c <= hi
-        int64_t lo64 = tok_abs - w + 1 - j0, hi64 = tok_abs - j0;
-        const int lo = int(lo64 < 0 ? 0 : (lo64 > kKT ? kKT : lo64));
-        const int hi = int(hi64 < -1 ? -1 : (hi64 > kKT - 1 ? kKT - 1 : hi64));
-        // pass 1: row maximum of the valid raw scores (the scale is positive: it is applied to the maximum)
-        float mx = -CUDART_INF_F;
-#pragma unroll 1
-        for (int c0 = 0; c0 < kKT; c0 += 32) {
-          uint32_t r[32];
-          tmem_ld32(tS + c0, r);
-          float m4[4] = {-CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F};
-          if (interior) {
-#pragma unroll
-            for (int i = 0; i < 32; ++i) m4[i & 3] = fmaxf(m4[i & 3], __uint_as_float(r[i]));
-          } else {
-#pragma unroll
-            for (int i = 0; i < 32; ++i)
-              if (c0 + i >= lo && c0 + i <= hi) m4[i & 3] = fmaxf(m4[i & 3], __uint_as_float(r[i]));
-          }
-          mx = fmaxf(mx, fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3])));
+        if (j0 + kKT - 1 <= tqX0 && j0 > tqX_last - w) {
+          soft_tile(IntTag<0>{}, 0, kKT - 1, t == tf);
+        } else {
+          // valid columns of this row: lo <= c <= hi
+          const int64_t lo64 = tok_abs - w + 1 - j0, hi64 = tok_abs - j0;
+          soft_tile(IntTag<1>{}, int(lo64 < 0 ? 0 : (lo64 > kKT ? kKT : lo64)),
+                    int(hi64 < -1 ? -1 : (hi64 > kKT - 1 ? kKT - 1 : hi64)), t == tf);
         }
-        mx *= p.scale_log2;
-        // lazy reference: move it (and rescale O, l) only when the maximum grows by more than 2^kLazy
-        float f = 1.f;
-        if (mx > m_ref + kLazy || (m_ref == -CUDART_INF_F && mx > -CUDART_INF_F)) {
-          f = m_ref == -CUDART_INF_F ? 0.f : ex2(m_ref - mx);
-          m_ref = mx;
-        }
-        if (o_written && __any_sync(0xffffffffu, f != 1.f)) scale_o(f);
-        l_sum *= f;
-        const float mr = m_ref == -CUDART_INF_F ? 0.f : m_ref;
-        if (interior) l_sum += write_p(IntTag<0>{}, lo, hi, mr, p.scale_log2);
-        else l_sum += write_p(IntTag<1>{}, lo, hi, mr, p.scale_log2);
         tc_fence_before();      // this thread's TMEM accesses precede the MMAs that read P and overwrite S
         mbar_arrive(smem_u32(&sm.bar_p[X]));
-        o_written = true;
+        if (t == tf) PF_CLK(13); else PF_CLK(14);
       }
-    }
-    if (n_tiles > 0) mbar_wait(smem_u32(&sm.bar_done), 0u, failed);
-    tc_fence_after();
-  } else if (warp == kMmaWarp) {
-    if (lane == 0 && n_tiles > 0) {
-      bool ok = mbar_wait(smem_u32(&sm.bar_q[0]), 0u, failed);
-      if (ok && hasB) ok = mbar_wait(smem_u32(&sm.bar_q[1]), 0u, failed);
-      if (ok) ok = mbar_wait(smem_u32(&sm.bar_full[0]), 0u, failed);   // K_0
-      if (ok) {
-        tc_fence_after();
-        issue_mma(tmem, sQ[0], kv_addr(0), false, false);
-        mma_commit(smem_u32(&sm.bar_s[0]));
-        if (hasB) {
-          issue_mma(tmem + 128, sQ[1], kv_addr(0), false, false);
-          mma_commit(smem_u32(&sm.bar_s[1]));
-        }
-        mma_commit(smem_u32(&sm.bar_free[0]));
-      }
-      for (int t = 0; t < n_tiles && ok; ++t) {
-        const int seqV = 2 * t + 1, seqK = 2 * t + 2;
-        const bool more = t + 1 < n_tiles;
-        ok = mbar_wait(smem_u32(&sm.bar_full[seqV % kStages]), uint32_t(seqV / kStages) & 1u, failed);
-        if (ok && more) ok = mbar_wait(smem_u32(&sm.bar_full[seqK % kStages]), uint32_t(seqK / kStages) & 1u, failed);
-        for (int x = 0; x < 2 && ok; ++x) {
-          if (x == 1 && !hasB) break;
-          ok = mbar_wait(smem_u32(&sm.bar_p[x]), uint32_t(t) & 1u, failed);
-          if (!ok) break;
-          tc_fence_after();
-          issue_mma_ts(tmem + 256 + x * 128, tmem + x * 128, kv_addr(seqV % kStages), t > 0);
-          if (more) {
-            issue_mma(tmem + x * 128, sQ[x], kv_addr(seqK % kStages), false, false);
-            mma_commit(smem_u32(&sm.bar_s[x]));
+      const bool windowed = te > tf;               // O_X holds a valid accumulation
+      if (linear) {
+        if (!windowed) mbar_wait(smem_u32(&sm.bar_q[X]), 0u, failed);   // (a window product implies it)
+        // Any common reference M >= m_ref gives the same quotient O / l.  M = max(m_ref, 0) would rescale O for every
+        // row whose window maximum is negative; a floor of -64 keeps 2^-M and everything scaled by it far inside the
+        // fp32 / bf16 range (phi <= 1) and makes that rescale a rarity.
+        // A row without evicted tokens (position below the window size) keeps its own reference and gets phi(q) = 0:
+        // a floor there would only push its window weights towards underflow.
+        // Sum of two normalised terms instead: the window part is normalised now (O / l), and phi(q) is divided by the
+        // row's linear normaliser phi(q) . (z + running sum of phi(K') up to the row's own delayed token), so that what
+        // the linear products add to O is the normalised linear term; the final division is by 1.
+        const bool has_lin = tok_abs >= wl;
+        const float M = has_lin ? fmaxf(m_ref, -64.f) : m_ref;
+        float fw = m_ref == -CUDART_INF_F ? 0.f : ex2(m_ref - M);
+        const float fl = has_lin ? ex2(-M) : 0.f;
+        if (SUM) fw = l_sum > 0.f ? 1.0f / l_sum : 0.f;
+        l_sum = SUM ? 1.f : l_sum * fw;
+        if (PHI2 || (SUM && need_state)) mbar_wait(smem_u32(&sm.bar_state), 0u, failed);   // phi(Q); z
+        unsigned char *tileX = sm.q[X];
+        float dot = 0.f;
+        if constexpr (!PHI2) {
+          // this row of Q is still in the shared tile, and every S product of X has completed: phi(q) takes its place,
+          // eight values at a time: maximum, then exponentials (left as bf16) and their sum, then the scaled values
+          float mx = -CUDART_INF_F;
+#pragma unroll 4
+          for (int c = 0; c < 16; ++c) {
+            const uint4 v4 = *reinterpret_cast<const uint4 *>(tileX + sw128(row, c));
+            const uint32_t w4[4] = {v4.x, v4.y, v4.z, v4.w};
+#pragma unroll
+            for (int e = 0; e < 4; ++e) mx = fmaxf(mx, fmaxf(__uint_as_float(w4[e] << 16), __uint_as_float(w4[e] & 0xffff0000u)));
+          }
+          float sum0 = 0.f, sum1 = 0.f, dz0 = 0.f, dz1 = 0.f;
+          const float mxl = mx * kLog2e;
+          const float2 *zrow = reinterpret_cast<const float2 *>(p.zcum + (size_t(uc) * p.SC + size_t(tok_r < ntokX ? tl : tok0)) * kD);
+#pragma unroll 4
+          for (int c = 0; c < 16; ++c) {
+            uint4 *at = reinterpret_cast<uint4 *>(tileX + sw128(row, c));
+            const uint4 v4 = *at;
+            uint32_t w4[4] = {v4.x, v4.y, v4.z, v4.w};
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+              float a0, a1;
+              fma2(a0, a1, __uint_as_float(w4[e] << 16), __uint_as_float(w4[e] & 0xffff0000u), kLog2e, -mxl);
+              const float e0 = ex2(a0), e1 = ex2(a1);
+              add2(sum0, sum1, e0, e1);
+              if (SUM) {
+                const float2 zc = __ldg(zrow + c * 4 + e);
+                dz0 = fmaf(e0, zc.x + (need_state ? sm.z[c * 8 + e * 2] : 0.f), dz0);
+                dz1 = fmaf(e1, zc.y + (need_state ? sm.z[c * 8 + e * 2 + 1] : 0.f), dz1);
+              }
+              w4[e] = pack_bf16x2(e0, e1);
+            }
+            *at = make_uint4(w4[0], w4[1], w4[2], w4[3]);
+          }
+          // shared normaliser: phi(q) 2^-M;  sum of terms: phi(q) / (phi(q) . z_row) = e / (e . z_row)
+          const float dz = dz0 + dz1;
+          const float sc = SUM ? ((has_lin && dz > 0.f) ? 1.0f / dz : 0.f) : fl * __frcp_rn(sum0 + sum1);
+          const bool with_z = !SUM && need_state;
+          if (with_z) mbar_wait(smem_u32(&sm.bar_state), 0u, failed);   // z has landed
+          float dot1 = 0.f;
+#pragma unroll 4
+          for (int c = 0; c < 16; ++c) {
+            uint4 *at = reinterpret_cast<uint4 *>(tileX + sw128(row, c));
+            const uint4 v4 = *at;
+            uint32_t w4[4] = {v4.x, v4.y, v4.z, v4.w};
+#pragma unroll
+            for (int e = 0; e < 4; ++e) w4[e] = pack_bf16x2(__uint_as_float(w4[e] << 16) * sc, __uint_as_float(w4[e] & 0xffff0000u) * sc);
+            *at = make_uint4(w4[0], w4[1], w4[2], w4[3]);
+            if (with_z) {
+#pragma unroll
+              for (int e = 0; e < 4; ++e) {
+                const float2 zz = *reinterpret_cast<const float2 *>(&sm.z[c * 8 + e * 2]);
+                dot = fmaf(__uint_as_float(w4[e] << 16), zz.x, dot);
+                dot1 = fmaf(__uint_as_float(w4[e] & 0xffff0000u), zz.y, dot1);
+              }
+            }
+          }
+          dot += dot1;
+        } else {
+          // this thread's row of phi+ and of phi-: times 2^-M, back as bf16; the dot with z uses the rounded values
+#pragma unroll 1
+          for (int hf = 0; hf < 2; ++hf) {
+            unsigned char *tile = hf == 0 ? tileX : sm.kv[X];
+#pragma unroll 4
+            for (int c = 0; c < 16; ++c) {
+              uint4 *at = reinterpret_cast<uint4 *>(tile + sw128(row, c));
+              const uint4 v4 = *at;
+              uint32_t w4[4] = {v4.x, v4.y, v4.z, v4.w};
+#pragma unroll
+              for (int e = 0; e < 4; ++e) {
+                w4[e] = pack_bf16x2(__uint_as_float(w4[e] << 16) * fl, __uint_as_float(w4[e] & 0xffff0000u) * fl);
+                if (need_state)
+                  dot += __uint_as_float(w4[e] << 16) * sm.z[hf * kD + c * 8 + e * 2] +
+                         __uint_as_float(w4[e] & 0xffff0000u) * sm.z[hf * kD + c * 8 + e * 2 + 1];
+              }
+              *at = make_uint4(w4[0], w4[1], w4[2], w4[3]);
+            }
           }
         }
-        if (ok) {
-          mma_commit(smem_u32(&sm.bar_free[seqV % kStages]));
-          if (more) mma_commit(smem_u32(&sm.bar_free[seqK % kStages]));
+        l_sum += dot;
+        if (windowed) {
+          ok = wait_s() && ok;                     // the last P V has completed
+          if (ok && __any_sync(0xffffffffu, fw != 1.f)) scale_o(fw);
+        }
+        fence_async_smem();
+        tc_fence_before();
+        mbar_arrive(smem_u32(&sm.bar_p[X]));
+        PF_CLK(10);
+        // C row -> bf16 over the same TMEM columns, masked to the delayed tokens j' <= i of the row (the values already
+        // carry 2^-M); the row's weight sum goes to l
+        for (int t = 0; t < n_itiles && ok; ++t) {
+          ok = wait_s();
+          if (!ok) break;
+          PF_CLK(3);
+          const int i0 = it0 + t * kKT;
+          float sum0 = 0.f, sum1 = 0.f;
+          const int lo = i_lo - i0, hi = tl - i0;
+          // a tile that lies wholly before the row tile's first token (and after the first delayed token) needs no mask
+          const bool whole = i0 + kKT - 1 <= tok0 + X * TOKT && i0 >= i_lo;
+          uint32_t r[2][32];
+          tmem_ld32_nowait(tS, r[0]);
+#pragma unroll 1
+          for (int c0 = 0; c0 < kKT; c0 += 64) {
+#pragma unroll
+            for (int hf = 0; hf < 2; ++hf) {
+              uint32_t (&x)[32] = r[hf];
+              const int c = c0 + hf * 32;
+              uint32_t pk[16];
+              tmem_wait_ld(x);
+              if (hf == 0) tmem_ld32_nowait(tS + c + 32, r[1]);
+              else if (c + 32 < kKT) tmem_ld32_nowait(tS + c + 32, r[0]);
+              if (!whole) {
+                const uint32_t m = column_mask(c, lo, hi);
+#pragma unroll
+                for (int i = 0; i < 32; ++i) x[i] = (m >> i) & 1u ? x[i] : 0u;
+              }
+#pragma unroll
+              for (int e = 0; e < 16; ++e) {
+                pk[e] = pack_bf16x2(__uint_as_float(x[e * 2]), __uint_as_float(x[e * 2 + 1]));
+                add2(sum0, sum1, __uint_as_float(pk[e] << 16), __uint_as_float(pk[e] & 0xffff0000u));
+              }
+              tmem_st16(tS + (c >> 1), pk);
+            }
+          }
+          tmem_wait_st();
+          if (!SUM) l_sum += sum0 + sum1;
+          tc_fence_before();
+          mbar_arrive(smem_u32(&sm.bar_p[X]));
+          PF_CLK(4);
         }
       }
-      if (ok) mma_commit(smem_u32(&sm.bar_done));
+      // ---- normalise and store: through the Q tile (every product that read it has completed), so that a warp's stores
+      // are whole rows ----
+      if (ok && (windowed || linear)) ok = wait_s();   // every product of X has completed
+      PF_CLK(5);
+      if (ok && (windowed || linear)) {
+        const float inv = tok_r < ntokX ? 1.0f / l_sum : 0.f;
+#pragma unroll 1
+        for (int c0 = 0; c0 < kD; c0 += 32) {
+          uint32_t r[32];
+          tmem_ld32(tO + c0, r);
+#pragma unroll
+          for (int q4 = 0; q4 < 4; ++q4) {
+            uint32_t pk[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+              pk[e] = pack_bf16x2(__uint_as_float(r[q4 * 8 + e * 2]) * inv, __uint_as_float(r[q4 * 8 + e * 2 + 1]) * inv);
+            *reinterpret_cast<uint4 *>(sm.q[X] + sw128(row, (c0 >> 3) + q4)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+          }
+        }
+        // a warp stores the 32 rows its own threads have written (lanes 0-15 one row, lanes 16-31 the next); a lane's rows
+        // are 2 apart
+        __syncwarp();
+        const int c = lane & 15, r0 = (row & ~31) + (lane >> 4);
+#pragma unroll 4
+        for (int i = 0; i < 16; ++i) {
+          const int rr = r0 + 2 * i, tk = rr / G;
+          if (tk < ntokX) {
+            const uint4 val = *reinterpret_cast<const uint4 *>(sm.q[X] + sw128(rr, c));
+            bf16 *op = reinterpret_cast<bf16 *>(p.out) +
+                       ((seq + size_t(chunk_c0 + tok0 + X * TOKT + tk)) * p.H + p.heads_of[g * G + (rr - tk * G)]) * kD + c * 8;
+            *reinterpret_cast<uint4 *>(op) = val;
+          }
+        }
+      }
     }
-  } else if (warp == kLoadWarp) {
+  } else if (warp == kMmaWarp) {
+    // =========================== MMA warp ===========================
+    // The warp stays together (every wait ends in a vote), one elected lane issues.
+    const bool leader = elect_one();
+    const uint32_t tm = __shfl_sync(0xffffffffu, tmem, 0);
+    const int nx = hasB ? 2 : 1;
+    const int tf0 = t_first(0), tf1 = t_first(1), te0 = t_end(0), te1 = hasB ? t_end(1) : 0;
+    uint32_t p_phase = 0;                          // bit x: parity of the next operand of X
+    bool ok = true;
+    auto wait = [&](uint64_t &bar, uint32_t parity) {
+      ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&bar), parity, failed));
+      tc_fence_after();
+      return ok;
+    };
+    auto wait_p = [&](int x) {
+      const uint32_t par = (p_phase >> x) & 1u;
+      p_phase ^= 1u << x;
+      return wait(sm.bar_p[x], par);
+    };
+    auto commit = [&](uint64_t &bar) {
+      if (leader) mma_commit(smem_u32(&bar));
+    };
+    PF_LAP_INIT();
+    // t = -1: the first S products; then per key tile P V of the tile and S of the next one
+    for (int t = -1; t < n_tiles && ok; ++t) {
+      const int seqV = 2 * t + 1, seqK = 2 * t + 2;
+      const bool more = t + 1 < n_tiles;
+      PF_LAP(18);
+      if (t >= 0) wait(sm.bar_full[seqV % kStages], uint32_t(seqV / kStages) & 1u);
+      PF_LAP(16);
+      if (ok && more) wait(sm.bar_full[seqK % kStages], uint32_t(seqK / kStages) & 1u);
+      PF_LAP(17);
+#pragma unroll 1
+      for (int x = 0; x < nx && ok; ++x) {
+        const int tf = x ? tf1 : tf0, te = x ? te1 : te0;
+        if (t >= tf && t < te) {
+          PF_LAP(18);
+          if (!wait_p(x)) break;
+          PF_LAP(19);
+          issue_mma_ts(leader, tm + 256 + x * 128, tm + x * 128, kv_addr(seqV % kStages), t > tf);
+          if (t + 1 == te) commit(sm.bar_s[x]);   // the window part of O_X
+        }
+        if (t + 1 >= tf && t + 1 < te) {
+          if (t + 1 == tf && !wait(sm.bar_q[x], 0u)) break;
+          issue_mma(leader, tm + x * 128, q_addr(x), kv_addr(seqK % kStages), false, false);
+          commit(sm.bar_s[x]);
+        }
+      }
+      if (ok) {
+        if (t >= 0) commit(sm.bar_free[seqV % kStages]);
+        if (more) commit(sm.bar_free[seqK % kStages]);
+      }
+    }
+    if (ok) commit(sm.bar_done);
+    if (ok && linear && !PHI2) {
+      // per row tile: phi(Q) S (inter-chunk) and the first C = phi(Q) phi(K')^T in one batch
+#pragma unroll 1
+      for (int x = 0; x < nx && ok; ++x) {
+        if (!wait_p(x)) break;
+        if (need_state && wait(sm.bar_state, 0u))
+          issue_mma(leader, tm + 256 + x * 128, q_addr(x), kv_addr(slot_state()), true, x ? te1 > tf1 : te0 > tf0);
+        if (ok && n_itiles > 0 && wait(sm.bar_pk[0], 0u))
+          issue_mma(leader, tm + x * 128, q_addr(x), kv_addr(slot_pk(0)), false, false);
+        if (ok) commit(sm.bar_s[x]);
+      }
+      for (int t = 0; t < n_itiles && ok; ++t) {
+        wait(sm.bar_vp[t & 1], uint32_t(t >> 1) & 1u);
+        if (ok && t + 1 < n_itiles) wait(sm.bar_pk[(t + 1) & 1], uint32_t((t + 1) >> 1) & 1u);
+#pragma unroll 1
+        for (int x = 0; x < nx && ok; ++x) {
+          if (!wait_p(x)) break;
+          issue_mma_ts(leader, tm + 256 + x * 128, tm + x * 128, kv_addr(slot_vp(t)), (x ? te1 > tf1 : te0 > tf0) || need_state || t > 0);
+          if (t + 1 < n_itiles) issue_mma(leader, tm + x * 128, q_addr(x), kv_addr(slot_pk(t + 1)), false, false);
+          commit(sm.bar_s[x]);
+        }
+        if (ok) commit(sm.bar_lfree[t & 1]);   // V'(t) has been read, and phi(K')(t) before it
+      }
+    }
+    if (ok && linear && PHI2) {
+      // phi+ S+ and phi- S-, then per step C = phi+ phi+(K')^T + phi- phi-(K')^T (accumulated before the causal mask)
+      // and C V'; the phi(K') halves of a step take the buffers of the state, or of the step before
+#pragma unroll 1
+      for (int x = 0; x < nx && ok; ++x) {
+        if (!wait_p(x)) break;
+        if (need_state) {
+          issue_mma(leader, tm + 256 + x * 128, q_addr(x), kv_addr(2), true, x ? te1 > tf1 : te0 > tf0);
+          issue_mma(leader, tm + 256 + x * 128, kv_addr(x), kv_addr(3), true, true);
+        }
+        if (n_itiles == 0) commit(sm.bar_s[x]);
+      }
+      if (ok) commit(sm.bar_lfree[0]);
+      for (int t = 0; t < n_itiles && ok; ++t) {
+        wait(sm.bar_pk[0], uint32_t(t) & 1u);
+#pragma unroll 1
+        for (int x = 0; x < nx && ok; ++x) {
+          issue_mma(leader, tm + x * 128, q_addr(x), kv_addr(2), false, false);
+          issue_mma(leader, tm + x * 128, kv_addr(x), kv_addr(3), false, true);
+          commit(sm.bar_s[x]);
+        }
+        if (ok) wait(sm.bar_vp[0], uint32_t(t) & 1u);
+#pragma unroll 1
+        for (int x = 0; x < nx && ok; ++x) {
+          if (!wait_p(x)) break;
+          issue_mma_ts(leader, tm + 256 + x * 128, tm + x * 128, kv_addr(4), (x ? te1 > tf1 : te0 > tf0) || need_state || t > 0);
+          if (t + 1 == n_itiles) commit(sm.bar_s[x]);
+        }
+        if (ok) commit(sm.bar_lfree[0]);
+      }
+    }
+  } else {
+    // =========================== loader warp ===========================
     // A 128-key tile is eight groups of 16 tokens.  A group that lies in one source (ring or call) and is contiguous
     // there is fetched by TMA, lane gi issuing the two boxes (column halves) of group gi so that the address
     // arithmetic of the groups runs in parallel.  A group that straddles the call boundary or a ring wrap is copied
@@ -546,28 +867,114 @@ prefill_attn_tc_kernel(const PrefillParams p, const CUtensorMap *ring_maps, cons
     // expect-tx one before the TMA boxes are issued and a plain one after the row copies.
     const CUtensorMap *ringK = ring_maps + 3 * layer, *ringV = ringK + 1;
     const CUtensorMap *ringK128 = ring_maps + 3 * p.L + 2 * layer, *ringV128 = ringK128 + 1;
+    const CUtensorMap *map_pk = ring_maps + 5 * p.L, *map_s16 = map_pk + 1, *map_pq = map_pk + 2;
     const bf16 *ringKp = reinterpret_cast<const bf16 *>(p.ws + ld.ringK) + unit_rows * kD;
     const bf16 *ringVp = reinterpret_cast<const bf16 *>(p.ws + ld.ringV) + unit_rows * kD;
     const bf16 *callKp = reinterpret_cast<const bf16 *>(p.k) + (seq * p.Hkv + g) * kD;
     const bf16 *callVp = reinterpret_cast<const bf16 *>(p.v) + (seq * p.Hkv + g) * kD;
     const int64_t call_stride = int64_t(p.Hkv) * kD;
     const int gi = lane;
-    // Rows of tokens j0 .. j0 + 127 (K or V) into buffer `slot` (the whole warp); rows of tokens below 0 are zero;
-    // 16-row groups that lie wholly above j_max are zero too (zero_rest) or not written at all.  j0 need
-    // not be a multiple of the box size: a ring row or a token of the call is a TMA coordinate like any other.
-    auto load_tile = [&](int64_t j0, bool is_v, int slot, uint32_t bar, int64_t j_max, bool zero_rest) {
-      const int64_t left = j_max - j0;                         // >= 0: the tile holds at least one valid token
+    bool ok = true;
+    auto tma_tile = [&](uint32_t dst, const CUtensorMap *m, int y, uint32_t bar) {
+      tma_load_2d(dst, m, 0, y, bar);
+      tma_load_2d(dst + kBoxBytes, m, 64, y, bar);
+    };
+    // Jobs of the warp in order: the K and V tiles of the window (2 n_tiles), one job for the operands of the linear part
+    // that one thread fetches, then the V' tiles of the intra-chunk steps (with the phi(K') tiles of later steps).
+    const int n_window = 2 * n_tiles;
+    const int n_jobs = n_window + (linear ? 1 + n_itiles : 0);
+#pragma unroll 1
+    for (int job = 0; job < n_jobs; ++job) {
+      if (job == n_window) {
+        if (lane == 0 && !PHI2) {
+          // the bf16 state (with z), then the phi(K') tiles of the first two intra-chunk steps
+          const int n_late = 1 + (n_itiles < 2 ? n_itiles : 2);
+#pragma unroll 1
+          for (int k = 0; k < n_late && ok; ++k) {
+            if (k == 0 && !need_state) continue;
+            const int sq = late_seq(k);
+            if (sq >= 0) ok = mbar_wait(smem_u32(&sm.bar_free[sq % kStages]), uint32_t(sq / kStages) & 1u, failed);
+            if (!ok) break;
+            const uint32_t bar = k == 0 ? smem_u32(&sm.bar_state) : smem_u32(&sm.bar_pk[k - 1]);
+            mbar_expect_tx(bar, kTileBytes + (k == 0 ? uint32_t(kD * sizeof(float)) : 0u));
+            if (k == 0) bulk_load(smem_u32(sm.z), p.zsnap + size_t(uc) * kD, uint32_t(kD * sizeof(float)), bar);
+            tma_tile(kv_addr(late_slot(k)), k == 0 ? map_s16 : map_pk, k == 0 ? int(uc) * kD : int(uc) * p.SC + it0 + (k - 1) * kKT, bar);
+          }
+        }
+        if (lane == 0 && PHI2) {
+          const uint32_t bar = smem_u32(&sm.bar_state);
+          const int rows_q = int(p.units_cap) * p.SC * G, rows_s = int(p.units_cap) * kD;
+          ok = mbar_wait(smem_u32(&sm.bar_done), 0u, failed);
+          if (ok && n_tiles == 0) {                // no window: phi+ takes the place of Q when Q's copies have landed
+            ok = mbar_wait(smem_u32(&sm.bar_q[0]), 0u, failed);
+            if (ok && hasB) ok = mbar_wait(smem_u32(&sm.bar_q[1]), 0u, failed);
+          }
+          if (ok) {
+            mbar_expect_tx(bar, (hasB ? 4u : 2u) * kTileBytes + (need_state ? 2u * kTileBytes + uint32_t(2 * kD * sizeof(float)) : 0u));
+#pragma unroll 1
+            for (int i = 0; i < (hasB ? 4 : 2); ++i) {
+              const int x = i >> 1, hf = i & 1;
+              tma_tile(hf == 0 ? q_addr(x) : kv_addr(x), map_pq, hf * rows_q + (int(uc) * p.SC + tok0 + x * TOKT) * G, bar);
+            }
+            if (need_state) {
+              tma_tile(kv_addr(2), map_s16, int(uc) * kD, bar);
+              tma_tile(kv_addr(3), map_s16, rows_s + int(uc) * kD, bar);
+              bulk_load(smem_u32(sm.z), p.zsnap + size_t(uc) * 2 * kD, uint32_t(2 * kD * sizeof(float)), bar);
+            }
+          }
+        }
+        ok = __all_sync(0xffffffffu, ok);
+        if (!ok) break;
+        continue;
+      }
+      // Rows of tokens j0 .. j0 + 127 (K or V) into buffer `slot` (the whole warp); 16-row groups that lie wholly above
+      // the CTA's last token are not written in the window, but zero in a V' tile, as are rows of tokens below 0 (their
+      // weights are zero, and 0 x anything must stay 0).  j0 need not be a multiple of the box size: a ring row or a token
+      // of the call is a TMA coordinate like any other.
+      const bool late = job > n_window;
+      const int ts = late ? job - n_window - 1 : job >> 1;       // intra-chunk step, or key tile
+      const bool is_v = late || (job & 1);
+      const int slot = late ? slot_vp(ts) : job % kStages;
+      const uint32_t bar = late ? smem_u32(&sm.bar_vp[PHI2 ? 0 : ts & 1]) : smem_u32(&sm.bar_full[slot]);
+      const int64_t j0 = late ? folded + it0 + int64_t(ts) * kKT : j_lo + int64_t(ts) * kKT;
+      if (!late) {
+        PF_LAP_INIT();
+        if (job >= kStages) ok = mbar_wait(smem_u32(&sm.bar_free[slot]), uint32_t(job / kStages - 1) & 1u, failed);
+        PF_LAP(20);
+      } else if (!PHI2) {
+        const int sq = late_seq(3 + ts);
+        if (ts < 2) {
+          if (sq >= 0) ok = mbar_wait(smem_u32(&sm.bar_free[sq % kStages]), uint32_t(sq / kStages) & 1u, failed);
+        } else {   // the buffers of step ts - 2: its phi(K') tile was read before its V' tile
+          ok = mbar_wait(smem_u32(&sm.bar_lfree[ts & 1]), uint32_t((ts >> 1) - 1) & 1u, failed);
+          if (ok && lane == 0) {
+            const uint32_t pkb = smem_u32(&sm.bar_pk[ts & 1]);
+            mbar_expect_tx(pkb, kTileBytes);
+            tma_tile(kv_addr(slot_pk(ts)), map_pk, int(uc) * p.SC + it0 + ts * kKT, pkb);
+          }
+        }
+      } else {   // learned map: the state's or the previous step's products have completed
+        ok = mbar_wait(smem_u32(&sm.bar_lfree[0]), uint32_t(ts) & 1u, failed);
+        if (ok && lane == 0) {
+          const uint32_t pkb = smem_u32(&sm.bar_pk[0]);
+          const int rows_k = int(p.units_cap) * p.SC, y = int(uc) * p.SC + it0 + ts * kKT;
+          mbar_expect_tx(pkb, 2u * kTileBytes);
+          tma_tile(kv_addr(2), map_pk, y, pkb);
+          tma_tile(kv_addr(3), map_pk, rows_k + y, pkb);
+        }
+      }
+      ok = __all_sync(0xffffffffu, ok);
+      if (!ok) break;
+      const int64_t left = tq_last - j0;                         // >= 0: the tile holds at least one valid token
       const int ngroups = left >= kKT - 1 ? kKT / kGroup : int(left / kGroup) + 1;
       // A full tile that lies in one source without a wrap takes two boxes of 128 rows (the layout in shared memory
       // is that of eight 16-row boxes).  Tiles that reach past the last token keep the 16-row path, which never
-      // loads a later token's row.
-      if (j0 >= 0) {
+      // loads a later token's row.  (left >= kKT - 1: every row of the tile is a token up to the last one; eight groups
+      // alone would also admit a last group that is only partly valid)
+      if (j0 >= 0 && left >= kKT - 1) {
         const uint32_t slot_row0 = (j0 >> 32) == 0 ? uint32_t(j0) % cap : uint32_t(uint64_t(j0) % cap);
         const bool all_call = j0 >= p.n0;
-        const bool all_ring = j0 + kKT <= p.n0 && slot_row0 + kKT <= cap;
-        // (left >= kKT - 1: every row of the tile is a token up to the last one; eight groups alone would also
-        // admit a last group that is only partly valid)
-        if (left >= kKT - 1 && (all_call || all_ring)) {
+        if (all_call || (j0 + kKT <= p.n0 && slot_row0 + kKT <= cap)) {
           if (lane == 0) {
             mbar_expect_tx(bar, kTileBytes);
             const uint32_t dst = kv_addr(slot);
@@ -576,19 +983,17 @@ prefill_attn_tc_kernel(const PrefillParams p, const CUtensorMap *ring_maps, cons
               tma_load_4d(dst, m, 0, g, int(j0 - p.n0), lrel * p.B + b, bar);
               tma_load_4d(dst + kBoxBytes, m, 64, g, int(j0 - p.n0), lrel * p.B + b, bar);
             } else {
-              const CUtensorMap *m = is_v ? ringV128 : ringK128;
-              const int y = int(unit_rows + slot_row0);
-              tma_load_2d(dst, m, 0, y, bar);
-              tma_load_2d(dst + kBoxBytes, m, 64, y, bar);
+              tma_tile(dst, is_v ? ringV128 : ringK128, int(unit_rows + slot_row0), bar);
             }
             mbar_arrive(bar);   // the barrier's second arrival (after the row copies on the other path)
           }
-          return;
+          __syncwarp();
+          continue;
         }
       }
       // this lane's group: where it comes from and whether one box covers it
       const int64_t j = j0 + gi * kGroup;
-      const bool mine = gi < kKT / kGroup && (zero_rest || gi < ngroups);
+      const bool mine = gi < kKT / kGroup && (late || gi < ngroups);
       const bool from_call = j >= p.n0;
       const uint32_t slot_row = j < 0 ? 0u : ((j >> 32) == 0 ? uint32_t(j) % cap : uint32_t(uint64_t(j) % cap));
       const bool boxed = mine && gi < ngroups && j >= 0 && (from_call || (j + kGroup <= p.n0 && slot_row + kGroup <= cap));
@@ -603,24 +1008,23 @@ prefill_attn_tc_kernel(const PrefillParams p, const CUtensorMap *ring_maps, cons
           tma_load_4d(dst, m, 0, g, int(j - p.n0), lrel * p.B + b, bar);
           tma_load_4d(dst + kBoxBytes, m, 64, g, int(j - p.n0), lrel * p.B + b, bar);
         } else {
-          const CUtensorMap *m = is_v ? ringV : ringK;
-          const int y = int(unit_rows + slot_row);
-          tma_load_2d(dst, m, 0, y, bar);
-          tma_load_2d(dst + kBoxBytes, m, 64, y, bar);
+          tma_tile(dst, is_v ? ringV : ringK, int(unit_rows + slot_row), bar);
         }
       }
+#pragma unroll 1
       for (unsigned mm = manual_mask; mm; mm &= mm - 1) {
         const int gm = __ffs(int(mm)) - 1;
         unsigned char *tile = sm.kv[slot];
-#pragma unroll
+#pragma unroll 2
         for (int i = 0; i < kGroup * 16 / 32; ++i) {
           const int id = lane + 32 * i;
           const int r = id >> 4, c = id & 15;
           const int64_t jj = j0 + gm * kGroup + r;
           uint4 val = make_uint4(0u, 0u, 0u, 0u);
-          if (jj >= 0 && jj <= j_max) {
+          if (jj >= 0 && jj <= tq_last) {
+            const uint32_t sr = (jj >> 32) == 0 ? uint32_t(jj) % cap : uint32_t(uint64_t(jj) % cap);
             const bf16 *src = jj >= p.n0 ? (is_v ? callVp : callKp) + size_t(jj - p.n0) * call_stride
-                                         : (is_v ? ringVp : ringKp) + size_t(uint64_t(jj) % cap) * kD;
+                                         : (is_v ? ringVp : ringKp) + size_t(sr) * kD;
             val = *reinterpret_cast<const uint4 *>(src + c * 8);
           }
           *reinterpret_cast<uint4 *>(tile + sw128(gm * kGroup + r, c)) = val;
@@ -629,412 +1033,17 @@ prefill_attn_tc_kernel(const PrefillParams p, const CUtensorMap *ring_maps, cons
       fence_async_smem();   // the row copies are read by the tensor core (async proxy)
       __syncwarp();
       if (lane == 0) mbar_arrive(bar);
-    };
-    bool ok = true;
-    for (int sq = 0; sq < 2 * n_tiles; ++sq) {
-      const int t = sq >> 1, slot = sq % kStages;
-      if (sq >= kStages) ok = mbar_wait(smem_u32(&sm.bar_free[slot]), uint32_t(sq / kStages - 1) & 1u, failed);
-      if (!__all_sync(0xffffffffu, ok)) break;
-      load_tile(j_lo + int64_t(t) * kKT, sq & 1, slot, smem_u32(&sm.bar_full[slot]), tq_last, false);
-    }
-    if (!PHI2 && lane == 0 && linear && !*failed) {
-      // the linear part's operands into the buffers the window loop leaves first: the bf16 state (with z), then the
-      // phi(K') tiles of the first two intra-chunk steps
-      const int n_late = 1 + (n_itiles < 2 ? n_itiles : 2);
-      for (int k = 0; k < n_late; ++k) {
-        const int sq = late_seq(k);
-        if (sq >= 0 && !mbar_wait(smem_u32(&sm.bar_free[sq % kStages]), uint32_t(sq / kStages) & 1u, failed)) break;
-        if (k == 0) {
-          if (!need_state) continue;
-          const uint32_t bar = smem_u32(&sm.bar_state);
-          mbar_expect_tx(bar, kTileBytes + uint32_t(kD * sizeof(float)));
-          tma_load_2d(kv_addr(slotSb), map_s16, 0, int(uc * kD), bar);
-          tma_load_2d(kv_addr(slotSb) + kBoxBytes, map_s16, 64, int(uc * kD), bar);
-          bulk_load(smem_u32(sm.z), p.zsnap + size_t(uc) * kD, uint32_t(kD * sizeof(float)), bar);
-        } else {
-          load_pk(k - 1);
-        }
-      }
-    }
-    __syncwarp();
-    // the V rows of the delayed tokens of the first two intra-chunk steps, behind the window loop's last tiles (the
-    // rows of tokens that do not exist yet, below 0, are zero: their weights are, and 0 x anything must stay 0)
-    for (int t = 0; !PHI2 && t < n_itiles && t < 2 && __all_sync(0xffffffffu, ok && !*failed); ++t) {
-      const int sq = late_seq(3 + t);
-      if (sq >= 0) ok = mbar_wait(smem_u32(&sm.bar_free[sq % kStages]), uint32_t(sq / kStages) & 1u, failed);
-      if (!__all_sync(0xffffffffu, ok)) break;
-      load_tile(folded + it0 + int64_t(t) * kKT, true, slotVp[t], smem_u32(&sm.bar_vp[t]), tq_last, true);
     }
   }
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-
-  PF_CLK(1);
-  // =========================== linear part: the whole CTA in step ===========================
-  // (no early exits from here on: every thread passes the same __syncthreads; after a time-out the waits return
-  // at once and the results are discarded)
-  // Operands: phi(Q) 2^-M from the softmax threads; the bf16 state and the phi(K') tiles by TMA (issued by the loader
-  // behind the window loop, see above); the delayed tokens' V rows row by row (they come from the ring or from the
-  // call, with a wrap or the call boundary anywhere) by the loader as well, with the key tiles' own routine.
-  bool o_init = n_tiles > 0;   // O_X holds a valid accumulation (uniform over the CTA)
-  uint32_t lin_phase = 0;
-  const int mma_tid = kMmaWarp * 32;
-  auto wait_lin = [&]() {
-    mbar_wait(smem_u32(&sm.bar_lin), lin_phase & 1u, failed);
-    ++lin_phase;
-    tc_fence_after();
-  };
-  // C row of this thread -> bf16 over the same TMEM columns, masked to the delayed tokens j' <= i of the row (the
-  // values already carry 2^-m*); the row's weight sum goes to l
-  auto convert_c = [&](int i0) {
-    if (activeX) {
-      // C row -> bf16, masked to delayed tokens j' <= i of this row (the values already carry 2^-m*)
-      float sum0 = 0.f, sum1 = 0.f;
-      const int lo = i_lo - i0, hi = tl - i0;
-      // a tile that lies wholly before the row tile's first token (and after the first delayed token) needs no mask
-      const bool whole = i0 + kKT - 1 <= tok0 + X * TOKT && i0 >= i_lo;
-      uint32_t ra[32], rb[32];
-      tmem_ld32_nowait(tS, ra);
-#pragma unroll
-      for (int c0 = 0; c0 < kKT; c0 += 32) {
-        uint32_t (&r)[32] = ((c0 >> 5) & 1) ? rb : ra;
-        uint32_t pk[16];
-        tmem_wait_ld();
-        if (c0 + 32 < kKT) tmem_ld32_nowait(tS + c0 + 32, ((c0 >> 5) & 1) ? ra : rb);
-        if (whole) {
-#pragma unroll
-          for (int e = 0; e < 16; ++e) pk[e] = pack_bf16x2(__uint_as_float(r[e * 2]), __uint_as_float(r[e * 2 + 1]));
-        } else {
-#pragma unroll
-          for (int e = 0; e < 16; ++e) {
-            const int i = c0 + e * 2;
-            const float a0 = (i >= lo && i <= hi) ? __uint_as_float(r[e * 2]) : 0.f;
-            const float a1 = (i + 1 >= lo && i + 1 <= hi) ? __uint_as_float(r[e * 2 + 1]) : 0.f;
-            pk[e] = pack_bf16x2(a0, a1);
-          }
-        }
-#pragma unroll
-        for (int e = 0; e < 16; ++e) {
-          sum0 += __uint_as_float(pk[e] << 16);
-          sum1 += __uint_as_float(pk[e] & 0xffff0000u);
-        }
-        tmem_st16(tS + (c0 >> 1), pk);
-      }
-      tmem_wait_st();
-      if (!sum_terms) l_sum += sum0 + sum1;
-    }
-    PF_CLK(4);
-  };
-  if (linear && !PHI2) {
-    const bf16 *ringV = reinterpret_cast<const bf16 *>(p.ws + ld.ringV) + unit_rows * kD;
-    const bf16 *callV = reinterpret_cast<const bf16 *>(p.v) + (seq * p.Hkv + g) * kD;
-    const int64_t call_stride = int64_t(p.Hkv) * kD;
-    auto load_vp = [&](int t) {   // softmax threads, steps after the second: V rows of the delayed tokens (MN-major), zero where none
-      const int i0 = it0 + t * kKT;
-      const uint32_t dst = kv_addr(slotVp[t & 1]);
-#pragma unroll 4
-      for (int i = 0; i < kKT * 16 / kSoftmaxThreads; ++i) {
-        const int id = tid + kSoftmaxThreads * i;
-        const int r = id >> 4, c = id & 15;
-        const int ii = i0 + r;
-        const bool valid = ii >= i_lo && ii <= i_hi;
-        const int64_t jj = valid ? folded + ii : 0;
-        const bool from_call = jj >= p.n0;
-        const uint32_t slot_row = (jj >> 32) == 0 ? uint32_t(jj) % cap : uint32_t(uint64_t(jj) % cap);
-        const bf16 *src = from_call ? callV + size_t(jj - p.n0) * call_stride : ringV + size_t(slot_row) * kD;
-        cp_async16(dst + sw128(r, c), src + c * 8, valid);
-      }
-      cp_async_commit();
-    };
-    uint32_t phq[kD / 2];                      // phi(q) 2^-m* of this row, packed bf16
-    if (activeX) {
-      // Any common reference M >= m_ref gives the same quotient O / l.  M = max(m_ref, 0) would rescale O for every
-      // row whose window maximum is negative; a floor of -64 keeps 2^-M and everything scaled by it far inside the
-      // fp32 / bf16 range (phi <= 1) and makes that rescale a rarity.
-      // A row without evicted tokens (position below the window size) keeps its own reference and gets phi(q) = 0:
-      // a floor there would only push its window weights towards underflow.
-      // Sum of two normalised terms instead: the window part is normalised now (O / l), and phi(q) is divided by the
-      // row's linear normaliser phi(q) . (z + running sum of phi(K') up to the row's own delayed token), so that what
-      // the linear products add to O is the normalised linear term; the final division is by 1.
-      const bool has_lin = tok_abs >= wl;
-      const float M = has_lin ? fmaxf(m_ref, -64.f) : m_ref;
-      float fw = m_ref == -CUDART_INF_F ? 0.f : ex2(m_ref - M);
-      const float fl = has_lin ? ex2(-M) : 0.f;
-      if (sum_terms) fw = l_sum > 0.f ? 1.0f / l_sum : 0.f;
-      if (o_init && __any_sync(0xffffffffu, fw != 1.f)) scale_o(fw);
-      l_sum = sum_terms ? 1.f : l_sum * fw;
-      if (sum_terms && need_state) mbar_wait(smem_u32(&sm.bar_state), 0u, failed);   // z is needed for the normaliser
-      // this row of Q is still in the shared tile (every S product has completed)
-#pragma unroll
-      for (int i = 0; i < kD / 8; ++i) {
-        const uint4 v4 = *reinterpret_cast<const uint4 *>(sm.q[X] + sw128(row, i));
-        phq[i * 4 + 0] = v4.x;
-        phq[i * 4 + 1] = v4.y;
-        phq[i * 4 + 2] = v4.z;
-        phq[i * 4 + 3] = v4.w;
-      }
-      float mx = -CUDART_INF_F;
-#pragma unroll
-      for (int i = 0; i < kD / 2; ++i)
-        mx = fmaxf(mx, fmaxf(__uint_as_float(phq[i] << 16), __uint_as_float(phq[i] & 0xffff0000u)));
-      // one pass of exponentials: kept as packed bf16, normalised by the sum of the unrounded values afterwards
-      float sum0 = 0.f, sum1 = 0.f, dz0 = 0.f, dz1 = 0.f;
-      const float mxl = mx * kLog2e;
-      const float4 *zrow = reinterpret_cast<const float4 *>(p.zcum + (size_t(uc) * p.SC + size_t(tok_r < ntokX ? tl : tok0)) * kD);
-#pragma unroll
-      for (int i4 = 0; i4 < kD / 4; ++i4) {
-        float zz[4] = {0.f, 0.f, 0.f, 0.f};
-        if (sum_terms) {
-          const float4 zc = __ldg(zrow + i4);
-          zz[0] = zc.x, zz[1] = zc.y, zz[2] = zc.z, zz[3] = zc.w;
-          if (need_state) {
-#pragma unroll
-            for (int e = 0; e < 4; ++e) zz[e] += sm.z[i4 * 4 + e];
-          }
-        }
-#pragma unroll
-        for (int hf = 0; hf < 2; ++hf) {
-          const int i = i4 * 2 + hf;
-          const float e0 = ex2(fmaf(__uint_as_float(phq[i] << 16), kLog2e, -mxl));
-          const float e1 = ex2(fmaf(__uint_as_float(phq[i] & 0xffff0000u), kLog2e, -mxl));
-          sum0 += e0;
-          sum1 += e1;
-          dz0 = fmaf(e0, zz[hf * 2], dz0);
-          dz1 = fmaf(e1, zz[hf * 2 + 1], dz1);
-          phq[i] = pack_bf16x2(e0, e1);
-        }
-      }
-      // shared normaliser: phi(q) 2^-M;  sum of terms: phi(q) / (phi(q) . z_row) = e / (e . z_row)
-      const float dz = dz0 + dz1;
-      const float sc = sum_terms ? ((has_lin && dz > 0.f) ? 1.0f / dz : 0.f) : fl * __frcp_rn(sum0 + sum1);
-#pragma unroll
-      for (int i = 0; i < kD / 2; ++i)
-        phq[i] = pack_bf16x2(__uint_as_float(phq[i] << 16) * sc, __uint_as_float(phq[i] & 0xffff0000u) * sc);
-#pragma unroll
-      for (int c = 0; c < 16; ++c)
-        *reinterpret_cast<uint4 *>(sm.q[X] + sw128(row, c)) = make_uint4(phq[c * 4], phq[c * 4 + 1], phq[c * 4 + 2], phq[c * 4 + 3]);
-    }
-    PF_CLK(10);
-    fence_async_smem();
-    tc_fence_before();
-    __syncthreads();
-    PF_CLK(2);
-    // inter-chunk product into O and the first intra-chunk C in one batch
-    if (tid == mma_tid) {
-      tc_fence_after();
-      if (need_state) {
-        mbar_wait(smem_u32(&sm.bar_state), 0u, failed);
-        issue_mma(tmem + 256, sQ[0], kv_addr(slotSb), true, o_init);
-        if (hasB) issue_mma(tmem + 384, sQ[1], kv_addr(slotSb), true, o_init);
-      }
-      if (n_itiles > 0) {
-        mbar_wait(smem_u32(&sm.bar_pk[0]), 0u, failed);
-        issue_mma(tmem, sQ[0], kv_addr(slotPk[0]), false, false);   // C_X = (phi(Q_X) 2^-m*) phi(K')^T
-        if (hasB) issue_mma(tmem + 128, sQ[1], kv_addr(slotPk[0]), false, false);
-      }
-      if (need_state || n_itiles > 0) mma_commit(smem_u32(&sm.bar_lin));
-    }
-    if (need_state && activeX) {
-      mbar_wait(smem_u32(&sm.bar_state), 0u, failed);   // z has landed
-      float dot = 0.f;
-#pragma unroll
-      for (int i = 0; i < kD / 2; ++i)
-        dot += __uint_as_float(phq[i] << 16) * sm.z[2 * i] + __uint_as_float(phq[i] & 0xffff0000u) * sm.z[2 * i + 1];
-      if (!sum_terms) l_sum += dot;
-    }
-    if (need_state || n_itiles > 0) wait_lin();
-    if (need_state) o_init = true;
-    PF_CLK(3);
-    for (int t = 0; t < n_itiles; ++t) {
-      const int i0 = it0 + t * kKT;
-      convert_c(i0);
-      if (t >= 2 && tid < kSoftmaxThreads) cp_async_wait_all();   // (steps after the second: rows copied by these threads)
-      fence_async_smem();
-      tc_fence_before();
-      __syncthreads();
-      if (tid == mma_tid) {
-        if (t < 2) mbar_wait(smem_u32(&sm.bar_vp[t]), 0u, failed);   // the loader's V' tile
-        tc_fence_after();
-        issue_mma_ts(tmem + 256, tmem, kv_addr(slotVp[t & 1]), o_init);
-        if (hasB) issue_mma_ts(tmem + 384, tmem + 128, kv_addr(slotVp[t & 1]), o_init);
-        if (t + 1 < n_itiles) {   // the next step's C follows in the same batch (the tensor pipe keeps the order)
-          mbar_wait(smem_u32(&sm.bar_pk[(t + 1) & 1]), uint32_t((t + 1) >> 1) & 1u, failed);
-          issue_mma(tmem, sQ[0], kv_addr(slotPk[(t + 1) & 1]), false, false);
-          if (hasB) issue_mma(tmem + 128, sQ[1], kv_addr(slotPk[(t + 1) & 1]), false, false);
-        }
-        mma_commit(smem_u32(&sm.bar_lin));
-      }
-      wait_lin();
-      PF_CLK(5);
-      o_init = true;
-      if (t + 2 < n_itiles) {   // this step's buffers are free again: the operands of the step after the next
-        if (tid == mma_tid) load_pk(t + 2);
-        if (tid < kSoftmaxThreads) load_vp(t + 2);
-      }
-    }
-  }
-
-  // Learned feature map (shared normaliser): phi(q) = [softmax(W^T q); softmax(-W^T q)] has 2 d entries, and
-  // phi(q)^T S, phi(q)^T z and phi(Q) phi(K')^T are sums over its two halves; every half is a linear part of the
-  // kind above with its own 128-column tensors.  phi(Q) comes from a kernel in front of this one (the projections
-  // differ per head, and a row tile mixes the heads of the group), as bf16 rows that this thread only scales by
-  // 2^-M.  Everything arrives by TMA after the window loop (the Q tiles and all five K/V buffers are free then):
-  // phi+ of the two row tiles in the Q tiles, phi- in buffers 0 and 1, the state halves and then the phi(K') halves of
-  // each intra-chunk step in buffers 2 and 3, the step's V' rows in buffer 4.
-  if (linear && PHI2) {
-    const bf16 *ringV = reinterpret_cast<const bf16 *>(p.ws + ld.ringV) + unit_rows * kD;
-    const bf16 *callV = reinterpret_cast<const bf16 *>(p.v) + (seq * p.Hkv + g) * kD;
-    const int64_t call_stride = int64_t(p.Hkv) * kD;
-    auto load_vp = [&](int t) {   // softmax threads: V rows of the delayed tokens of step t (MN-major), zero where none
-      const int i0 = it0 + t * kKT;
-      const uint32_t dst = kv_addr(4);
-#pragma unroll 4
-      for (int i = 0; i < kKT * 16 / kSoftmaxThreads; ++i) {
-        const int id = tid + kSoftmaxThreads * i;
-        const int r = id >> 4, c = id & 15;
-        const int ii = i0 + r;
-        const bool valid = ii >= i_lo && ii <= i_hi;
-        const int64_t jj = valid ? folded + ii : 0;
-        const bool from_call = jj >= p.n0;
-        const uint32_t slot_row = (jj >> 32) == 0 ? uint32_t(jj) % cap : uint32_t(uint64_t(jj) % cap);
-        const bf16 *src = from_call ? callV + size_t(jj - p.n0) * call_stride : ringV + size_t(slot_row) * kD;
-        cp_async16(dst + sw128(r, c), src + c * 8, valid);
-      }
-      cp_async_commit();
-    };
-    const CUtensorMap *map_pq = map_pk + 2;
-    const int rows_q = int(p.units_cap) * p.SC * G, rows_s = int(p.units_cap) * kD, rows_k = int(p.units_cap) * p.SC;
-    auto tma_tile = [&](uint32_t dst, const CUtensorMap *m, int y, uint32_t bar) {
-      tma_load_2d(dst, m, 0, y, bar);
-      tma_load_2d(dst + kBoxBytes, m, 64, y, bar);
-    };
-    if (tid == mma_tid) {
-      const uint32_t bar = smem_u32(&sm.bar_state);
-      mbar_expect_tx(bar, (hasB ? 4u : 2u) * kTileBytes + (need_state ? 2u * kTileBytes + uint32_t(2 * kD * sizeof(float)) : 0u));
-      for (int hf = 0; hf < 2; ++hf)
-        for (int x = 0; x < 2; ++x) {
-          if (x == 1 && !hasB) break;
-          tma_tile(hf == 0 ? sQ[x] : kv_addr(x), map_pq, hf * rows_q + (int(uc) * p.SC + tok0 + x * TOKT) * G, bar);
-        }
-      if (need_state) {
-        tma_tile(kv_addr(2), map_s16, int(uc) * kD, bar);
-        tma_tile(kv_addr(3), map_s16, rows_s + int(uc) * kD, bar);
-        bulk_load(smem_u32(sm.z), p.zsnap + size_t(uc) * 2 * kD, uint32_t(2 * kD * sizeof(float)), bar);
-      }
-    }
-    if (tid < kSoftmaxThreads && n_itiles > 0) load_vp(0);
-    float dot = 0.f;
-    if (activeX) {
-      const bool has_lin = tok_abs >= wl;
-      const float M = has_lin ? fmaxf(m_ref, -64.f) : m_ref;   // (the reference of the shared normaliser, as above)
-      const float fw = m_ref == -CUDART_INF_F ? 0.f : ex2(m_ref - M);
-      const float fl = has_lin ? ex2(-M) : 0.f;
-      if (o_init && __any_sync(0xffffffffu, fw != 1.f)) scale_o(fw);
-      l_sum *= fw;
-      mbar_wait(smem_u32(&sm.bar_state), 0u, failed);
-      // this thread's row of phi+ and of phi-: times 2^-M, back as bf16; the dot with z uses the rounded values
-#pragma unroll 1
-      for (int hf = 0; hf < 2; ++hf) {
-        unsigned char *tile = hf == 0 ? sm.q[X] : sm.kv[X];
-#pragma unroll
-        for (int c = 0; c < 16; ++c) {
-          uint4 v4 = *reinterpret_cast<const uint4 *>(tile + sw128(row, c));
-          uint32_t w4[4] = {v4.x, v4.y, v4.z, v4.w};
-#pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            w4[e] = pack_bf16x2(__uint_as_float(w4[e] << 16) * fl, __uint_as_float(w4[e] & 0xffff0000u) * fl);
-            if (need_state)
-              dot += __uint_as_float(w4[e] << 16) * sm.z[hf * kD + c * 8 + e * 2] +
-                     __uint_as_float(w4[e] & 0xffff0000u) * sm.z[hf * kD + c * 8 + e * 2 + 1];
-          }
-          *reinterpret_cast<uint4 *>(tile + sw128(row, c)) = make_uint4(w4[0], w4[1], w4[2], w4[3]);
-        }
-      }
-    }
-    fence_async_smem();
-    tc_fence_before();
-    __syncthreads();
-    if (need_state) {
-      if (tid == mma_tid) {
-        tc_fence_after();
-        mbar_wait(smem_u32(&sm.bar_state), 0u, failed);
-        for (int x = 0; x < 2; ++x) {
-          if (x == 1 && !hasB) break;
-          issue_mma(tmem + 256 + x * 128, sQ[x], kv_addr(2), true, o_init);
-          issue_mma(tmem + 256 + x * 128, kv_addr(x), kv_addr(3), true, true);
-        }
-        mma_commit(smem_u32(&sm.bar_lin));
-      }
-      if (activeX) l_sum += dot;
-      wait_lin();
-      o_init = true;
-    }
-    for (int t = 0; t < n_itiles; ++t) {
-      const int i0 = it0 + t * kKT;
-      if (tid == mma_tid) {
-        // buffers 2 and 3 are free: the products that read them have completed
-        const uint32_t bar = smem_u32(&sm.bar_pk[0]);
-        mbar_expect_tx(bar, 2u * kTileBytes);
-        tma_tile(kv_addr(2), map_pk, int(uc) * p.SC + i0, bar);
-        tma_tile(kv_addr(3), map_pk, rows_k + int(uc) * p.SC + i0, bar);
-        mbar_wait(bar, uint32_t(t) & 1u, failed);
-        tc_fence_after();
-        for (int x = 0; x < 2; ++x) {
-          if (x == 1 && !hasB) break;
-          issue_mma(tmem + x * 128, sQ[x], kv_addr(2), false, false);      // C_X = phi+(Q_X) phi+(K')^T ...
-          issue_mma(tmem + x * 128, kv_addr(x), kv_addr(3), false, true);  // ... + phi-(Q_X) phi-(K')^T
-        }
-        mma_commit(smem_u32(&sm.bar_lin));
-      }
-      wait_lin();
-      convert_c(i0);
-      if (tid < kSoftmaxThreads) cp_async_wait_all();   // the step's V' rows
-      fence_async_smem();
-      tc_fence_before();
-      __syncthreads();
-      if (tid == mma_tid) {
-        tc_fence_after();
-        issue_mma_ts(tmem + 256, tmem, kv_addr(4), o_init);
-        if (hasB) issue_mma_ts(tmem + 384, tmem + 128, kv_addr(4), o_init);
-        mma_commit(smem_u32(&sm.bar_lin));
-      }
-      wait_lin();
-      o_init = true;
-      if (t + 1 < n_itiles && tid < kSoftmaxThreads) load_vp(t + 1);
-    }
-  }
-  // ---- shared normaliser and store: one contiguous 256-byte row per thread ------------------------------------
-  __syncthreads();
-  const bool bad = sm.failed != 0;
-  if (bad) {
-    if (tid == 0) atomicExch(&p.ctl->status, kDevWaitTimeout);
-  } else if (activeX && o_init) {
-    const bool store = tok_r < ntokX;   // the TMEM loads below are warp-collective: only the store is per row
-    const float inv = store ? 1.0f / l_sum : 0.f;
-    bf16 *op = reinterpret_cast<bf16 *>(p.out) +
-               ((seq + size_t(chunk_c0 + (store ? tl : tok0))) * p.H + p.heads_of[g * G + hh]) * kD;
-    uint32_t ra[32], rb[32];
-    tmem_ld32_nowait(tO, ra);
-#pragma unroll
-    for (int c0 = 0; c0 < kD; c0 += 32) {
-      uint32_t (&r)[32] = ((c0 >> 5) & 1) ? rb : ra;
-      tmem_wait_ld();
-      if (c0 + 32 < kD) tmem_ld32_nowait(tO + c0 + 32, ((c0 >> 5) & 1) ? ra : rb);   // the next columns are on their way
-#pragma unroll
-      for (int q4 = 0; q4 < 4; ++q4) {
-        uint32_t pk[4];
-#pragma unroll
-        for (int e = 0; e < 4; ++e)
-          pk[e] = pack_bf16x2(__uint_as_float(r[q4 * 8 + e * 2]) * inv, __uint_as_float(r[q4 * 8 + e * 2 + 1]) * inv);
-        if (store) *reinterpret_cast<uint4 *>(op + c0 + q4 * 8) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
-      }
-    }
-  }
+  // after a time-out the waits return at once and nothing is stored; the CTA meets here either way
   tc_fence_before();
   __syncthreads();
   PF_CLK(6);
-  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem) : "memory");
+  if (tid == 0 && sm.failed) atomicExch(&p.ctl->status, kDevWaitTimeout);
+  if (warp == kLoadWarp) {
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem) : "memory");
+  }
 }
 
 }  // namespace
@@ -1042,10 +1051,10 @@ prefill_attn_tc_kernel(const PrefillParams p, const CUtensorMap *ring_maps, cons
 
 // The kernel needs the ring descriptors made for the tensor-core decode kernels.
 #ifdef GLIDE_PF_CLOCKS
-extern "C" int glide_debug_pf_clocks(unsigned long long *host16, int reset) {
-  if (cudaMemcpyFromSymbol(host16, g_pf_clk, sizeof(g_pf_clk)) != cudaSuccess) return 6;
+extern "C" int glide_debug_pf_clocks(unsigned long long *host32, int reset) {
+  if (cudaMemcpyFromSymbol(host32, g_pf_clk, sizeof(g_pf_clk)) != cudaSuccess) return 6;
   if (reset) {
-    unsigned long long z[16] = {};
+    unsigned long long z[32] = {};
     if (cudaMemcpyToSymbol(g_pf_clk, z, sizeof(z)) != cudaSuccess) return 6;
   }
   return 0;
@@ -1109,8 +1118,8 @@ int launch_prefill_attn_tc(glide_ctx *ctx, const PrefillParams &p, cudaStream_t 
       kern<<<unsigned(blocks), kThreads, smem, stream>>>(p, ring_maps, cm);
       return cudaGetLastError() == cudaSuccess ? GLIDE_OK : GLIDE_ERR_CUDA;
     };
-    if (p.phiq16) return run(prefill_attn_tc_kernel<G, false, true>);   // learned map (shared normaliser only)
-    return p.merge == GLIDE_MERGE_SHARED ? run(prefill_attn_tc_kernel<G, false, false>) : run(prefill_attn_tc_kernel<G, true, false>);
+    if (p.phiq16) return run(prefill_attn_tc_kernel<G, kModeLearned>);   // (shared normaliser only)
+    return p.merge == GLIDE_MERGE_SHARED ? run(prefill_attn_tc_kernel<G, kModeShared>) : run(prefill_attn_tc_kernel<G, kModeSum>);
   };
   switch (ctx->G) {
     case 1: return launch(IntTag<1>{});
