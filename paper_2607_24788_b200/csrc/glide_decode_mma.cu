@@ -725,7 +725,7 @@ int build_ring_tensor_maps(glide_ctx *ctx) {
     // rows), the bf16 copy of S ([unit][128] rows) and, for the learned map, phi(Q) ([unit][chunk][G] rows); with the
     // learned map every array holds its two 128-column halves one after the other
     const cuuint64_t units = cuuint64_t(L) * ctx->cfg.batch * ctx->cfg.n_kv_heads;
-    const cuuint64_t halves = cuuint64_t(ctx->dp / D);
+    const cuuint64_t halves = ctx->cfg.gated ? 2 : cuuint64_t(ctx->dp / D);   // (gated: hi and lo)
     const cuuint64_t strides[1] = {cuuint64_t(D) * 2};
     const cuuint32_t box128[2] = {64, 128};
     const cuuint32_t estr[2] = {1, 1};

@@ -199,16 +199,19 @@ int glide::plan_context(const glide_config *cfg, glide_ctx *ctx, std::vector<Wor
   if (cfg->gated) off = align_up(off + sizeof(float) * size_t(L) * units_per_layer * ctx->prefill_chunk, 256);
   // tcgen05 prefill kernel (bf16, head_dim 128, plain feature map): bf16 copies of the chunk's phi(K') rows and of S,
   // which its CTAs fetch by TMA instead of converting the fp32 arrays themselves
-  if (cfg->io_dtype == GLIDE_BF16 && d == 128 && !cfg->gated &&
-      (cfg->phi == GLIDE_PHI_SOFTMAX || cfg->merge == GLIDE_MERGE_SHARED)) {
-    const size_t halves = size_t(dp / d);   // the learned map's two softmax halves are kept apart (one 128-column tensor each)
+  // (the learned map under the shared normaliser and, with the plain map, gates too; not both)
+  if (cfg->io_dtype == GLIDE_BF16 && d == 128 &&
+      (cfg->gated ? cfg->phi == GLIDE_PHI_SOFTMAX && cfg->merge == GLIDE_MERGE_SHARED
+                  : cfg->phi == GLIDE_PHI_SOFTMAX || cfg->merge == GLIDE_MERGE_SHARED)) {
+    // the learned map's two softmax halves are kept apart (one 128-column tensor each), as are hi and lo of a gated context
+    const size_t halves = cfg->gated ? 2 : size_t(dp / d);
     ctx->off_phik16 = off;
     off = align_up(off + 2 * halves * size_t(L) * units_per_layer * ctx->prefill_chunk * d, 256);
     ctx->off_s16 = off;
     off = align_up(off + 2 * halves * size_t(L) * units_per_layer * d * d, 256);
     ctx->off_zsnap = off;
     off = align_up(off + sizeof(float) * size_t(L) * units_per_layer * dp, 256);
-    if (halves == 2) {
+    if (dp == 2 * d) {
       ctx->off_phiq16 = off;
       off = align_up(off + 2 * halves * size_t(L) * units_per_layer * ctx->prefill_chunk * ctx->G * d, 256);
     }

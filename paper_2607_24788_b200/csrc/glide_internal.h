@@ -156,13 +156,14 @@ struct PrefillParams {
   const int32_t *heads_of;
   Control *ctl;
   float *phik;               // scratch: [layer_count][B][Hkv][nsub * SC][dp] fp32, phi of the delayed keys
-  void *phik16;              // tcgen05 kernel: the same rows as bf16 (read by TMA), [dp / d halves][units_cap * Cmax][d];
+  void *phik16;              // tcgen05 kernel: the same rows as bf16 (read by TMA), [halves][units_cap * SC][d], where the
+                             // halves are the learned map's, or hi and lo of a gated context's rows;
                              // nullptr when that kernel is not in use
   void *s16;                 // tcgen05 kernel: bf16 copy of every unit's S as it is at the start of every chunk of the pass,
-                             // [dp / d halves][units_cap][d][d], index (unit of the pass * nsub + chunk)
+                             // [halves][units_cap][d][d], index (unit of the pass * nsub + chunk)
   float *zsnap;              // tcgen05 kernel: z at the start of every chunk of the pass, [units_cap][dp], the same index
   void *phiq16;              // tcgen05 kernel, learned map: phi(q) of the chunk's query rows as bf16,
-                             // [2 halves][units_cap * Cmax * G][d], row = (unit * Cmax + token) * G + head of the group
+                             // [2 halves][units_cap * SC * G][d], row = (unit * Cmax + token) * G + head of the group
   int64_t units_cap;         // L * B * H_kv of the context: what separates the halves in the three arrays above
   float *zcum;               // sum-of-terms merges on the tcgen05 kernel: running sums of phik over the chunk, same shape
   int32_t merge;             // glide_merge

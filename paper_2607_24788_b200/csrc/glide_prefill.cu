@@ -108,6 +108,11 @@ __global__ void __launch_bounds__(kPrefillThreads) prefill_phi_kernel(const Pref
         __nv_bfloat16 *d16 = reinterpret_cast<__nv_bfloat16 *>(p.phik16) + (size_t(u) * p.Cmax + i0 + r) * D + lane * E;
 #pragma unroll
         for (int e = 0; e < E; ++e) d16[e] = __float2bfloat16_rn(x[r][e]);
+        if (p.gated) {   // and what the rounding left, in the second half of the array
+          d16 += size_t(p.units_cap) * p.SC * D;
+#pragma unroll
+          for (int e = 0; e < E; ++e) d16[e] = __float2bfloat16_rn(x[r][e] - __bfloat162float(__float2bfloat16_rn(x[r][e])));
+        }
       }
     }
   } else {
@@ -144,23 +149,46 @@ __global__ void __launch_bounds__(kPrefillThreads) prefill_phi_kernel(const Pref
 // 1c. (gated contexts) running sums of log(gate) over the chunk's delayed tokens: gcum[i] = sum over the valid delayed
 // indices ii <= i of log gate(k'_ii).  exp(gcum[i] - gcum[ii]) is then the decay a delayed token ii has suffered when
 // delayed token i has entered the state, exp(gcum[i]) the decay of the state the chunk started from.
-// One thread per unit, sequential over the chunk (C <= 1024).
+// One warp per (unit, chunk), 32 tokens at a time by a warp scan, all of the chunk's gates asked for first (one thread per
+// unit, token after token, took 92 us for 256 tokens of 256 units: a memory round trip and a logarithm each).
 template <typename T, int D>
 __global__ void __launch_bounds__(kPrefillThreads) prefill_gcum_kernel(const PrefillParams p) {
-  const int64_t u = int64_t(blockIdx.x) * kPrefillThreads + threadIdx.x;
+  const int lane = threadIdx.x & 31;
+  const int64_t uc = (int64_t(blockIdx.x) * kPrefillThreads + threadIdx.x) >> 5;
   const int64_t units = int64_t(p.layer_count) * p.B * p.Hkv;
-  if (u >= units) return;
+  if (uc >= units * p.nsub) return;
+  const int64_t u = uc / p.nsub;
+  const int chunk_c0 = int(uc - u * p.nsub) * p.SC, chunk_n = min(p.SC, p.C - chunk_c0);
   const int g = int(u % p.Hkv);
   const int b = int((u / p.Hkv) % p.B);
   const int lrel = int(u / (int64_t(p.Hkv) * p.B));
   const LayerDev ld = p.layers[p.layer_begin + lrel];
   if (!ld.evicts) return;
   const RowSource<T> src = make_source<T, D>(p, ld, lrel, b, g);
+  const int64_t first = p.n0 + p.c0 + chunk_c0 - ld.wlin;   // delayed token of chunk index 0
+  float *out = p.gcum + size_t(u) * p.Cmax + chunk_c0;
+  constexpr int kAhead = 8;
   float run = 0.f;
-  for (int i = 0; i < p.C; ++i) {
-    const int64_t j = p.n0 + p.c0 + i - ld.wlin;
-    if (j >= 0) run += logf(src.gate(j));
-    p.gcum[size_t(u) * p.Cmax + i] = run;
+  for (int i0 = 0; i0 < chunk_n; i0 += 32 * kAhead) {
+    float x[kAhead];
+#pragma unroll
+    for (int a = 0; a < kAhead; ++a) {
+      const int i = i0 + a * 32 + lane;
+      x[a] = i < chunk_n && first + i >= 0 ? src.gate(first + i) : 1.f;
+    }
+#pragma unroll
+    for (int a = 0; a < kAhead; ++a) {
+      float s = logf(x[a]);
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const float y = __shfl_up_sync(0xffffffffu, s, o);
+        if (lane >= o) s += y;
+      }
+      s += run;
+      const int i = i0 + a * 32 + lane;
+      if (i < chunk_n) out[i] = s;
+      run = __shfl_sync(0xffffffffu, s, 31);
+    }
   }
 }
 
@@ -572,9 +600,11 @@ int launch_prefill(glide_ctx *ctx, int layer_begin, int layer_count, int64_t T, 
   p.gcum = reinterpret_cast<float *>(ctx->ws + ctx->off_gcum);
   const int64_t units = int64_t(layer_count) * p.B * p.Hkv;
   const bool plain = ctx->cfg.phi == GLIDE_PHI_SOFTMAX && !ctx->cfg.gated;   // what the tensor-core kernels compute
+  const bool plain_gated = ctx->cfg.gated && ctx->cfg.phi == GLIDE_PHI_SOFTMAX && ctx->cfg.merge == GLIDE_MERGE_SHARED;
   int impl = ctx->cfg.prefill_impl;
   // the tcgen05 kernel also takes the learned map under the shared normaliser (its two halves as two linear parts)
-  const bool tc_kind = !ctx->cfg.gated && (ctx->cfg.phi == GLIDE_PHI_SOFTMAX || ctx->cfg.merge == GLIDE_MERGE_SHARED);
+  // and, under the shared normaliser, gates with the plain map (its operands split in two)
+  const bool tc_kind = ctx->cfg.gated ? plain_gated : (ctx->cfg.phi == GLIDE_PHI_SOFTMAX || ctx->cfg.merge == GLIDE_MERGE_SHARED);
   if (impl == GLIDE_PREFILL_AUTO)
     impl = (tc_kind && prefill_attn_mma_supported(ctx) && ctx->cfg.decode_impl != GLIDE_DECODE_FMA) ? GLIDE_PREFILL_TCGEN05
                                                                                                 : GLIDE_PREFILL_FMA;
@@ -591,7 +621,7 @@ int launch_prefill(glide_ctx *ctx, int layer_begin, int layer_count, int64_t T, 
                        prefill_attn_mma_supported(ctx) && ctx->cfg.merge == GLIDE_MERGE_SHARED;
   // carry of the chunk scan: tensor cores with an error-free three-way bf16 split of phi(K') (bf16, d = 128), or the
   // CUDA-core kernel (fp32 I/O, d = 64, and whenever the CUDA-core prefill is asked for)
-  const bool state_mma = !ctx->cfg.gated && prefill_state_mma_supported(ctx) && impl != GLIDE_PREFILL_FMA;   // (either feature map)
+  const bool state_mma = prefill_state_mma_supported(ctx) && impl != GLIDE_PREFILL_FMA;   // (either feature map, gated or not)
   auto evicts_in = [&](int first, int count) {
     bool any = false;
     for (int l = first; l < first + count; ++l) any = any || ctx->layers[l].evicts;
@@ -625,6 +655,7 @@ int launch_prefill(glide_ctx *ctx, int layer_begin, int layer_count, int64_t T, 
         s.v = static_cast<const unsigned char *>(v) + seqs * p.Hkv * D * elem;
         if (q) s.q = static_cast<const unsigned char *>(q) + seqs * p.H * D * elem;
         if (out) s.out = static_cast<unsigned char *>(out) + seqs * p.H * D * elem;
+        if (gate) s.gate = gate + seqs * p.Hkv;
         s.c0 = c0;
         s.C = int(std::min<int64_t>(int64_t(nsub_max) * p.SC, T - c0));
         s.nsub = (s.C + p.SC - 1) / p.SC;
@@ -638,6 +669,8 @@ int launch_prefill(glide_ctx *ctx, int layer_begin, int layer_count, int64_t T, 
           } else {
             prefill_phi_kernel<TT, D, DP><<<warp4_blocks, kPrefillThreads, 0, stream>>>(s);
           }
+          if (p.gated)
+            prefill_gcum_kernel<TT, D><<<unsigned((units * s.nsub * 32 + kPrefillThreads - 1) / kPrefillThreads), kPrefillThreads, 0, stream>>>(s);
           if (out && s.phiq16 && launch_prefill_project(ctx, s, false, stream) != GLIDE_OK) return GLIDE_ERR_CUDA;
           if (out && p.merge != GLIDE_MERGE_SHARED)   // (before the carry: the chunk sums overwrite rows of phi(K'))
             prefill_zcum_kernel<D><<<unsigned((units * s.nsub * D + kPrefillThreads - 1) / kPrefillThreads), kPrefillThreads, 0, stream>>>(s);
@@ -669,7 +702,7 @@ int launch_prefill(glide_ctx *ctx, int layer_begin, int layer_count, int64_t T, 
         prefill_phi_kernel<TT, D, DP><<<warp4_blocks, kPrefillThreads, 0, stream>>>(p);
       }
       if (any_evicts && p.gated)
-        prefill_gcum_kernel<TT, D><<<unsigned((units + kPrefillThreads - 1) / kPrefillThreads), kPrefillThreads, 0, stream>>>(p);
+        prefill_gcum_kernel<TT, D><<<unsigned((units * 32 + kPrefillThreads - 1) / kPrefillThreads), kPrefillThreads, 0, stream>>>(p);
       if (out) {
         if (use_mma) {
           if (launch_prefill_attn_mma(ctx, p, stream) != GLIDE_OK) return GLIDE_ERR_CUDA;

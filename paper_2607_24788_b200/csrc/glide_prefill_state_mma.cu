@@ -55,6 +55,13 @@ __device__ __forceinline__ void split3(float x0, float x1, uint32_t &hi, uint32_
   lo = *reinterpret_cast<const uint32_t *>(&l);
 }
 
+// the bf16 copy of two values of S (gated: hi here and lo `lo_half` elements further on)
+__device__ __forceinline__ void store_s16(__nv_bfloat16 *at, size_t lo_half, float x, float y) {
+  const __nv_bfloat162 h = __floats2bfloat162_rn(x, y);
+  *reinterpret_cast<__nv_bfloat162 *>(at) = h;
+  if (lo_half) *reinterpret_cast<__nv_bfloat162 *>(at + lo_half) = __floats2bfloat162_rn(x - __low2float(h), y - __high2float(h));
+}
+
 // PARTIAL (passes of several chunks): the chunk's own sum goes to the scratch rows that the CTA has just consumed instead
 // of S (64 state rows x 128 values = 128 scratch rows x the CTA's 64 columns, z in row 128: chunks of more than 128
 // tokens), and prefill_scan_kernel adds the sums up in chunk order.  Otherwise S is updated in place, and its value
@@ -63,6 +70,7 @@ template <bool PARTIAL>
 __global__ void __launch_bounds__(kThreads) prefill_state_mma_kernel(const PrefillParams p) {
   using bf16 = __nv_bfloat16;
   __shared__ __align__(16) unsigned char stage[2][kPhiBytes + kVBytes];
+  __shared__ float decay[2][kTok];   // gated: what each staged token has decayed to by the end of the chunk
   const int blocks_per_unit = p.dp / kRowsPerCta;   // rows of S: d, or 2 d with the learned feature map
   const int64_t uc = blockIdx.x / blocks_per_unit;   // (unit, chunk of the pass)
   const int rb = blockIdx.x % blocks_per_unit;
@@ -91,6 +99,8 @@ __global__ void __launch_bounds__(kThreads) prefill_state_mma_kernel(const Prefi
 #pragma unroll
   for (int n = 0; n < kD / 8; ++n) acc[n][0] = acc[n][1] = acc[n][2] = acc[n][3] = 0.f;
   float zacc = 0.f;   // threads 0..63: z of row rb*64 + tid
+  const float *gc = p.gated ? p.gcum + size_t(u) * p.Cmax + chunk_c0 : nullptr;
+  const float g_end = gc ? gc[chunk_n - 1] : 0.f;
 
   // tokens past the chunk's end are filled with zeros
   auto issue = [&](int buf, int i0) {
@@ -107,6 +117,7 @@ __global__ void __launch_bounds__(kThreads) prefill_state_mma_kernel(const Prefi
       cp16(sv + uint32_t(i * kVStride + c * 16), row + c * 8, i < nt);
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
+    if (tid < kTok) decay[buf][tid] = (gc && tid < nt) ? expf(g_end - gc[i0 + tid]) : 1.f;   // (rows past the end are zero)
   };
   issue(0, i_lo);
   int buf = 0;
@@ -126,10 +137,11 @@ __global__ void __launch_bounds__(kThreads) prefill_state_mma_kernel(const Prefi
       // a1: (gid + 8, ..), a2: (gid, 2 tig + 8 + {0,1}), a3: (gid + 8, ..)
       const float *base = sphi + (kk * 16 + 2 * tig) * kPhiStride + warp * 16 + gid;
       uint32_t ah[4], am[4], al[4];
-      split3(base[0], base[kPhiStride], ah[0], am[0], al[0]);
-      split3(base[8], base[kPhiStride + 8], ah[1], am[1], al[1]);
-      split3(base[8 * kPhiStride], base[9 * kPhiStride], ah[2], am[2], al[2]);
-      split3(base[8 * kPhiStride + 8], base[9 * kPhiStride + 8], ah[3], am[3], al[3]);
+      const float *dk = decay[buf] + kk * 16 + 2 * tig;   // (without gates: exact products with 1)
+      split3(base[0] * dk[0], base[kPhiStride] * dk[1], ah[0], am[0], al[0]);
+      split3(base[8] * dk[0], base[kPhiStride + 8] * dk[1], ah[1], am[1], al[1]);
+      split3(base[8 * kPhiStride] * dk[8], base[9 * kPhiStride] * dk[9], ah[2], am[2], al[2]);
+      split3(base[8 * kPhiStride + 8] * dk[8], base[9 * kPhiStride + 8] * dk[9], ah[3], am[3], al[3]);
       const int krow = kk * 16 + (lane & 7) + ((lane >> 3) & 1) * 8;
 #pragma unroll
       for (int dp = 0; dp < kD / 16; ++dp) {
@@ -146,7 +158,7 @@ __global__ void __launch_bounds__(kThreads) prefill_state_mma_kernel(const Prefi
     }
     if (tid < kRowsPerCta) {
 #pragma unroll 8
-      for (int i = 0; i < kTok; ++i) zacc += sphi[i * kPhiStride + tid];
+      for (int i = 0; i < kTok; ++i) zacc = fmaf(sphi[i * kPhiStride + tid], decay[buf][i], zacc);
     }
     __syncthreads();   // the stage is refilled by the next iteration's issue
   }
@@ -164,7 +176,9 @@ __global__ void __launch_bounds__(kThreads) prefill_state_mma_kernel(const Prefi
     return;
   }
   float *Sb = reinterpret_cast<float *>(p.ws + ld.S) + size_t(ub) * p.dp * kD + size_t(rb * kRowsPerCta + warp * 16) * kD;
-  // the halves of a state with 2 d rows are units_cap units apart in the bf16 copy
+  // the halves of a state with 2 d rows are units_cap units apart in the bf16 copy, as are hi and lo of a gated one
+  const size_t lo_half = p.gated ? size_t(p.units_cap) * kD * kD : 0;
+  const float dec_all = gc ? expf(g_end) : 1.f;   // the state the chunk started from, after the whole chunk has entered
   bf16 *s16 = p.s16 ? reinterpret_cast<bf16 *>(p.s16) + (size_t(rb * kRowsPerCta / kD) * p.units_cap + u) * kD * kD +
                           size_t(rb * kRowsPerCta % kD + warp * 16) * kD
                     : nullptr;
@@ -175,16 +189,16 @@ __global__ void __launch_bounds__(kThreads) prefill_state_mma_kernel(const Prefi
       const size_t at = size_t(gid + h * 8) * kD + n * 8 + 2 * tig;
       float2 *dst = reinterpret_cast<float2 *>(Sb + at);
       float2 c = *dst;
-      if (s16) *reinterpret_cast<__nv_bfloat162 *>(s16 + at) = __floats2bfloat162_rn(c.x, c.y);
-      c.x += acc[n][2 * h];
-      c.y += acc[n][2 * h + 1];
+      if (s16) store_s16(s16 + at, lo_half, c.x, c.y);
+      c.x = fmaf(c.x, dec_all, acc[n][2 * h]);
+      c.y = fmaf(c.y, dec_all, acc[n][2 * h + 1]);
       *dst = c;
     }
   if (tid < kRowsPerCta) {
     float *zb = reinterpret_cast<float *>(p.ws + ld.z) + size_t(ub) * p.dp + rb * kRowsPerCta;
     const float z0 = zb[tid];
     if (s16) p.zsnap[size_t(u) * p.dp + rb * kRowsPerCta + tid] = z0;
-    zb[tid] = z0 + zacc;
+    zb[tid] = fmaf(z0, dec_all, zacc);
   }
 }
 
@@ -215,6 +229,10 @@ __global__ void __launch_bounds__(kThreads) prefill_scan_kernel(const PrefillPar
   bf16 *snap = p.s16 ? reinterpret_cast<bf16 *>(p.s16) + ((size_t(half) * p.units_cap + u * p.nsub) * kD + (r - half * kD)) * kD + col
                      : nullptr;
   float4 s = *Sp;
+  const size_t lo_half = p.gated ? size_t(p.units_cap) * kD * kD : 0;
+  // gated: what the state has decayed by over chunk k (tokens before the first delayed one count as gates of 1)
+  const float *gc = p.gated ? p.gcum + size_t(u) * p.Cmax - 1 : nullptr;
+  auto chunk_decay = [&](int k) { return gc ? expf(gc[min((k + 1) * p.SC, p.C)]) : 1.f; };
   constexpr int kAhead = 4;
   for (int k = k0; k < p.nsub; k += kAhead) {
     float4 x[kAhead];
@@ -225,14 +243,14 @@ __global__ void __launch_bounds__(kThreads) prefill_scan_kernel(const PrefillPar
     for (int a = 0; a < kAhead; ++a) {
       if (k + a >= p.nsub) break;
       if (snap) {
-        const __nv_bfloat162 lo = __floats2bfloat162_rn(s.x, s.y), hi = __floats2bfloat162_rn(s.z, s.w);
-        *reinterpret_cast<uint2 *>(snap + size_t(k + a) * kD * kD) =
-            make_uint2(*reinterpret_cast<const uint32_t *>(&lo), *reinterpret_cast<const uint32_t *>(&hi));
+        store_s16(snap + size_t(k + a) * kD * kD, lo_half, s.x, s.y);
+        store_s16(snap + size_t(k + a) * kD * kD + 2, lo_half, s.z, s.w);
       }
-      s.x += x[a].x;
-      s.y += x[a].y;
-      s.z += x[a].z;
-      s.w += x[a].w;
+      const float dec = chunk_decay(k + a);
+      s.x = fmaf(s.x, dec, x[a].x);
+      s.y = fmaf(s.y, dec, x[a].y);
+      s.z = fmaf(s.z, dec, x[a].z);
+      s.w = fmaf(s.w, dec, x[a].w);
     }
   }
   *Sp = s;
@@ -243,7 +261,7 @@ __global__ void __launch_bounds__(kThreads) prefill_scan_kernel(const PrefillPar
     float z = *zp;
     for (int k = k0; k < p.nsub; ++k) {
       if (snap) p.zsnap[(size_t(u) * p.nsub + k) * p.dp + rz] = z;
-      z += pz[size_t(k) * step];
+      z = fmaf(z, chunk_decay(k), pz[size_t(k) * step]);
     }
     *zp = z;
   }

@@ -102,7 +102,8 @@ __device__ __forceinline__ void issue_mma(bool leader, uint32_t tmem_d, uint32_t
   }
 }
 // the same product with the A operand in TMEM: lane = row, 32-bit column c = elements 2c (low half) and 2c+1 of
-// the row, 8 columns per k16 step; B MN-major in shared memory
+// the row, 8 columns per k16 step (PAIRS: two steps, then a gap of 16 columns); B MN-major in shared memory
+template <bool PAIRS>
 __device__ __forceinline__ void issue_mma_ts(bool leader, uint32_t tmem_d, uint32_t tmem_a, uint32_t b_tile, bool accumulate) {
   const uint32_t idesc = make_idesc(true);
   const uint32_t b0 = desc_lo(b_tile, kBoxBytes);
@@ -112,7 +113,7 @@ __device__ __forceinline__ void issue_mma_ts(bool leader, uint32_t tmem_d, uint3
       asm volatile(
           "{\n\t.reg .pred p;\n\t.reg .b64 b;\n\tsetp.ne.b32 p, %4, 0;\n\tmov.b64 b, {%2, %5};\n\t"
           "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], b, %3, p;\n\t}" ::"r"(tmem_d),
-          "r"(tmem_a + ks * 8), "r"(b0 + uint32_t(ks * 2048 >> 4)), "r"(idesc), "r"((accumulate || ks > 0) ? 1u : 0u), "r"(kDescHi)
+          "r"(tmem_a + (PAIRS ? (ks >> 1) * 32 + (ks & 1) * 8 : ks * 8)), "r"(b0 + uint32_t(ks * 2048 >> 4)), "r"(idesc), "r"((accumulate || ks > 0) ? 1u : 0u), "r"(kDescHi)
           : "memory");
   }
 }
@@ -262,7 +263,10 @@ struct CallMaps {
   CUtensorMap k128, v128;   // boxes of a whole 128-key tile
 };
 
-enum : int { kModeShared = 0, kModeSum = 1, kModeLearned = 2 };
+// Gated: the weights stay fp32 quantities (the gated recurrence has no other tensor-core form whose precision it could
+// share): every A operand (P, phi(Q), C) and the state and phi(K') are split into two bf16 terms, hi + lo, and the
+// products of two split operands leave out lo x lo (2^-18 of the result).
+enum : int { kModeShared = 0, kModeSum = 1, kModeLearned = 2, kModeGated = 3 };
 
 // bit i: column c + i of a key tile is valid for a row whose valid columns are lo .. hi
 __device__ __forceinline__ uint32_t column_mask(int c, int lo, int hi) {
@@ -283,6 +287,11 @@ __device__ __forceinline__ void add2(float &a0, float &a1, float x0, float x1) {
       : "+f"(a0), "+f"(a1)
       : "f"(x0), "f"(x1));
 }
+// x0, x1 -> bf16 pairs hi (rounded) and lo (the rounded rest)
+__device__ __forceinline__ void split2(float x0, float x1, uint32_t &hi, uint32_t &lo) {
+  hi = pack_bf16x2(x0, x1);
+  lo = pack_bf16x2(x0 - __uint_as_float(hi << 16), x1 - __uint_as_float(hi & 0xffff0000u));
+}
 __device__ __forceinline__ void prefetch_map(const void *m) {
   asm volatile("prefetch.tensormap [%0];" ::"l"(m) : "memory");
 }
@@ -293,6 +302,8 @@ prefill_attn_tc_kernel(const PrefillParams p, const CUtensorMap *ring_maps, cons
   using bf16 = __nv_bfloat16;
   constexpr bool SUM = MODE == kModeSum;          // sum of two normalised terms instead of the shared normaliser
   constexpr bool PHI2 = MODE == kModeLearned;
+  constexpr bool GATED = MODE == kModeGated;
+  constexpr bool TWO = PHI2 || GATED;             // two tiles of phi(Q), S and phi(K'): the map's halves, or hi and lo
   constexpr int TOKT = kRows / G;    // tokens per row tile
   constexpr int TOKC = 2 * TOKT;     // tokens per CTA
   extern __shared__ __align__(1024) unsigned char smem_raw[];
@@ -429,13 +440,14 @@ prefill_attn_tc_kernel(const PrefillParams p, const CUtensorMap *ring_maps, cons
   // copy of the unit's state, the next two the phi(K') tiles of the first two intra-chunk steps, the last two the V'
   // tiles of those steps; all are on their way while the last key tiles are still being processed.  Later steps take the
   // buffers of the step before the previous one.
-  // Learned map: twice the operands, so they come when every window product has completed: phi- of the two row tiles in
-  // buffers 0 and 1 (phi+ in the Q tiles), the state halves and then the phi(K') halves of each step in 2 and 3, V' in 4.
+  // Learned map and gated: twice the operands, so they come when every window product has completed: phi- (or phi's lo) of
+  // the two row tiles in buffers 0 and 1 (phi+ or hi in the Q tiles), the state's two tiles and then the two phi(K') tiles
+  // of each step in 2 and 3, V' in 4.
   auto late_seq = [&](int k) { return 2 * n_tiles - kStages + k; };
   auto late_slot = [&](int k) { const int sq = late_seq(k); return sq >= 0 ? sq % kStages : sq + kStages; };
-  auto slot_state = [&]() { return PHI2 ? 2 : late_slot(0); };
-  auto slot_pk = [&](int t) { return PHI2 ? 2 : late_slot(1 + (t & 1)); };
-  auto slot_vp = [&](int t) { return PHI2 ? 4 : late_slot(3 + (t & 1)); };
+  auto slot_state = [&]() { return TWO ? 2 : late_slot(0); };
+  auto slot_pk = [&](int t) { return TWO ? 2 : late_slot(1 + (t & 1)); };
+  auto slot_vp = [&](int t) { return TWO ? 4 : late_slot(3 + (t & 1)); };
 
   if (tid < kSoftmaxThreads) {
     // =========================== softmax threads: one row each ===========================
@@ -464,6 +476,19 @@ prefill_attn_tc_kernel(const PrefillParams p, const CUtensorMap *ring_maps, cons
 #pragma unroll
         for (int i = 0; i < 32; ++i) r[i] = __float_as_uint(__uint_as_float(r[i]) * f);
         tmem_st32(tO + c0, r);
+      }
+    };
+    // weights of columns c .. c + 31 over columns c / 2 .. c / 2 + 15; gated: hi over c .. c + 15, lo (first half of x)
+    // over c + 16 .. c + 31
+    auto store_p = [&](int c, const uint32_t (&pk)[16], const uint32_t (&x)[32]) {
+      if constexpr (GATED) {
+        uint32_t lo[16];
+#pragma unroll
+        for (int e = 0; e < 16; ++e) lo[e] = x[e];
+        tmem_st16(tS + c, pk);
+        tmem_st16(tS + c + 16, lo);
+      } else {
+        tmem_st16(tS + (c >> 1), pk);
       }
     };
     // One key tile: maximum, reference, weights.  Tiles without a masked key keep their loops unrolled; the others, one or
@@ -530,10 +555,16 @@ prefill_attn_tc_kernel(const PrefillParams p, const CUtensorMap *ring_maps, cons
           for (int e = 0; e < 16; ++e) {
             float a0, a1;
             fma2(a0, a1, __uint_as_float(x[e * 2]), __uint_as_float(x[e * 2 + 1]), p.scale_log2, -mr);
-            pk[e] = pack_bf16x2(ex2(a0), ex2(a1));
-            add2(sum0, sum1, __uint_as_float(pk[e] << 16), __uint_as_float(pk[e] & 0xffff0000u));
+            if constexpr (GATED) {
+              a0 = ex2(a0), a1 = ex2(a1);
+              add2(sum0, sum1, a0, a1);
+              split2(a0, a1, pk[e], x[e]);   // (x[e] has been read: element e comes from x[2 e] and x[2 e + 1])
+            } else {
+              pk[e] = pack_bf16x2(ex2(a0), ex2(a1));
+              add2(sum0, sum1, __uint_as_float(pk[e] << 16), __uint_as_float(pk[e] & 0xffff0000u));
+            }
           }
-          tmem_st16(tS + (c >> 1), pk);
+          store_p(c, pk, x);
         }
       }
       tmem_wait_st();
@@ -583,6 +614,8 @@ prefill_attn_tc_kernel(const PrefillParams p, const CUtensorMap *ring_maps, cons
         if (PHI2 || (SUM && need_state)) mbar_wait(smem_u32(&sm.bar_state), 0u, failed);   // phi(Q); z
         unsigned char *tileX = sm.q[X];
         float dot = 0.f;
+        const float g_own = GATED ? p.gcum[size_t(uc) * p.SC + min(tl, chunk_n - 1)] : 0.f;
+        const float dec0 = GATED ? ex2(g_own * kLog2e) : 1.f;   // what the chunk-start state has decayed to
         if constexpr (!PHI2) {
           // this row of Q is still in the shared tile, and every S product of X has completed: phi(q) takes its place,
           // eight values at a time: maximum, then exponentials (left as bf16) and their sum, then the scaled values
@@ -615,7 +648,7 @@ prefill_attn_tc_kernel(const PrefillParams p, const CUtensorMap *ring_maps, cons
               }
               w4[e] = pack_bf16x2(e0, e1);
             }
-            *at = make_uint4(w4[0], w4[1], w4[2], w4[3]);
+            if (!GATED) *at = make_uint4(w4[0], w4[1], w4[2], w4[3]);
           }
           // shared normaliser: phi(q) 2^-M;  sum of terms: phi(q) / (phi(q) . z_row) = e / (e . z_row)
           const float dz = dz0 + dz1;
@@ -623,6 +656,32 @@ prefill_attn_tc_kernel(const PrefillParams p, const CUtensorMap *ring_maps, cons
           const bool with_z = !SUM && need_state;
           if (with_z) mbar_wait(smem_u32(&sm.bar_state), 0u, failed);   // z has landed
           float dot1 = 0.f;
+          if constexpr (GATED) {
+            // the values in fp32 (the exponentials once more), hi in place, lo in a buffer of the finished window part
+            mbar_wait(smem_u32(&sm.bar_done), 0u, failed);
+#pragma unroll 2
+            for (int c = 0; c < 16; ++c) {
+              uint4 *at = reinterpret_cast<uint4 *>(tileX + sw128(row, c));
+              const uint4 v4 = *at;
+              uint32_t w4[4] = {v4.x, v4.y, v4.z, v4.w}, lo4[4];
+#pragma unroll
+              for (int e = 0; e < 4; ++e) {
+                float a0, a1;
+                fma2(a0, a1, __uint_as_float(w4[e] << 16), __uint_as_float(w4[e] & 0xffff0000u), kLog2e, -mxl);
+                a0 = ex2(a0) * sc, a1 = ex2(a1) * sc;
+                split2(a0, a1, w4[e], lo4[e]);
+                if (with_z) {
+                  const float2 zz = *reinterpret_cast<const float2 *>(&sm.z[c * 8 + e * 2]);
+                  dot = fmaf(a0, zz.x, dot);
+                  dot1 = fmaf(a1, zz.y, dot1);
+                }
+              }
+              *at = make_uint4(w4[0], w4[1], w4[2], w4[3]);
+              *reinterpret_cast<uint4 *>(sm.kv[X] + sw128(row, c)) = make_uint4(lo4[0], lo4[1], lo4[2], lo4[3]);
+            }
+            dot = (dot + dot1) * dec0;
+            dot1 = 0.f;
+          } else
 #pragma unroll 4
           for (int c = 0; c < 16; ++c) {
             uint4 *at = reinterpret_cast<uint4 *>(tileX + sw128(row, c));
@@ -671,6 +730,24 @@ prefill_attn_tc_kernel(const PrefillParams p, const CUtensorMap *ring_maps, cons
         tc_fence_before();
         mbar_arrive(smem_u32(&sm.bar_p[X]));
         PF_CLK(10);
+        if (GATED && need_state && ok) {
+          // phi(q) S is in the S columns: it has decayed by dec0 since the chunk began, row by row, so it is added here
+          ok = wait_s();
+#pragma unroll 1
+          for (int c0 = 0; c0 < kD && ok; c0 += 32) {
+            uint32_t o[32], x[32];
+            tmem_ld32_nowait(tS + c0, x);
+            if (windowed) tmem_ld32_nowait(tO + c0, o);
+            tmem_wait_ld(x);
+            if (windowed) tmem_wait_ld(o);
+#pragma unroll
+            for (int i = 0; i < 32; ++i)
+              o[i] = __float_as_uint(fmaf(__uint_as_float(x[i]), dec0, windowed ? __uint_as_float(o[i]) : 0.f));
+            tmem_st32(tO + c0, o);
+          }
+          tc_fence_before();
+          mbar_arrive(smem_u32(&sm.bar_p[X]));
+        }
         // C row -> bf16 over the same TMEM columns, masked to the delayed tokens j' <= i of the row (the values already
         // carry 2^-M); the row's weight sum goes to l
         for (int t = 0; t < n_itiles && ok; ++t) {
@@ -691,6 +768,8 @@ prefill_attn_tc_kernel(const PrefillParams p, const CUtensorMap *ring_maps, cons
               uint32_t (&x)[32] = r[hf];
               const int c = c0 + hf * 32;
               uint32_t pk[16];
+              // the running log-gates of the 32 columns' tokens, one per lane
+              const float gl = GATED ? __ldg(p.gcum + size_t(uc) * p.SC + min(i0 + c + lane, chunk_n - 1)) : 0.f;
               tmem_wait_ld(x);
               if (hf == 0) tmem_ld32_nowait(tS + c + 32, r[1]);
               else if (c + 32 < kKT) tmem_ld32_nowait(tS + c + 32, r[0]);
@@ -701,10 +780,20 @@ prefill_attn_tc_kernel(const PrefillParams p, const CUtensorMap *ring_maps, cons
               }
 #pragma unroll
               for (int e = 0; e < 16; ++e) {
-                pk[e] = pack_bf16x2(__uint_as_float(x[e * 2]), __uint_as_float(x[e * 2 + 1]));
-                add2(sum0, sum1, __uint_as_float(pk[e] << 16), __uint_as_float(pk[e] & 0xffff0000u));
+                if constexpr (GATED) {
+                  // a delayed token ii <= i has decayed by exp(g_own - gc[ii]) <= 1 (columns past the row's own are zero:
+                  // the limit keeps 0 x inf out)
+                  const float g0 = __shfl_sync(0xffffffffu, gl, e * 2), g1 = __shfl_sync(0xffffffffu, gl, e * 2 + 1);
+                  const float a0 = __uint_as_float(x[e * 2]) * ex2(fminf(g_own - g0, 0.f) * kLog2e);
+                  const float a1 = __uint_as_float(x[e * 2 + 1]) * ex2(fminf(g_own - g1, 0.f) * kLog2e);
+                  add2(sum0, sum1, a0, a1);
+                  split2(a0, a1, pk[e], x[e]);
+                } else {
+                  pk[e] = pack_bf16x2(__uint_as_float(x[e * 2]), __uint_as_float(x[e * 2 + 1]));
+                  add2(sum0, sum1, __uint_as_float(pk[e] << 16), __uint_as_float(pk[e] & 0xffff0000u));
+                }
               }
-              tmem_st16(tS + (c >> 1), pk);
+              store_p(c, pk, x);
             }
           }
           tmem_wait_st();
@@ -771,6 +860,25 @@ prefill_attn_tc_kernel(const PrefillParams p, const CUtensorMap *ring_maps, cons
     auto commit = [&](uint64_t &bar) {
       if (leader) mma_commit(smem_u32(&bar));
     };
+    // O_X (+)= A_X B with A_X in the S columns of X: packed bf16 behind one another, or hi and lo in turn every 32 columns
+    auto issue_ts = [&](int x, uint32_t b_tile, bool accumulate) {
+      if (!GATED) {
+        issue_mma_ts<false>(leader, tm + 256 + x * 128, tm + x * 128, b_tile, accumulate);
+      } else {
+        issue_mma_ts<true>(leader, tm + 256 + x * 128, tm + x * 128, b_tile, accumulate);
+        issue_mma_ts<true>(leader, tm + 256 + x * 128, tm + x * 128 + 16, b_tile, true);
+      }
+    };
+    // D (+)= [Q tile of X | buffer X] . [buffer 2 | buffer 3], the map's halves or hi and lo
+    auto issue_two = [&](int x, uint32_t d, bool b_mn, bool accumulate) {
+      issue_mma(leader, d, q_addr(x), kv_addr(2), b_mn, accumulate);
+      if (GATED) {
+        issue_mma(leader, d, kv_addr(x), kv_addr(2), b_mn, true);
+        issue_mma(leader, d, q_addr(x), kv_addr(3), b_mn, true);
+      } else {
+        issue_mma(leader, d, kv_addr(x), kv_addr(3), b_mn, true);
+      }
+    };
     PF_LAP_INIT();
     // t = -1: the first S products; then per key tile P V of the tile and S of the next one
     for (int t = -1; t < n_tiles && ok; ++t) {
@@ -788,7 +896,7 @@ prefill_attn_tc_kernel(const PrefillParams p, const CUtensorMap *ring_maps, cons
           PF_LAP(18);
           if (!wait_p(x)) break;
           PF_LAP(19);
-          issue_mma_ts(leader, tm + 256 + x * 128, tm + x * 128, kv_addr(seqV % kStages), t > tf);
+          issue_ts(x, kv_addr(seqV % kStages), t > tf);
           if (t + 1 == te) commit(sm.bar_s[x]);   // the window part of O_X
         }
         if (t + 1 >= tf && t + 1 < te) {
@@ -803,7 +911,7 @@ prefill_attn_tc_kernel(const PrefillParams p, const CUtensorMap *ring_maps, cons
       }
     }
     if (ok) commit(sm.bar_done);
-    if (ok && linear && !PHI2) {
+    if (ok && linear && !TWO) {
       // per row tile: phi(Q) S (inter-chunk) and the first C = phi(Q) phi(K')^T in one batch
 #pragma unroll 1
       for (int x = 0; x < nx && ok; ++x) {
@@ -820,39 +928,39 @@ prefill_attn_tc_kernel(const PrefillParams p, const CUtensorMap *ring_maps, cons
 #pragma unroll 1
         for (int x = 0; x < nx && ok; ++x) {
           if (!wait_p(x)) break;
-          issue_mma_ts(leader, tm + 256 + x * 128, tm + x * 128, kv_addr(slot_vp(t)), (x ? te1 > tf1 : te0 > tf0) || need_state || t > 0);
+          issue_ts(x, kv_addr(slot_vp(t)), (x ? te1 > tf1 : te0 > tf0) || need_state || t > 0);
           if (t + 1 < n_itiles) issue_mma(leader, tm + x * 128, q_addr(x), kv_addr(slot_pk(t + 1)), false, false);
           commit(sm.bar_s[x]);
         }
         if (ok) commit(sm.bar_lfree[t & 1]);   // V'(t) has been read, and phi(K')(t) before it
       }
     }
-    if (ok && linear && PHI2) {
+    if (ok && linear && TWO) {
       // phi+ S+ and phi- S-, then per step C = phi+ phi+(K')^T + phi- phi-(K')^T (accumulated before the causal mask)
-      // and C V'; the phi(K') halves of a step take the buffers of the state, or of the step before
+      // and C V'; the phi(K') halves of a step take the buffers of the state, or of the step before.  Gated: phi(Q) S goes
+      // to the S columns, from where the softmax threads add it to O with the row's decay.
+      if (GATED && need_state) wait(sm.bar_state, 0u);
 #pragma unroll 1
       for (int x = 0; x < nx && ok; ++x) {
         if (!wait_p(x)) break;
-        if (need_state) {
-          issue_mma(leader, tm + 256 + x * 128, q_addr(x), kv_addr(2), true, x ? te1 > tf1 : te0 > tf0);
-          issue_mma(leader, tm + 256 + x * 128, kv_addr(x), kv_addr(3), true, true);
-        }
-        if (n_itiles == 0) commit(sm.bar_s[x]);
+        if (need_state) issue_two(x, GATED ? tm + x * 128 : tm + 256 + x * 128, true, !GATED && (x ? te1 > tf1 : te0 > tf0));
+        if (GATED && need_state) commit(sm.bar_s[x]);
       }
       if (ok) commit(sm.bar_lfree[0]);
+#pragma unroll 1
+      for (int x = 0; GATED && need_state && x < nx && ok; ++x) wait_p(x);   // the state's part has left the S columns
       for (int t = 0; t < n_itiles && ok; ++t) {
         wait(sm.bar_pk[0], uint32_t(t) & 1u);
 #pragma unroll 1
         for (int x = 0; x < nx && ok; ++x) {
-          issue_mma(leader, tm + x * 128, q_addr(x), kv_addr(2), false, false);
-          issue_mma(leader, tm + x * 128, kv_addr(x), kv_addr(3), false, true);
+          issue_two(x, tm + x * 128, false, false);
           commit(sm.bar_s[x]);
         }
         if (ok) wait(sm.bar_vp[0], uint32_t(t) & 1u);
 #pragma unroll 1
         for (int x = 0; x < nx && ok; ++x) {
           if (!wait_p(x)) break;
-          issue_mma_ts(leader, tm + 256 + x * 128, tm + x * 128, kv_addr(4), (x ? te1 > tf1 : te0 > tf0) || need_state || t > 0);
+          issue_ts(x, kv_addr(4), (x ? te1 > tf1 : te0 > tf0) || need_state || t > 0);
           if (t + 1 == n_itiles) commit(sm.bar_s[x]);
         }
         if (ok) commit(sm.bar_lfree[0]);
@@ -886,7 +994,7 @@ prefill_attn_tc_kernel(const PrefillParams p, const CUtensorMap *ring_maps, cons
 #pragma unroll 1
     for (int job = 0; job < n_jobs; ++job) {
       if (job == n_window) {
-        if (lane == 0 && !PHI2) {
+        if (lane == 0 && !TWO) {
           // the bf16 state (with z), then the phi(K') tiles of the first two intra-chunk steps
           const int n_late = 1 + (n_itiles < 2 ? n_itiles : 2);
 #pragma unroll 1
@@ -901,25 +1009,26 @@ prefill_attn_tc_kernel(const PrefillParams p, const CUtensorMap *ring_maps, cons
             tma_tile(kv_addr(late_slot(k)), k == 0 ? map_s16 : map_pk, k == 0 ? int(uc) * kD : int(uc) * p.SC + it0 + (k - 1) * kKT, bar);
           }
         }
-        if (lane == 0 && PHI2) {
+        if (lane == 0 && TWO && (PHI2 || need_state)) {
           const uint32_t bar = smem_u32(&sm.bar_state);
           const int rows_q = int(p.units_cap) * p.SC * G, rows_s = int(p.units_cap) * kD;
           ok = mbar_wait(smem_u32(&sm.bar_done), 0u, failed);
-          if (ok && n_tiles == 0) {                // no window: phi+ takes the place of Q when Q's copies have landed
+          if (PHI2 && ok && n_tiles == 0) {        // no window: phi+ takes the place of Q when Q's copies have landed
             ok = mbar_wait(smem_u32(&sm.bar_q[0]), 0u, failed);
             if (ok && hasB) ok = mbar_wait(smem_u32(&sm.bar_q[1]), 0u, failed);
           }
           if (ok) {
-            mbar_expect_tx(bar, (hasB ? 4u : 2u) * kTileBytes + (need_state ? 2u * kTileBytes + uint32_t(2 * kD * sizeof(float)) : 0u));
+            const uint32_t zbytes = uint32_t((PHI2 ? 2 : 1) * kD * sizeof(float));
+            mbar_expect_tx(bar, (PHI2 ? (hasB ? 4u : 2u) * kTileBytes : 0u) + (need_state ? 2u * kTileBytes + zbytes : 0u));
 #pragma unroll 1
-            for (int i = 0; i < (hasB ? 4 : 2); ++i) {
+            for (int i = 0; PHI2 && i < (hasB ? 4 : 2); ++i) {
               const int x = i >> 1, hf = i & 1;
               tma_tile(hf == 0 ? q_addr(x) : kv_addr(x), map_pq, hf * rows_q + (int(uc) * p.SC + tok0 + x * TOKT) * G, bar);
             }
             if (need_state) {
               tma_tile(kv_addr(2), map_s16, int(uc) * kD, bar);
               tma_tile(kv_addr(3), map_s16, rows_s + int(uc) * kD, bar);
-              bulk_load(smem_u32(sm.z), p.zsnap + size_t(uc) * 2 * kD, uint32_t(2 * kD * sizeof(float)), bar);
+              bulk_load(smem_u32(sm.z), p.zsnap + size_t(uc) * p.dp, zbytes, bar);
             }
           }
         }
@@ -935,13 +1044,13 @@ prefill_attn_tc_kernel(const PrefillParams p, const CUtensorMap *ring_maps, cons
       const int ts = late ? job - n_window - 1 : job >> 1;       // intra-chunk step, or key tile
       const bool is_v = late || (job & 1);
       const int slot = late ? slot_vp(ts) : job % kStages;
-      const uint32_t bar = late ? smem_u32(&sm.bar_vp[PHI2 ? 0 : ts & 1]) : smem_u32(&sm.bar_full[slot]);
+      const uint32_t bar = late ? smem_u32(&sm.bar_vp[TWO ? 0 : ts & 1]) : smem_u32(&sm.bar_full[slot]);
       const int64_t j0 = late ? folded + it0 + int64_t(ts) * kKT : j_lo + int64_t(ts) * kKT;
       if (!late) {
         PF_LAP_INIT();
         if (job >= kStages) ok = mbar_wait(smem_u32(&sm.bar_free[slot]), uint32_t(job / kStages - 1) & 1u, failed);
         PF_LAP(20);
-      } else if (!PHI2) {
+      } else if (!TWO) {
         const int sq = late_seq(3 + ts);
         if (ts < 2) {
           if (sq >= 0) ok = mbar_wait(smem_u32(&sm.bar_free[sq % kStages]), uint32_t(sq / kStages) & 1u, failed);
@@ -953,7 +1062,7 @@ prefill_attn_tc_kernel(const PrefillParams p, const CUtensorMap *ring_maps, cons
             tma_tile(kv_addr(slot_pk(ts)), map_pk, int(uc) * p.SC + it0 + ts * kKT, pkb);
           }
         }
-      } else {   // learned map: the state's or the previous step's products have completed
+      } else {   // learned map, gated: the state's or the previous step's products have completed
         ok = mbar_wait(smem_u32(&sm.bar_lfree[0]), uint32_t(ts) & 1u, failed);
         if (ok && lane == 0) {
           const uint32_t pkb = smem_u32(&sm.bar_pk[0]);
@@ -1118,7 +1227,8 @@ int launch_prefill_attn_tc(glide_ctx *ctx, const PrefillParams &p, cudaStream_t 
       kern<<<unsigned(blocks), kThreads, smem, stream>>>(p, ring_maps, cm);
       return cudaGetLastError() == cudaSuccess ? GLIDE_OK : GLIDE_ERR_CUDA;
     };
-    if (p.phiq16) return run(prefill_attn_tc_kernel<G, kModeLearned>);   // (shared normaliser only)
+    if (p.gated) return run(prefill_attn_tc_kernel<G, kModeGated>);      // (shared normaliser only, both)
+    if (p.phiq16) return run(prefill_attn_tc_kernel<G, kModeLearned>);
     return p.merge == GLIDE_MERGE_SHARED ? run(prefill_attn_tc_kernel<G, kModeShared>) : run(prefill_attn_tc_kernel<G, kModeSum>);
   };
   switch (ctx->G) {

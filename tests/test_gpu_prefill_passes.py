@@ -1,0 +1,25 @@
+"""Prefill passes of the tensor-core pipeline: several chunks per pass (their sums go over consumed scratch rows and are added
+up by a scan), passes of few layers, and the gated recurrence on the tcgen05 kernel with split operands; against the oracle."""
+import pytest
+import torch
+
+from paper_2607_24788_b200 import glide
+from tests.parity_util import run_case
+
+pytestmark = pytest.mark.gpu
+BF16 = torch.bfloat16
+
+
+# chunk 144: the smallest with room for a chunk's sums (129 rows) that is no multiple of 128; 64: passes of one chunk.
+# Calls of 1 token, of a chunk and one token, and of more chunks than a pass holds for one layer (6 layers: 6 chunks).
+@pytest.mark.parametrize("chunk,calls", [(144, [145, 1, 300]), (256, [1, 600, 257]), (144, [1000]), (64, [130, 65])])
+@pytest.mark.parametrize("kw", [dict(), dict(merge=glide.GLIDE_MERGE_SUM_EVICTED), dict(phi=1), dict(gated=True)],
+                         ids=["shared", "sum", "learned", "gated"])
+def test_passes_of_several_chunks(chunk, calls, kw):
+    run_case([0, 16, 100, 128, 304, 1 << 20], 1, 4, 2, 128, BF16, calls, 2, amp=128 ** -0.5 * 4, seed=41, prefill_chunk=chunk, **kw)
+
+
+# one query head per KV head to eight (rows of a tile per token), two sequences, the call boundary inside a key tile
+@pytest.mark.parametrize("G,chunk,calls", [(1, 0, [300, 131]), (2, 512, [40, 520]), (8, 0, [70, 33, 5])])
+def test_gated_prefill_on_tcgen05(G, chunk, calls):
+    run_case([0, 33, 129, 1 << 20], 2, 2 * G, 2, 128, BF16, calls, 2, amp=128 ** -0.5 * 4, seed=43 + G, gated=True, prefill_chunk=chunk)
