@@ -484,11 +484,6 @@ __global__ void __launch_bounds__(kPhiSplit * kPhiHeads * 32) glide_decode_phi_k
   }
 }
 
-__global__ void glide_advance_kernel(int64_t *n_dev, int layer_begin, int layer_count, int64_t T) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < layer_count) n_dev[layer_begin + i] += T;
-}
-
 }  // namespace
 
 // q, k, v, out are the tensors of the layer range [layer_begin, layer_begin + layer_count).  The per-item kernels
@@ -678,13 +673,6 @@ int launch_decode_noalloc(glide_ctx *ctx, const void *q, const void *k, const vo
     if (cudaGetLastError() != cudaSuccess) return GLIDE_ERR_CUDA;
     return GLIDE_OK;
   });
-}
-
-int launch_advance(glide_ctx *ctx, int layer_begin, int layer_count, int64_t T, cudaStream_t stream) {
-  int64_t *n_dev = reinterpret_cast<int64_t *>(ctx->ws + ctx->off_ndev);
-  glide_advance_kernel<<<(layer_count + 63) / 64, 64, 0, stream>>>(n_dev, layer_begin, layer_count, T);
-  if (cudaGetLastError() != cudaSuccess) return GLIDE_ERR_CUDA;
-  return GLIDE_OK;
 }
 
 }  // namespace glide

@@ -188,7 +188,11 @@ int glide::plan_context(const glide_config *cfg, glide_ctx *ctx, std::vector<Wor
   // per layer 3 maps of 16-row boxes, then (from 3 L on) 2 of 128-row boxes, then the three bf16 scratch arrays of prefill
   off = align_up(off + size_t(128) * (5 * L + 3), 256);
   ctx->off_phik = off;
-  off = align_up(off + sizeof(float) * size_t(L) * units_per_layer * ctx->prefill_chunk * dp, 256);
+  // one chunk's phi(K'), or the CUDA-core passes' chunk sums: at least one [d][d] (with z) per unit
+  ctx->phik_rows = size_t(std::max(ctx->prefill_chunk, d));
+  off = align_up(off + sizeof(float) * size_t(L) * units_per_layer * ctx->phik_rows * dp, 256);
+  ctx->off_zsnap = off;
+  off = align_up(off + sizeof(float) * size_t(L) * units_per_layer * std::max<size_t>(1, ctx->phik_rows / d) * dp, 256);
   ctx->off_zcum = off;   // running sums of phi(K') over the chunk: only the sum-of-terms merges use them
   if (cfg->merge != GLIDE_MERGE_SHARED)
     off = align_up(off + sizeof(float) * size_t(L) * units_per_layer * ctx->prefill_chunk * dp, 256);
@@ -209,8 +213,6 @@ int glide::plan_context(const glide_config *cfg, glide_ctx *ctx, std::vector<Wor
     off = align_up(off + 2 * halves * size_t(L) * units_per_layer * ctx->prefill_chunk * d, 256);
     ctx->off_s16 = off;
     off = align_up(off + 2 * halves * size_t(L) * units_per_layer * d * d, 256);
-    ctx->off_zsnap = off;
-    off = align_up(off + sizeof(float) * size_t(L) * units_per_layer * dp, 256);
     if (dp == 2 * d) {
       ctx->off_phiq16 = off;
       off = align_up(off + 2 * halves * size_t(L) * units_per_layer * ctx->prefill_chunk * ctx->G * d, 256);

@@ -161,7 +161,9 @@ struct PrefillParams {
                              // nullptr when that kernel is not in use
   void *s16;                 // tcgen05 kernel: bf16 copy of every unit's S as it is at the start of every chunk of the pass,
                              // [halves][units_cap][d][d], index (unit of the pass * nsub + chunk)
-  float *zsnap;              // tcgen05 kernel: z at the start of every chunk of the pass, [units_cap][dp], the same index
+  float *zsnap;              // tcgen05 kernel: z at the start of every chunk of the pass, [units_cap][dp], the same index;
+                             // CUDA-core passes: every chunk's sum of phi(K') (their S sums, [unit * nsub + chunk][d][d], are
+                             // in phik)
   void *phiq16;              // tcgen05 kernel, learned map: phi(q) of the chunk's query rows as bf16,
                              // [2 halves][units_cap * SC * G][d], row = (unit * Cmax + token) * G + head of the group
   int64_t units_cap;         // L * B * H_kv of the context: what separates the halves in the three arrays above
@@ -186,6 +188,8 @@ struct PrefillParams {
   const void *wq, *wk;       // learned feature map: [L][H][d][d], [L][Hkv][d][d] in the I/O dtype
   int32_t gated;
   const float *gate;         // the call's gates [layer_count][B][T][Hkv], or null for gates of 1
+  int64_t *n_dev;            // [L] position counters
+  int64_t advance;           // the pass's last kernel adds this to its layers' counters (0: none)
   float *gcum;               // gated: running sums of log(gate) of the chunk's delayed tokens, [units][Cmax]
 };
 
@@ -230,6 +234,7 @@ struct glide_ctx {
   mutable bool launch_wrapped = false;   // the counter has passed 2^32: the records are cleared before the next launch
   int stream_rec_floats = 0;        // record size of the streaming kernel (twice as large for the sum-of-terms merges)
   int prefill_chunk = 0;
+  size_t phik_rows = 0;             // rows of d_phi floats per unit of the fp32 prefill scratch
   float scale = 0.f;
   size_t elem = 0;
   unsigned char *ws = nullptr;
@@ -271,6 +276,6 @@ bool prefill_attn_mma_supported(const glide_ctx *ctx);
 int launch_prefill_attn_mma(glide_ctx *ctx, const PrefillParams &p, cudaStream_t stream);
 bool prefill_state_mma_supported(const glide_ctx *ctx);
 int launch_prefill_state_mma(glide_ctx *ctx, const PrefillParams &p, cudaStream_t stream);
-int launch_advance(glide_ctx *ctx, int layer_begin, int layer_count, int64_t T, cudaStream_t stream);
+int launch_prefill_fma(glide_ctx *ctx, const PrefillParams &p, cudaStream_t stream);
 
 }  // namespace glide

@@ -509,7 +509,7 @@ __global__ void __launch_bounds__(kPrefillThreads) prefill_zcum_kernel(const Pre
   }
 }
 
-// 4. ring fill: the chunk's newest min(C, cap) tokens; one warp per (unit, kTokPerWarp consecutive chunk tokens)
+// 4. ring fill: the pass's newest min(C, cap) tokens, and the layers' counters on the last pass; one warp per (unit, kTokPerWarp consecutive chunk tokens)
 template <typename T, int D>
 __global__ void __launch_bounds__(kPrefillThreads) prefill_ring_kernel(const PrefillParams p) {
   constexpr int E = D / 32;
@@ -517,6 +517,8 @@ __global__ void __launch_bounds__(kPrefillThreads) prefill_ring_kernel(const Pre
   const int64_t wid = (int64_t(blockIdx.x) * kPrefillThreads + threadIdx.x) >> 5;
   const int64_t units = int64_t(p.layer_count) * p.B * p.Hkv;
   const int groups = (p.C + kTokPerWarp - 1) / kTokPerWarp;
+  if (blockIdx.x == 0 && p.advance)
+    for (int l = threadIdx.x; l < p.layer_count; l += kPrefillThreads) p.n_dev[p.layer_begin + l] += p.advance;
   if (wid >= units * groups) return;
   const int i0 = int(wid % groups) * kTokPerWarp;
   const int64_t u = wid / groups;
@@ -596,6 +598,7 @@ int launch_prefill(glide_ctx *ctx, int layer_begin, int layer_count, int64_t T, 
   p.wq = ctx->cfg.phi_wq;
   p.wk = ctx->cfg.phi_wk;
   p.gated = ctx->cfg.gated;
+  p.n_dev = reinterpret_cast<int64_t *>(ctx->ws + ctx->off_ndev);
   p.gate = gate;
   p.gcum = reinterpret_cast<float *>(ctx->ws + ctx->off_gcum);
   const int64_t units = int64_t(layer_count) * p.B * p.Hkv;
@@ -629,21 +632,13 @@ int launch_prefill(glide_ctx *ctx, int layer_begin, int layer_count, int64_t T, 
   };
   const bool any_evicts = evicts_in(layer_begin, layer_count);
 
-  // Tensor-core pipeline (outputs by the tcgen05 kernel, or no outputs and the tensor-core carry).  Nothing in a pass
-  // waits for the ring update of its own tokens, and the chunks of a pass depend on one another through S alone, which
-  // a scan over the chunk sums supplies: so a pass takes many chunks of few layers rather than one chunk of all
-  // layers, as many as the scratch holds (it is sized for one chunk of every unit).  Chunk by chunk, one layer of 8 KV
-  // heads left most of the chip idle: 32 CTAs of 40 us per chunk (32 layers, 8001 tokens, layer by layer: 76.2 ms).
-  auto run_passes = [&](auto tt, auto dd, auto pp) -> int {
-    using TT = typename decltype(tt)::type;
-    constexpr int D = decltype(dd)::value, DP = decltype(pp)::value;
-    constexpr bool kCanProject = DP == 2 * D && D == 128 && std::is_same<TT, __nv_bfloat16>::value;
-    const int64_t units_layer = int64_t(p.B) * p.Hkv;
-    const int64_t most = p.SC > 128 ? p.units_cap / units_layer : 1;   // (the chunk sums take 129 scratch rows of a chunk)
+  // Passes over the call: run(s) for every pass s, which holds some of the layers and up to `most` chunks of p.SC tokens of
+  // their units, `slots` (unit, chunk) pairs at most (what the scratch holds).
+  const int64_t units_layer = int64_t(p.B) * p.Hkv;
+  auto for_passes = [&](int64_t slots, int64_t most, int D, size_t elem, auto &&run) -> int {
     const int nsub_max = int(std::min<int64_t>(most, (T + p.SC - 1) / p.SC));
-    const int fit = int(std::min<int64_t>(layer_count, p.units_cap / (units_layer * nsub_max)));
+    const int fit = int(std::min<int64_t>(layer_count, slots / (units_layer * nsub_max)));
     const int n_groups = (layer_count + fit - 1) / fit;
-    const size_t elem = sizeof(TT);
     for (int64_t c0 = 0; c0 < T; c0 += int64_t(nsub_max) * p.SC) {
       for (int gi = 0; gi < n_groups; ++gi) {
         const int l0 = int(int64_t(layer_count) * gi / n_groups), l1 = int(int64_t(layer_count) * (gi + 1) / n_groups);
@@ -660,30 +655,56 @@ int launch_prefill(glide_ctx *ctx, int layer_begin, int layer_count, int64_t T, 
         s.C = int(std::min<int64_t>(int64_t(nsub_max) * p.SC, T - c0));
         s.nsub = (s.C + p.SC - 1) / p.SC;
         s.Cmax = s.nsub * p.SC;
-        const int64_t units = int64_t(s.layer_count) * units_layer;
-        const int64_t warps4 = units * ((s.C + kTokPerWarp - 1) / kTokPerWarp);
-        const unsigned warp4_blocks = unsigned((warps4 * 32 + kPrefillThreads - 1) / kPrefillThreads);
-        if (evicts_in(s.layer_begin, s.layer_count)) {
-          if (kCanProject) {
-            if (launch_prefill_project(ctx, s, true, stream) != GLIDE_OK) return GLIDE_ERR_CUDA;
-          } else {
-            prefill_phi_kernel<TT, D, DP><<<warp4_blocks, kPrefillThreads, 0, stream>>>(s);
-          }
-          if (p.gated)
-            prefill_gcum_kernel<TT, D><<<unsigned((units * s.nsub * 32 + kPrefillThreads - 1) / kPrefillThreads), kPrefillThreads, 0, stream>>>(s);
-          if (out && s.phiq16 && launch_prefill_project(ctx, s, false, stream) != GLIDE_OK) return GLIDE_ERR_CUDA;
-          if (out && p.merge != GLIDE_MERGE_SHARED)   // (before the carry: the chunk sums overwrite rows of phi(K'))
-            prefill_zcum_kernel<D><<<unsigned((units * s.nsub * D + kPrefillThreads - 1) / kPrefillThreads), kPrefillThreads, 0, stream>>>(s);
-          if (launch_prefill_state_mma(ctx, s, stream) != GLIDE_OK) return GLIDE_ERR_CUDA;
-        }
-        if (out && launch_prefill_attn_tc(ctx, s, stream) != GLIDE_OK) return GLIDE_ERR_CUDA;
-        prefill_ring_kernel<TT, D><<<warp4_blocks, kPrefillThreads, 0, stream>>>(s);
-        if (cudaGetLastError() != cudaSuccess) return GLIDE_ERR_CUDA;
+        s.advance = seq < 0 && c0 + s.C == T ? T : 0;
+        const int rc = run(s);
+        if (rc) return rc;
       }
     }
     return GLIDE_OK;
   };
+  // Tensor-core pipeline (outputs by the tcgen05 kernel, or no outputs and the tensor-core carry).  Nothing in a pass
+  // waits for the ring update of its own tokens, and the chunks of a pass depend on one another through S alone, which
+  // a scan over the chunk sums supplies: so a pass takes many chunks of few layers rather than one chunk of all
+  // layers, as many as the scratch holds (it is sized for one chunk of every unit).  Chunk by chunk, one layer of 8 KV
+  // heads left most of the chip idle: 32 CTAs of 40 us per chunk (32 layers, 8001 tokens, layer by layer: 76.2 ms).
+  auto run_passes = [&](auto tt, auto dd, auto pp) -> int {
+    using TT = typename decltype(tt)::type;
+    constexpr int D = decltype(dd)::value, DP = decltype(pp)::value;
+    constexpr bool kCanProject = DP == 2 * D && D == 128 && std::is_same<TT, __nv_bfloat16>::value;
+    const int64_t most = p.SC > 128 ? p.units_cap / units_layer : 1;   // (the chunk sums take 129 scratch rows of a chunk)
+    return for_passes(p.units_cap, most, D, sizeof(TT), [&](const PrefillParams &s) -> int {
+      const int64_t units = int64_t(s.layer_count) * units_layer;
+      const int64_t warps4 = units * ((s.C + kTokPerWarp - 1) / kTokPerWarp);
+      const unsigned warp4_blocks = unsigned((warps4 * 32 + kPrefillThreads - 1) / kPrefillThreads);
+      if (evicts_in(s.layer_begin, s.layer_count)) {
+        if (kCanProject) {
+          if (launch_prefill_project(ctx, s, true, stream) != GLIDE_OK) return GLIDE_ERR_CUDA;
+        } else {
+          prefill_phi_kernel<TT, D, DP><<<warp4_blocks, kPrefillThreads, 0, stream>>>(s);
+        }
+        if (p.gated)
+          prefill_gcum_kernel<TT, D><<<unsigned((units * s.nsub * 32 + kPrefillThreads - 1) / kPrefillThreads), kPrefillThreads, 0, stream>>>(s);
+        if (out && s.phiq16 && launch_prefill_project(ctx, s, false, stream) != GLIDE_OK) return GLIDE_ERR_CUDA;
+        if (out && p.merge != GLIDE_MERGE_SHARED)   // (before the carry: the chunk sums overwrite rows of phi(K'))
+          prefill_zcum_kernel<D><<<unsigned((units * s.nsub * D + kPrefillThreads - 1) / kPrefillThreads), kPrefillThreads, 0, stream>>>(s);
+        if (launch_prefill_state_mma(ctx, s, stream) != GLIDE_OK) return GLIDE_ERR_CUDA;
+      }
+      if (out && launch_prefill_attn_tc(ctx, s, stream) != GLIDE_OK) return GLIDE_ERR_CUDA;
+      prefill_ring_kernel<TT, D><<<warp4_blocks, kPrefillThreads, 0, stream>>>(s);
+      return cudaGetLastError() == cudaSuccess ? GLIDE_OK : GLIDE_ERR_CUDA;
+    });
+  };
   const bool passes = state_mma && (use_tc || !out);
+
+  // CUDA-core passes (parameter-free map, no gates): the scratch holds phik_rows / d chunk sums per unit.  Chunks as short as
+  // that allows for the whole call in one pass (a query goes through its chunk's delayed tokens one by one, 64 at a time),
+  // but not below 64 tokens, where a chunk's sum costs as much as the tokens it saves, nor above 256.
+  if (!passes && !use_mma && !state_mma && plain) {
+    const int64_t slots = p.units_cap * int64_t(ctx->phik_rows / size_t(ctx->cfg.head_dim));
+    const int64_t most = slots / units_layer;
+    p.SC = int(std::min<int64_t>(256, std::max<int64_t>(64, ((T + most - 1) / most + 15) / 16 * 16)));
+    return for_passes(slots, most, ctx->cfg.head_dim, ctx->elem, [&](const PrefillParams &s) -> int { return launch_prefill_fma(ctx, s, stream); });
+  }
 
   auto run_chunks = [&](auto tt, auto dd, auto gg, auto pp) -> int {
     using TT = typename decltype(tt)::type;
@@ -691,6 +712,7 @@ int launch_prefill(glide_ctx *ctx, int layer_begin, int layer_count, int64_t T, 
     for (int64_t c0 = 0; c0 < T; c0 += p.Cmax) {
       p.c0 = c0;
       p.C = int(std::min<int64_t>(p.Cmax, T - c0));
+      p.advance = seq < 0 && c0 + p.C == T ? T : 0;
       const int64_t warps = units * p.C;
       const unsigned warp_blocks = unsigned((warps * 32 + kPrefillThreads - 1) / kPrefillThreads);
       const int64_t warps4 = units * ((p.C + kTokPerWarp - 1) / kTokPerWarp);
@@ -729,8 +751,7 @@ int launch_prefill(glide_ctx *ctx, int layer_begin, int layer_count, int64_t T, 
     if (ctx->dp == D) return run_chunks(tt, dd, gg, IntTag<D>{});
     return run_chunks(tt, dd, gg, IntTag<2 * D>{});
   });
-  if (rc) return rc;
-  return seq < 0 ? launch_advance(ctx, layer_begin, layer_count, T, stream) : GLIDE_OK;
+  return rc;
 }
 
 }  // namespace glide

@@ -23,3 +23,13 @@ def test_passes_of_several_chunks(chunk, calls, kw):
 @pytest.mark.parametrize("G,chunk,calls", [(1, 0, [300, 131]), (2, 512, [40, 520]), (8, 0, [70, 33, 5])])
 def test_gated_prefill_on_tcgen05(G, chunk, calls):
     run_case([0, 33, 129, 1 << 20], 2, 2 * G, 2, 128, BF16, calls, 2, amp=128 ** -0.5 * 4, seed=43 + G, gated=True, prefill_chunk=chunk)
+
+
+# CUDA-core passes: chunk sums per unit from one (prefill_chunk 16) to four, calls of one token, of a chunk and one token, of
+# several passes; row tiles of 16 to 2 tokens; every merge
+@pytest.mark.parametrize("dtype,d,G,merge,chunk,calls", [
+    (torch.float32, 64, 1, 0, 0, [1, 65, 512]), (torch.float32, 64, 4, 1, 0, [700, 3]), (torch.float32, 128, 2, 2, 0, [130, 257]),
+    (torch.float32, 64, 8, 0, 16, [40, 300]), (torch.float32, 128, 1, 0, 512, [600]), (BF16, 64, 2, 0, 0, [65, 300])])
+def test_cuda_core_passes(dtype, d, G, merge, chunk, calls):
+    amp = 4 * d ** -0.5
+    run_case([0, 16, 100, 300, 1 << 20], 2, 2 * G, 2, d, dtype, calls, 2, amp=amp, seed=47 + G, merge=merge, prefill_chunk=chunk)
