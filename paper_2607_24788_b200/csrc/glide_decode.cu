@@ -388,6 +388,252 @@ __global__ void __launch_bounds__(kDecodeThreads) glide_decode_kernel(const Deco
   }
 }
 
+// ---- small units: one CTA per unit ---------------------------------------------------------------
+// The list above costs a small problem a chain of some ten memory round trips (item from the work counter, item, layer,
+// rows, record, ticket, records again, completion count: 12.5 us for 4 units of 64 slots).  Here a CTA holds a whole unit:
+// eight warps take its ring rows (with the current token), four warps its state, they meet once in shared memory,
+// and nothing leaves the CTA but the results.  The position is read by every CTA, so the counters move on when the last
+// one has read it (a count that nobody waits for).
+constexpr int kUnitStateThreads = 128;
+template <int D, int G>
+constexpr int kUnitWinWarps = D * G >= 1024 ? 4 : 8;   // (their partial results are the CTA's shared memory)
+template <int D, int G>
+constexpr int kUnitThreads = kUnitWinWarps<D, G> * 32 + kUnitStateThreads;
+// Longest ring for it: a CTA has 64 rows in flight and scores them for all heads of the group itself, so longer rings are
+// read faster by several CTAs.  Per launch, here against the list above: d = 64, one head per unit, 4 units: w = 64 5.8 us
+// against 12.6, 256 8.4 / 15.6, 500 11.6 / 15.6; d = 128, four heads, 2 units: w = 300 18.3 / 22.6, 500 26.4 / 21.6;
+// 64 units of w = 300 (d = 64): 9.1 / 17.2.
+inline int64_t unit_max_cap(int d, int G) { return d * G <= 128 ? 512 : 320; }
+
+template <typename T, int D, int G, int DP>
+__global__ void __launch_bounds__(kUnitThreads<D, G>) glide_decode_unit_kernel(const DecodeParams p) {
+  constexpr int E = D / 32;
+  constexpr int WW = kUnitWinWarps<D, G>;
+  constexpr int U = 8;                           // rows a warp has in flight
+  constexpr int TPR = D / 4, RPI = kUnitStateThreads / TPR;   // threads per state row, rows at a time
+  __shared__ __align__(16) float win[WW][G][D];
+  __shared__ float win_m[WW][G], win_l[WW][G];
+  __shared__ __align__(16) float lin[RPI][G][D];
+  __shared__ __align__(16) float phiq[G][DP], phik[DP], ve_s[D];
+  __shared__ float lin_b[G];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int unit_rel = blockIdx.x, per_layer = p.B * p.Hkv;
+  const int layer = p.layer_begin + unit_rel / per_layer, ub = unit_rel % per_layer;
+  const int b = ub / p.Hkv, g = ub - b * p.Hkv;
+  const size_t unit = size_t(layer) * per_layer + ub;
+  const int64_t n = p.n_dev[layer];
+  const LayerDev ld = p.layers[layer];
+  const int64_t t = n + (p.seq_off ? p.seq_off[b] : 0);
+  const T *kt = reinterpret_cast<const T *>(p.k) + unit * D, *vt = reinterpret_cast<const T *>(p.v) + unit * D;
+  const T *qb = reinterpret_cast<const T *>(p.q) + (size_t(layer) * p.B + b) * p.H * D;
+  const bool live = t >= 0;                      // (a parked slot: nothing is read or written for it)
+  const bool has_win = live && ld.cap > 0, has_state = live && ld.evicts && t >= ld.wlin;
+  const size_t ring0 = size_t(ub) * size_t(ld.cap);
+  const int cur = ld.cap > 0 ? int(uint32_t(t) % uint32_t(ld.cap)) : 0;   // the slot of the token that leaves the window
+
+  if (warp < WW) {
+    if (has_win) {
+      const T *Kb = reinterpret_cast<const T *>(p.ws + ld.ringK) + ring0 * D + lane * E;
+      const T *Vb = reinterpret_cast<const T *>(p.ws + ld.ringV) + ring0 * D + lane * E;
+      // slots [0, t) until the ring is full, then every slot but `cur`; the current token is row `lim`
+      const int lim = int(t < ld.cap ? t : ld.cap);
+      float q[G][E], acc[G][E], m[G], l[G];
+#pragma unroll
+      for (int h = 0; h < G; ++h) {
+        load_elems<T, E>(qb + size_t(p.heads_of[g * G + h]) * D + lane * E, q[h]);
+        m[h] = -CUDART_INF_F;
+        l[h] = 0.f;
+#pragma unroll
+        for (int i = 0; i < E; ++i) {
+          q[h][i] *= p.scale_log2;
+          acc[h][i] = 0.f;
+        }
+      }
+      for (int s0 = warp; s0 <= lim; s0 += WW * U) {
+        float kx[U][E], vx[U][E];
+        bool ok[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const int s = s0 + u * WW;
+          ok[u] = s <= lim && (s == lim || s != cur);   // (before the ring is full `cur` is lim itself)
+#pragma unroll
+          for (int i = 0; i < E; ++i) kx[u][i] = vx[u][i] = 0.f;
+          if (ok[u]) {
+            load_elems<T, E>(s == lim ? kt + lane * E : Kb + size_t(s) * D, kx[u]);
+            load_elems<T, E>(s == lim ? vt + lane * E : Vb + size_t(s) * D, vx[u]);
+          }
+        }
+#pragma unroll
+        for (int h = 0; h < G; ++h) {
+          float sc[U], mx = m[h];
+#pragma unroll
+          for (int u = 0; u < U; ++u) {
+            float part = 0.f;
+#pragma unroll
+            for (int i = 0; i < E; ++i) part = fmaf(q[h][i], kx[u][i], part);
+            sc[u] = warp_sum(part);
+            if (ok[u]) mx = fmaxf(mx, sc[u]);
+          }
+          const float f = m[h] == -CUDART_INF_F ? 0.f : exp2f(m[h] - mx);
+          m[h] = mx;
+          l[h] *= f;
+#pragma unroll
+          for (int i = 0; i < E; ++i) acc[h][i] *= f;
+#pragma unroll
+          for (int u = 0; u < U; ++u) {
+            const float e = ok[u] ? exp2f(sc[u] - mx) : 0.f;
+            l[h] += e;
+#pragma unroll
+            for (int i = 0; i < E; ++i) acc[h][i] = fmaf(e, vx[u][i], acc[h][i]);
+          }
+        }
+      }
+#pragma unroll
+      for (int h = 0; h < G; ++h) {
+#pragma unroll
+        for (int i = 0; i < E; ++i) win[warp][h][lane * E + i] = acc[h][i];
+        if (lane == 0) {
+          win_m[warp][h] = m[h];
+          win_l[warp][h] = l[h];
+        }
+      }
+    }
+  } else if (has_state) {
+    const int st = tid - WW * 32, swarp = st >> 5;
+    const int c4 = (st % TPR) * 4, rsub = st / TPR;
+    float *Sb = reinterpret_cast<float *>(p.ws + ld.S) + size_t(ub) * DP * D + c4;
+    constexpr int kAhead = DP / RPI < 8 ? DP / RPI : 8;
+    float4 s[kAhead];
+#pragma unroll
+    for (int a = 0; a < kAhead; ++a) s[a] = *reinterpret_cast<const float4 *>(Sb + size_t(rsub + a * RPI) * D);
+    // the token that enters the state: the one that leaves the ring, or the current one
+    const bool from_ring = ld.wlin != 0;
+    const T *ke = from_ring ? reinterpret_cast<const T *>(p.ws + ld.ringK) + (ring0 + cur) * D : kt;
+    const T *ve = from_ring ? reinterpret_cast<const T *>(p.ws + ld.ringV) + (ring0 + cur) * D : vt;
+    float gamma = 1.f;
+    if (p.gated) gamma = from_ring ? reinterpret_cast<const float *>(p.ws + ld.ringG)[ring0 + cur] : (p.gate ? p.gate[unit] : 1.f);
+    for (int c = st; c < D; c += kUnitStateThreads) ve_s[c] = to_f32(ve[c]);
+    if constexpr (DP == D) {
+      for (int h = swarp; h <= G; h += 4) {      // row G: the key
+        float x[E];
+        load_elems<T, E>((h == G ? ke : qb + size_t(p.heads_of[g * G + h]) * D) + lane * E, x);
+        warp_phi<E>(x);
+        float *dst = (h == G ? phik : phiq[h < G ? h : 0]) + lane * E;
+#pragma unroll
+        for (int i = 0; i < E; ++i) dst[i] = x[i];
+      }
+    } else {
+      const float *ph = p.phit + size_t(unit_rel) * DP * (G + 1);   // [DP / 16][G + 1][16]
+      for (int idx = st; idx < (G + 1) * DP; idx += kUnitStateThreads) {
+        const int r16 = idx / ((G + 1) * 16), h = idx / 16 % (G + 1), r = r16 * 16 + idx % 16;
+        (h < G ? phiq[h < G ? h : 0] : phik)[r] = ph[idx];
+      }
+    }
+    asm volatile("bar.sync 1, %0;" ::"n"(kUnitStateThreads) : "memory");
+    const float4 v4 = *reinterpret_cast<const float4 *>(&ve_s[c4]);
+    float4 a4[G];
+#pragma unroll
+    for (int h = 0; h < G; ++h) a4[h] = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int r0 = rsub; r0 < DP; r0 += RPI * kAhead) {
+      float4 nx[kAhead];
+      const bool more = r0 + RPI * kAhead < DP;
+#pragma unroll
+      for (int a = 0; a < kAhead; ++a)
+        if (more) nx[a] = *reinterpret_cast<const float4 *>(Sb + size_t(r0 + (kAhead + a) * RPI) * D);
+#pragma unroll
+      for (int a = 0; a < kAhead; ++a) {
+        const int r = r0 + a * RPI;
+        const float pk = phik[r];
+        float4 x = s[a];
+        x.x = fmaf(pk, v4.x, gamma * x.x);
+        x.y = fmaf(pk, v4.y, gamma * x.y);
+        x.z = fmaf(pk, v4.z, gamma * x.z);
+        x.w = fmaf(pk, v4.w, gamma * x.w);
+        *reinterpret_cast<float4 *>(Sb + size_t(r) * D) = x;
+#pragma unroll
+        for (int h = 0; h < G; ++h) {
+          const float f = phiq[h][r];
+          a4[h].x = fmaf(f, x.x, a4[h].x);
+          a4[h].y = fmaf(f, x.y, a4[h].y);
+          a4[h].z = fmaf(f, x.z, a4[h].z);
+          a4[h].w = fmaf(f, x.w, a4[h].w);
+        }
+      }
+#pragma unroll
+      for (int a = 0; a < kAhead; ++a) s[a] = nx[a];
+    }
+#pragma unroll
+    for (int h = 0; h < G; ++h) *reinterpret_cast<float4 *>(&lin[rsub][h][c4]) = a4[h];
+    if (swarp == 3) {   // z and its readout
+      float *zb = reinterpret_cast<float *>(p.ws + ld.z) + size_t(ub) * DP;
+      float bp[G];
+#pragma unroll
+      for (int h = 0; h < G; ++h) bp[h] = 0.f;
+#pragma unroll 4
+      for (int r = lane; r < DP; r += 32) {
+        const float zn = fmaf(gamma, zb[r], phik[r]);
+        zb[r] = zn;
+#pragma unroll
+        for (int h = 0; h < G; ++h) bp[h] = fmaf(phiq[h][r], zn, bp[h]);
+      }
+#pragma unroll
+      for (int h = 0; h < G; ++h) {
+        const float bs = warp_sum(bp[h]);
+        if (lane == 0) lin_b[h] = bs;
+      }
+    }
+  }
+  __syncthreads();   // also: every thread of the CTA has read the position
+  if (tid == 0) {
+    __threadfence();
+    if (atomicAdd(&p.ctl->done_counter, 1) == int(gridDim.x) - 1) {
+      p.ctl->done_counter = 0;
+      for (int i = 0; i < p.layer_count; ++i) p.n_dev[p.layer_begin + i] += 1;
+    }
+  }
+  if (!live) return;
+  const bool shared = ld.merge == GLIDE_MERGE_SHARED;
+  for (int idx = tid; idx < G * D; idx += kUnitThreads<D, G>) {
+    const int h = idx / D, c = idx - h * D;
+    // shared normaliser: m* = max(window max, 0), the floor belongs to the linear terms (logit 0); sum of two normalised
+    // terms: the window is normalised on its own, against its own maximum
+    float M = shared && has_state ? 0.f : -CUDART_INF_F, num = 0.f, den = 0.f, add = 0.f;
+    if (has_win) {
+#pragma unroll
+      for (int wi = 0; wi < WW; ++wi) M = fmaxf(M, win_m[wi][h]);
+#pragma unroll
+      for (int wi = 0; wi < WW; ++wi) {
+        const float f = win_m[wi][h] == -CUDART_INF_F ? 0.f : exp2f(win_m[wi][h] - M);
+        num = fmaf(win[wi][h][c], f, num);
+        den = fmaf(win_l[wi][h], f, den);
+      }
+    }
+    if (has_state) {
+      float a = 0.f;
+#pragma unroll
+      for (int r = 0; r < RPI; ++r) a += lin[r][h][c];
+      if (shared) {
+        const float f = exp2f(-M);
+        num = fmaf(f, a, num);
+        den = fmaf(f, lin_b[h], den);
+      } else if (lin_b[h] > 0.f) {
+        add = a / lin_b[h];
+      }
+    }
+    const float inv = den > 0.f ? 1.0f / den : 0.f;   // den = 0 only for a sum-of-terms layer without a window
+    from_f32(reinterpret_cast<T *>(p.out) + ((size_t(layer) * p.B + b) * p.H + p.heads_of[g * G + h]) * D + c, fmaf(num, inv, add));
+  }
+  if (has_win) {  // every reader of slot `cur` has passed the barrier: store the new row
+    T *Kd = reinterpret_cast<T *>(p.ws + ld.ringK) + (ring0 + cur) * D, *Vd = reinterpret_cast<T *>(p.ws + ld.ringV) + (ring0 + cur) * D;
+    for (int c = tid; c < D; c += kUnitThreads<D, G>) {
+      Kd[c] = kt[c];
+      Vd[c] = vt[c];
+    }
+    if (p.gated && tid == 0)   // the token's gate waits in the ring with it
+      reinterpret_cast<float *>(p.ws + ld.ringG)[ring0 + cur] = p.gate ? p.gate[unit] : 1.f;
+  }
+}
+
 // ---- learned feature map of one decode step ------------------------------------------------------
 // phi_W(x) = [softmax(W^T x); softmax(-W^T x)] of the step's queries and of the key that enters the state, for every
 // unit of the launch, into p.phit [unit][DP / 16][G + 1][16] (row G: the key).  kPhiSplit warps per (layer, KV head,
@@ -581,6 +827,13 @@ int launch_decode_phi(glide_ctx *ctx, const DecodeParams &p, cudaStream_t stream
   });
 }
 
+// the CUDA-core decode step of these layers takes one CTA per unit
+bool decode_by_unit(const glide_ctx *ctx, int layer_begin, int layer_count) {
+  for (int l = layer_begin; l < layer_begin + layer_count; ++l)
+    if (ctx->layers[size_t(l)].cap > unit_max_cap(ctx->cfg.head_dim, ctx->G)) return false;
+  return true;
+}
+
 int launch_decode(glide_ctx *ctx, int layer_begin, int layer_count, const void *q, const void *k, const void *v,
                   const float *gate, void *out, cudaStream_t stream) {
   const int L = ctx->cfg.n_layers;
@@ -610,7 +863,10 @@ int launch_decode(glide_ctx *ctx, int layer_begin, int layer_count, const void *
   return dispatch_decode(ctx, [&](auto tt, auto dd, auto gg, auto pp) -> int {
     using T = typename decltype(tt)::type;
     constexpr int D = decltype(dd)::value, G = decltype(gg)::value, DP = decltype(pp)::value;
-    glide_decode_kernel<T, D, G, DP><<<ctx->decode_grid, kDecodeThreads, 0, stream>>>(p);
+    if (decode_by_unit(ctx, layer_begin, layer_count))
+      glide_decode_unit_kernel<T, D, G, DP><<<unsigned(layer_count * p.B * p.Hkv), kUnitThreads<D, G>, 0, stream>>>(p);
+    else
+      glide_decode_kernel<T, D, G, DP><<<ctx->decode_grid, kDecodeThreads, 0, stream>>>(p);
     if (cudaGetLastError() != cudaSuccess) return GLIDE_ERR_CUDA;
     return GLIDE_OK;
   });

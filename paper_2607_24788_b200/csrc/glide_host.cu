@@ -200,7 +200,9 @@ int glide::plan_context(const glide_config *cfg, glide_ctx *ctx, std::vector<Wor
   if (cfg->phi == GLIDE_PHI_PROJ_SOFTMAX2)
     off = align_up(off + sizeof(float) * size_t(L) * units_per_layer * dp * (ctx->G + 1), 256);
   ctx->off_gcum = off;   // gated: running sums of log(gate) over the chunk's delayed tokens
-  if (cfg->gated) off = align_up(off + sizeof(float) * size_t(L) * units_per_layer * ctx->prefill_chunk, 256);
+  // (as many chunks of up to 256 tokens as the CUDA-core passes have sums for)
+  if (cfg->gated)
+    off = align_up(off + sizeof(float) * size_t(L) * units_per_layer * std::max<size_t>(ctx->prefill_chunk, 256 * (ctx->phik_rows / d)), 256);
   // tcgen05 prefill kernel (bf16, head_dim 128, plain feature map): bf16 copies of the chunk's phi(K') rows and of S,
   // which its CTAs fetch by TMA instead of converting the fp32 arrays themselves
   // (the learned map under the shared normaliser and, with the plain map, gates too; not both)
@@ -369,6 +371,7 @@ int glide_create(const glide_config *cfg, void *dev_workspace, size_t workspace_
   if (ok && ctx->decode_kind == 0) {
     ok = decode_occupancy(ctx, &per_sm) == GLIDE_OK && per_sm > 0;
     if (ok) ctx->decode_grid = std::max(1, std::min(ctx->n_items, ctx->sm_count * per_sm));
+    if (ok && decode_by_unit(ctx, 0, cfg->n_layers)) ctx->decode_grid = cfg->n_layers * cfg->batch * cfg->n_kv_heads;   // (one CTA per unit)
   }
   if (ok) {
     if (!ctx->tmaps_host.empty())
@@ -671,14 +674,13 @@ int glide_import_gates(glide_ctx *ctx, int32_t layer, const float *dev_gates, vo
 int glide_reset(glide_ctx *ctx, void *stream) {
   if (!ctx) return GLIDE_ERR_INVALID_ARG;
   cudaStream_t st = as_stream(stream);
-  bool ok = cudaMemsetAsync(ctx->ws, 0, ctx->off_layers, st) == cudaSuccess &&
-            cudaMemsetAsync(ctx->ws + ctx->off_seqoff, 0, sizeof(int64_t) * size_t(ctx->cfg.batch), st) == cudaSuccess &&
-            cudaMemsetAsync(ctx->ws + ctx->off_tickets, 0, ctx->off_partials - ctx->off_tickets, st) == cudaSuccess &&
-            cudaMemsetAsync(ctx->ws + ctx->off_state, 0, ctx->state_bytes, st) == cudaSuccess;
-  if (!ok) {
-    cudaGetLastError();
-    return GLIDE_ERR_CUDA;
-  }
+  // control words and counters, slot offsets, tickets, S and z
+  ZeroRanges z{};
+  z.ptr[0] = ctx->ws, z.bytes[0] = ctx->off_layers;
+  z.ptr[1] = ctx->ws + ctx->off_seqoff, z.bytes[1] = sizeof(int64_t) * size_t(ctx->cfg.batch);
+  z.ptr[2] = ctx->ws + ctx->off_tickets, z.bytes[2] = ctx->off_partials - ctx->off_tickets;
+  z.ptr[3] = ctx->ws + ctx->off_state, z.bytes[3] = ctx->state_bytes;
+  if (launch_zero(ctx, z, st) != GLIDE_OK) return GLIDE_ERR_CUDA;
   std::fill(ctx->n_host.begin(), ctx->n_host.end(), 0);
   std::fill(ctx->seq_off.begin(), ctx->seq_off.end(), 0);
   std::fill(ctx->parked.begin(), ctx->parked.end(), 0);

@@ -266,6 +266,7 @@ int launch_decode_noalloc(glide_ctx *ctx, const void *q, const void *k, const vo
 int launch_decode(glide_ctx *ctx, int layer_begin, int layer_count, const void *q, const void *k, const void *v,
                   const float *gate, void *out, cudaStream_t stream);
 int decode_occupancy(const glide_ctx *ctx, int *blocks_per_sm);
+bool decode_by_unit(const glide_ctx *ctx, int layer_begin, int layer_count);
 // seq < 0: the call's tensors hold all B sequences, the layers' counters advance; otherwise they hold sequence slot
 // `seq` alone ([layer_count][1][T]...), which is at position n0, and no counter is touched
 int launch_prefill(glide_ctx *ctx, int layer_begin, int layer_count, int64_t T, const void *q, const void *k,
@@ -276,6 +277,12 @@ bool prefill_attn_mma_supported(const glide_ctx *ctx);
 int launch_prefill_attn_mma(glide_ctx *ctx, const PrefillParams &p, cudaStream_t stream);
 bool prefill_state_mma_supported(const glide_ctx *ctx);
 int launch_prefill_state_mma(glide_ctx *ctx, const PrefillParams &p, cudaStream_t stream);
+// up to four ranges of the workspace (8-byte aligned, sizes multiples of 8) set to zero by one launch
+struct ZeroRanges {
+  unsigned char *ptr[4];
+  size_t bytes[4];
+};
+int launch_zero(const glide_ctx *ctx, const ZeroRanges &z, cudaStream_t stream);
 int launch_prefill_fma(glide_ctx *ctx, const PrefillParams &p, cudaStream_t stream);
 
 }  // namespace glide

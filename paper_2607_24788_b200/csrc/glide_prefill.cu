@@ -564,7 +564,30 @@ __global__ void __launch_bounds__(kPrefillThreads) prefill_ring_kernel(const Pre
   }
 }
 
+// The ranges one after the other, 16 bytes per store where the address allows (S and z start on a 2 MiB multiple).  One
+// launch: as four memsets a reset of a small context took four launches of 1.6 us and the gaps between them.
+__global__ void __launch_bounds__(256) zero_kernel(const ZeroRanges z) {
+  const size_t first = size_t(blockIdx.x) * 256 + threadIdx.x, step = size_t(gridDim.x) * 256;
+#pragma unroll
+  for (int r = 0; r < 4; ++r) {
+    unsigned char *ptr = z.ptr[r];
+    const size_t n16 = (reinterpret_cast<uintptr_t>(ptr) & 15u) ? 0 : z.bytes[r] / 16;
+    for (size_t i = first; i < n16; i += step) reinterpret_cast<uint4 *>(ptr)[i] = make_uint4(0u, 0u, 0u, 0u);
+    for (size_t i = n16 * 2 + first; i < z.bytes[r] / 8; i += step) reinterpret_cast<uint64_t *>(ptr)[i] = 0u;
+  }
+}
+
 }  // namespace
+
+int launch_zero(const glide_ctx *ctx, const ZeroRanges &z, cudaStream_t stream) {
+  size_t most = 0;
+  for (size_t n : z.bytes) most = std::max(most, n);
+  // 16 bytes a thread up to a full chip, more rounds per thread above
+  const size_t blocks = std::min<size_t>((most / 16 + 255) / 256 + 1, size_t(ctx->sm_count) * 8);
+  zero_kernel<<<unsigned(blocks), 256, 0, stream>>>(z);
+  if (cudaGetLastError() != cudaSuccess) return GLIDE_ERR_CUDA;
+  return GLIDE_OK;
+}
 
 int launch_prefill(glide_ctx *ctx, int layer_begin, int layer_count, int64_t T, const void *q, const void *k,
                    const void *v, const float *gate, void *out, int seq, int64_t n0, cudaStream_t stream) {
@@ -696,14 +719,24 @@ int launch_prefill(glide_ctx *ctx, int layer_begin, int layer_count, int64_t T, 
   };
   const bool passes = state_mma && (use_tc || !out);
 
-  // CUDA-core passes (parameter-free map, no gates): the scratch holds phik_rows / d chunk sums per unit.  Chunks as short as
+  // CUDA-core passes (parameter-free map): the scratch holds phik_rows / d chunk sums per unit.  Chunks as short as
   // that allows for the whole call in one pass (a query goes through its chunk's delayed tokens one by one, 64 at a time),
   // but not below 64 tokens, where a chunk's sum costs as much as the tokens it saves, nor above 256.
-  if (!passes && !use_mma && !state_mma && plain) {
+  if (!passes && !use_mma && !state_mma && ctx->cfg.phi == GLIDE_PHI_SOFTMAX) {
     const int64_t slots = p.units_cap * int64_t(ctx->phik_rows / size_t(ctx->cfg.head_dim));
     const int64_t most = slots / units_layer;
     p.SC = int(std::min<int64_t>(256, std::max<int64_t>(64, ((T + most - 1) / most + 15) / 16 * 16)));
-    return for_passes(slots, most, ctx->cfg.head_dim, ctx->elem, [&](const PrefillParams &s) -> int { return launch_prefill_fma(ctx, s, stream); });
+    return for_passes(slots, most, ctx->cfg.head_dim, ctx->elem, [&](const PrefillParams &s) -> int {
+      if (p.gated && evicts_in(s.layer_begin, s.layer_count)) {
+        const unsigned blocks = unsigned((int64_t(s.layer_count) * units_layer * s.nsub * 32 + kPrefillThreads - 1) / kPrefillThreads);
+        const int rc = dispatch_config(ctx->cfg.io_dtype, ctx->cfg.head_dim, 1, [&](auto tt, auto dd, auto) -> int {
+          prefill_gcum_kernel<typename decltype(tt)::type, decltype(dd)::value><<<blocks, kPrefillThreads, 0, stream>>>(s);
+          return cudaGetLastError() == cudaSuccess ? GLIDE_OK : GLIDE_ERR_CUDA;
+        });
+        if (rc) return rc;
+      }
+      return launch_prefill_fma(ctx, s, stream);
+    });
   }
 
   auto run_chunks = [&](auto tt, auto dd, auto gg, auto pp) -> int {

@@ -1,15 +1,18 @@
 // GLIDE prefill on the CUDA cores with fp32 arithmetic throughout (fp32 I/O, d = 64, and whenever the CUDA-core prefill is
-// asked for) for the parameter-free feature map without gates.  A pass takes up to nsub chunks of CH tokens of every unit
+// asked for) for the parameter-free feature map, gated or not.  A pass takes up to nsub chunks of CH tokens of every unit
 // (unit = layer, sequence, KV head) in three launches:
 //   1. prefill_fma_sums_kernel    per chunk phi(K')^T V' and sum phi(K') of its delayed tokens k'_i = k_{i-w}
 //   2. prefill_fma_attn_kernel    per 16 query rows: window softmax, the chunk's own delayed tokens, and the state at
 //                                 the chunk's start = S + the sums of the chunks before it; out
 //   3. prefill_fma_finish_kernel  S and z move on by the pass, the pass's newest tokens go to the ring, counters advance
+// Gated: the running log-gates of the chunks' delayed tokens (gcum) come from a kernel in front; without gates every decay
+// is an exact 1, so that a gated context driven without gates keeps the bits of a plain one.
 // All three read K and V rows where they are (ring for tokens older than the call) and make phi in registers; the ring
 // and S change in the third only.  The problems are small (a few units of a few hundred tokens), so what bounds them is the
 // length of the dependent chain and not the arithmetic: the rows of a tile are shared by 16 query rows and the next
-// tile's loads are in flight while one is used.  512 tokens of 4 units (fp32, d = 64, w = 64): attention 103 us per 256
-// tokens with a warp per query and one key row at a time.
+// tile's loads are in flight while one is used, and a CTA's two groups of four warps work side by side on the window and
+// the linear part (the sums kernel: on every other tile).  512 tokens of 4 units (fp32, d = 64, w = 64): attention 103 us
+// per 256 tokens with a warp per query and one key row at a time, 20 us for all 512 now.
 #include <algorithm>
 #include <type_traits>
 
@@ -19,7 +22,7 @@ namespace glide {
 
 namespace {
 
-constexpr int kThreads = 128;
+constexpr int kThreads = 128;     // of a group; the sums and the attention kernel run two groups per CTA
 constexpr int kRows = 16;         // query rows (token, head of the group) per CTA: 8 half-warps of two rows
 
 __device__ __forceinline__ float4 load4(const float *p) { return *reinterpret_cast<const float4 *>(p); }
@@ -33,6 +36,8 @@ __device__ __forceinline__ void store4(__nv_bfloat16 *p, float4 v) {
   const __nv_bfloat162 lo = __floats2bfloat162_rn(v.x, v.y), hi = __floats2bfloat162_rn(v.z, v.w);
   *reinterpret_cast<uint2 *>(p) = make_uint2(*reinterpret_cast<const uint32_t *>(&lo), *reinterpret_cast<const uint32_t *>(&hi));
 }
+// the barrier of one group of kThreads threads
+__device__ __forceinline__ void group_sync(int grp) { asm volatile("bar.sync %0, 128;" ::"r"(1 + grp) : "memory"); }
 // reductions over N consecutive lanes (N = 16 or 32), the result in all of them
 template <int N>
 __device__ __forceinline__ float lanes_max(float x) {
@@ -92,17 +97,27 @@ __device__ __forceinline__ int first_delayed(int64_t first, int chunk_n) {
   return first >= 0 ? 0 : (first <= -int64_t(chunk_n) ? chunk_n : int(-first));
 }
 
+// gated: running log-gates of chunk uc of the pass (chunk index 0 on); null without gates
+__device__ __forceinline__ const float *chunk_gates(const PrefillParams &p, int64_t uc) {
+  return p.gated ? p.gcum + size_t(uc) * p.SC : nullptr;
+}
+// what a state has decayed by over chunk k of unit u
+__device__ __forceinline__ float chunk_decay(const PrefillParams &p, int64_t u, int k) {
+  return p.gated ? expf(chunk_gates(p, u * p.nsub + k)[min(p.SC, p.C - k * p.SC) - 1]) : 1.f;
+}
+
 // 1. One CTA per (unit, chunk, 16 rows of S): every half-warp owns two rows, a lane D / 16 columns of them.  The rows of phi
 // are made from K' as they are loaded (all of them in every CTA of a unit: cheaper than a launch in front and a trip
 // through memory), the CTA keeps its 16 columns of them.
 constexpr int kSumTok = 32;    // tokens per tile
 template <typename T, int D>
-__global__ void __launch_bounds__(kThreads) prefill_fma_sums_kernel(const PrefillParams p) {
+__global__ void __launch_bounds__(2 * kThreads) prefill_fma_sums_kernel(const PrefillParams p) {
   constexpr int LD = kSumTok * D / 4 / kThreads;   // float4 per thread and tile
   constexpr int CG = D / 64;                       // groups of four columns per thread
-  __shared__ __align__(16) float ph[2][kSumTok][16];
+  static_assert(2 * kThreads * (4 * CG + 1) <= kSumTok * D, "the second group's sums fit its tile");
+  __shared__ __align__(16) float ph[2][kSumTok][16];   // [group]
   __shared__ __align__(16) float vt[2][kSumTok][D];
-  const int tid = threadIdx.x;
+  const int grp = threadIdx.x / kThreads, tid = threadIdx.x % kThreads;
   const int rb = int(blockIdx.x % (D / 16));
   const int64_t uc = blockIdx.x / (D / 16);
   const UnitId id = unit_id(p, uc / p.nsub);
@@ -113,6 +128,8 @@ __global__ void __launch_bounds__(kThreads) prefill_fma_sums_kernel(const Prefil
   const int i_lo = first_delayed(first, chunk_n);
   if (i_lo >= chunk_n) return;                     // (the readers of the sums leave such chunks out as well)
   const Rows<T, D> rows(p, ld, id.lrel, id.b, id.g);
+  const float *gc = chunk_gates(p, uc);
+  const float g_end = gc ? gc[chunk_n - 1] : 0.f;
   float4 kr[LD], vr[LD];
   auto fetch = [&](int i0) {
 #pragma unroll
@@ -130,25 +147,28 @@ __global__ void __launch_bounds__(kThreads) prefill_fma_sums_kernel(const Prefil
   float acc[2][4 * CG], zacc = 0.f;
 #pragma unroll
   for (int c = 0; c < 4 * CG; ++c) acc[0][c] = acc[1][c] = 0.f;
-  fetch(i_lo);
-  int buf = 0;
-  for (int i0 = i_lo; i0 < chunk_n; i0 += kSumTok, buf ^= 1) {
+  fetch(i_lo + grp * kSumTok);
+  for (int i0 = i_lo + grp * kSumTok; i0 < chunk_n; i0 += 2 * kSumTok) {
 #pragma unroll
     for (int i = 0; i < LD; ++i) {
       const int e = tid + kThreads * i, r = e / (D / 4), c = e % (D / 4) * 4;
       float4 f = row_phi<D>(kr[i]);
       if (i0 + r >= chunk_n) f = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (c >> 4 == rb) *reinterpret_cast<float4 *>(&ph[buf][r][c & 15]) = f;
-      *reinterpret_cast<float4 *>(&vt[buf][r][c]) = vr[i];
+      else if (gc) {   // what the token has decayed to by the end of the chunk
+        const float dec = expf(g_end - gc[i0 + r]);
+        f = make_float4(f.x * dec, f.y * dec, f.z * dec, f.w * dec);
+      }
+      if (c >> 4 == rb) *reinterpret_cast<float4 *>(&ph[grp][r][c & 15]) = f;
+      *reinterpret_cast<float4 *>(&vt[grp][r][c]) = vr[i];
     }
-    __syncthreads();   // (two buffers: the tile before the previous one has been read by everyone)
-    if (i0 + kSumTok < chunk_n) fetch(i0 + kSumTok);
+    group_sync(grp);
+    if (i0 + 2 * kSumTok < chunk_n) fetch(i0 + 2 * kSumTok);
 #pragma unroll 8
     for (int i = 0; i < kSumTok; ++i) {
-      const float2 f = *reinterpret_cast<const float2 *>(&ph[buf][i][row]);
+      const float2 f = *reinterpret_cast<const float2 *>(&ph[grp][i][row]);
 #pragma unroll
       for (int q = 0; q < CG; ++q) {
-        const float4 v = *reinterpret_cast<const float4 *>(&vt[buf][i][q * 64 + cg * 4]);
+        const float4 v = *reinterpret_cast<const float4 *>(&vt[grp][i][q * 64 + cg * 4]);
         acc[0][q * 4 + 0] = fmaf(f.x, v.x, acc[0][q * 4 + 0]);
         acc[0][q * 4 + 1] = fmaf(f.x, v.y, acc[0][q * 4 + 1]);
         acc[0][q * 4 + 2] = fmaf(f.x, v.z, acc[0][q * 4 + 2]);
@@ -161,9 +181,26 @@ __global__ void __launch_bounds__(kThreads) prefill_fma_sums_kernel(const Prefil
     }
     if (tid < 16) {
 #pragma unroll 8
-      for (int i = 0; i < kSumTok; ++i) zacc += ph[buf][i][tid];
+      for (int i = 0; i < kSumTok; ++i) zacc += ph[grp][i][tid];
     }
+    group_sync(grp);
   }
+  // the second group's sums on top of the first's, through the second group's tile
+  float (*other)[4 * CG + 1] = reinterpret_cast<float (*)[4 * CG + 1]>(&vt[1][0][0]);   // [2 * kThreads]
+  if (grp == 1) {
+#pragma unroll
+    for (int r = 0; r < 2; ++r)
+#pragma unroll
+      for (int c = 0; c < 4 * CG; ++c) other[r * kThreads + tid][c] = acc[r][c];
+    if (tid < 16) ph[1][0][tid] = zacc;
+  }
+  __syncthreads();
+  if (grp == 1) return;
+#pragma unroll
+  for (int r = 0; r < 2; ++r)
+#pragma unroll
+    for (int c = 0; c < 4 * CG; ++c) acc[r][c] += other[r * kThreads + tid][c];
+  if (tid < 16) zacc += ph[1][0][tid];
   float *dst = p.phik + (size_t(uc) * D + rb * 16 + row) * D + cg * 4;
 #pragma unroll
   for (int r = 0; r < 2; ++r)
@@ -173,29 +210,32 @@ __global__ void __launch_bounds__(kThreads) prefill_fma_sums_kernel(const Prefil
   if (tid < 16) p.zsnap[size_t(uc) * D + rb * 16 + tid] = zacc;
 }
 
-// 2. Tiles of KT rows in turn: the window's keys, the chunk's delayed tokens, the rows of the state.  Per tile a half-warp
+// 2. Tiles of KT rows: group 0 takes the window's keys, group 1 the chunk's delayed tokens and the rows of the state; group
+// 0 merges and stores.  Per tile a half-warp
 // computes the weights of its two rows (a lane KT / 16 keys), keeps them in shared memory for itself, and adds the weighted
 // V (or S) rows (a lane D / 16 columns).
 template <int D>
 struct AttnSmem {
   static constexpr int KT = 4096 / D;             // 64 rows for d = 64, 32 for d = 128: 16 float4 per thread and tile
-  float q[kRows][D + 4];                          // scaled to the log2 domain
-  float pq[kRows][D + 4];                         // phi(q)
-  float k[KT][D + 4];                             // (+ 4: rows start four banks apart)
-  float v[KT][D];
-  float p[kRows][KT + 4];
+  struct Group {
+    float a[kRows][D + 4];                        // q in the log2 domain, or phi(q)
+    float k[KT][D + 4];                           // (+ 4: rows start four banks apart)
+    float v[KT][D];
+    float p[kRows][KT + 4];
+  } grp[2];
 };
 
 template <typename T, int D, int G>
-__global__ void __launch_bounds__(kThreads) prefill_fma_attn_kernel(const PrefillParams p) {
+__global__ void __launch_bounds__(2 * kThreads) prefill_fma_attn_kernel(const PrefillParams p) {
   constexpr int KT = AttnSmem<D>::KT;
   constexpr int LD = KT * D / 4 / kThreads;        // float4 of K (and of V) per thread and tile
   constexpr int KPT = KT / 16;                     // keys per lane
   constexpr int CG = D / 64;
   constexpr int TOK = kRows / G;                   // tokens per CTA
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  AttnSmem<D> &sm = *reinterpret_cast<AttnSmem<D> *>(smem_raw);
-  const int tid = threadIdx.x;
+  const int grp = threadIdx.x / kThreads, tid = threadIdx.x % kThreads;
+  auto &all = *reinterpret_cast<AttnSmem<D> *>(smem_raw);
+  typename AttnSmem<D>::Group &sm = all.grp[grp];
   const int per_chunk = (p.SC + TOK - 1) / TOK;
   const int per_unit = (p.nsub - 1) * per_chunk + (p.C - (p.nsub - 1) * p.SC + TOK - 1) / TOK;
   const UnitId id = unit_id(p, blockIdx.x / per_unit);
@@ -203,21 +243,32 @@ __global__ void __launch_bounds__(kThreads) prefill_fma_attn_kernel(const Prefil
   const int sub = cta / per_chunk, tok0 = (cta - sub * per_chunk) * TOK;
   const int chunk_c0 = sub * p.SC, chunk_n = min(p.SC, p.C - chunk_c0);
   const int ntok = min(TOK, chunk_n - tok0);
+  const size_t seq_row = (size_t(id.lrel) * p.B + id.b) * size_t(p.T) + size_t(p.c0 + chunk_c0 + tok0);
+  // the 16 query rows (D / 4 lanes of one row, as in the tiles), asked for before anything else
+  constexpr int LQ = kRows * D / 4 / kThreads;
+  float4 qr[LQ];
+#pragma unroll
+  for (int i = 0; i < LQ; ++i) {
+    const int e = tid + kThreads * i, r = e / (D / 4), c = e % (D / 4) * 4;
+    qr[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (r / G < ntok)
+      qr[i] = load4(reinterpret_cast<const T *>(p.q) + ((seq_row + r / G) * p.H + p.heads_of[id.g * G + r % G]) * D + c);
+  }
   const LayerDev ld = p.layers[p.layer_begin + id.lrel];
   const Rows<T, D> rows(p, ld, id.lrel, id.b, id.g);
   const int64_t tq0 = p.n0 + p.c0 + chunk_c0 + tok0, tq_last = tq0 + ntok - 1;
-  const size_t seq_row = (size_t(id.lrel) * p.B + id.b) * size_t(p.T) + size_t(p.c0 + chunk_c0 + tok0);
 
-  // tiles: n_win of window keys from j_lo on, n_int of delayed tokens from chunk index i_lo on, n_st of state rows
-  const int64_t w_lo = tq0 - ld.w + 1;
-  const int64_t j_lo = w_lo < 0 ? 0 : w_lo;
-  const int n_win = ld.w > 0 ? int((tq_last - j_lo) / KT) + 1 : 0;
+  // the group's tiles: n_st of state rows (they decay with the row, so they come first), then n_rows of key rows from token
+  // j_lo on, up to token j_hi
   const bool linear = ld.evicts && tq_last >= ld.wlin;
   const int64_t first = p.n0 + p.c0 + chunk_c0 - ld.wlin;      // delayed token of chunk index 0
-  const int i_lo = first_delayed(first, chunk_n), i_hi = tok0 + ntok - 1;
-  const int n_int = linear && i_lo <= i_hi ? (i_hi - i_lo) / KT + 1 : 0;
-  const int n_st = linear && first > 0 ? D / KT : 0;
-  const int n_tiles = n_win + n_int + n_st;
+  const int64_t w_lo = tq0 - ld.w + 1;
+  const int64_t j_lo = grp == 0 ? (w_lo < 0 ? 0 : w_lo) : (first < 0 ? 0 : first);
+  const int64_t j_hi = grp == 0 ? tq_last : first + tok0 + ntok - 1;
+  const bool any = grp == 0 ? ld.w > 0 : linear;
+  const int n_rows = any && j_hi >= j_lo ? int((j_hi - j_lo) / KT) + 1 : 0;
+  const int n_st = grp == 1 && linear && first > 0 ? D / KT : 0;
+  const int n_tiles = n_rows + n_st;
   // sums of the chunks before this one that hold delayed tokens: [sub0, sub)
   const int sub0 = first - int64_t(chunk_c0) >= 0 ? 0 : int(-(first - chunk_c0) / p.SC);
   const float *sums = p.phik + size_t(id.u) * p.nsub * D * D;
@@ -226,70 +277,59 @@ __global__ void __launch_bounds__(kThreads) prefill_fma_attn_kernel(const Prefil
 
   float4 kr[LD], vr[LD];
   auto fetch = [&](int t) {
+    if (t >= n_st) {
 #pragma unroll
-    for (int i = 0; i < LD; ++i) {
-      const int e = tid + kThreads * i, r = e / (D / 4), c = e % (D / 4) * 4;
-      kr[i] = vr[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (t < n_win + n_int) {
-        const bool win = t < n_win;
-        const int64_t j = win ? j_lo + int64_t(t) * KT + r : first + i_lo + (t - n_win) * KT + r;
-        if (j <= (win ? tq_last : first + i_hi)) {
+      for (int i = 0; i < LD; ++i) {
+        const int e = tid + kThreads * i, r = e / (D / 4), c = e % (D / 4) * 4;
+        kr[i] = vr[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+        const int64_t j = j_lo + int64_t(t - n_st) * KT + r;
+        if (j <= j_hi) {
           const int64_t off = rows.at(j);
           kr[i] = rows.k(off, c);
           vr[i] = rows.v(off, c);
         }
-      } else {
-        const size_t at = size_t((t - n_win - n_int) * KT + r) * D + c;
-        float4 s = *reinterpret_cast<const float4 *>(Sb + at);
-        for (int k = sub0; k < sub; ++k) {
-          const float4 x = *reinterpret_cast<const float4 *>(sums + size_t(k) * D * D + at);
-          s.x += x.x, s.y += x.y, s.z += x.z, s.w += x.w;
-        }
-        vr[i] = s;
+      }
+    } else {
+      const size_t at0 = size_t(t) * KT * D + tid * 4;   // (a tile's rows are contiguous)
+#pragma unroll
+      for (int i = 0; i < LD; ++i) vr[i] = *reinterpret_cast<const float4 *>(Sb + at0 + i * kThreads * 4);
+      for (int k = sub0; k < sub; ++k) {
+        const float dec = chunk_decay(p, id.u, k);
+#pragma unroll
+        for (int i = 0; i < LD; ++i) kr[i] = *reinterpret_cast<const float4 *>(sums + size_t(k) * D * D + at0 + i * kThreads * 4);
+#pragma unroll
+        for (int i = 0; i < LD; ++i)
+          vr[i] = make_float4(fmaf(vr[i].x, dec, kr[i].x), fmaf(vr[i].y, dec, kr[i].y), fmaf(vr[i].z, dec, kr[i].z), fmaf(vr[i].w, dec, kr[i].w));
       }
     }
   };
   if (n_tiles > 0) fetch(0);
-  // the 16 query rows, and phi of them (D / 4 lanes of one row, as in the tiles)
 #pragma unroll
-  for (int i = 0; i < kRows * D / 4 / kThreads; ++i) {
+  for (int i = 0; i < LQ; ++i) {
     const int e = tid + kThreads * i, r = e / (D / 4), c = e % (D / 4) * 4;
-    const int tk = r / G, head = p.heads_of[id.g * G + r % G];
-    float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (tk < ntok) x = load4(reinterpret_cast<const T *>(p.q) + ((seq_row + tk) * p.H + head) * D + c);
-    *reinterpret_cast<float4 *>(&sm.pq[r][c]) = row_phi<D>(x);
-    *reinterpret_cast<float4 *>(&sm.q[r][c]) = make_float4(x.x * p.scale_log2, x.y * p.scale_log2, x.z * p.scale_log2, x.w * p.scale_log2);
+    const float4 x = qr[i];
+    *reinterpret_cast<float4 *>(&sm.a[r][c]) =
+        grp ? row_phi<D>(x) : make_float4(x.x * p.scale_log2, x.y * p.scale_log2, x.z * p.scale_log2, x.w * p.scale_log2);
   }
 
+  // o: window accumulator or linear one; l: the lane's part of the row's weight sum
   const int row = (tid >> 4) * 2, cg = tid & 15;
-  float acc[2][4 * CG], lin[2][4 * CG], m[2], l[2], bl[2];
-  int64_t tq[2];
+  float o[2][4 * CG], m[2], l[2];
+  const float *gc = grp == 1 && linear ? chunk_gates(p, id.u * p.nsub + sub) : nullptr;
+  float g_own[2];
+  int64_t last[2];                                 // last token that counts for the row: its own, or its own delayed one
 #pragma unroll
   for (int r = 0; r < 2; ++r) {
     m[r] = -CUDART_INF_F;
-    l[r] = bl[r] = 0.f;
-    tq[r] = tq0 + (row + r) / G;
+    l[r] = 0.f;
+    last[r] = (grp == 0 ? tq0 : first + tok0) + (row + r) / G;
+    g_own[r] = gc ? gc[min(tok0 + (row + r) / G, chunk_n - 1)] : 0.f;
 #pragma unroll
-    for (int c = 0; c < 4 * CG; ++c) acc[r][c] = lin[r][c] = 0.f;
+    for (int c = 0; c < 4 * CG; ++c) o[r][c] = 0.f;
   }
-  // s[r][x] = a[row + r] . k[cg + 16 x]
-  auto scores = [&](const float (*a)[D + 4], float (&s)[2][KPT]) {
-#pragma unroll
-    for (int x = 0; x < KPT; ++x) s[0][x] = s[1][x] = 0.f;
+  // o[r] += the weights w0, w1 of rows row, row + 1 times the tile's V rows
+  auto add_rows = [&](const float *w0, const float *w1) {
 #pragma unroll 4
-    for (int c = 0; c < D; c += 4) {
-      const float4 a0 = *reinterpret_cast<const float4 *>(&a[row][c]), a1 = *reinterpret_cast<const float4 *>(&a[row + 1][c]);
-#pragma unroll
-      for (int x = 0; x < KPT; ++x) {
-        const float4 b = *reinterpret_cast<const float4 *>(&sm.k[cg + 16 * x][c]);
-        s[0][x] = fmaf(a0.w, b.w, fmaf(a0.z, b.z, fmaf(a0.y, b.y, fmaf(a0.x, b.x, s[0][x]))));
-        s[1][x] = fmaf(a1.w, b.w, fmaf(a1.z, b.z, fmaf(a1.y, b.y, fmaf(a1.x, b.x, s[1][x]))));
-      }
-    }
-  };
-  // o[r] += weights of row + r (wt, row stride ws) times the tile's V rows
-  auto add_rows = [&](const float *w0, const float *w1, float (&o)[2][4 * CG]) {
-#pragma unroll 2
     for (int i = 0; i < KT; i += 4) {
       const float4 p0 = *reinterpret_cast<const float4 *>(w0 + i), p1 = *reinterpret_cast<const float4 *>(w1 + i);
       const float f0[4] = {p0.x, p0.y, p0.z, p0.w}, f1[4] = {p1.x, p1.y, p1.z, p1.w};
@@ -311,80 +351,103 @@ __global__ void __launch_bounds__(kThreads) prefill_fma_attn_kernel(const Prefil
   };
 
   for (int t = 0; t < n_tiles; ++t) {
-    const bool win = t < n_win, intra = !win && t < n_win + n_int;
+    const bool keyed = t >= n_st;
 #pragma unroll
     for (int i = 0; i < LD; ++i) {
       const int e = tid + kThreads * i, r = e / (D / 4), c = e % (D / 4) * 4;
-      if (win) *reinterpret_cast<float4 *>(&sm.k[r][c]) = kr[i];
-      if (intra) *reinterpret_cast<float4 *>(&sm.k[r][c]) = row_phi<D>(kr[i]);   // (uniform over the CTA)
+      if (keyed) *reinterpret_cast<float4 *>(&sm.k[r][c]) = grp ? row_phi<D>(kr[i]) : kr[i];   // (uniform over the group)
       *reinterpret_cast<float4 *>(&sm.v[r][c]) = vr[i];
     }
-    __syncthreads();
+    group_sync(grp);
     if (t + 1 < n_tiles) fetch(t + 1);
-    if (win) {
+    if (keyed) {
+      // s[r][x] = a[row + r] . k[cg + 16 x]
       float s[2][KPT];
-      scores(sm.q, s);
-      const int64_t j0 = j_lo + int64_t(t) * KT + cg;
+#pragma unroll
+      for (int x = 0; x < KPT; ++x) s[0][x] = s[1][x] = 0.f;
+#pragma unroll 4
+      for (int c = 0; c < D; c += 4) {
+        const float4 a0 = *reinterpret_cast<const float4 *>(&sm.a[row][c]), a1 = *reinterpret_cast<const float4 *>(&sm.a[row + 1][c]);
+#pragma unroll
+        for (int x = 0; x < KPT; ++x) {
+          const float4 b = *reinterpret_cast<const float4 *>(&sm.k[cg + 16 * x][c]);
+          s[0][x] = fmaf(a0.w, b.w, fmaf(a0.z, b.z, fmaf(a0.y, b.y, fmaf(a0.x, b.x, s[0][x]))));
+          s[1][x] = fmaf(a1.w, b.w, fmaf(a1.z, b.z, fmaf(a1.y, b.y, fmaf(a1.x, b.x, s[1][x]))));
+        }
+      }
+      const int64_t j0 = j_lo + int64_t(t - n_st) * KT + cg;
 #pragma unroll
       for (int r = 0; r < 2; ++r) {
-        float mx = -CUDART_INF_F;
+        if (grp == 0) {
+          float mx = -CUDART_INF_F;
+#pragma unroll
+          for (int x = 0; x < KPT; ++x) {
+            const int64_t j = j0 + 16 * x;
+            if (j > last[r] || j <= last[r] - ld.w) s[r][x] = -CUDART_INF_F;
+            mx = fmaxf(mx, s[r][x]);
+          }
+          const float mn = fmaxf(m[r], lanes_max<16>(mx));
+          const float f = m[r] == -CUDART_INF_F ? 0.f : exp2f(m[r] - mn);
+          m[r] = mn;
+          l[r] *= f;
+#pragma unroll
+          for (int c = 0; c < 4 * CG; ++c) o[r][c] *= f;
+        }
 #pragma unroll
         for (int x = 0; x < KPT; ++x) {
           const int64_t j = j0 + 16 * x;
-          if (j > tq[r] || j <= tq[r] - ld.w) s[r][x] = -CUDART_INF_F;
-          mx = fmaxf(mx, s[r][x]);
-        }
-        const float mn = fmaxf(m[r], lanes_max<16>(mx));
-        const float f = m[r] == -CUDART_INF_F ? 0.f : exp2f(m[r] - mn);
-        m[r] = mn;
-        l[r] *= f;
-#pragma unroll
-        for (int c = 0; c < 4 * CG; ++c) acc[r][c] *= f;
-#pragma unroll
-        for (int x = 0; x < KPT; ++x) {
-          const float e = s[r][x] == -CUDART_INF_F ? 0.f : exp2f(s[r][x] - mn);
+          float e = grp == 0 ? (s[r][x] == -CUDART_INF_F ? 0.f : exp2f(s[r][x] - m[r])) : (j <= last[r] ? s[r][x] : 0.f);
+          if (gc && j <= last[r]) e *= expf(g_own[r] - gc[j - first]);   // what delayed token j has decayed to
           l[r] += e;
           sm.p[row + r][cg + 16 * x] = e;
         }
       }
       __syncwarp();
-      add_rows(sm.p[row], sm.p[row + 1], acc);
-    } else if (intra) {
-      float s[2][KPT];
-      scores(sm.pq, s);
-      const int ii = i_lo + (t - n_win) * KT + cg;
+      add_rows(sm.p[row], sm.p[row + 1]);
+    } else {
+      add_rows(&sm.a[row][t * KT], &sm.a[row + 1][t * KT]);
+      if (t + 1 == n_st) {   // the state's part is complete: phi(q) . z, and what both have decayed to by the row's token
+        const float *zb = reinterpret_cast<const float *>(p.ws + ld.z) + size_t(ub) * D;
+        const float *zs = p.zsnap + size_t(id.u) * p.nsub * D;
+        float z[D / 16];
 #pragma unroll
-      for (int r = 0; r < 2; ++r) {
-        const int own = tok0 + (row + r) / G;      // delayed tokens up to and including the query's own
+        for (int i = 0; i < D / 16; ++i) z[i] = zb[cg + 16 * i];
+        for (int k = sub0; k < sub; ++k) {
+          const float dec = chunk_decay(p, id.u, k);
 #pragma unroll
-        for (int x = 0; x < KPT; ++x) {
-          const float e = ii + 16 * x <= own ? s[r][x] : 0.f;
-          bl[r] += e;
-          sm.p[row + r][cg + 16 * x] = e;
+          for (int i = 0; i < D / 16; ++i) z[i] = fmaf(z[i], dec, zs[size_t(k) * D + cg + 16 * i]);
+        }
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+#pragma unroll
+          for (int i = 0; i < D / 16; ++i) l[r] = fmaf(sm.a[row + r][cg + 16 * i], z[i], l[r]);
+          const float dec = gc ? expf(g_own[r]) : 1.f;
+          l[r] *= dec;
+#pragma unroll
+          for (int c = 0; c < 4 * CG; ++c) o[r][c] *= dec;
         }
       }
-      __syncwarp();
-      add_rows(sm.p[row], sm.p[row + 1], lin);
-    } else {
-      const int r0 = (t - n_win - n_int) * KT;
-      add_rows(&sm.pq[row][r0], &sm.pq[row + 1][r0], lin);
     }
-    __syncthreads();
+    group_sync(grp);
   }
-  if (n_st > 0) {   // phi(q) . z
-    const float *zb = reinterpret_cast<const float *>(p.ws + ld.z) + size_t(ub) * D;
-    const float *zs = p.zsnap + size_t(id.u) * p.nsub * D;
 #pragma unroll
-    for (int i = 0; i < D / 16; ++i) {
-      float z = zb[cg + 16 * i];
-      for (int k = sub0; k < sub; ++k) z += zs[size_t(k) * D + cg + 16 * i];
-      bl[0] = fmaf(sm.pq[row][cg + 16 * i], z, bl[0]);
-      bl[1] = fmaf(sm.pq[row + 1][cg + 16 * i], z, bl[1]);
+  for (int r = 0; r < 2; ++r) l[r] = lanes_sum<16>(l[r]);
+  // group 1 hands its part over in its V tile (16 x d floats) and the row sums in its weights
+  float *lin = &all.grp[1].v[0][0], *lsum = &all.grp[1].p[0][0];
+  if (grp == 1) {
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+#pragma unroll
+      for (int q = 0; q < CG; ++q)
+        *reinterpret_cast<float4 *>(lin + (row + r) * D + q * 64 + cg * 4) = make_float4(o[r][q * 4], o[r][q * 4 + 1], o[r][q * 4 + 2], o[r][q * 4 + 3]);
+      if (cg == 0) lsum[row + r] = l[r];
     }
   }
+  __syncthreads();
+  if (grp == 1) return;
 #pragma unroll
   for (int r = 0; r < 2; ++r) {
-    const float L = lanes_sum<16>(l[r]), Bl = lanes_sum<16>(bl[r]);
+    const float L = l[r], Bl = lsum[row + r];
     const int tk = (row + r) / G, head = p.heads_of[id.g * G + (row + r) % G];
     // shared normaliser (reference max(window maximum, 0): the floor belongs to the linear terms, logit 0), or the sum of
     // the two separately normalised terms (an empty term counts as zero)
@@ -402,9 +465,11 @@ __global__ void __launch_bounds__(kThreads) prefill_fma_attn_kernel(const Prefil
     if (tk < ntok) {
       T *op = reinterpret_cast<T *>(p.out) + ((seq_row + tk) * p.H + head) * D + cg * 4;
 #pragma unroll
-      for (int q = 0; q < CG; ++q)
-        store4(op + q * 64, make_float4(fmaf(acc[r][q * 4], fa, lin[r][q * 4] * fb), fmaf(acc[r][q * 4 + 1], fa, lin[r][q * 4 + 1] * fb),
-                                        fmaf(acc[r][q * 4 + 2], fa, lin[r][q * 4 + 2] * fb), fmaf(acc[r][q * 4 + 3], fa, lin[r][q * 4 + 3] * fb)));
+      for (int q = 0; q < CG; ++q) {
+        const float4 x = *reinterpret_cast<const float4 *>(lin + (row + r) * D + q * 64 + cg * 4);
+        store4(op + q * 64, make_float4(fmaf(o[r][q * 4], fa, x.x * fb), fmaf(o[r][q * 4 + 1], fa, x.y * fb),
+                                        fmaf(o[r][q * 4 + 2], fa, x.z * fb), fmaf(o[r][q * 4 + 3], fa, x.w * fb)));
+      }
     }
   }
 }
@@ -431,7 +496,8 @@ __global__ void __launch_bounds__(kThreads) prefill_fma_finish_kernel(const Pref
 #pragma unroll 4
     for (int k = k0; k < p.nsub; ++k) {
       const float4 x = *reinterpret_cast<const float4 *>(sums + size_t(k) * D * D);
-      s.x += x.x, s.y += x.y, s.z += x.z, s.w += x.w;
+      const float dec = chunk_decay(p, id.u, k);
+      s = make_float4(fmaf(s.x, dec, x.x), fmaf(s.y, dec, x.y), fmaf(s.z, dec, x.z), fmaf(s.w, dec, x.w));
     }
     *Sp = s;
     if (at < D) {
@@ -439,7 +505,8 @@ __global__ void __launch_bounds__(kThreads) prefill_fma_finish_kernel(const Pref
       float4 z = *zp;
       for (int k = k0; k < p.nsub; ++k) {
         const float4 x = *reinterpret_cast<const float4 *>(p.zsnap + (size_t(id.u) * p.nsub + k) * D + at);
-        z.x += x.x, z.y += x.y, z.z += x.z, z.w += x.w;
+        const float dec = chunk_decay(p, id.u, k);
+        z = make_float4(fmaf(z.x, dec, x.x), fmaf(z.y, dec, x.y), fmaf(z.z, dec, x.z), fmaf(z.w, dec, x.w));
       }
       *zp = z;
     }
@@ -458,6 +525,8 @@ __global__ void __launch_bounds__(kThreads) prefill_fma_finish_kernel(const Pref
   const size_t dst = ((size_t(id.b + p.b0) * p.Hkv + id.g) * size_t(ld.cap) + slot) * D + c;
   store4(reinterpret_cast<T *>(p.ws + ld.ringK) + dst, load4(reinterpret_cast<const T *>(p.k) + src));
   store4(reinterpret_cast<T *>(p.ws + ld.ringV) + dst, load4(reinterpret_cast<const T *>(p.v) + src));
+  if (p.gated && c == 0)   // the token's gate waits in the ring with it
+    reinterpret_cast<float *>(p.ws + ld.ringG)[dst / D] = p.gate ? p.gate[src / D] : 1.f;   // ([layer][B][T][Hkv], as K's rows)
 }
 
 }  // namespace
@@ -470,7 +539,7 @@ int launch_prefill_fma(glide_ctx *ctx, const PrefillParams &p, cudaStream_t stre
   return dispatch_config(ctx->cfg.io_dtype, ctx->cfg.head_dim, ctx->G, [&](auto tt, auto dd, auto gg) -> int {
     using T = typename decltype(tt)::type;
     constexpr int D = decltype(dd)::value, G = decltype(gg)::value, TOK = kRows / G;
-    if (any_evicts) prefill_fma_sums_kernel<T, D><<<unsigned(units * p.nsub * (D / 16)), kThreads, 0, stream>>>(p);
+    if (any_evicts) prefill_fma_sums_kernel<T, D><<<unsigned(units * p.nsub * (D / 16)), 2 * kThreads, 0, stream>>>(p);
     if (p.out) {
       auto kern = prefill_fma_attn_kernel<T, D, G>;
       if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(sizeof(AttnSmem<D>))) != cudaSuccess) {
@@ -478,7 +547,7 @@ int launch_prefill_fma(glide_ctx *ctx, const PrefillParams &p, cudaStream_t stre
         return GLIDE_ERR_CUDA;
       }
       const int64_t blocks = units * (int64_t(p.nsub - 1) * ((p.SC + TOK - 1) / TOK) + (p.C - (p.nsub - 1) * p.SC + TOK - 1) / TOK);
-      kern<<<unsigned(blocks), kThreads, sizeof(AttnSmem<D>), stream>>>(p);
+      kern<<<unsigned(blocks), 2 * kThreads, sizeof(AttnSmem<D>), stream>>>(p);
     }
     const unsigned state_blocks = any_evicts ? unsigned(units * (D * D / 4 / kThreads)) : 0u;
     const unsigned ring_blocks = unsigned((units * p.C * (D / 4) + kThreads - 1) / kThreads);

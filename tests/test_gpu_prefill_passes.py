@@ -30,6 +30,18 @@ def test_gated_prefill_on_tcgen05(G, chunk, calls):
 @pytest.mark.parametrize("dtype,d,G,merge,chunk,calls", [
     (torch.float32, 64, 1, 0, 0, [1, 65, 512]), (torch.float32, 64, 4, 1, 0, [700, 3]), (torch.float32, 128, 2, 2, 0, [130, 257]),
     (torch.float32, 64, 8, 0, 16, [40, 300]), (torch.float32, 128, 1, 0, 512, [600]), (BF16, 64, 2, 0, 0, [65, 300])])
-def test_cuda_core_passes(dtype, d, G, merge, chunk, calls):
+@pytest.mark.parametrize("gated", [False, True])
+def test_cuda_core_passes(dtype, d, G, merge, chunk, calls, gated):
     amp = 4 * d ** -0.5
-    run_case([0, 16, 100, 300, 1 << 20], 2, 2 * G, 2, d, dtype, calls, 2, amp=amp, seed=47 + G, merge=merge, prefill_chunk=chunk)
+    run_case([0, 16, 100, 300, 1 << 20], 2, 2 * G, 2, d, dtype, calls, 2, amp=amp, seed=47 + G, merge=merge, gated=gated and merge == 0,
+             prefill_chunk=chunk)
+
+
+# one CTA per unit (decode on the CUDA cores): rings at and beside the length where the work list takes over, rows not
+# filling a warp's batch, every merge, the learned map, gates
+@pytest.mark.parametrize("dtype,d,G,windows,kw", [
+    (torch.float32, 64, 1, [0, 1, 63, 512], dict()), (torch.float32, 64, 1, [513, 64], dict()), (torch.float32, 128, 8, [320, 7], dict()),
+    (torch.float32, 128, 2, [321], dict(merge=1)), (BF16, 128, 4, [40, 0], dict(merge=2, decode_impl=glide.GLIDE_DECODE_FMA)),
+    (torch.float32, 128, 4, [33, 0, 1 << 20], dict(phi=1)), (torch.float32, 64, 2, [31, 0], dict(gated=True))])
+def test_decode_by_unit(dtype, d, G, windows, kw):
+    run_case(windows, 2, 2 * G, 2, d, dtype, [70], 3, amp=4 * d ** -0.5, seed=53 + G, max_tokens=600, **kw)
