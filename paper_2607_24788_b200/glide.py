@@ -136,8 +136,14 @@ def _ptr(t: Optional[torch.Tensor]) -> Optional[int]:
 
 
 def _stream(stream: Optional[torch.cuda.Stream]) -> Optional[int]:
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return s.cuda_stream or None
+    if stream is None:   # the raw handle of the current device's current stream, without a Stream object around it
+        return _raw_stream(_current_device()) or None
+    return stream.cuda_stream or None
+
+
+# torch.cuda.current_stream() builds an object per call (2.5 us of a step's host time); these are what it asks
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None) or (lambda dev: torch.cuda.current_stream(dev).cuda_stream)
+_current_device = getattr(torch._C, "_cuda_getDevice", None) or torch.cuda.current_device
 
 
 def make_config(windows: Sequence[int], batch: int, n_q_heads: int, n_kv_heads: int, head_dim: int, max_tokens: int,
@@ -203,6 +209,17 @@ class Glide:
             _check(self.lib.glide_create(ctypes.byref(self.cfg), self._ws_ptr, self.workspace_bytes, _stream(None),
                                          ctypes.byref(handle)), "glide_create")
         self._h = handle
+        self._q_row, self._kv_row = (batch, n_q_heads, head_dim), (batch, n_kv_heads, head_dim)   # a layer's tensors
+
+    def _step_args(self, q, k, v, out, layer_count: int):
+        """Checks of a decode step's tensors (layer_count layers); their addresses."""
+        q_shape, kv_shape = (layer_count, *self._q_row), (layer_count, *self._kv_row)
+        assert q.shape == q_shape and out.shape == q_shape and k.shape == kv_shape and v.shape == kv_shape
+        dt = self.dtype
+        assert q.dtype is dt and k.dtype is dt and v.dtype is dt and out.dtype is dt
+        assert (q.is_cuda and k.is_cuda and v.is_cuda and out.is_cuda and q.is_contiguous() and k.is_contiguous()
+                and v.is_contiguous() and out.is_contiguous()), "device buffers must be contiguous CUDA tensors"
+        return q.data_ptr(), k.data_ptr(), v.data_ptr(), out.data_ptr()
 
     # -- the four calls of the hot path ---------------------------------------------------------
     def glide_prefill(self, q: Optional[torch.Tensor], k: torch.Tensor, v: torch.Tensor,
@@ -218,11 +235,9 @@ class Glide:
 
     def glide_decode_step(self, q: torch.Tensor, k: torch.Tensor, v: torch.Tensor, out: torch.Tensor,
                           stream=None) -> None:
-        assert q.shape == (self.L, self.B, self.H, self.d) and out.shape == q.shape
-        assert k.shape == (self.L, self.B, self.Hkv, self.d) and v.shape == k.shape
-        assert q.dtype == k.dtype == v.dtype == out.dtype == self.dtype
-        _check(self.lib.glide_decode_step(self._h, _ptr(q), _ptr(k), _ptr(v), _ptr(out), _stream(stream)),
-               "glide_decode_step")
+        rc = self.lib.glide_decode_step(self._h, *self._step_args(q, k, v, out, self.L), _stream(stream))
+        if rc:
+            _check(rc, "glide_decode_step")
 
     def glide_prefill_gated(self, q: Optional[torch.Tensor], k: torch.Tensor, v: torch.Tensor,
                             gate: Optional[torch.Tensor], out: Optional[torch.Tensor] = None, layer_begin: int = 0,
@@ -240,21 +255,18 @@ class Glide:
     def glide_decode_step_gated(self, q: torch.Tensor, k: torch.Tensor, v: torch.Tensor, gate: Optional[torch.Tensor],
                                 out: torch.Tensor, stream=None) -> None:
         """glide_decode_step of a gated context: gate fp32 [L][B][H_kv] in (0, 1], or None for gates of 1."""
-        assert q.shape == (self.L, self.B, self.H, self.d) and out.shape == q.shape
-        assert k.shape == (self.L, self.B, self.Hkv, self.d) and v.shape == k.shape
-        assert q.dtype == k.dtype == v.dtype == out.dtype == self.dtype
+        args = self._step_args(q, k, v, out, self.L)
         assert gate is None or (gate.shape == (self.L, self.B, self.Hkv) and gate.dtype == torch.float32)
-        _check(self.lib.glide_decode_step_gated(self._h, _ptr(q), _ptr(k), _ptr(v), _ptr(gate), _ptr(out),
-                                                _stream(stream)), "glide_decode_step_gated")
+        _check(self.lib.glide_decode_step_gated(self._h, *args[:3], _ptr(gate), args[3], _stream(stream)),
+               "glide_decode_step_gated")
 
     def glide_decode_step_layers(self, q: torch.Tensor, k: torch.Tensor, v: torch.Tensor, out: torch.Tensor,
                                  layer_begin: int, layer_count: int, stream=None) -> None:
         """glide_decode_step for the layers [layer_begin, layer_begin + layer_count); tensors are the range's."""
-        assert q.shape == (layer_count, self.B, self.H, self.d) and out.shape == q.shape
-        assert k.shape == (layer_count, self.B, self.Hkv, self.d) and v.shape == k.shape
-        assert q.dtype == k.dtype == v.dtype == out.dtype == self.dtype
-        _check(self.lib.glide_decode_step_layers(self._h, int(layer_begin), int(layer_count), _ptr(q), _ptr(k), _ptr(v),
-                                                 _ptr(out), _stream(stream)), "glide_decode_step_layers")
+        rc = self.lib.glide_decode_step_layers(self._h, int(layer_begin), int(layer_count), *self._step_args(q, k, v, out, layer_count),
+                                               _stream(stream))
+        if rc:
+            _check(rc, "glide_decode_step_layers")
 
     def glide_decode_step_noalloc(self, q: torch.Tensor, k: torch.Tensor, v: torch.Tensor, out: torch.Tensor,
                                   stream=None) -> None:
