@@ -189,6 +189,8 @@ struct PrefillParams {
   int32_t gated;
   const float *gate;         // the call's gates [layer_count][B][T][Hkv], or null for gates of 1
   int64_t *n_dev;            // [L] position counters
+  int32_t sm_count;
+  int32_t q_tma;             // tcgen05 kernel: the query rows come by TMA (every group's heads lie side by side)
   int64_t advance;           // the pass's last kernel adds this to its layers' counters (0: none)
   float *gcum;               // gated: running sums of log(gate) of the chunk's delayed tokens, [units][Cmax]
 };

@@ -621,6 +621,7 @@ int launch_prefill(glide_ctx *ctx, int layer_begin, int layer_count, int64_t T, 
   p.wq = ctx->cfg.phi_wq;
   p.wk = ctx->cfg.phi_wk;
   p.gated = ctx->cfg.gated;
+  p.sm_count = ctx->sm_count;
   p.n_dev = reinterpret_cast<int64_t *>(ctx->ws + ctx->off_ndev);
   p.gate = gate;
   p.gcum = reinterpret_cast<float *>(ctx->ws + ctx->off_gcum);

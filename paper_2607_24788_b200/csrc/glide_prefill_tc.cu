@@ -165,6 +165,13 @@ __device__ __forceinline__ void tma_load_4d(uint32_t dst, const void *tmap, int 
       "l"(tmap), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(bar)
       : "memory");
 }
+__device__ __forceinline__ void tma_prefetch_2d(const void *tmap, int x, int y) {
+  asm volatile("cp.async.bulk.prefetch.tensor.2d.L2.global.tile [%0, {%1, %2}];" ::"l"(tmap), "r"(x), "r"(y) : "memory");
+}
+__device__ __forceinline__ void tma_prefetch_4d(const void *tmap, int c0, int c1, int c2, int c3) {
+  asm volatile("cp.async.bulk.prefetch.tensor.4d.L2.global.tile [%0, {%1, %2, %3, %4}];" ::"l"(tmap), "r"(c0), "r"(c1), "r"(c2), "r"(c3)
+               : "memory");
+}
 // 32 columns of this thread's lane; the registers are valid only after tmem_wait_ld(r)
 __device__ __forceinline__ void tmem_ld32_nowait(uint32_t taddr, uint32_t (&r)[32]) {
   asm volatile(
@@ -244,7 +251,7 @@ struct Smem {
   float z[2 * kD];                       // z of the unit (both halves with the learned map)
   uint64_t bar_full[kStages];            // the buffer's K or V tile has landed
   uint64_t bar_free[kStages];            // the MMAs that read the buffer have completed
-  uint64_t bar_q[2];                     // Q_X staged (128 arrivals)
+  uint64_t bar_q[2];                     // Q_X staged (TMA, or the 128 threads that copied it)
   uint64_t bar_s[2];                     // MMA -> softmax threads of X: the products issued for X so far have completed
   uint64_t bar_p[2];                     // softmax threads of X -> MMA: the A operand of X's next products is ready (128)
   uint64_t bar_done;                     // every window MMA has completed
@@ -261,6 +268,7 @@ static_assert(sizeof(Smem) + 1024 <= 232448, "shared memory of one CTA");
 struct CallMaps {
   CUtensorMap k, v;         // boxes of 16 tokens
   CUtensorMap k128, v128;   // boxes of a whole 128-key tile
+  CUtensorMap q;            // {d, H, T, layers x sequences}: boxes of one row tile's tokens x the G heads of a group x 64 columns
 };
 
 // Gated: the weights stay fp32 quantities (the gated recurrence has no other tensor-core form whose precision it could
@@ -361,7 +369,7 @@ prefill_attn_tc_kernel(const PrefillParams p, const CUtensorMap *ring_maps, cons
       mbar_init(smem_u32(&sm.bar_free[s]), 1);
     }
     for (int x = 0; x < 2; ++x) {
-      mbar_init(smem_u32(&sm.bar_q[x]), kRows);
+      mbar_init(smem_u32(&sm.bar_q[x]), p.q_tma ? 1 : kRows);
       mbar_init(smem_u32(&sm.bar_s[x]), 1);
       mbar_init(smem_u32(&sm.bar_p[x]), kRows);
       mbar_init(smem_u32(&sm.bar_pk[x]), 1);
@@ -372,6 +380,14 @@ prefill_attn_tc_kernel(const PrefillParams p, const CUtensorMap *ring_maps, cons
     mbar_init(smem_u32(&sm.bar_state), 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     sm.failed = 0;
+    // Q_X, when the group's heads lie side by side: before anything else and before the other warps have set up.  (Tokens
+    // past the tile's last one are zeros or the next tile's rows: their results are not stored.)
+    for (int x = 0; p.q_tma && x < (hasB ? 2 : 1); ++x) {
+      const uint32_t bar = smem_u32(&sm.bar_q[x]), dst = smem_u32(sm.q[x]);
+      mbar_expect_tx(bar, kTileBytes);
+      tma_load_4d(dst, &cm.q, 0, g * G, chunk_c0 + tok0 + x * TOKT, lrel * p.B + b, bar);
+      tma_load_4d(dst + kBoxBytes, &cm.q, 64, g * G, chunk_c0 + tok0 + x * TOKT, lrel * p.B + b, bar);
+    }
   }
   if (warp == kLoadWarp) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(smem_u32(&sm.tmem_base)) : "memory");
@@ -396,14 +412,14 @@ prefill_attn_tc_kernel(const PrefillParams p, const CUtensorMap *ring_maps, cons
       for (int i = tid; i < n16; i += kThreads) dst[i] = make_uint4(0u, 0u, 0u, 0u);
     }
   }
-  // Q_X: 128 rows x 16 chunks by the 128 threads of each row tile, asked for before the set-up's barrier so that the copy
+  // Q_X otherwise: 128 rows x 16 chunks by the 128 threads of each row tile, asked for before the set-up's barrier so that the copy
   // runs while the other warps finish setting up (it needs nothing of that; nothing else writes these tiles).  A thread's
   // rows are 8 apart, so all of them belong to one head of the group (G divides 8).
   const int X = (tid >> 7) & 1;                   // row tile of this thread (softmax warps only)
   const int row = tid & 127;
   const int ntokX = X ? ntokB : ntokA;
   const bool activeX = tid < kSoftmaxThreads && ntokX > 0;
-  if (activeX) {
+  if (activeX && !p.q_tma) {
     const int c = row & 15, r0 = row >> 4, h2 = r0 % G;
     const bf16 *src = reinterpret_cast<const bf16 *>(p.q) +
                       ((seq + size_t(chunk_c0 + tok0 + X * TOKT)) * p.H + p.heads_of[g * G + h2]) * kD + c * 8;
@@ -571,9 +587,11 @@ prefill_attn_tc_kernel(const PrefillParams p, const CUtensorMap *ring_maps, cons
       l_sum += sum0 + sum1;
     };
     if (activeX) {
-      cp_async_wait_all();   // Q_X (asked for before the set-up's barrier) has landed
-      fence_async_smem();
-      mbar_arrive(smem_u32(&sm.bar_q[X]));
+      if (!p.q_tma) {
+        cp_async_wait_all();   // Q_X (asked for before the set-up's barrier) has landed
+        fence_async_smem();
+        mbar_arrive(smem_u32(&sm.bar_q[X]));
+      }
       const int64_t tqX0 = tq0 + X * TOKT, tqX_last = tqX0 + ntokX - 1;
       const int tf = t_first(X), te = t_end(X);
       bool ok = true;
@@ -619,36 +637,51 @@ prefill_attn_tc_kernel(const PrefillParams p, const CUtensorMap *ring_maps, cons
         if constexpr (!PHI2) {
           // this row of Q is still in the shared tile, and every S product of X has completed: phi(q) takes its place,
           // eight values at a time: maximum, then exponentials (left as bf16) and their sum, then the scaled values
+          // (four chunks are loaded before any of them is used: a store to the tile in between would hold the loads back)
           float mx = -CUDART_INF_F;
-#pragma unroll 4
-          for (int c = 0; c < 16; ++c) {
-            const uint4 v4 = *reinterpret_cast<const uint4 *>(tileX + sw128(row, c));
-            const uint32_t w4[4] = {v4.x, v4.y, v4.z, v4.w};
+          uint4 v4[4];
+          auto load_chunks = [&](int c0) {
 #pragma unroll
-            for (int e = 0; e < 4; ++e) mx = fmaxf(mx, fmaxf(__uint_as_float(w4[e] << 16), __uint_as_float(w4[e] & 0xffff0000u)));
+            for (int i = 0; i < 4; ++i) v4[i] = *reinterpret_cast<const uint4 *>(tileX + sw128(row, c0 + i));
+          };
+#pragma unroll 1
+          for (int c0 = 0; c0 < 16; c0 += 4) {
+            load_chunks(c0);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+              const uint32_t w4[4] = {v4[i].x, v4[i].y, v4[i].z, v4[i].w};
+#pragma unroll
+              for (int e = 0; e < 4; ++e) mx = fmaxf(mx, fmaxf(__uint_as_float(w4[e] << 16), __uint_as_float(w4[e] & 0xffff0000u)));
+            }
           }
           float sum0 = 0.f, sum1 = 0.f, dz0 = 0.f, dz1 = 0.f;
           const float mxl = mx * kLog2e;
           const float2 *zrow = reinterpret_cast<const float2 *>(p.zcum + (size_t(uc) * p.SC + size_t(tok_r < ntokX ? tl : tok0)) * kD);
-#pragma unroll 4
-          for (int c = 0; c < 16; ++c) {
-            uint4 *at = reinterpret_cast<uint4 *>(tileX + sw128(row, c));
-            const uint4 v4 = *at;
-            uint32_t w4[4] = {v4.x, v4.y, v4.z, v4.w};
+#pragma unroll 1
+          for (int c0 = 0; c0 < 16; c0 += 4) {
+            load_chunks(c0);
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {
-              float a0, a1;
-              fma2(a0, a1, __uint_as_float(w4[e] << 16), __uint_as_float(w4[e] & 0xffff0000u), kLog2e, -mxl);
-              const float e0 = ex2(a0), e1 = ex2(a1);
-              add2(sum0, sum1, e0, e1);
-              if (SUM) {
-                const float2 zc = __ldg(zrow + c * 4 + e);
-                dz0 = fmaf(e0, zc.x + (need_state ? sm.z[c * 8 + e * 2] : 0.f), dz0);
-                dz1 = fmaf(e1, zc.y + (need_state ? sm.z[c * 8 + e * 2 + 1] : 0.f), dz1);
+            for (int i = 0; i < 4; ++i) {
+              const int c = c0 + i;
+              uint32_t w4[4] = {v4[i].x, v4[i].y, v4[i].z, v4[i].w};
+#pragma unroll
+              for (int e = 0; e < 4; ++e) {
+                float a0, a1;
+                fma2(a0, a1, __uint_as_float(w4[e] << 16), __uint_as_float(w4[e] & 0xffff0000u), kLog2e, -mxl);
+                const float e0 = ex2(a0), e1 = ex2(a1);
+                add2(sum0, sum1, e0, e1);
+                if (SUM) {
+                  const float2 zc = __ldg(zrow + c * 4 + e);
+                  dz0 = fmaf(e0, zc.x + (need_state ? sm.z[c * 8 + e * 2] : 0.f), dz0);
+                  dz1 = fmaf(e1, zc.y + (need_state ? sm.z[c * 8 + e * 2 + 1] : 0.f), dz1);
+                }
+                w4[e] = pack_bf16x2(e0, e1);
               }
-              w4[e] = pack_bf16x2(e0, e1);
+              if (!GATED) v4[i] = make_uint4(w4[0], w4[1], w4[2], w4[3]);
             }
-            if (!GATED) *at = make_uint4(w4[0], w4[1], w4[2], w4[3]);
+            if (!GATED)
+#pragma unroll
+              for (int i = 0; i < 4; ++i) *reinterpret_cast<uint4 *>(tileX + sw128(row, c0 + i)) = v4[i];
           }
           // shared normaliser: phi(q) 2^-M;  sum of terms: phi(q) / (phi(q) . z_row) = e / (e . z_row)
           const float dz = dz0 + dz1;
@@ -662,8 +695,8 @@ prefill_attn_tc_kernel(const PrefillParams p, const CUtensorMap *ring_maps, cons
 #pragma unroll 2
             for (int c = 0; c < 16; ++c) {
               uint4 *at = reinterpret_cast<uint4 *>(tileX + sw128(row, c));
-              const uint4 v4 = *at;
-              uint32_t w4[4] = {v4.x, v4.y, v4.z, v4.w}, lo4[4];
+              const uint4 v = *at;
+              uint32_t w4[4] = {v.x, v.y, v.z, v.w}, lo4[4];
 #pragma unroll
               for (int e = 0; e < 4; ++e) {
                 float a0, a1;
@@ -681,22 +714,27 @@ prefill_attn_tc_kernel(const PrefillParams p, const CUtensorMap *ring_maps, cons
             }
             dot = (dot + dot1) * dec0;
             dot1 = 0.f;
-          } else
-#pragma unroll 4
-          for (int c = 0; c < 16; ++c) {
-            uint4 *at = reinterpret_cast<uint4 *>(tileX + sw128(row, c));
-            const uint4 v4 = *at;
-            uint32_t w4[4] = {v4.x, v4.y, v4.z, v4.w};
+          } else {
+#pragma unroll 1
+            for (int c0 = 0; c0 < 16; c0 += 4) {
+              load_chunks(c0);
 #pragma unroll
-            for (int e = 0; e < 4; ++e) w4[e] = pack_bf16x2(__uint_as_float(w4[e] << 16) * sc, __uint_as_float(w4[e] & 0xffff0000u) * sc);
-            *at = make_uint4(w4[0], w4[1], w4[2], w4[3]);
-            if (with_z) {
+              for (int i = 0; i < 4; ++i) {
+                uint32_t w4[4] = {v4[i].x, v4[i].y, v4[i].z, v4[i].w};
 #pragma unroll
-              for (int e = 0; e < 4; ++e) {
-                const float2 zz = *reinterpret_cast<const float2 *>(&sm.z[c * 8 + e * 2]);
-                dot = fmaf(__uint_as_float(w4[e] << 16), zz.x, dot);
-                dot1 = fmaf(__uint_as_float(w4[e] & 0xffff0000u), zz.y, dot1);
+                for (int e = 0; e < 4; ++e) w4[e] = pack_bf16x2(__uint_as_float(w4[e] << 16) * sc, __uint_as_float(w4[e] & 0xffff0000u) * sc);
+                v4[i] = make_uint4(w4[0], w4[1], w4[2], w4[3]);
+                if (with_z) {
+#pragma unroll
+                  for (int e = 0; e < 4; ++e) {
+                    const float2 zz = *reinterpret_cast<const float2 *>(&sm.z[(c0 + i) * 8 + e * 2]);
+                    dot = fmaf(__uint_as_float(w4[e] << 16), zz.x, dot);
+                    dot1 = fmaf(__uint_as_float(w4[e] & 0xffff0000u), zz.y, dot1);
+                  }
+                }
               }
+#pragma unroll
+              for (int i = 0; i < 4; ++i) *reinterpret_cast<uint4 *>(tileX + sw128(row, c0 + i)) = v4[i];
             }
           }
           dot += dot1;
@@ -826,14 +864,18 @@ prefill_attn_tc_kernel(const PrefillParams p, const CUtensorMap *ring_maps, cons
         // are 2 apart
         __syncwarp();
         const int c = lane & 15, r0 = (row & ~31) + (lane >> 4);
-#pragma unroll 4
-        for (int i = 0; i < 16; ++i) {
-          const int rr = r0 + 2 * i, tk = rr / G;
-          if (tk < ntokX) {
-            const uint4 val = *reinterpret_cast<const uint4 *>(sm.q[X] + sw128(rr, c));
-            bf16 *op = reinterpret_cast<bf16 *>(p.out) +
-                       ((seq + size_t(chunk_c0 + tok0 + X * TOKT + tk)) * p.H + p.heads_of[g * G + (rr - tk * G)]) * kD + c * 8;
-            *reinterpret_cast<uint4 *>(op) = val;
+        const int my_head = p.heads_of[g * G + lane % G];   // (head of group member h: lane h has it)
+        bf16 *obase = reinterpret_cast<bf16 *>(p.out) + (seq + size_t(chunk_c0 + tok0 + X * TOKT)) * p.H * kD + c * 8;
+#pragma unroll 1
+        for (int i0 = 0; i0 < 16; i0 += 4) {
+          uint4 val[4];
+#pragma unroll
+          for (int i = 0; i < 4; ++i) val[i] = *reinterpret_cast<const uint4 *>(sm.q[X] + sw128(r0 + 2 * (i0 + i), c));
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const int rr = r0 + 2 * (i0 + i), tk = rr / G;
+            const int head = __shfl_sync(0xffffffffu, my_head, rr - tk * G);
+            if (tk < ntokX) *reinterpret_cast<uint4 *>(obase + (size_t(tk) * p.H + head) * kD) = val[i];
           }
         }
       }
@@ -860,6 +902,20 @@ prefill_attn_tc_kernel(const PrefillParams p, const CUtensorMap *ring_maps, cons
     auto commit = [&](uint64_t &bar) {
       if (leader) mma_commit(smem_u32(&bar));
     };
+    // The query rows of the CTA that will take this place one wave later are asked into L2 while nothing can be issued yet
+    // (line by line: bulk prefetches of the rows took the memory pipe 12000 cycles).
+    if (int64_t(blockIdx.x) + p.sm_count < int64_t(gridDim.x)) {
+      const int64_t nb = int64_t(blockIdx.x) + p.sm_count, nu = nb / ctas_per_unit;
+      const int ncta = ctas_per_unit - 1 - int(nb % ctas_per_unit), nsub = ncta / ctas_per_chunk;
+      const int ntok0 = nsub * p.SC + (ncta - nsub * ctas_per_chunk) * TOKC;      // relative to the pass
+      const int nrows = min(TOKC, min(p.SC - (ncta - nsub * ctas_per_chunk) * TOKC, p.C - ntok0)) * G;
+      const int head = p.heads_of[int(nu % p.Hkv) * G + (lane >> 1) % G];         // (rows are 16 apart: one head per lane)
+      const bf16 *nq = reinterpret_cast<const bf16 *>(p.q) + ((nu / p.Hkv) * size_t(p.T) + size_t(p.c0 + ntok0)) * p.H * kD +
+                       size_t(head) * kD + (lane & 1) * 64;
+#pragma unroll 4
+      for (int r = lane >> 1; r < nrows; r += 16)
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(nq + size_t(r / G) * p.H * kD));
+    }
     // O_X (+)= A_X B with A_X in the S columns of X: packed bf16 behind one another, or hi and lo in turn every 32 columns
     auto issue_ts = [&](int x, uint32_t b_tile, bool accumulate) {
       if (!GATED) {
@@ -912,16 +968,18 @@ prefill_attn_tc_kernel(const PrefillParams p, const CUtensorMap *ring_maps, cons
     }
     if (ok) commit(sm.bar_done);
     if (ok && linear && !TWO) {
-      // per row tile: phi(Q) S (inter-chunk) and the first C = phi(Q) phi(K')^T in one batch
+      // the first C = phi(Q) phi(K')^T of each row tile, then phi(Q) S (inter-chunk): the softmax threads convert C while the
+      // state's products run (their completion shows in the next batch)
 #pragma unroll 1
       for (int x = 0; x < nx && ok; ++x) {
-        if (!wait_p(x)) break;
-        if (need_state && wait(sm.bar_state, 0u))
-          issue_mma(leader, tm + 256 + x * 128, q_addr(x), kv_addr(slot_state()), true, x ? te1 > tf1 : te0 > tf0);
-        if (ok && n_itiles > 0 && wait(sm.bar_pk[0], 0u))
-          issue_mma(leader, tm + x * 128, q_addr(x), kv_addr(slot_pk(0)), false, false);
-        if (ok) commit(sm.bar_s[x]);
+        if (!wait_p(x) || !wait(sm.bar_pk[0], 0u)) break;
+        issue_mma(leader, tm + x * 128, q_addr(x), kv_addr(slot_pk(0)), false, false);
+        commit(sm.bar_s[x]);
       }
+      if (ok && need_state && wait(sm.bar_state, 0u))
+#pragma unroll 1
+        for (int x = 0; x < nx; ++x)
+          issue_mma(leader, tm + 256 + x * 128, q_addr(x), kv_addr(slot_state()), true, x ? te1 > tf1 : te0 > tf0);
       for (int t = 0; t < n_itiles && ok; ++t) {
         wait(sm.bar_vp[t & 1], uint32_t(t >> 1) & 1u);
         if (ok && t + 1 < n_itiles) wait(sm.bar_pk[(t + 1) & 1], uint32_t((t + 1) >> 1) & 1u);
@@ -1087,12 +1145,25 @@ prefill_attn_tc_kernel(const PrefillParams p, const CUtensorMap *ring_maps, cons
           if (lane == 0) {
             mbar_expect_tx(bar, kTileBytes);
             const uint32_t dst = kv_addr(slot);
+            // (the same rows kAhead key tiles further on are asked into L2: a buffer is refilled one key tile before it is
+            // needed, which covers a trip to L2 but not one to memory)
+            constexpr int kAhead = 3;
+            const bool ahead = !late && ts + kAhead < n_tiles;
             if (all_call) {
               const CUtensorMap *m = is_v ? &cm.v128 : &cm.k128;
               tma_load_4d(dst, m, 0, g, int(j0 - p.n0), lrel * p.B + b, bar);
               tma_load_4d(dst + kBoxBytes, m, 64, g, int(j0 - p.n0), lrel * p.B + b, bar);
+              if (ahead) {
+                tma_prefetch_4d(m, 0, g, int(j0 - p.n0) + kAhead * kKT, lrel * p.B + b);
+                tma_prefetch_4d(m, 64, g, int(j0 - p.n0) + kAhead * kKT, lrel * p.B + b);
+              }
             } else {
-              tma_tile(dst, is_v ? ringV128 : ringK128, int(unit_rows + slot_row0), bar);
+              const CUtensorMap *m = is_v ? ringV128 : ringK128;
+              tma_tile(dst, m, int(unit_rows + slot_row0), bar);
+              if (ahead && slot_row0 + (kAhead + 1) * kKT <= cap) {
+                tma_prefetch_2d(m, 0, int(unit_rows + slot_row0) + kAhead * kKT);
+                tma_prefetch_2d(m, 64, int(unit_rows + slot_row0) + kAhead * kKT);
+              }
             }
             mbar_arrive(bar);   // the barrier's second arrival (after the row copies on the other path)
           }
@@ -1193,7 +1264,8 @@ EncodeFn tensor_map_encoder() {
 }
 }  // namespace
 
-int launch_prefill_attn_tc(glide_ctx *ctx, const PrefillParams &p, cudaStream_t stream) {
+int launch_prefill_attn_tc(glide_ctx *ctx, const PrefillParams &pass, cudaStream_t stream) {
+  PrefillParams p = pass;
   EncodeFn encode = tensor_map_encoder();
   if (!encode) return GLIDE_ERR_CUDA;
   CallMaps cm;
@@ -1209,6 +1281,17 @@ int launch_prefill_attn_tc(glide_ctx *ctx, const PrefillParams &p, cudaStream_t 
       CUresult r = encode(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void *>((kv & 1) == 0 ? p.k : p.v), dims,
                           strides, kv < 2 ? box : box128, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
                           CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+      if (r != CUDA_SUCCESS) return GLIDE_ERR_UNSUPPORTED;
+    }
+    p.q_tma = 1;
+    for (int h = 0; h < p.H; ++h) p.q_tma = p.q_tma && ctx->heads_of[size_t(h)] == h;   // groups of neighbouring heads
+    if (p.q_tma) {
+      const cuuint64_t qdims[4] = {cuuint64_t(kD), cuuint64_t(p.H), cuuint64_t(p.T), cuuint64_t(p.layer_count) * cuuint64_t(p.B)};
+      const cuuint64_t qstrides[3] = {cuuint64_t(kD) * 2, cuuint64_t(p.H) * kD * 2, cuuint64_t(p.T) * p.H * kD * 2};
+      const cuuint32_t qbox[4] = {64, cuuint32_t(ctx->G), cuuint32_t(kRows / ctx->G), 1};
+      CUresult r = encode(&cm.q, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void *>(p.q), qdims, qstrides, qbox, estr,
+                          CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                          CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
       if (r != CUDA_SUCCESS) return GLIDE_ERR_UNSUPPORTED;
     }
   }
