@@ -300,9 +300,6 @@ __device__ __forceinline__ void split2(float x0, float x1, uint32_t &hi, uint32_
   hi = pack_bf16x2(x0, x1);
   lo = pack_bf16x2(x0 - __uint_as_float(hi << 16), x1 - __uint_as_float(hi & 0xffff0000u));
 }
-__device__ __forceinline__ void prefetch_map(const void *m) {
-  asm volatile("prefetch.tensormap [%0];" ::"l"(m) : "memory");
-}
 
 template <int G, int MODE>
 __global__ void __launch_bounds__(kThreads, 1)   // 10 warps = 3 on one scheduler: 168 registers per thread at most
@@ -321,16 +318,14 @@ prefill_attn_tc_kernel(const PrefillParams p, const CUtensorMap *ring_maps, cons
   // longest of a new prompt); from here on "the chunk" is the CTA's own
   const int ctas_per_chunk = (p.SC + TOKC - 1) / TOKC;
   const int ctas_per_unit = (p.nsub - 1) * ctas_per_chunk + (p.C - (p.nsub - 1) * p.SC + TOKC - 1) / TOKC;
-  const int64_t u = blockIdx.x / ctas_per_unit;
-  const int cta_u = ctas_per_unit - 1 - int(blockIdx.x % ctas_per_unit);
+  const int u = int(blockIdx.x / unsigned(ctas_per_unit));
+  const int cta_u = ctas_per_unit - 1 - int(blockIdx.x - unsigned(u) * unsigned(ctas_per_unit));
   const int sub = cta_u / ctas_per_chunk;
   const int tok0 = (cta_u - sub * ctas_per_chunk) * TOKC;
   const int chunk_c0 = int(p.c0) + sub * p.SC;                // first token of the chunk, relative to the call
   const int chunk_n = min(p.SC, p.C - sub * p.SC);            // its tokens
-  const int64_t uc = u * p.nsub + sub;                        // (unit, chunk): index into the scratch arrays
-  const int g = int(u % p.Hkv);
-  const int b = int((u / p.Hkv) % p.B);
-  const int lrel = int(u / (int64_t(p.Hkv) * p.B));
+  const int64_t uc = int64_t(u) * p.nsub + sub;                        // (unit, chunk): index into the scratch arrays
+  const int ug = u / p.Hkv, g = u - ug * p.Hkv, lrel = ug / p.B, b = ug - lrel * p.B;
   const int layer = p.layer_begin + lrel;
   const LayerDev ld = p.layers[layer];
   const int ntok = min(TOKC, chunk_n - tok0);
@@ -363,54 +358,54 @@ prefill_attn_tc_kernel(const PrefillParams p, const CUtensorMap *ring_maps, cons
   };
   auto t_end = [&](int x) { return n_tiles == 0 ? 0 : int((tq0 + x * TOKT + (x ? ntokB : ntokA) - 1 - j_lo) / kKT) + 1; };
 
-  if (tid == kSoftmaxThreads) {
-    for (int s = 0; s < kStages; ++s) {
-      mbar_init(smem_u32(&sm.bar_full[s]), 2);
-      mbar_init(smem_u32(&sm.bar_free[s]), 1);
-    }
-    for (int x = 0; x < 2; ++x) {
-      mbar_init(smem_u32(&sm.bar_q[x]), p.q_tma ? 1 : kRows);
-      mbar_init(smem_u32(&sm.bar_s[x]), 1);
-      mbar_init(smem_u32(&sm.bar_p[x]), kRows);
-      mbar_init(smem_u32(&sm.bar_pk[x]), 1);
-      mbar_init(smem_u32(&sm.bar_vp[x]), 2);
-      mbar_init(smem_u32(&sm.bar_lfree[x]), 1);
-    }
-    mbar_init(smem_u32(&sm.bar_done), 1);
-    mbar_init(smem_u32(&sm.bar_state), 1);
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    sm.failed = 0;
-    // Q_X, when the group's heads lie side by side: before anything else and before the other warps have set up.  (Tokens
-    // past the tile's last one are zeros or the next tile's rows: their results are not stored.)
-    for (int x = 0; p.q_tma && x < (hasB ? 2 : 1); ++x) {
-      const uint32_t bar = smem_u32(&sm.bar_q[x]), dst = smem_u32(sm.q[x]);
-      mbar_expect_tx(bar, kTileBytes);
-      tma_load_4d(dst, &cm.q, 0, g * G, chunk_c0 + tok0 + x * TOKT, lrel * p.B + b, bar);
-      tma_load_4d(dst + kBoxBytes, &cm.q, 64, g * G, chunk_c0 + tok0 + x * TOKT, lrel * p.B + b, bar);
-    }
-  }
-  if (warp == kLoadWarp) {
+  if (warp == kMmaWarp) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(smem_u32(&sm.tmem_base)) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-    if (lane == 0) {
-      prefetch_map(&cm.k128);
-      prefetch_map(&cm.v128);
-      prefetch_map(&cm.k);
-      prefetch_map(&cm.v);
-    }
   }
-  // Token groups past the CTA's last token are never loaded (only the last tile has such groups), and what a
-  // masked key's V row holds is multiplied by a zero weight, so it has to be finite: those rows of the buffer that
-  // will hold the last V tile start at zero (earlier tiles that pass through the buffer leave real rows behind).
-  if (n_tiles > 0) {
-    const int last_slot = (2 * (n_tiles - 1) + 1) % kStages;
-    const int64_t j0_last = j_lo + int64_t(n_tiles - 1) * kKT;
-    const int first_skipped = int((tq_last - j0_last) / kGroup) + 1;   // groups [first_skipped, 8) are not loaded
-    const int n16 = (kKT / kGroup - first_skipped) * int(kGroupBytes / 16);
-    for (int half = 0; half < 2; ++half) {
-      uint4 *dst = reinterpret_cast<uint4 *>(&sm.kv[last_slot][half * kBoxBytes + first_skipped * kGroupBytes]);
-      for (int i = tid; i < n16; i += kThreads) dst[i] = make_uint4(0u, 0u, 0u, 0u);
+  // The loader warp sets up the barriers and is the first to go on: Q and the first K tile are on their way before the CTA
+  // meets for the first time (it needs nothing from the other warps: it zeroes what has to be zero itself).
+  if (warp == kLoadWarp) {
+    if (lane == 0) {
+      for (int s = 0; s < kStages; ++s) {
+        mbar_init(smem_u32(&sm.bar_full[s]), 2);
+        mbar_init(smem_u32(&sm.bar_free[s]), 1);
+      }
+      for (int x = 0; x < 2; ++x) {
+        mbar_init(smem_u32(&sm.bar_q[x]), p.q_tma ? 1 : kRows);
+        mbar_init(smem_u32(&sm.bar_s[x]), 1);
+        mbar_init(smem_u32(&sm.bar_p[x]), kRows);
+        mbar_init(smem_u32(&sm.bar_pk[x]), 1);
+        mbar_init(smem_u32(&sm.bar_vp[x]), 2);
+        mbar_init(smem_u32(&sm.bar_lfree[x]), 1);
+      }
+      mbar_init(smem_u32(&sm.bar_done), 1);
+      mbar_init(smem_u32(&sm.bar_state), 1);
+      asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+      sm.failed = 0;
+      // Q_X, when the group's heads lie side by side.  (Tokens past the tile's last one are zeros or the next tile's rows:
+      // their results are not stored.)
+      for (int x = 0; p.q_tma && x < (hasB ? 2 : 1); ++x) {
+        const uint32_t bar = smem_u32(&sm.bar_q[x]), dst = smem_u32(sm.q[x]);
+        mbar_expect_tx(bar, kTileBytes);
+        tma_load_4d(dst, &cm.q, 0, g * G, chunk_c0 + tok0 + x * TOKT, lrel * p.B + b, bar);
+        tma_load_4d(dst + kBoxBytes, &cm.q, 64, g * G, chunk_c0 + tok0 + x * TOKT, lrel * p.B + b, bar);
+      }
     }
+    // Token groups past the CTA's last token are never loaded (only the last tile has such groups), and what a
+    // masked key's V row holds is multiplied by a zero weight, so it has to be finite: those rows of the buffer that
+    // will hold the last V tile start at zero (earlier tiles that pass through the buffer leave real rows behind).
+    if (n_tiles > 0) {
+      const int last_slot = (2 * (n_tiles - 1) + 1) % kStages;
+      const int64_t j0_last = j_lo + int64_t(n_tiles - 1) * kKT;
+      const int first_skipped = int((tq_last - j0_last) / kGroup) + 1;   // groups [first_skipped, 8) are not loaded
+      const int n16 = (kKT / kGroup - first_skipped) * int(kGroupBytes / 16);
+      for (int half = 0; half < 2; ++half) {
+        uint4 *dst = reinterpret_cast<uint4 *>(&sm.kv[last_slot][half * kBoxBytes + first_skipped * kGroupBytes]);
+        for (int i = lane; i < n16; i += 32) dst[i] = make_uint4(0u, 0u, 0u, 0u);
+      }
+      fence_async_smem();
+    }
+    __syncwarp();   // (the barriers are set up for every lane)
   }
   // Q_X otherwise: 128 rows x 16 chunks by the 128 threads of each row tile, asked for before the set-up's barrier so that the copy
   // runs while the other warps finish setting up (it needs nothing of that; nothing else writes these tiles).  A thread's
@@ -432,12 +427,17 @@ prefill_attn_tc_kernel(const PrefillParams p, const CUtensorMap *ring_maps, cons
     }
     cp_async_commit();
   }
-  fence_async_smem();
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  const uint32_t tmem = sm.tmem_base;
-  PF_CLK(0);
+  // the CTA's first meeting: barriers and TMEM are set up (the loader comes to it with its second tile)
+  uint32_t tmem = 0;
+  auto meet = [&]() {
+    fence_async_smem();
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    tmem = sm.tmem_base;
+    PF_CLK(0);
+  };
+  if (warp != kLoadWarp) meet();
   const uint32_t sQ0 = smem_u32(sm.q[0]);
   const uint32_t sKV0 = smem_u32(sm.kv[0]);
   auto q_addr = [&](int x) { return sQ0 + uint32_t(x) * kTileBytes; };
@@ -507,81 +507,99 @@ prefill_attn_tc_kernel(const PrefillParams p, const CUtensorMap *ring_maps, cons
         tmem_st16(tS + (c >> 1), pk);
       }
     };
-    // One key tile: maximum, reference, weights.  Tiles without a masked key keep their loops unrolled; the others, one or
-    // two per row tile, keep them rolled: with everything unrolled the kernel was 210 KB of code that a CTA fetched once
-    // per phase (a CTA's first key tile took 12000 cycles, a later one 2500).
-    auto soft_tile = [&](auto masked, int lo, int hi, bool first) {
-      constexpr bool kMasked = decltype(masked)::value != 0;
-      constexpr int kUnroll = kMasked ? 1 : 2;
-      // pass 1: row maximum of the valid raw scores (the scale is positive: it is applied to the maximum)
-      float mx = -CUDART_INF_F;
-      uint32_t r[2][32];
-      tmem_ld32_nowait(tS, r[0]);
-#pragma unroll kUnroll
-      for (int c0 = 0; c0 < kKT; c0 += 64) {
-#pragma unroll
-        for (int hf = 0; hf < 2; ++hf) {
-          uint32_t (&x)[32] = r[hf];
-          const int c = c0 + hf * 32;
-          tmem_wait_ld(x);
-          if (hf == 0) tmem_ld32_nowait(tS + c + 32, r[1]);
-          else tmem_ld32_nowait(tS + ((c + 32) & (kKT - 1)), r[0]);   // (after the last columns: the first of pass 2)
-          if (kMasked) {
-            const uint32_t m = column_mask(c, lo, hi);
-#pragma unroll
-            for (int i = 0; i < 32; ++i) x[i] = (m >> i) & 1u ? x[i] : 0xff800000u;
-          }
-          float m4[4] = {mx, -CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F};
-#pragma unroll
-          for (int i = 0; i < 32; ++i) m4[i & 3] = fmaxf(m4[i & 3], __uint_as_float(x[i]));
-          mx = fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3]));
-        }
-      }
-      mx *= p.scale_log2;
-      // lazy reference: move it (and rescale O, l) only when the maximum grows by more than 2^kLazy
+    // the lazy reference for a tile whose row maximum (raw) is mx: it moves, and O and l are rescaled, only when the maximum
+    // grows by more than 2^kLazy; returns what the weights are taken against
+    auto move_ref = [&](float mx, bool first) {
+      mx *= p.scale_log2;   // (the scale is positive: it is applied to the maximum)
       float f = 1.f;
       if (mx > m_ref + kLazy || (m_ref == -CUDART_INF_F && mx > -CUDART_INF_F)) {
         f = m_ref == -CUDART_INF_F ? 0.f : ex2(m_ref - mx);
         m_ref = mx;
       }
-      tmem_wait_ld(r[0]);
       if (!first && __any_sync(0xffffffffu, f != 1.f)) scale_o(f);
       l_sum *= f;
-      const float mr = m_ref == -CUDART_INF_F ? 0.f : m_ref;
-      // pass 2: weights against the reference -> bf16, over the S columns this thread has already consumed (keys
-      // c .. c + 31 -> columns c / 2 .. c / 2 + 15); the sum uses the weights as the tensor core sees them
-      float sum0 = 0.f, sum1 = 0.f;
-#pragma unroll kUnroll
-      for (int c0 = 0; c0 < kKT; c0 += 64) {
+      return m_ref == -CUDART_INF_F ? 0.f : m_ref;
+    };
+    auto row_max = [&](const uint32_t (&x)[32], float mx) {
+      float m4[4] = {mx, -CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F};
 #pragma unroll
-        for (int hf = 0; hf < 2; ++hf) {
-          uint32_t (&x)[32] = r[hf];
-          const int c = c0 + hf * 32;
-          uint32_t pk[16];
-          tmem_wait_ld(x);
-          // the next 32 columns are on their way while these are turned into weights
-          if (hf == 0) tmem_ld32_nowait(tS + c + 32, r[1]);
-          else if (c + 32 < kKT) tmem_ld32_nowait(tS + c + 32, r[0]);
-          if (kMasked) {
-            const uint32_t m = column_mask(c, lo, hi);
+      for (int i = 0; i < 32; ++i) m4[i & 3] = fmaxf(m4[i & 3], __uint_as_float(x[i]));
+      return fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3]));
+    };
+    // weights of columns c .. c + 31 (scores x) over the S columns this thread has already consumed (columns c / 2 ..
+    // c / 2 + 15); the sum uses the weights as the tensor core sees them
+    auto weights = [&](int c, uint32_t (&x)[32], float mr, float &sum0, float &sum1) {
+      uint32_t pk[16];
 #pragma unroll
-            for (int i = 0; i < 32; ++i) x[i] = (m >> i) & 1u ? x[i] : 0xff800000u;
-          }
-#pragma unroll
-          for (int e = 0; e < 16; ++e) {
-            float a0, a1;
-            fma2(a0, a1, __uint_as_float(x[e * 2]), __uint_as_float(x[e * 2 + 1]), p.scale_log2, -mr);
-            if constexpr (GATED) {
-              a0 = ex2(a0), a1 = ex2(a1);
-              add2(sum0, sum1, a0, a1);
-              split2(a0, a1, pk[e], x[e]);   // (x[e] has been read: element e comes from x[2 e] and x[2 e + 1])
-            } else {
-              pk[e] = pack_bf16x2(ex2(a0), ex2(a1));
-              add2(sum0, sum1, __uint_as_float(pk[e] << 16), __uint_as_float(pk[e] & 0xffff0000u));
-            }
-          }
-          store_p(c, pk, x);
+      for (int e = 0; e < 16; ++e) {
+        float a0, a1;
+        fma2(a0, a1, __uint_as_float(x[e * 2]), __uint_as_float(x[e * 2 + 1]), p.scale_log2, -mr);
+        if constexpr (GATED) {
+          a0 = ex2(a0), a1 = ex2(a1);
+          add2(sum0, sum1, a0, a1);
+          split2(a0, a1, pk[e], x[e]);   // (x[e] has been read: element e comes from x[2 e] and x[2 e + 1])
+        } else {
+          pk[e] = pack_bf16x2(ex2(a0), ex2(a1));
+          add2(sum0, sum1, __uint_as_float(pk[e] << 16), __uint_as_float(pk[e] & 0xffff0000u));
         }
+      }
+      store_p(c, pk, x);
+    };
+    // One key tile without a masked key: two passes over its columns, the next 32 on their way while some are used.
+    auto soft_tile = [&](bool first) {
+      float mx = -CUDART_INF_F, sum0 = 0.f, sum1 = 0.f;
+      uint32_t r[2][32];
+      tmem_ld32_nowait(tS, r[0]);
+#pragma unroll
+      for (int c = 0; c < kKT; c += 32) {
+        uint32_t (&x)[32] = r[(c >> 5) & 1];
+        tmem_wait_ld(x);
+        tmem_ld32_nowait(tS + ((c + 32) & (kKT - 1)), r[((c >> 5) & 1) ^ 1]);   // (after the last columns: the first of pass 2)
+        mx = row_max(x, mx);
+      }
+      tmem_wait_ld(r[0]);
+      const float mr = move_ref(mx, first);
+#pragma unroll
+      for (int c = 0; c < kKT; c += 32) {
+        uint32_t (&x)[32] = r[(c >> 5) & 1];
+        tmem_wait_ld(x);
+        if (c + 32 < kKT) tmem_ld32_nowait(tS + c + 32, r[((c >> 5) & 1) ^ 1]);
+        weights(c, x, mr, sum0, sum1);
+      }
+      tmem_wait_st();
+      l_sum += sum0 + sum1;
+    };
+    // One key tile with masked keys (valid columns lo .. hi of this row).  32 columns at a time, those in which no row of the
+    // warp has a valid one left out; the loops stay rolled: with everything unrolled the kernel was 210 KB of code that a CTA
+    // fetched once per phase (a CTA's first key tile took 12000 cycles, a later one 2500).
+    auto soft_tile_masked = [&](int lo, int hi, bool first) {
+      float mx = -CUDART_INF_F, sum0 = 0.f, sum1 = 0.f;
+#pragma unroll 1
+      for (int c = 0; c < kKT; c += 32) {
+        const uint32_t m = column_mask(c, lo, hi);
+        if (!__any_sync(0xffffffffu, m)) continue;
+        uint32_t x[32];
+        tmem_ld32(tS + c, x);
+#pragma unroll
+        for (int i = 0; i < 32; ++i) x[i] = (m >> i) & 1u ? x[i] : 0xff800000u;
+        mx = row_max(x, mx);
+      }
+      const float mr = move_ref(mx, first);
+#pragma unroll 1
+      for (int c = 0; c < kKT; c += 32) {
+        const uint32_t m = column_mask(c, lo, hi);
+        uint32_t x[32];
+        if (!__any_sync(0xffffffffu, m)) {
+          uint32_t pk[16];
+#pragma unroll
+          for (int e = 0; e < 16; ++e) pk[e] = x[e] = 0u;
+          store_p(c, pk, x);
+          continue;
+        }
+        tmem_ld32(tS + c, x);
+#pragma unroll
+        for (int i = 0; i < 32; ++i) x[i] = (m >> i) & 1u ? x[i] : 0xff800000u;
+        weights(c, x, mr, sum0, sum1);
       }
       tmem_wait_st();
       l_sum += sum0 + sum1;
@@ -601,12 +619,12 @@ prefill_attn_tc_kernel(const PrefillParams p, const CUtensorMap *ring_maps, cons
         if (t == tf) PF_CLK(11); else PF_CLK(12);
         const int64_t j0 = j_lo + int64_t(t) * kKT;
         if (j0 + kKT - 1 <= tqX0 && j0 > tqX_last - w) {
-          soft_tile(IntTag<0>{}, 0, kKT - 1, t == tf);
+          soft_tile(t == tf);
         } else {
           // valid columns of this row: lo <= c <= hi
           const int64_t lo64 = tok_abs - w + 1 - j0, hi64 = tok_abs - j0;
-          soft_tile(IntTag<1>{}, int(lo64 < 0 ? 0 : (lo64 > kKT ? kKT : lo64)),
-                    int(hi64 < -1 ? -1 : (hi64 > kKT - 1 ? kKT - 1 : hi64)), t == tf);
+          soft_tile_masked(int(lo64 < 0 ? 0 : (lo64 > kKT ? kKT : lo64)), int(hi64 < -1 ? -1 : (hi64 > kKT - 1 ? kKT - 1 : hi64)),
+                           t == tf);
         }
         tc_fence_before();      // this thread's TMEM accesses precede the MMAs that read P and overwrite S
         mbar_arrive(smem_u32(&sm.bar_p[X]));
@@ -797,42 +815,39 @@ prefill_attn_tc_kernel(const PrefillParams p, const CUtensorMap *ring_maps, cons
           const int lo = i_lo - i0, hi = tl - i0;
           // a tile that lies wholly before the row tile's first token (and after the first delayed token) needs no mask
           const bool whole = i0 + kKT - 1 <= tok0 + X * TOKT && i0 >= i_lo;
-          uint32_t r[2][32];
-          tmem_ld32_nowait(tS, r[0]);
 #pragma unroll 1
-          for (int c0 = 0; c0 < kKT; c0 += 64) {
+          for (int c = 0; c < kKT; c += 32) {
+            uint32_t pk[16], x[32];
+            const uint32_t m = whole ? ~0u : column_mask(c, lo, hi);
+            // the running log-gates of the 32 columns' tokens, one per lane
+            const float gl = GATED ? __ldg(p.gcum + size_t(uc) * p.SC + min(i0 + c + lane, chunk_n - 1)) : 0.f;
+            if (!__any_sync(0xffffffffu, m)) {   // no row of the warp has a delayed token here
 #pragma unroll
-            for (int hf = 0; hf < 2; ++hf) {
-              uint32_t (&x)[32] = r[hf];
-              const int c = c0 + hf * 32;
-              uint32_t pk[16];
-              // the running log-gates of the 32 columns' tokens, one per lane
-              const float gl = GATED ? __ldg(p.gcum + size_t(uc) * p.SC + min(i0 + c + lane, chunk_n - 1)) : 0.f;
-              tmem_wait_ld(x);
-              if (hf == 0) tmem_ld32_nowait(tS + c + 32, r[1]);
-              else if (c + 32 < kKT) tmem_ld32_nowait(tS + c + 32, r[0]);
-              if (!whole) {
-                const uint32_t m = column_mask(c, lo, hi);
-#pragma unroll
-                for (int i = 0; i < 32; ++i) x[i] = (m >> i) & 1u ? x[i] : 0u;
-              }
-#pragma unroll
-              for (int e = 0; e < 16; ++e) {
-                if constexpr (GATED) {
-                  // a delayed token ii <= i has decayed by exp(g_own - gc[ii]) <= 1 (columns past the row's own are zero:
-                  // the limit keeps 0 x inf out)
-                  const float g0 = __shfl_sync(0xffffffffu, gl, e * 2), g1 = __shfl_sync(0xffffffffu, gl, e * 2 + 1);
-                  const float a0 = __uint_as_float(x[e * 2]) * ex2(fminf(g_own - g0, 0.f) * kLog2e);
-                  const float a1 = __uint_as_float(x[e * 2 + 1]) * ex2(fminf(g_own - g1, 0.f) * kLog2e);
-                  add2(sum0, sum1, a0, a1);
-                  split2(a0, a1, pk[e], x[e]);
-                } else {
-                  pk[e] = pack_bf16x2(__uint_as_float(x[e * 2]), __uint_as_float(x[e * 2 + 1]));
-                  add2(sum0, sum1, __uint_as_float(pk[e] << 16), __uint_as_float(pk[e] & 0xffff0000u));
-                }
-              }
+              for (int e = 0; e < 16; ++e) pk[e] = x[e] = 0u;
               store_p(c, pk, x);
+              continue;
             }
+            tmem_ld32(tS + c, x);
+            if (!whole) {
+#pragma unroll
+              for (int i = 0; i < 32; ++i) x[i] = (m >> i) & 1u ? x[i] : 0u;
+            }
+#pragma unroll
+            for (int e = 0; e < 16; ++e) {
+              if constexpr (GATED) {
+                // a delayed token ii <= i has decayed by exp(g_own - gc[ii]) <= 1 (columns past the row's own are zero:
+                // the limit keeps 0 x inf out)
+                const float g0 = __shfl_sync(0xffffffffu, gl, e * 2), g1 = __shfl_sync(0xffffffffu, gl, e * 2 + 1);
+                const float a0 = __uint_as_float(x[e * 2]) * ex2(fminf(g_own - g0, 0.f) * kLog2e);
+                const float a1 = __uint_as_float(x[e * 2 + 1]) * ex2(fminf(g_own - g1, 0.f) * kLog2e);
+                add2(sum0, sum1, a0, a1);
+                split2(a0, a1, pk[e], x[e]);
+              } else {
+                pk[e] = pack_bf16x2(__uint_as_float(x[e * 2]), __uint_as_float(x[e * 2 + 1]));
+                add2(sum0, sum1, __uint_as_float(pk[e] << 16), __uint_as_float(pk[e] & 0xffff0000u));
+              }
+            }
+            store_p(c, pk, x);
           }
           tmem_wait_st();
           if (!SUM) l_sum += sum0 + sum1;
@@ -902,20 +917,6 @@ prefill_attn_tc_kernel(const PrefillParams p, const CUtensorMap *ring_maps, cons
     auto commit = [&](uint64_t &bar) {
       if (leader) mma_commit(smem_u32(&bar));
     };
-    // The query rows of the CTA that will take this place one wave later are asked into L2 while nothing can be issued yet
-    // (line by line: bulk prefetches of the rows took the memory pipe 12000 cycles).
-    if (int64_t(blockIdx.x) + p.sm_count < int64_t(gridDim.x)) {
-      const int64_t nb = int64_t(blockIdx.x) + p.sm_count, nu = nb / ctas_per_unit;
-      const int ncta = ctas_per_unit - 1 - int(nb % ctas_per_unit), nsub = ncta / ctas_per_chunk;
-      const int ntok0 = nsub * p.SC + (ncta - nsub * ctas_per_chunk) * TOKC;      // relative to the pass
-      const int nrows = min(TOKC, min(p.SC - (ncta - nsub * ctas_per_chunk) * TOKC, p.C - ntok0)) * G;
-      const int head = p.heads_of[int(nu % p.Hkv) * G + (lane >> 1) % G];         // (rows are 16 apart: one head per lane)
-      const bf16 *nq = reinterpret_cast<const bf16 *>(p.q) + ((nu / p.Hkv) * size_t(p.T) + size_t(p.c0 + ntok0)) * p.H * kD +
-                       size_t(head) * kD + (lane & 1) * 64;
-#pragma unroll 4
-      for (int r = lane >> 1; r < nrows; r += 16)
-        asm volatile("prefetch.global.L2 [%0];" ::"l"(nq + size_t(r / G) * p.H * kD));
-    }
     // O_X (+)= A_X B with A_X in the S columns of X: packed bf16 behind one another, or hi and lo in turn every 32 columns
     auto issue_ts = [&](int x, uint32_t b_tile, bool accumulate) {
       if (!GATED) {
@@ -964,6 +965,20 @@ prefill_attn_tc_kernel(const PrefillParams p, const CUtensorMap *ring_maps, cons
       if (ok) {
         if (t >= 0) commit(sm.bar_free[seqV % kStages]);
         if (more) commit(sm.bar_free[seqK % kStages]);
+      }
+      // The query rows of the CTA that will take this place one wave later are asked into L2 (line by line: bulk prefetches of
+      // the rows took the memory pipe 12000 cycles; before the first products the address arithmetic held them up by 1900).
+      if (t < 0 && blockIdx.x + unsigned(p.sm_count) < gridDim.x) {
+        const unsigned nb = blockIdx.x + unsigned(p.sm_count), nu = nb / unsigned(ctas_per_unit);
+        const int ncta = ctas_per_unit - 1 - int(nb - nu * unsigned(ctas_per_unit)), nsub = ncta / ctas_per_chunk;
+        const int ncol = (ncta - nsub * ctas_per_chunk) * TOKC, ntok0 = nsub * p.SC + ncol;   // relative to the pass
+        const int nrows = min(TOKC, min(p.SC - ncol, p.C - ntok0)) * G;
+        const int head = p.heads_of[(nu % unsigned(p.Hkv)) * G + (lane >> 1) % G];            // (rows are 16 apart: one head per lane)
+        const bf16 *nq = reinterpret_cast<const bf16 *>(p.q) + (size_t(nu / unsigned(p.Hkv)) * size_t(p.T) + size_t(p.c0 + ntok0)) * p.H * kD +
+                         size_t(head) * kD + (lane & 1) * 64;
+#pragma unroll 4
+        for (int r = lane >> 1; r < nrows; r += 16)
+          asm volatile("prefetch.global.L2 [%0];" ::"l"(nq + size_t(r / G) * p.H * kD));
       }
     }
     if (ok) commit(sm.bar_done);
@@ -1049,8 +1064,11 @@ prefill_attn_tc_kernel(const PrefillParams p, const CUtensorMap *ring_maps, cons
     // that one thread fetches, then the V' tiles of the intra-chunk steps (with the phi(K') tiles of later steps).
     const int n_window = 2 * n_tiles;
     const int n_jobs = n_window + (linear ? 1 + n_itiles : 0);
+    const int meet_job = n_window > 0 ? 1 : 0;   // (a CTA has no job or at least two; only a window's first tile waits for nobody)
+    if (n_jobs == 0) meet();
 #pragma unroll 1
     for (int job = 0; job < n_jobs; ++job) {
+      if (job == meet_job) meet();
       if (job == n_window) {
         if (lane == 0 && !TWO) {
           // the bf16 state (with z), then the phi(K') tiles of the first two intra-chunk steps
@@ -1220,7 +1238,7 @@ prefill_attn_tc_kernel(const PrefillParams p, const CUtensorMap *ring_maps, cons
   __syncthreads();
   PF_CLK(6);
   if (tid == 0 && sm.failed) atomicExch(&p.ctl->status, kDevWaitTimeout);
-  if (warp == kLoadWarp) {
+  if (warp == kMmaWarp) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem) : "memory");
   }
