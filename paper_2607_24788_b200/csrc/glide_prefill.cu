@@ -108,11 +108,6 @@ __global__ void __launch_bounds__(kPrefillThreads) prefill_phi_kernel(const Pref
         __nv_bfloat16 *d16 = reinterpret_cast<__nv_bfloat16 *>(p.phik16) + (size_t(u) * p.Cmax + i0 + r) * D + lane * E;
 #pragma unroll
         for (int e = 0; e < E; ++e) d16[e] = __float2bfloat16_rn(x[r][e]);
-        if (p.gated) {   // and what the rounding left, in the second half of the array
-          d16 += size_t(p.units_cap) * p.SC * D;
-#pragma unroll
-          for (int e = 0; e < E; ++e) d16[e] = __float2bfloat16_rn(x[r][e] - __bfloat162float(__float2bfloat16_rn(x[r][e])));
-        }
       }
     }
   } else {
@@ -695,6 +690,8 @@ int launch_prefill(glide_ctx *ctx, int layer_begin, int layer_count, int64_t T, 
     using TT = typename decltype(tt)::type;
     constexpr int D = decltype(dd)::value, DP = decltype(pp)::value;
     constexpr bool kCanProject = DP == 2 * D && D == 128 && std::is_same<TT, __nv_bfloat16>::value;
+    // the carry makes phi(K') itself, unless it is the learned map's or its running sums are needed before
+    const bool make_phi = DP == D && !(out && p.merge != GLIDE_MERGE_SHARED);
     const int64_t most = p.SC > 128 ? p.units_cap / units_layer : 1;   // (the chunk sums take 129 scratch rows of a chunk)
     return for_passes(p.units_cap, most, D, sizeof(TT), [&](const PrefillParams &s) -> int {
       const int64_t units = int64_t(s.layer_count) * units_layer;
@@ -703,7 +700,7 @@ int launch_prefill(glide_ctx *ctx, int layer_begin, int layer_count, int64_t T, 
       if (evicts_in(s.layer_begin, s.layer_count)) {
         if (kCanProject) {
           if (launch_prefill_project(ctx, s, true, stream) != GLIDE_OK) return GLIDE_ERR_CUDA;
-        } else {
+        } else if (!make_phi) {
           prefill_phi_kernel<TT, D, DP><<<warp4_blocks, kPrefillThreads, 0, stream>>>(s);
         }
         if (p.gated)
@@ -711,7 +708,7 @@ int launch_prefill(glide_ctx *ctx, int layer_begin, int layer_count, int64_t T, 
         if (out && s.phiq16 && launch_prefill_project(ctx, s, false, stream) != GLIDE_OK) return GLIDE_ERR_CUDA;
         if (out && p.merge != GLIDE_MERGE_SHARED)   // (before the carry: the chunk sums overwrite rows of phi(K'))
           prefill_zcum_kernel<D><<<unsigned((units * s.nsub * D + kPrefillThreads - 1) / kPrefillThreads), kPrefillThreads, 0, stream>>>(s);
-        if (launch_prefill_state_mma(ctx, s, stream) != GLIDE_OK) return GLIDE_ERR_CUDA;
+        if (launch_prefill_state_mma(ctx, s, make_phi, stream) != GLIDE_OK) return GLIDE_ERR_CUDA;
       }
       if (out && launch_prefill_attn_tc(ctx, s, stream) != GLIDE_OK) return GLIDE_ERR_CUDA;
       prefill_ring_kernel<TT, D><<<warp4_blocks, kPrefillThreads, 0, stream>>>(s);
@@ -768,7 +765,7 @@ int launch_prefill(glide_ctx *ctx, int layer_begin, int layer_count, int64_t T, 
       }
       if (any_evicts) {
         if (state_mma) {
-          if (launch_prefill_state_mma(ctx, p, stream) != GLIDE_OK) return GLIDE_ERR_CUDA;
+          if (launch_prefill_state_mma(ctx, p, false, stream) != GLIDE_OK) return GLIDE_ERR_CUDA;
         } else {
           prefill_state_kernel<TT, D><<<unsigned(units * (DP / kStateRows)), kPrefillThreads, 0, stream>>>(p);
         }

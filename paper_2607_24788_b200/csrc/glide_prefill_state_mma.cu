@@ -10,7 +10,10 @@
 // One CTA of 4 warps per (unit, 64 state rows); warp w owns rows 16 w .. 16 w + 15 and all 128 columns
 // (16 n-tiles of m16n8k16, 64 accumulators per thread).  Tokens are staged 32 at a time through two shared-memory
 // buffers filled by cp.async; row strides are padded (272 bytes) so that the scalar reads of the A fragments and
-// the ldmatrix reads of V' are free of bank conflicts.
+// the ldmatrix reads of V' are free of bank conflicts.  With the parameter-free map the kernel makes phi(K') itself from the
+// staged K' rows (both CTAs of a unit's chunk the whole row, for its normaliser, each keeping its 64 columns) and leaves
+// the bf16 rows for the attention kernel: as a kernel in front, phi cost a trip of 512 bytes per token through memory.
+// 8 x 2048 tokens, 4 layers: 107 us for phi and 126 for the carry, 188 together.
 #include <algorithm>
 
 #include "glide_device.cuh"
@@ -66,10 +69,14 @@ __device__ __forceinline__ void store_s16(__nv_bfloat16 *at, size_t lo_half, flo
 // of S (64 state rows x 128 values = 128 scratch rows x the CTA's 64 columns, z in row 128: chunks of more than 128
 // tokens), and prefill_scan_kernel adds the sums up in chunk order.  Otherwise S is updated in place, and its value
 // before the chunk is left as bf16 (z: fp32) for the attention kernel, which runs after this one.
-template <bool PARTIAL>
+// MAKE_PHI: phi(K') is made here (parameter-free map); otherwise it is in the scratch.
+template <bool PARTIAL, bool MAKE_PHI>
 __global__ void __launch_bounds__(kThreads) prefill_state_mma_kernel(const PrefillParams p) {
   using bf16 = __nv_bfloat16;
-  __shared__ __align__(16) unsigned char stage[2][kPhiBytes + kVBytes];
+  // per stage phi columns (or K' rows, 16 bytes more per row) and V' rows; made phi columns
+  constexpr int kInBytes = MAKE_PHI ? kVBytes : kPhiBytes;
+  __shared__ __align__(16) unsigned char stage[2][kInBytes + kVBytes];
+  __shared__ __align__(16) float made[MAKE_PHI ? kTok * kPhiStride : 4];
   __shared__ float decay[2][kTok];   // gated: what each staged token has decayed to by the end of the chunk
   const int blocks_per_unit = p.dp / kRowsPerCta;   // rows of S: d, or 2 d with the learned feature map
   const int64_t uc = blockIdx.x / blocks_per_unit;   // (unit, chunk of the pass)
@@ -92,7 +99,10 @@ __global__ void __launch_bounds__(kThreads) prefill_state_mma_kernel(const Prefi
   const int64_t cap = ld.cap > 0 ? ld.cap : 1;
   const bf16 *ringV = reinterpret_cast<const bf16 *>(p.ws + ld.ringV) + size_t(ub) * size_t(ld.cap) * kD;
   const bf16 *callV = reinterpret_cast<const bf16 *>(p.v) + ((size_t(lrel) * p.B + b) * size_t(p.T) * p.Hkv + g) * kD;
+  const bf16 *ringK = reinterpret_cast<const bf16 *>(p.ws + ld.ringK) + size_t(ub) * size_t(ld.cap) * kD;
+  const bf16 *callK = reinterpret_cast<const bf16 *>(p.k) + ((size_t(lrel) * p.B + b) * size_t(p.T) * p.Hkv + g) * kD;
   const int64_t call_stride = int64_t(p.Hkv) * kD;
+  bf16 *p16 = MAKE_PHI && p.phik16 ? reinterpret_cast<bf16 *>(p.phik16) + (size_t(u) * p.Cmax + chunk_c0) * kD + rb * kRowsPerCta : nullptr;
   float *pk = p.phik + (size_t(u) * p.Cmax + chunk_c0) * p.dp + rb * kRowsPerCta;
 
   float acc[kD / 8][4];
@@ -105,16 +115,17 @@ __global__ void __launch_bounds__(kThreads) prefill_state_mma_kernel(const Prefi
   // tokens past the chunk's end are filled with zeros
   auto issue = [&](int buf, int i0) {
     const int nt = min(kTok, chunk_n - i0);
-    const uint32_t sphi = smem_addr(stage[buf]), sv = sphi + kPhiBytes;
-    for (int e = tid; e < kTok * (kRowsPerCta / 4); e += kThreads) {
+    const uint32_t sphi = smem_addr(stage[buf]), sv = sphi + kInBytes;
+    for (int e = tid; !MAKE_PHI && e < kTok * (kRowsPerCta / 4); e += kThreads) {
       const int i = e / (kRowsPerCta / 4), c4 = e % (kRowsPerCta / 4);
       cp16(sphi + uint32_t(i * kPhiStride + c4 * 4) * 4u, pk + size_t(i0 + (i < nt ? i : 0)) * p.dp + c4 * 4, i < nt);
     }
     for (int e = tid; e < kTok * 16; e += kThreads) {
       const int i = e >> 4, c = e & 15;
       const int64_t j = first + i0 + (i < nt ? i : 0);
-      const bf16 *row = j >= p.n0 ? callV + (j - p.n0) * call_stride : ringV + (j % cap) * kD;
-      cp16(sv + uint32_t(i * kVStride + c * 16), row + c * 8, i < nt);
+      const int64_t at = j >= p.n0 ? (j - p.n0) * call_stride : int64_t(uint32_t(j) % uint32_t(cap)) * kD;   // (tokens stay below 2^31)
+      cp16(sv + uint32_t(i * kVStride + c * 16), (j >= p.n0 ? callV : ringV) + at + c * 8, i < nt);
+      if (MAKE_PHI) cp16(sphi + uint32_t(i * kVStride + c * 16), (j >= p.n0 ? callK : ringK) + at + c * 8, i < nt);
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
     if (tid < kTok) decay[buf][tid] = (gc && tid < nt) ? expf(g_end - gc[i0 + tid]) : 1.f;   // (rows past the end are zero)
@@ -129,8 +140,68 @@ __global__ void __launch_bounds__(kThreads) prefill_state_mma_kernel(const Prefi
       asm volatile("cp.async.wait_group 0;" ::: "memory");
     }
     __syncthreads();
-    const float *sphi = reinterpret_cast<const float *>(stage[buf]);
-    const uint32_t sv = smem_addr(stage[buf]) + kPhiBytes;
+    if constexpr (MAKE_PHI) {
+      // four threads per token, 32 entries each; those of this CTA's columns go to `made`, rounded to the bf16 rows
+      const int tok = tid >> 2, part = tid & 3;
+      const uint4 *src = reinterpret_cast<const uint4 *>(stage[buf] + tok * kVStride + part * 64);
+      float x[32];
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        const uint4 v = src[c];
+        const uint32_t w4[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          x[c * 8 + e * 2] = __uint_as_float(w4[e] << 16);
+          x[c * 8 + e * 2 + 1] = __uint_as_float(w4[e] & 0xffff0000u);
+        }
+      }
+      float mx = x[0];
+#pragma unroll
+      for (int i = 1; i < 32; ++i) mx = fmaxf(mx, x[i]);
+      mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
+      mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
+      float sum = 0.f;
+#pragma unroll
+      for (int i = 0; i < 32; ++i) {
+        x[i] = exp2f((x[i] - mx) * kLog2e);
+        sum += x[i];
+      }
+      sum += __shfl_xor_sync(0xffffffffu, sum, 1);
+      sum += __shfl_xor_sync(0xffffffffu, sum, 2);
+      const bool there = i0 + tok < chunk_n;
+      const float inv = there ? 1.0f / sum : 0.f;   // (rows past the chunk's end stay zero)
+      if (part >> 1 == rb) {
+        float *dst = made + tok * kPhiStride + (part & 1) * 32;
+#pragma unroll
+        for (int i = 0; i < 32; i += 4) {
+#pragma unroll
+          for (int e = 0; e < 4; ++e) x[i + e] *= inv;
+          *reinterpret_cast<float4 *>(dst + i) = make_float4(x[i], x[i + 1], x[i + 2], x[i + 3]);
+        }
+        if (p16 && there) {
+          bf16 *out = p16 + size_t(i0 + tok) * kD + (part & 1) * 32;
+#pragma unroll
+          for (int hl = 0; hl < 2; ++hl) {   // gated: what the rounding left, in the second half of the array
+            if (hl == 1 && !p.gated) break;
+#pragma unroll
+            for (int i = 0; i < 32; i += 8) {
+              uint32_t o[4];
+#pragma unroll
+              for (int e = 0; e < 4; ++e) {
+                const __nv_bfloat162 h = __floats2bfloat162_rn(x[i + e * 2], x[i + e * 2 + 1]);
+                o[e] = *reinterpret_cast<const uint32_t *>(&h);
+                x[i + e * 2] -= __low2float(h);
+                x[i + e * 2 + 1] -= __high2float(h);
+              }
+              *reinterpret_cast<uint4 *>(out + (hl ? size_t(p.units_cap) * p.SC * kD : 0) + i) = make_uint4(o[0], o[1], o[2], o[3]);
+            }
+          }
+        }
+      }
+      __syncthreads();
+    }
+    const float *sphi = MAKE_PHI ? made : reinterpret_cast<const float *>(stage[buf]);
+    const uint32_t sv = smem_addr(stage[buf]) + kInBytes;
 #pragma unroll
     for (int kk = 0; kk < kTok / 16; ++kk) {
       // A = phi(K')^T: element (row r, k i) = phi(k'_i)[r]; fragment registers a0: (gid, 2 tig + {0,1}),
@@ -273,16 +344,18 @@ bool prefill_state_mma_supported(const glide_ctx *ctx) {
   return ctx->cfg.io_dtype == GLIDE_BF16 && ctx->cfg.head_dim == kD;
 }
 
-int launch_prefill_state_mma(glide_ctx *ctx, const PrefillParams &p, cudaStream_t stream) {
+int launch_prefill_state_mma(glide_ctx *ctx, const PrefillParams &p, bool make_phi, cudaStream_t stream) {
   (void)ctx;
   const int64_t units = int64_t(p.layer_count) * p.B * p.Hkv;
   const unsigned blocks = unsigned(units * p.nsub * (p.dp / kRowsPerCta));
-  if (p.nsub == 1) {
-    prefill_state_mma_kernel<false><<<blocks, kThreads, 0, stream>>>(p);
+  if (make_phi) {
+    if (p.nsub == 1) prefill_state_mma_kernel<false, true><<<blocks, kThreads, 0, stream>>>(p);
+    else prefill_state_mma_kernel<true, true><<<blocks, kThreads, 0, stream>>>(p);
   } else {
-    prefill_state_mma_kernel<true><<<blocks, kThreads, 0, stream>>>(p);
-    prefill_scan_kernel<<<unsigned(units * (p.dp / 4)), kThreads, 0, stream>>>(p);
+    if (p.nsub == 1) prefill_state_mma_kernel<false, false><<<blocks, kThreads, 0, stream>>>(p);
+    else prefill_state_mma_kernel<true, false><<<blocks, kThreads, 0, stream>>>(p);
   }
+  if (p.nsub > 1) prefill_scan_kernel<<<unsigned(units * (p.dp / 4)), kThreads, 0, stream>>>(p);
   return cudaGetLastError() == cudaSuccess ? GLIDE_OK : GLIDE_ERR_CUDA;
 }
 
