@@ -124,7 +124,8 @@ typedef struct {
                               that enters it: S <- gamma S + phi(k) v^T, z <- gamma z + phi(k).  Gates are passed to
                               glide_prefill_gated / glide_decode_step_gated; the calls without gates use gamma = 1.
                               Decode: the streaming kernel (bf16, head_dim 128) or the CUDA-core kernel (decode_impl
-                              AUTO, STREAM or FMA); prefill: the CUDA-core kernels (prefill_impl AUTO or FMA). */
+                              AUTO, STREAM or FMA); prefill: the tcgen05 kernel with split operands (bf16, head_dim 128,
+                              parameter-free map, shared normaliser, prefill_impl AUTO) or the CUDA-core kernels. */
   int32_t reserved_;       /* must be 0 */
 } glide_config;
 

@@ -369,8 +369,9 @@ glide_decode_stream_kernel(const DecodeParams p, const StreamParams sp) {
   }
   __syncthreads();   // segment table and barriers ready
   // A sequence's position is the layers' common counter, which comes with the launch, plus the sequence's own offset
-  // (zero unless sequences were reset or prefilled one by one; written by copies from the host, never by a kernel,
-  // so it may be read before the preceding kernel has completed).  Level batches (RAGGED false: an instantiation of
+  // (zero unless sequences were reset or prefilled one by one; written by copies from the host, so it may be read before
+  // the preceding kernel has completed; glide_reset's kernel zeroes the offsets, after which they are not read until the
+  // next copy).  Level batches (RAGGED false: an instantiation of
   // its own, so that the B = 1 step carries none of this) take the position from the launch parameters.
   constexpr bool ragged = RAGGED;
   if (ragged) {

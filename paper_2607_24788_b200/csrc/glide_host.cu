@@ -69,7 +69,7 @@ int validate_config(const glide_config *c) {
   } else if (c->phi_wq || c->phi_wk) {
     return GLIDE_ERR_INVALID_ARG;
   }
-  if (c->gated) {   // the gated recurrence runs on the CUDA-core kernels and on the streaming decode kernel
+  if (c->gated) {   // the CUDA-core kernels, the streaming decode kernel and (by AUTO alone) the tcgen05 prefill kernel
     if (c->decode_impl == GLIDE_DECODE_MMA) return GLIDE_ERR_UNSUPPORTED;
     if (c->prefill_impl == GLIDE_PREFILL_MMA_SYNC || c->prefill_impl == GLIDE_PREFILL_TCGEN05) return GLIDE_ERR_UNSUPPORTED;
   }

@@ -1,16 +1,20 @@
-// GLIDE prefill: append T prompt tokens, chunk by chunk (C tokens per chunk).
+// GLIDE prefill: append T prompt tokens in passes over the call's chunks and layers.
 //
 // For a layer with window w the linear part of query i sums over tokens j <= i - w, i.e. it is
 // ordinary causal (inclusive) linear attention on the stream delayed by w tokens:
-// k'_i = k_{i-w}, v'_i = v_{i-w}.  Per chunk, in stream order:
+// k'_i = k_{i-w}, v'_i = v_{i-w}.  Three routes (launch_prefill chooses):
+//   tensor-core passes (bf16, head_dim 128): carry with the chunks' bf16 phi(k') and state copies, scan over the chunks,
+//                 tcgen05 attention, ring; several chunks of some layers per pass
+//   CUDA-core passes (glide_prefill_fma.cu): parameter-free map, fp32 or head_dim 64
+//   chunk by chunk, all layers at once (the learned map on the CUDA cores, the mma.sync attention kernel):
 //   1. phi kernel    phi(k') of the chunk's delayed tokens -> scratch (fp32)
 //   2. attn kernel   per query: sliding-window online softmax over ring-or-call rows, the readout
 //                    phi(q) S / phi(q) z of the state at chunk start, the intra-chunk delayed terms
 //                    (phi(q).phi(k'_j)) v'_j, merged under the shared normaliser -> out
 //   3. state kernel  S += phi(K'_c)^T V'_c, z += sum phi(K'_c)   (fp32 carry)
 //   4. ring kernel   the chunk's newest min(C, cap) tokens -> slot (position mod cap)
-// The delayed rows and the window rows older than the call come from the ring, which step 4 of
-// the same chunk overwrites only after steps 1-3 have read it.
+// The delayed rows and the window rows older than the call come from the ring, which the last kernel of a chunk or pass
+// overwrites only after the others have read it.
 #include <algorithm>
 #include <type_traits>
 
