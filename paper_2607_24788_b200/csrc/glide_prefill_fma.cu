@@ -16,7 +16,7 @@
 #include <algorithm>
 #include <type_traits>
 
-#include "glide_device.cuh"
+#include "glide_prefill_rows.cuh"
 
 namespace glide {
 
@@ -59,31 +59,6 @@ __device__ __forceinline__ float4 row_phi(float4 x) {
   const float inv = 1.0f / lanes_sum<D / 4>(e.x + e.y + e.z + e.w);
   return make_float4(e.x * inv, e.y * inv, e.z * inv, e.w * inv);
 }
-
-// K and V rows of one unit by absolute token
-template <typename T, int D>
-struct Rows {
-  const T *ringK, *ringV, *callK, *callV;
-  int64_t n0, call_stride;
-  uint32_t cap;
-  __device__ __forceinline__ Rows(const PrefillParams &p, const LayerDev &ld, int lrel, int b, int g) {
-    const size_t base = (size_t(b + p.b0) * p.Hkv + g) * size_t(ld.cap) * D;   // b + b0: the sequence's slot in the context
-    ringK = reinterpret_cast<const T *>(p.ws + ld.ringK) + base;
-    ringV = reinterpret_cast<const T *>(p.ws + ld.ringV) + base;
-    const size_t seq = (size_t(lrel) * p.B + b) * size_t(p.T) * p.Hkv * D + size_t(g) * D;
-    callK = reinterpret_cast<const T *>(p.k) + seq;
-    callV = reinterpret_cast<const T *>(p.v) + seq;
-    n0 = p.n0;
-    call_stride = int64_t(p.Hkv) * D;
-    cap = ld.cap > 0 ? uint32_t(ld.cap) : 1u;
-  }
-  // element offset of token j's row in the call's tensors (>= 0) or, as ~offset, in the rings; tokens stay below 2^31
-  __device__ __forceinline__ int64_t at(int64_t j) const {
-    return j >= n0 ? (j - n0) * call_stride : ~(int64_t(uint32_t(j) % cap) * D);
-  }
-  __device__ __forceinline__ float4 k(int64_t off, int c) const { return load4(off >= 0 ? callK + off + c : ringK + ~off + c); }
-  __device__ __forceinline__ float4 v(int64_t off, int c) const { return load4(off >= 0 ? callV + off + c : ringV + ~off + c); }
-};
 
 struct UnitId {
   int64_t u;
@@ -138,8 +113,8 @@ __global__ void __launch_bounds__(2 * kThreads) prefill_fma_sums_kernel(const Pr
       kr[i] = vr[i] = make_float4(0.f, 0.f, 0.f, 0.f);
       if (i0 + r < chunk_n) {
         const int64_t off = rows.at(first + i0 + r);
-        kr[i] = rows.k(off, c);
-        vr[i] = rows.v(off, c);
+        kr[i] = load4(rows.k(off) + c);
+        vr[i] = load4(rows.v(off) + c);
       }
     }
   };
@@ -225,8 +200,31 @@ struct AttnSmem {
   } grp[2];
 };
 
+// The state at a chunk's start for a single row: S and z with the sums of chunks [sub0, sub) on top
+template <int D>
+struct SumsState {
+  const float *S, *z0, *sums, *zs, *gates;   // gates: gcum of the unit's first chunk, or null
+  int sub0, sub, SC;
+  __device__ __forceinline__ float after(int k) const { return gates ? expf(gates[(k + 1) * SC - 1]) : 1.f; }   // (these chunks are whole)
+  template <int E>
+  __device__ __forceinline__ void row(int r, int c, float (&x)[E]) const {
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+      x[e] = S[r * D + c + e];
+      for (int k = sub0; k < sub; ++k) x[e] = fmaf(x[e], after(k), sums[(size_t(k) * D + r) * D + c + e]);
+    }
+  }
+  __device__ __forceinline__ float z(int r) const {
+    float x = z0[r];
+    for (int k = sub0; k < sub; ++k) x = fmaf(x, after(k), zs[size_t(k) * D + r]);
+    return x;
+  }
+};
+
+// (One CTA per SM is what fits with 170 registers a thread as with 250, which the second bound allows: 512 tokens of 4 units,
+// fp32, d = 64, w = 64, 20.5 us without it, 18.2 with it.)
 template <typename T, int D, int G>
-__global__ void __launch_bounds__(2 * kThreads) prefill_fma_attn_kernel(const PrefillParams p) {
+__global__ void __launch_bounds__(2 * kThreads, 1) prefill_fma_attn_kernel(const PrefillParams p) {
   constexpr int KT = AttnSmem<D>::KT;
   constexpr int LD = KT * D / 4 / kThreads;        // float4 of K (and of V) per thread and tile
   constexpr int KPT = KT / 16;                     // keys per lane
@@ -285,8 +283,8 @@ __global__ void __launch_bounds__(2 * kThreads) prefill_fma_attn_kernel(const Pr
         const int64_t j = j_lo + int64_t(t - n_st) * KT + r;
         if (j <= j_hi) {
           const int64_t off = rows.at(j);
-          kr[i] = rows.k(off, c);
-          vr[i] = rows.v(off, c);
+          kr[i] = load4(rows.k(off) + c);
+          vr[i] = load4(rows.v(off) + c);
         }
       }
     } else {
@@ -445,6 +443,7 @@ __global__ void __launch_bounds__(2 * kThreads) prefill_fma_attn_kernel(const Pr
   }
   __syncthreads();
   if (grp == 1) return;
+  unsigned again[2];
 #pragma unroll
   for (int r = 0; r < 2; ++r) {
     const float L = l[r], Bl = lsum[row + r];
@@ -462,14 +461,33 @@ __global__ void __launch_bounds__(2 * kThreads) prefill_fma_attn_kernel(const Pr
       fa = fw * inv;
       fb = fl * inv;
     }
+    bool bad = false;
     if (tk < ntok) {
       T *op = reinterpret_cast<T *>(p.out) + ((seq_row + tk) * p.H + head) * D + cg * 4;
 #pragma unroll
       for (int q = 0; q < CG; ++q) {
         const float4 x = *reinterpret_cast<const float4 *>(lin + (row + r) * D + q * 64 + cg * 4);
-        store4(op + q * 64, make_float4(fmaf(o[r][q * 4], fa, x.x * fb), fmaf(o[r][q * 4 + 1], fa, x.y * fb),
-                                        fmaf(o[r][q * 4 + 2], fa, x.z * fb), fmaf(o[r][q * 4 + 3], fa, x.w * fb)));
+        const float4 y = make_float4(fmaf(o[r][q * 4], fa, x.x * fb), fmaf(o[r][q * 4 + 1], fa, x.y * fb),
+                                     fmaf(o[r][q * 4 + 2], fa, x.z * fb), fmaf(o[r][q * 4 + 3], fa, x.w * fb));
+        store4(op + q * 64, y);
+        bad = bad || !isfinite(y.x + y.y + y.z + y.w);
       }
+    }
+    again[r] = __ballot_sync(0xffffffffu, bad);
+  }
+  // rows with a result that is not finite (or a sum of four that is not): from the rows that count for them alone
+  if (again[0] | again[1]) {
+    __syncwarp();
+#pragma unroll 1
+    for (int i = 0; i < 4; ++i) {   // the warp's rows: lanes 0-15 have rows 0 and 1 of them, lanes 16-31 rows 2 and 3
+      if (!((again[i & 1] >> (i >> 1) * 16) & 0xffffu)) continue;
+      const int rw = (tid >> 5) * 4 + i, tk = rw / G, head = p.heads_of[id.g * G + rw % G];
+      const size_t at = ((seq_row + tk) * p.H + head) * D;
+      const RowJob<T, D> job{rows, reinterpret_cast<const T *>(p.q) + at, reinterpret_cast<T *>(p.out) + at,
+                             chunk_gates(p, id.u * p.nsub + sub), p.n0 + p.c0 + chunk_c0, tok0 + tk, ld.w, ld.wlin, ld.evicts, ld.merge,
+                             p.scale_log2};
+      recompute_row(job, SumsState<D>{Sb, reinterpret_cast<const float *>(p.ws + ld.z) + size_t(ub) * D, sums, p.zsnap + size_t(id.u) * p.nsub * D,
+                                      chunk_gates(p, id.u * p.nsub), sub0, sub, p.SC});
     }
   }
 }
