@@ -1,14 +1,16 @@
 // GLIDE prefill on the CUDA cores with fp32 arithmetic throughout (fp32 I/O, d = 64, and whenever the CUDA-core prefill is
 // asked for) for the parameter-free feature map, gated or not.  A pass takes up to nsub chunks of CH tokens of every unit
-// (unit = layer, sequence, KV head) in three launches:
-//   1. prefill_fma_sums_kernel    per chunk phi(K')^T V' and sum phi(K') of its delayed tokens k'_i = k_{i-w}
-//   2. prefill_fma_attn_kernel    per 16 query rows: window softmax, the chunk's own delayed tokens, and the state at
-//                                 the chunk's start = S + the sums of the chunks before it; out
-//   3. prefill_fma_finish_kernel  S and z move on by the pass, the pass's newest tokens go to the ring, counters advance
+// (unit = layer, sequence, KV head) in three launches, or four where it has many chunks:
+//   1.  prefill_fma_sums_kernel    per chunk phi(K')^T V' and sum phi(K') of its delayed tokens k'_i = k_{i-w}
+//   1b. prefill_fma_scan_kernel    (many chunks) the sums added up: S and z move on, the state at every chunk's start is left
+//   2.  prefill_fma_attn_kernel    per 16 query rows: window softmax, the chunk's own delayed tokens, and the state at
+//                                  the chunk's start, the scan's or S + the sums of the chunks before it; out
+//   3.  prefill_fma_finish_kernel  S and z move on by the pass if no scan did it, the pass's newest tokens go to the ring,
+//                                  counters advance
 // Gated: the running log-gates of the chunks' delayed tokens (gcum) come from a kernel in front; without gates every decay
 // is an exact 1, so that a gated context driven without gates keeps the bits of a plain one.
-// All three read K and V rows where they are (ring for tokens older than the call) and make phi in registers; the ring
-// and S change in the third only.  The problems are small (a few units of a few hundred tokens), so what bounds them is the
+// The kernels read K and V rows where they are (ring for tokens older than the call) and make phi in registers; the ring
+// changes in the last only.  The problems are small (a few units of a few hundred tokens), so what bounds them is the
 // length of the dependent chain and not the arithmetic: the rows of a tile are shared by 16 query rows and the next
 // tile's loads are in flight while one is used, and a CTA's two groups of four warps work side by side on the window and
 // the linear part (the sums kernel: on every other tile).  512 tokens of 4 units (fp32, d = 64, w = 64): attention 103 us
@@ -24,6 +26,12 @@ namespace {
 
 constexpr int kThreads = 128;     // of a group; the sums and the attention kernel run two groups per CTA
 constexpr int kRows = 16;         // query rows (token, head of the group) per CTA: 8 half-warps of two rows
+// Passes of more chunks than this are scanned.  Without a scan every CTA of 16 query rows reads S and the sums of all chunks
+// before its own, which grows with the square of the chunks; the scan is a launch more (4 us).  Per layer of a 32-layer
+// context with windows of 64, fp32, without / with a scan: 8 heads of 64, 8 chunks 42 / 45 us, 16 78 / 76, 64 383 / 223,
+// 128 1153 / 433; 32 heads of 128 (8 KV heads), 4 chunks 107 / 107 us, 8 202 / 187, 125 7462 / 3288.
+template <int D>
+constexpr int kDirectChunks = 512 / D;
 
 __device__ __forceinline__ float4 load4(const float *p) { return *reinterpret_cast<const float4 *>(p); }
 __device__ __forceinline__ float4 load4(const __nv_bfloat16 *p) {
@@ -267,11 +275,14 @@ __global__ void __launch_bounds__(2 * kThreads, 1) prefill_fma_attn_kernel(const
   const int n_rows = any && j_hi >= j_lo ? int((j_hi - j_lo) / KT) + 1 : 0;
   const int n_st = grp == 1 && linear && first > 0 ? D / KT : 0;
   const int n_tiles = n_rows + n_st;
-  // sums of the chunks before this one that hold delayed tokens: [sub0, sub)
-  const int sub0 = first - int64_t(chunk_c0) >= 0 ? 0 : int(-(first - chunk_c0) / p.SC);
-  const float *sums = p.phik + size_t(id.u) * p.nsub * D * D;
+  // The state at the chunk's start: left by the scan in the chunk's slot, or S and z with the sums of the chunks before this
+  // one that hold delayed tokens, [sub0, sub), on top
+  const bool scanned = p.nsub > kDirectChunks<D>;
+  const int sub0 = scanned ? sub : (first - int64_t(chunk_c0) >= 0 ? 0 : int(-(first - chunk_c0) / p.SC));
+  const float *sums = p.phik + size_t(id.u) * p.nsub * D * D, *zs = p.zsnap + size_t(id.u) * p.nsub * D;
   const int ub = (id.b + p.b0) * p.Hkv + id.g;
-  const float *Sb = reinterpret_cast<const float *>(p.ws + ld.S) + size_t(ub) * D * D;
+  const float *Sb = scanned ? sums + size_t(sub) * D * D : reinterpret_cast<const float *>(p.ws + ld.S) + size_t(ub) * D * D;
+  const float *zb = scanned ? zs + size_t(sub) * D : reinterpret_cast<const float *>(p.ws + ld.z) + size_t(ub) * D;
 
   float4 kr[LD], vr[LD];
   auto fetch = [&](int t) {
@@ -405,8 +416,6 @@ __global__ void __launch_bounds__(2 * kThreads, 1) prefill_fma_attn_kernel(const
     } else {
       add_rows(&sm.a[row][t * KT], &sm.a[row + 1][t * KT]);
       if (t + 1 == n_st) {   // the state's part is complete: phi(q) . z, and what both have decayed to by the row's token
-        const float *zb = reinterpret_cast<const float *>(p.ws + ld.z) + size_t(ub) * D;
-        const float *zs = p.zsnap + size_t(id.u) * p.nsub * D;
         float z[D / 16];
 #pragma unroll
         for (int i = 0; i < D / 16; ++i) z[i] = zb[cg + 16 * i];
@@ -486,48 +495,61 @@ __global__ void __launch_bounds__(2 * kThreads, 1) prefill_fma_attn_kernel(const
       const RowJob<T, D> job{rows, reinterpret_cast<const T *>(p.q) + at, reinterpret_cast<T *>(p.out) + at,
                              chunk_gates(p, id.u * p.nsub + sub), p.n0 + p.c0 + chunk_c0, tok0 + tk, ld.w, ld.wlin, ld.evicts, ld.merge,
                              p.scale_log2};
-      recompute_row(job, SumsState<D>{Sb, reinterpret_cast<const float *>(p.ws + ld.z) + size_t(ub) * D, sums, p.zsnap + size_t(id.u) * p.nsub * D,
-                                      chunk_gates(p, id.u * p.nsub), sub0, sub, p.SC});
+      recompute_row(job, SumsState<D>{Sb, zb, sums, zs, chunk_gates(p, id.u * p.nsub), sub0, sub, p.SC});
     }
   }
 }
 
-// 3. The first blocks: S and z plus the pass's sums (a thread four columns of one row); the others: the pass's newest
-// min(C, cap) tokens to slot (position mod cap), one thread per four entries of a K and a V row.
+// Four columns of one row of S (element index e over the units' states), and z for the first row's threads, move on by the
+// pass's sums; SNAP: every sum gives way to the state at its chunk's start
+template <int D, bool SNAP>
+__device__ __forceinline__ void add_sums(const PrefillParams &p, int64_t e) {
+  const UnitId id = unit_id(p, e / (D * D / 4));
+  const int at = int(e % (D * D / 4)) * 4;
+  const LayerDev ld = p.layers[p.layer_begin + id.lrel];
+  const int64_t first = p.n0 + p.c0 - ld.wlin;
+  if (!ld.evicts || first + p.C <= 0) return;
+  const int k0 = first >= 0 ? 0 : int(-first / p.SC);
+  const int ub = (id.b + p.b0) * p.Hkv + id.g;
+  // the sums are `stride` floats apart; those of four chunks are asked for together
+  auto run = [&](float *state, float *sum, size_t stride) {
+    constexpr int kAhead = 4;
+    float4 s = load4(state);
+    for (int k = k0; k < p.nsub; k += kAhead) {
+      float4 x[kAhead];
+#pragma unroll
+      for (int a = 0; a < kAhead; ++a)
+        if (k + a < p.nsub) x[a] = load4(sum + size_t(k + a) * stride);
+#pragma unroll
+      for (int a = 0; a < kAhead; ++a) {
+        if (k + a >= p.nsub) break;
+        if (SNAP) store4(sum + size_t(k + a) * stride, s);
+        const float dec = chunk_decay(p, id.u, k + a);
+        s = make_float4(fmaf(s.x, dec, x[a].x), fmaf(s.y, dec, x[a].y), fmaf(s.z, dec, x[a].z), fmaf(s.w, dec, x[a].w));
+      }
+    }
+    store4(state, s);
+  };
+  run(reinterpret_cast<float *>(p.ws + ld.S) + size_t(ub) * D * D + at, p.phik + size_t(id.u) * p.nsub * D * D + at, size_t(D) * D);
+  if (at < D) run(reinterpret_cast<float *>(p.ws + ld.z) + size_t(ub) * D + at, p.zsnap + size_t(id.u) * p.nsub * D + at, D);
+}
+
+// 1b. (passes of more than kDirectChunks chunks) the sums are added up once: S and z move on by the pass, and every chunk's
+// slot then holds the state at its start
+template <int D>
+__global__ void __launch_bounds__(kThreads) prefill_fma_scan_kernel(const PrefillParams p) {
+  add_sums<D, true>(p, int64_t(blockIdx.x) * kThreads + threadIdx.x);
+}
+
+// 3. The first blocks (passes without a scan): S and z plus the pass's sums; the others: the pass's newest min(C, cap) tokens
+// to slot (position mod cap), one thread per four entries of a K and a V row.
 template <typename T, int D>
 __global__ void __launch_bounds__(kThreads) prefill_fma_finish_kernel(const PrefillParams p, unsigned state_blocks) {
   const int tid = threadIdx.x;
   if (blockIdx.x == 0 && p.advance)
     for (int l = tid; l < p.layer_count; l += kThreads) p.n_dev[p.layer_begin + l] += p.advance;
   if (blockIdx.x < state_blocks) {
-    const int64_t e = int64_t(blockIdx.x) * kThreads + tid;
-    const UnitId id = unit_id(p, e / (D * D / 4));
-    const int at = int(e % (D * D / 4)) * 4;
-    const LayerDev ld = p.layers[p.layer_begin + id.lrel];
-    const int64_t first = p.n0 + p.c0 - ld.wlin;
-    if (!ld.evicts || first + p.C <= 0) return;
-    const int k0 = first >= 0 ? 0 : int(-first / p.SC);
-    const int ub = (id.b + p.b0) * p.Hkv + id.g;
-    float4 *Sp = reinterpret_cast<float4 *>(reinterpret_cast<float *>(p.ws + ld.S) + size_t(ub) * D * D + at);
-    const float *sums = p.phik + size_t(id.u) * p.nsub * D * D + at;
-    float4 s = *Sp;
-#pragma unroll 4
-    for (int k = k0; k < p.nsub; ++k) {
-      const float4 x = *reinterpret_cast<const float4 *>(sums + size_t(k) * D * D);
-      const float dec = chunk_decay(p, id.u, k);
-      s = make_float4(fmaf(s.x, dec, x.x), fmaf(s.y, dec, x.y), fmaf(s.z, dec, x.z), fmaf(s.w, dec, x.w));
-    }
-    *Sp = s;
-    if (at < D) {
-      float4 *zp = reinterpret_cast<float4 *>(reinterpret_cast<float *>(p.ws + ld.z) + size_t(ub) * D + at);
-      float4 z = *zp;
-      for (int k = k0; k < p.nsub; ++k) {
-        const float4 x = *reinterpret_cast<const float4 *>(p.zsnap + (size_t(id.u) * p.nsub + k) * D + at);
-        const float dec = chunk_decay(p, id.u, k);
-        z = make_float4(fmaf(z.x, dec, x.x), fmaf(z.y, dec, x.y), fmaf(z.z, dec, x.z), fmaf(z.w, dec, x.w));
-      }
-      *zp = z;
-    }
+    add_sums<D, false>(p, int64_t(blockIdx.x) * kThreads + tid);
     return;
   }
   const int64_t e = int64_t(blockIdx.x - state_blocks) * kThreads + tid;
@@ -557,7 +579,10 @@ int launch_prefill_fma(glide_ctx *ctx, const PrefillParams &p, cudaStream_t stre
   return dispatch_config(ctx->cfg.io_dtype, ctx->cfg.head_dim, ctx->G, [&](auto tt, auto dd, auto gg) -> int {
     using T = typename decltype(tt)::type;
     constexpr int D = decltype(dd)::value, G = decltype(gg)::value, TOK = kRows / G;
+    const unsigned state_ctas = any_evicts ? unsigned(units * (D * D / 4 / kThreads)) : 0u;
+    const bool scan = any_evicts && p.nsub > kDirectChunks<D>;
     if (any_evicts) prefill_fma_sums_kernel<T, D><<<unsigned(units * p.nsub * (D / 16)), 2 * kThreads, 0, stream>>>(p);
+    if (scan) prefill_fma_scan_kernel<D><<<state_ctas, kThreads, 0, stream>>>(p);
     if (p.out) {
       auto kern = prefill_fma_attn_kernel<T, D, G>;
       if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(sizeof(AttnSmem<D>))) != cudaSuccess) {
@@ -567,7 +592,7 @@ int launch_prefill_fma(glide_ctx *ctx, const PrefillParams &p, cudaStream_t stre
       const int64_t blocks = units * (int64_t(p.nsub - 1) * ((p.SC + TOK - 1) / TOK) + (p.C - (p.nsub - 1) * p.SC + TOK - 1) / TOK);
       kern<<<unsigned(blocks), 2 * kThreads, sizeof(AttnSmem<D>), stream>>>(p);
     }
-    const unsigned state_blocks = any_evicts ? unsigned(units * (D * D / 4 / kThreads)) : 0u;
+    const unsigned state_blocks = scan ? 0u : state_ctas;
     const unsigned ring_blocks = unsigned((units * p.C * (D / 4) + kThreads - 1) / kThreads);
     prefill_fma_finish_kernel<T, D><<<state_blocks + ring_blocks, kThreads, 0, stream>>>(p, state_blocks);
     return cudaGetLastError() == cudaSuccess ? GLIDE_OK : GLIDE_ERR_CUDA;

@@ -45,3 +45,12 @@ def test_cuda_core_passes(dtype, d, G, merge, chunk, calls, gated):
     (torch.float32, 128, 4, [33, 0, 1 << 20], dict(phi=1)), (torch.float32, 64, 2, [31, 0], dict(gated=True))])
 def test_decode_by_unit(dtype, d, G, windows, kw):
     run_case(windows, 2, 2 * G, 2, d, dtype, [70], 3, amp=4 * d ** -0.5, seed=53 + G, max_tokens=600, **kw)
+
+
+# CUDA-core passes of so many chunks that their sums are scanned (more than 8 of d = 64, 4 of d = 128), with the first delayed
+# token in the pass's first, a middle and its last chunk; gates
+@pytest.mark.parametrize("dtype,d,G,chunk,calls,gated", [
+    (torch.float32, 64, 1, 0, [700, 90], False), (torch.float32, 64, 4, 64, [640, 1], True), (torch.float32, 128, 2, 80, [500, 33], False),
+    (BF16, 64, 2, 0, [650], True)])
+def test_cuda_core_passes_with_a_scan(dtype, d, G, chunk, calls, gated):
+    run_case([0, 64, 300, 630], 2, 2 * G, 2, d, dtype, calls, 2, amp=4 * d ** -0.5, seed=73 + G, gated=gated, prefill_chunk=chunk)
