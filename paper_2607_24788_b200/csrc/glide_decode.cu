@@ -847,8 +847,9 @@ int launch_decode_phi(glide_ctx *ctx, const DecodeParams &p, cudaStream_t stream
   });
 }
 
-// the CUDA-core decode step of these layers takes one CTA per unit
+// the CUDA-core decode step of these layers takes one CTA per unit (a caller who chooses how units are cut gets the work list)
 bool decode_by_unit(const glide_ctx *ctx, int layer_begin, int layer_count) {
+  if (ctx->cfg.decode_chunk || ctx->cfg.decode_state_splits) return false;
   for (int l = layer_begin; l < layer_begin + layer_count; ++l)
     if (ctx->layers[size_t(l)].cap > unit_max_cap(ctx->cfg.head_dim, ctx->G)) return false;
   return true;

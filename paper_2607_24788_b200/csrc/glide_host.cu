@@ -371,7 +371,6 @@ int glide_create(const glide_config *cfg, void *dev_workspace, size_t workspace_
   if (ok && ctx->decode_kind == 0) {
     ok = decode_occupancy(ctx, &per_sm) == GLIDE_OK && per_sm > 0;
     if (ok) ctx->decode_grid = std::max(1, std::min(ctx->n_items, ctx->sm_count * per_sm));
-    if (ok && decode_by_unit(ctx, 0, cfg->n_layers)) ctx->decode_grid = cfg->n_layers * cfg->batch * cfg->n_kv_heads;   // (one CTA per unit)
   }
   if (ok) {
     if (!ctx->tmaps_host.empty())
@@ -704,8 +703,10 @@ int glide_device_status(glide_ctx *ctx, void *stream, int32_t *status_out) {
 int glide_decode_launch_info(glide_ctx *ctx, int32_t *n_launches, int32_t *n_work_items, int32_t *grid_size) {
   if (!ctx) return GLIDE_ERR_INVALID_ARG;
   if (n_launches) *n_launches = ctx->cfg.phi == GLIDE_PHI_PROJ_SOFTMAX2 ? 2 : 1;   // the feature kernel, then the step
-  if (n_work_items) *n_work_items = ctx->decode_kind == 2 ? int32_t(ctx->stream_scheds[0].n_segs) : ctx->n_items;
-  if (grid_size) *grid_size = ctx->decode_grid;
+  const bool by_unit = ctx->decode_kind == 0 && decode_by_unit(ctx, 0, ctx->cfg.n_layers);   // one CTA and one item per unit
+  const int32_t units = ctx->cfg.n_layers * ctx->cfg.batch * ctx->cfg.n_kv_heads;
+  if (n_work_items) *n_work_items = by_unit ? units : ctx->decode_kind == 2 ? int32_t(ctx->stream_scheds[0].n_segs) : ctx->n_items;
+  if (grid_size) *grid_size = by_unit ? units : ctx->decode_grid;
   return GLIDE_OK;
 }
 
