@@ -110,7 +110,10 @@ typedef struct {
                               h / (H/H_kv) (the Llama/Mistral GQA convention). Groups must be equal-sized. Copied. */
   int64_t max_tokens;      /* per-sequence capacity, prompt + generated tokens */
   float softmax_scale;     /* scale of the window logits; 0 selects 1/sqrt(head_dim) (appendix Eq. 1) */
-  int32_t prefill_chunk;   /* tokens per chunk of the chunked linear scan; 0 selects 256; multiple of 16, <= 1024 */
+  int32_t prefill_chunk;   /* tokens per chunk of the chunked linear scan; multiple of 16, <= 1024.  The prefill scratch is
+                              sized for one chunk of every unit.  0: 256, or what suits the call on the CUDA-core prefill
+                              kernels with the parameter-free map (64 to 256 in a scratch sized for 256; the order of the
+                              fp32 sums then depends on the call's length and on how many sequences it holds) */
   int32_t decode_chunk;    /* window slots per split-K work item of the decode kernel; 0 selects automatically */
   int32_t decode_state_splits; /* row blocks the S update/readout of one KV head is split into; 0 selects automatically */
   int32_t decode_impl;     /* glide_decode_impl */

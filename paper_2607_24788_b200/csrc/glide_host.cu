@@ -188,11 +188,14 @@ int glide::plan_context(const glide_config *cfg, glide_ctx *ctx, std::vector<Wor
   // per layer 3 maps of 16-row boxes, then (from 3 L on) 2 of 128-row boxes, then the three bf16 scratch arrays of prefill
   off = align_up(off + size_t(128) * (5 * L + 3), 256);
   ctx->off_phik = off;
-  // one chunk's phi(K'), or the CUDA-core passes' chunk sums: at least one [d][d] (with z) per unit
-  ctx->phik_rows = size_t(std::max(ctx->prefill_chunk, d));
-  off = align_up(off + sizeof(float) * size_t(L) * units_per_layer * ctx->phik_rows * dp, 256);
+  // phi(K') of one chunk of every unit, or the CUDA-core passes' chunk sums ([d][d] each): room for one sum of every unit of a layer
+  const size_t all_units = size_t(L) * units_per_layer;
+  size_t phik_rows = all_units * ctx->prefill_chunk;
+  if (cuda_core_passes(*cfg)) phik_rows = std::max(phik_rows, size_t(units_per_layer) * d);
+  ctx->sum_slots = int64_t(phik_rows / d);
+  off = align_up(off + sizeof(float) * phik_rows * dp, 256);
   ctx->off_zsnap = off;
-  off = align_up(off + sizeof(float) * size_t(L) * units_per_layer * std::max<size_t>(1, ctx->phik_rows / d) * dp, 256);
+  off = align_up(off + sizeof(float) * std::max(all_units, size_t(ctx->sum_slots)) * dp, 256);
   ctx->off_zcum = off;   // running sums of phi(K') over the chunk: only the sum-of-terms merges use them
   if (cfg->merge != GLIDE_MERGE_SHARED)
     off = align_up(off + sizeof(float) * size_t(L) * units_per_layer * ctx->prefill_chunk * dp, 256);
@@ -200,9 +203,12 @@ int glide::plan_context(const glide_config *cfg, glide_ctx *ctx, std::vector<Wor
   if (cfg->phi == GLIDE_PHI_PROJ_SOFTMAX2)
     off = align_up(off + sizeof(float) * size_t(L) * units_per_layer * dp * (ctx->G + 1), 256);
   ctx->off_gcum = off;   // gated: running sums of log(gate) over the chunk's delayed tokens
-  // (as many chunks of up to 256 tokens as the CUDA-core passes have sums for)
-  if (cfg->gated)
-    off = align_up(off + sizeof(float) * size_t(L) * units_per_layer * std::max<size_t>(ctx->prefill_chunk, 256 * (ctx->phik_rows / d)), 256);
+  // (the CUDA-core passes choose the chunk themselves, up to 256 tokens, unless the caller does: sums for all of their slots then)
+  if (cfg->gated) {
+    if (cuda_core_passes(*cfg) && cfg->prefill_chunk) ctx->sum_slots = std::min(ctx->sum_slots, int64_t(all_units));
+    const size_t sums = cuda_core_passes(*cfg) && !cfg->prefill_chunk ? size_t(ctx->sum_slots) * 256 : all_units * ctx->prefill_chunk;
+    off = align_up(off + sizeof(float) * sums, 256);
+  }
   // tcgen05 prefill kernel (bf16, head_dim 128, plain feature map): bf16 copies of the chunk's phi(K') rows and of S,
   // which its CTAs fetch by TMA instead of converting the fp32 arrays themselves
   // (the learned map under the shared normaliser and, with the plain map, gates too; not both)

@@ -236,7 +236,7 @@ struct glide_ctx {
   mutable bool launch_wrapped = false;   // the counter has passed 2^32: the records are cleared before the next launch
   int stream_rec_floats = 0;        // record size of the streaming kernel (twice as large for the sum-of-terms merges)
   int prefill_chunk = 0;
-  size_t phik_rows = 0;             // rows of d_phi floats per unit of the fp32 prefill scratch
+  int64_t sum_slots = 0;            // (unit, chunk) pairs that a CUDA-core prefill pass has room for
   float scale = 0.f;
   size_t elem = 0;
   unsigned char *ws = nullptr;
@@ -269,6 +269,21 @@ int launch_decode(glide_ctx *ctx, int layer_begin, int layer_count, const void *
                   const float *gate, void *out, cudaStream_t stream);
 int decode_occupancy(const glide_ctx *ctx, int *blocks_per_sm);
 bool decode_by_unit(const glide_ctx *ctx, int layer_begin, int layer_count);
+// What the tcgen05 prefill kernel takes beside the plain method: the learned map under the shared normaliser (its two halves
+// as two linear parts) and, with the plain map and the shared normaliser, gates (its operands split in two)
+inline bool tc_prefill_kind(const glide_config &c) {
+  return c.gated ? c.phi == GLIDE_PHI_SOFTMAX && c.merge == GLIDE_MERGE_SHARED : c.phi == GLIDE_PHI_SOFTMAX || c.merge == GLIDE_MERGE_SHARED;
+}
+// prefill_impl with AUTO resolved
+inline int resolved_prefill_impl(const glide_config &c) {
+  if (c.prefill_impl != GLIDE_PREFILL_AUTO) return c.prefill_impl;
+  return tc_prefill_kind(c) && c.io_dtype == GLIDE_BF16 && c.head_dim == 128 && c.decode_impl != GLIDE_DECODE_FMA ? GLIDE_PREFILL_TCGEN05
+                                                                                                                 : GLIDE_PREFILL_FMA;
+}
+// prefill by the CUDA-core passes (otherwise by the tensor-core pipeline or chunk by chunk)
+inline bool cuda_core_passes(const glide_config &c) {
+  return c.phi == GLIDE_PHI_SOFTMAX && resolved_prefill_impl(c) == GLIDE_PREFILL_FMA;
+}
 // seq < 0: the call's tensors hold all B sequences, the layers' counters advance; otherwise they hold sequence slot
 // `seq` alone ([layer_count][1][T]...), which is at position n0, and no counter is touched
 int launch_prefill(glide_ctx *ctx, int layer_begin, int layer_count, int64_t T, const void *q, const void *k,

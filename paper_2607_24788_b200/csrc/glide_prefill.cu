@@ -626,17 +626,10 @@ int launch_prefill(glide_ctx *ctx, int layer_begin, int layer_count, int64_t T, 
   p.gcum = reinterpret_cast<float *>(ctx->ws + ctx->off_gcum);
   const int64_t units = int64_t(layer_count) * p.B * p.Hkv;
   const bool plain = ctx->cfg.phi == GLIDE_PHI_SOFTMAX && !ctx->cfg.gated;   // what the tensor-core kernels compute
-  const bool plain_gated = ctx->cfg.gated && ctx->cfg.phi == GLIDE_PHI_SOFTMAX && ctx->cfg.merge == GLIDE_MERGE_SHARED;
-  int impl = ctx->cfg.prefill_impl;
-  // the tcgen05 kernel also takes the learned map under the shared normaliser (its two halves as two linear parts)
-  // and, under the shared normaliser, gates with the plain map (its operands split in two)
-  const bool tc_kind = ctx->cfg.gated ? plain_gated : (ctx->cfg.phi == GLIDE_PHI_SOFTMAX || ctx->cfg.merge == GLIDE_MERGE_SHARED);
-  if (impl == GLIDE_PREFILL_AUTO)
-    impl = (tc_kind && prefill_attn_mma_supported(ctx) && ctx->cfg.decode_impl != GLIDE_DECODE_FMA) ? GLIDE_PREFILL_TCGEN05
-                                                                                                : GLIDE_PREFILL_FMA;
+  const int impl = resolved_prefill_impl(ctx->cfg);
   // the tcgen05 kernel needs the ring descriptors of the tensor-core decode kernels (absent when decode_impl asks
   // for the CUDA-core kernel); without them the call uses the mma.sync kernel
-  const bool use_tc = impl == GLIDE_PREFILL_TCGEN05 && tc_kind && prefill_attn_tc_supported(ctx);
+  const bool use_tc = impl == GLIDE_PREFILL_TCGEN05 && tc_prefill_kind(ctx->cfg) && prefill_attn_tc_supported(ctx);
   p.phik16 = use_tc && out ? ctx->ws + ctx->off_phik16 : nullptr;
   p.s16 = use_tc && out ? ctx->ws + ctx->off_s16 : nullptr;
   p.zsnap = reinterpret_cast<float *>(ctx->ws + ctx->off_zsnap);
@@ -721,13 +714,12 @@ int launch_prefill(glide_ctx *ctx, int layer_begin, int layer_count, int64_t T, 
   };
   const bool passes = state_mma && (use_tc || !out);
 
-  // CUDA-core passes (parameter-free map): the scratch holds phik_rows / d chunk sums per unit.  Chunks as short as
-  // that allows for the whole call in one pass (a query goes through its chunk's delayed tokens one by one, 64 at a time),
-  // but not below 64 tokens, where a chunk's sum costs as much as the tokens it saves, nor above 256.
-  if (!passes && !use_mma && !state_mma && ctx->cfg.phi == GLIDE_PHI_SOFTMAX) {
-    const int64_t slots = p.units_cap * int64_t(ctx->phik_rows / size_t(ctx->cfg.head_dim));
-    const int64_t most = slots / units_layer;
-    p.SC = int(std::min<int64_t>(256, std::max<int64_t>(64, ((T + most - 1) / most + 15) / 16 * 16)));
+  // CUDA-core passes (parameter-free map).  The chunk is the caller's, or as short as the slots for chunk sums allow for the
+  // whole call in one pass (a query goes through its chunk's delayed tokens one by one, 64 at a time), but not below 64
+  // tokens, where a chunk's sum costs as much as the tokens it saves, nor above 256.
+  if (cuda_core_passes(ctx->cfg)) {
+    const int64_t slots = ctx->sum_slots, most = slots / units_layer;
+    if (!ctx->cfg.prefill_chunk) p.SC = int(std::min<int64_t>(256, std::max<int64_t>(64, ((T + most - 1) / most + 15) / 16 * 16)));
     return for_passes(slots, most, ctx->cfg.head_dim, ctx->elem, [&](const PrefillParams &s) -> int {
       if (p.gated && evicts_in(s.layer_begin, s.layer_count)) {
         const unsigned blocks = unsigned((int64_t(s.layer_count) * units_layer * s.nsub * 32 + kPrefillThreads - 1) / kPrefillThreads);

@@ -28,3 +28,36 @@ def test_decode_items_per_unit(kw, items):
 def test_decode_work_list_with_many_records(dtype, d, G, kw):
     run_case([0, 5, 150, 1 << 20], 2, 2 * G, 2, d, dtype, [260], 4, amp=4 * d ** -0.5, seed=59 + G, max_tokens=300, decode_chunk=8,
              **kw)
+
+
+# prefill_chunk is the chunk of the scan: a call of eight chunks, eight calls of one, and one slot after the other give the
+# same bits (the same sums in the same order); 16: less than a chunk sum's rows, 272: more than the kernels choose themselves
+@pytest.mark.parametrize("d,gated,chunk", [(64, False, 16), (64, True, 80), (128, False, 48), (128, True, 272)])
+def test_prefill_chunk_cuts_the_scan(d, gated, chunk):
+    L, B, H, Hkv, T = 2, 2, 4, 2, 8 * chunk
+    gen = torch.Generator(device="cuda").manual_seed(67)
+    q, k, v = (torch.randn((L, B, T, h, d), generator=gen, device="cuda") for h in (H, Hkv, Hkv))
+    gate = 0.99 + 0.01 * torch.rand((L, B, T, Hkv), generator=gen, device="cuda")
+
+    def prefill(cuts, by_slot):
+        g = glide.Glide([100, 0], B, H, Hkv, d, 1 << 20, dtype=F32, gated=gated, prefill_chunk=chunk)
+        out = torch.zeros_like(q)
+        for s in ([slice(b, b + 1) for b in range(B)] if by_slot else [slice(0, B)]):
+            for c in range(0, T, T // cuts):
+                part = [x[:, s, c:c + T // cuts].contiguous() for x in (q, k, v, out, gate)]
+                if by_slot:
+                    g.glide_prefill_seq(s.start, *(x[:, 0] for x in part[:4]))
+                elif gated:
+                    g.glide_prefill_gated(*part[:3], part[4], part[3])
+                else:
+                    g.glide_prefill(*part[:4])
+                out[:, s, c:c + T // cuts] = part[3]
+        states = [x.clone() for l in range(L) for x in g.glide_export_state(l)[2:]]
+        assert g.glide_device_status() == 0
+        g.glide_destroy()
+        return [out, *states]
+
+    one = prefill(1, False)
+    for other in [prefill(8, False)] + ([] if gated else [prefill(2, True)]):   # (a slot's call takes no gates)
+        for a, b in zip(one, other):
+            assert torch.equal(a, b)
