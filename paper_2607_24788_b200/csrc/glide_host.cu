@@ -209,12 +209,9 @@ int glide::plan_context(const glide_config *cfg, glide_ctx *ctx, std::vector<Wor
     const size_t sums = cuda_core_passes(*cfg) && !cfg->prefill_chunk ? size_t(ctx->sum_slots) * 256 : all_units * ctx->prefill_chunk;
     off = align_up(off + sizeof(float) * sums, 256);
   }
-  // tcgen05 prefill kernel (bf16, head_dim 128, plain feature map): bf16 copies of the chunk's phi(K') rows and of S,
-  // which its CTAs fetch by TMA instead of converting the fp32 arrays themselves
-  // (the learned map under the shared normaliser and, with the plain map, gates too; not both)
-  if (cfg->io_dtype == GLIDE_BF16 && d == 128 &&
-      (cfg->gated ? cfg->phi == GLIDE_PHI_SOFTMAX && cfg->merge == GLIDE_MERGE_SHARED
-                  : cfg->phi == GLIDE_PHI_SOFTMAX || cfg->merge == GLIDE_MERGE_SHARED)) {
+  // tcgen05 prefill kernel, where the context can run it: bf16 copies of the chunk's phi(K') rows and of S, which its CTAs
+  // fetch by TMA instead of converting the fp32 arrays themselves
+  if (tc_prefill_kind(*cfg) && resolved_prefill_impl(*cfg) == GLIDE_PREFILL_TCGEN05 && cfg->decode_impl != GLIDE_DECODE_FMA) {
     // the learned map's two softmax halves are kept apart (one 128-column tensor each), as are hi and lo of a gated context
     const size_t halves = cfg->gated ? 2 : size_t(dp / d);
     ctx->off_phik16 = off;

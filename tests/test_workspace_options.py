@@ -24,7 +24,18 @@ SLACK = 3 << 20   # alignment of the streamed arrays, small tables
 
 
 # the prefill scratch holds prefill_chunk rows of fp32 per unit (or one chunk sum for every unit of one layer, which is less here)
-@pytest.mark.parametrize("dtype,d,kw", [(F32, 64, {}), (F32, 128, {}), (F32, 128, dict(gated=True)), (BF16, 64, {})])
+@pytest.mark.parametrize("dtype,d,kw", [(F32, 64, {}), (F32, 128, {}), (F32, 128, dict(gated=True)), (BF16, 64, {}),
+                                        (BF16, 128, dict(prefill_impl=glide.GLIDE_PREFILL_FMA))])
 def test_prefill_chunk_bounds_the_scratch(dtype, d, kw):
     rows = (256 - 16) * UNITS
     assert abs(_bytes(dtype, d, prefill_chunk=256, **kw) - _bytes(dtype, d, prefill_chunk=16, **kw) - rows * d * 4) < rows * 8 + SLACK
+
+
+# the bf16 copies that the tcgen05 prefill kernel reads (phi(K') rows and S; two of each with gates) are laid out only where
+# the context can run that kernel
+@pytest.mark.parametrize("gated,halves", [(False, 1), (True, 2)])
+@pytest.mark.parametrize("kw", [dict(prefill_impl=glide.GLIDE_PREFILL_FMA), dict(decode_impl=glide.GLIDE_DECODE_FMA)])
+def test_no_scratch_for_a_kernel_that_is_ruled_out(gated, halves, kw):
+    copies = halves * UNITS * (64 + 128) * 128 * 2
+    more = _bytes(BF16, 128, gated=gated, prefill_chunk=64) - _bytes(BF16, 128, gated=gated, prefill_chunk=64, **kw)
+    assert abs(more - copies) < UNITS * 1024 + SLACK
