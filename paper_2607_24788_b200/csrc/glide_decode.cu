@@ -399,11 +399,23 @@ template <int D, int G>
 constexpr int kUnitWinWarps = D * G >= 1024 ? 4 : 8;   // (their partial results are the CTA's shared memory)
 template <int D, int G>
 constexpr int kUnitThreads = kUnitWinWarps<D, G> * 32 + kUnitStateThreads;
-// Longest ring for it: a CTA has 64 rows in flight and scores them for all heads of the group itself, so longer rings are
-// read faster by several CTAs.  Per launch, here against the list above: d = 64, one head per unit, 4 units: w = 64 5.8 us
-// against 12.6, 256 8.4 / 15.6, 500 11.6 / 15.6; d = 128, four heads, 2 units: w = 300 18.3 / 22.6, 500 26.4 / 21.6;
-// 64 units of w = 300 (d = 64): 9.1 / 17.2.
-inline int64_t unit_max_cap(int d, int G) { return d * G <= 128 ? 512 : 320; }
+// Longest ring for it (-1: none).  A CTA has 64 rows in flight and scores them for all heads of the group itself, so the list,
+// which cuts a ring in pieces of 128 rows, gains with the heads and rows of a unit; and once the units are several waves of
+// the chip, the time per row counts and no longer the list's chain of round trips: its leaner warps win with more heads,
+// with bf16 rows of 128 (converted for every head here) and, over few heads, with the learned map.  The lines lie where a
+// launch becomes slower than the list's.  Microseconds here / list, 8 units: d = 64, G = 1, w = 512 14.4 / 17.5; G = 4, w = 192
+// 16.5 / 21.0, w = 512 28.8 / 21.5; d = 128, G = 8, bf16, w = 64 22.6 / 24.9, w = 512 100 / 35.  4096 units: d = 64, G = 1, w = 512
+// 263 / 357, G = 4, w = 16 180 / 150; d = 128, G = 4, w = 320 627 / 701, bf16 1075 / 751.
+inline int64_t unit_max_cap(int d, int G, bool bf16, bool learned, bool one_wave) {
+  const int gi = G == 1 ? 0 : G == 2 ? 1 : G == 4 ? 2 : 3, di = d == 128;
+  static constexpr int16_t kOneWave[2][4] = {{512, 384, 192, 128}, {320, 320, 256, 64}};   // [d = 64, 128][G]
+  static constexpr int16_t kF32[2][4] = {{512, -1, -1, -1}, {320, 320, 320, 64}};          // several waves, from here on
+  static constexpr int16_t kBf16[2][4] = {{512, 512, -1, -1}, {64, 64, 64, 16}};
+  static constexpr int16_t kLearned[2][4] = {{-1, -1, -1, -1}, {-1, 320, 320, 128}};
+  if (one_wave) return kOneWave[di][gi];
+  const int cap = learned ? kLearned[di][gi] : kF32[di][gi];
+  return bf16 ? (learned ? std::min<int>(cap, kBf16[di][gi]) : kBf16[di][gi]) : cap;
+}
 
 template <typename T, int D, int G, int DP>
 __global__ void __launch_bounds__(kUnitThreads<D, G>) glide_decode_unit_kernel(const DecodeParams p) {
@@ -850,8 +862,11 @@ int launch_decode_phi(glide_ctx *ctx, const DecodeParams &p, cudaStream_t stream
 // the CUDA-core decode step of these layers takes one CTA per unit (a caller who chooses how units are cut gets the work list)
 bool decode_by_unit(const glide_ctx *ctx, int layer_begin, int layer_count) {
   if (ctx->cfg.decode_chunk || ctx->cfg.decode_state_splits) return false;
+  const int64_t units = int64_t(layer_count) * ctx->cfg.batch * ctx->cfg.n_kv_heads;
+  const int64_t longest = unit_max_cap(ctx->cfg.head_dim, ctx->G, ctx->cfg.io_dtype == GLIDE_BF16, ctx->cfg.phi == GLIDE_PHI_PROJ_SOFTMAX2,
+                                       units <= ctx->sm_count);
   for (int l = layer_begin; l < layer_begin + layer_count; ++l)
-    if (ctx->layers[size_t(l)].cap > unit_max_cap(ctx->cfg.head_dim, ctx->G)) return false;
+    if (ctx->layers[size_t(l)].cap > longest) return false;
   return true;
 }
 

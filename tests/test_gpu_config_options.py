@@ -61,3 +61,25 @@ def test_prefill_chunk_cuts_the_scan(d, gated, chunk):
     for other in [prefill(8, False)] + ([] if gated else [prefill(2, True)]):   # (a slot's call takes no gates)
         for a, b in zip(one, other):
             assert torch.equal(a, b)
+
+
+# one CTA per unit or the work list: the longest ring of the launch, head_dim, group size, type and map, and whether the units
+# are more than the chip has SMs (148 here): (L, B, H_kv, G, d, window) with one item per unit, and the same with one slot more
+@pytest.mark.parametrize("dtype,L,B,Hkv,G,d,w,kw", [
+    (F32, 1, 1, 4, 1, 64, 512, {}), (F32, 8, 8, 4, 1, 64, 512, {}), (F32, 1, 2, 4, 8, 128, 64, {}), (BF16, 8, 8, 4, 8, 128, 16, dict(decode_impl=2)),
+    (F32, 1, 2, 4, 4, 64, 192, {}), (F32, 8, 8, 4, 4, 128, 320, {}), (F32, 8, 8, 4, 2, 128, 320, dict(phi=1))])
+def test_decode_by_unit_or_by_list(dtype, L, B, Hkv, G, d, w, kw):
+    units = L * B * Hkv
+    if kw.get("phi"):
+        kw = dict(kw, phi_wq=torch.zeros((L, G * Hkv, d, d), device="cuda", dtype=dtype),
+                  phi_wk=torch.zeros((L, Hkv, d, d), device="cuda", dtype=dtype))
+    for longer in (0, 1):
+        g = glide.Glide([w + longer] + [w] * (L - 1), B, G * Hkv, Hkv, d, 1 << 20, dtype=dtype, **kw)
+        assert (g.glide_decode_launch_info()["work_items"] == units) == (longer == 0)
+        g.glide_destroy()
+
+
+@pytest.mark.parametrize("G,d,kw", [(4, 64, {}), (2, 64, dict(phi=1)), (8, 64, dict(merge=1))])
+def test_decode_many_small_units_take_the_work_list(G, d, kw):
+    """More units than SMs with several heads of 64: the list, against the oracle; a range of few of its layers: by unit."""
+    run_case([16] * 5, 16, 2 * G, 2, d, F32, [20], 2, amp=4 * d ** -0.5, seed=71 + G, max_tokens=40, **kw)
