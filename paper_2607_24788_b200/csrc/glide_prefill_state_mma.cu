@@ -15,6 +15,7 @@
 // the bf16 rows for the attention kernel: as a kernel in front, phi cost a trip of 512 bytes per token through memory.
 // 8 x 2048 tokens, 4 layers: 107 us for phi and 126 for the carry, 188 together.
 #include <algorithm>
+#include <type_traits>
 
 #include "glide_device.cuh"
 
@@ -65,12 +66,38 @@ __device__ __forceinline__ void store_s16(__nv_bfloat16 *at, size_t lo_half, flo
   if (lo_half) *reinterpret_cast<__nv_bfloat162 *>(at + lo_half) = __floats2bfloat162_rn(x - __low2float(h), y - __high2float(h));
 }
 
+// One element of a gated chunk's sum in fp32, token after token: what a split term times an infinity (0 x inf, or an infinity of
+// the other sign) must not decide.  Row `row` of S and column `col` of V'; phi(k') of the row from `phi` (stride dp), or made
+// from the K' rows with the tokens' maxima and 1 / sums.  Cold: called for sums that are not finite.
+struct CarryRows {
+  const __nv_bfloat16 *ringK, *ringV, *callK, *callV;
+  int64_t n0, first, cap, call_stride;
+  const float *gc;
+  float g_end;
+  int i_lo, chunk_n;
+  __device__ __forceinline__ int64_t at(int i) const {
+    const int64_t j = first + i;
+    return j >= n0 ? (j - n0) * call_stride : int64_t(uint32_t(j) % uint32_t(cap)) * kD;
+  }
+  __device__ __forceinline__ const __nv_bfloat16 *k(int i) const { return (first + i >= n0 ? callK : ringK) + at(i); }
+  __device__ __forceinline__ const __nv_bfloat16 *v(int i) const { return (first + i >= n0 ? callV : ringV) + at(i); }
+};
+__device__ __noinline__ float carry_element(const CarryRows &rows, const float *phi, int dp, const float2 *stats, int row, int col) {
+  float sum = 0.f;
+#pragma unroll 4
+  for (int i = rows.i_lo; i < rows.chunk_n; ++i) {
+    const float f = phi ? phi[size_t(i) * dp] : exp2f((__bfloat162float(rows.k(i)[row]) - stats[i].x) * kLog2e) * stats[i].y;
+    sum = fmaf(f * expf(rows.g_end - rows.gc[i]), __bfloat162float(rows.v(i)[col]), sum);
+  }
+  return sum;
+}
+
 // PARTIAL (passes of several chunks): the chunk's own sum goes to the scratch rows that the CTA has just consumed instead
 // of S (64 state rows x 128 values = 128 scratch rows x the CTA's 64 columns, z in row 128: chunks of more than 128
 // tokens), and prefill_scan_kernel adds the sums up in chunk order.  Otherwise S is updated in place, and its value
 // before the chunk is left as bf16 (z: fp32) for the attention kernel, which runs after this one.
 // MAKE_PHI: phi(K') is made here (parameter-free map); otherwise it is in the scratch.
-template <bool PARTIAL, bool MAKE_PHI>
+template <bool PARTIAL, bool MAKE_PHI, bool GATED>
 __global__ void __launch_bounds__(kThreads) prefill_state_mma_kernel(const PrefillParams p) {
   using bf16 = __nv_bfloat16;
   // per stage phi columns (or K' rows, 16 bytes more per row) and V' rows; made phi columns
@@ -109,8 +136,8 @@ __global__ void __launch_bounds__(kThreads) prefill_state_mma_kernel(const Prefi
 #pragma unroll
   for (int n = 0; n < kD / 8; ++n) acc[n][0] = acc[n][1] = acc[n][2] = acc[n][3] = 0.f;
   float zacc = 0.f;   // threads 0..63: z of row rb*64 + tid
-  const float *gc = p.gated ? p.gcum + size_t(u) * p.Cmax + chunk_c0 : nullptr;
-  const float g_end = gc ? gc[chunk_n - 1] : 0.f;
+  const float *gc = GATED ? p.gcum + size_t(u) * p.Cmax + chunk_c0 : nullptr;
+  const float g_end = GATED ? gc[chunk_n - 1] : 0.f;
 
   // tokens past the chunk's end are filled with zeros
   auto issue = [&](int buf, int i0) {
@@ -128,7 +155,7 @@ __global__ void __launch_bounds__(kThreads) prefill_state_mma_kernel(const Prefi
       if (MAKE_PHI) cp16(sphi + uint32_t(i * kVStride + c * 16), (j >= p.n0 ? callK : ringK) + at + c * 8, i < nt);
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
-    if (tid < kTok) decay[buf][tid] = (gc && tid < nt) ? expf(g_end - gc[i0 + tid]) : 1.f;   // (rows past the end are zero)
+    if (tid < kTok) decay[buf][tid] = (GATED && tid < nt) ? expf(g_end - gc[i0 + tid]) : 1.f;   // (rows past the end are zero)
   };
   issue(0, i_lo);
   int buf = 0;
@@ -182,7 +209,7 @@ __global__ void __launch_bounds__(kThreads) prefill_state_mma_kernel(const Prefi
           bf16 *out = p16 + size_t(i0 + tok) * kD + (part & 1) * 32;
 #pragma unroll
           for (int hl = 0; hl < 2; ++hl) {   // gated: what the rounding left, in the second half of the array
-            if (hl == 1 && !p.gated) break;
+            if (hl == 1 && !GATED) break;
 #pragma unroll
             for (int i = 0; i < 32; i += 8) {
               uint32_t o[4];
@@ -233,6 +260,35 @@ __global__ void __launch_bounds__(kThreads) prefill_state_mma_kernel(const Prefi
     }
     __syncthreads();   // the stage is refilled by the next iteration's issue
   }
+  if constexpr (GATED) {
+    float chk[4] = {};   // finite if every sum of the thread is
+#pragma unroll
+    for (int n = 0; n < kD / 8; ++n)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) chk[e] += acc[n][e];
+    if (__syncthreads_or(!isfinite(chk[0] + chk[1] + chk[2] + chk[3]))) {
+      const CarryRows rows{ringK, ringV, callK, callV, p.n0, first, cap, call_stride, gc, g_end, i_lo, chunk_n};
+      float2 *stats = reinterpret_cast<float2 *>(&stage[0][0]);   // [chunk token]: maximum of K', 1 / sum of its exponentials
+      static_assert(sizeof(stage) >= 1024 * sizeof(float2), "as many as a chunk has tokens");
+      for (int i = i_lo + tid; MAKE_PHI && i < chunk_n; i += kThreads) {
+        const bf16 *kr = rows.k(i);
+        float mx = __bfloat162float(kr[0]), sum = 0.f;
+        for (int c = 1; c < kD; ++c) mx = fmaxf(mx, __bfloat162float(kr[c]));
+        for (int c = 0; c < kD; ++c) sum += exp2f((__bfloat162float(kr[c]) - mx) * kLog2e);
+        stats[i] = make_float2(mx, 1.0f / sum);
+      }
+      __syncthreads();
+#pragma unroll
+      for (int n = 0; n < kD / 8; ++n)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const int row = warp * 16 + gid + (e >> 1) * 8;
+          if (!isfinite(acc[n][e]))
+            acc[n][e] = carry_element(rows, MAKE_PHI ? nullptr : pk + row, p.dp, stats, rb * kRowsPerCta + row, n * 8 + 2 * tig + (e & 1));
+        }
+      __syncthreads();   // (PARTIAL: the sums go over the scratch that was read)
+    }
+  }
   // accumulator fragment: c0, c1 -> (row gid, cols 2 tig + {0,1}); c2, c3 -> row gid + 8
   if (PARTIAL) {   // (every read of these scratch columns lies before the loop's last barrier)
 #pragma unroll
@@ -248,8 +304,8 @@ __global__ void __launch_bounds__(kThreads) prefill_state_mma_kernel(const Prefi
   }
   float *Sb = reinterpret_cast<float *>(p.ws + ld.S) + size_t(ub) * p.dp * kD + size_t(rb * kRowsPerCta + warp * 16) * kD;
   // the halves of a state with 2 d rows are units_cap units apart in the bf16 copy, as are hi and lo of a gated one
-  const size_t lo_half = p.gated ? size_t(p.units_cap) * kD * kD : 0;
-  const float dec_all = gc ? expf(g_end) : 1.f;   // the state the chunk started from, after the whole chunk has entered
+  const size_t lo_half = GATED ? size_t(p.units_cap) * kD * kD : 0;
+  const float dec_all = GATED ? expf(g_end) : 1.f;   // the state the chunk started from, after the whole chunk has entered
   bf16 *s16 = p.s16 ? reinterpret_cast<bf16 *>(p.s16) + (size_t(rb * kRowsPerCta / kD) * p.units_cap + u) * kD * kD +
                           size_t(rb * kRowsPerCta % kD + warp * 16) * kD
                     : nullptr;
@@ -348,12 +404,21 @@ int launch_prefill_state_mma(glide_ctx *ctx, const PrefillParams &p, bool make_p
   (void)ctx;
   const int64_t units = int64_t(p.layer_count) * p.B * p.Hkv;
   const unsigned blocks = unsigned(units * p.nsub * (p.dp / kRowsPerCta));
-  if (make_phi) {
-    if (p.nsub == 1) prefill_state_mma_kernel<false, true><<<blocks, kThreads, 0, stream>>>(p);
-    else prefill_state_mma_kernel<true, true><<<blocks, kThreads, 0, stream>>>(p);
+  auto run = [&](auto partial, auto make, auto gated) {
+    prefill_state_mma_kernel<decltype(partial)::value, decltype(make)::value, decltype(gated)::value><<<blocks, kThreads, 0, stream>>>(p);
+  };
+  const std::true_type yes{};
+  const std::false_type no{};
+  if (p.gated) {   // (a gated pass of several chunks makes its own phi)
+    if (p.nsub > 1) run(yes, yes, yes);
+    else if (make_phi) run(no, yes, yes);
+    else run(no, no, yes);
+  } else if (make_phi) {
+    if (p.nsub > 1) run(yes, yes, no);
+    else run(no, yes, no);
   } else {
-    if (p.nsub == 1) prefill_state_mma_kernel<false, false><<<blocks, kThreads, 0, stream>>>(p);
-    else prefill_state_mma_kernel<true, false><<<blocks, kThreads, 0, stream>>>(p);
+    if (p.nsub > 1) run(yes, no, no);
+    else run(no, no, no);
   }
   if (p.nsub > 1) prefill_scan_kernel<<<unsigned(units * (p.dp / 4)), kThreads, 0, stream>>>(p);
   return cudaGetLastError() == cudaSuccess ? GLIDE_OK : GLIDE_ERR_CUDA;

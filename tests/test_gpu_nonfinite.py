@@ -61,3 +61,11 @@ def _check(dtype, d, G, w, gated, calls, bad, value, **kw):
     (F32, 128, 8, 200, True, [300], (150, 280)), (BF16, 64, 2, 64, False, [257], (256,)), (F32, 64, 8, 90, False, [64, 100], tuple(range(120, 164)))])
 def test_cuda_core_prefill(dtype, d, G, w, gated, calls, bad, value):
     _check(dtype, d, G, w, gated, calls, bad, value)
+
+
+# gated bf16 states of d = 128 are carried by the tensor cores: chunks on their own and in a pass, phi made there and in front
+@pytest.mark.parametrize("value", [float("nan"), float("inf"), float("-inf")])
+@pytest.mark.parametrize("w,calls,kw", [(40, [300], {}), (0, [100, 60], dict(prefill_chunk=64)), (100, [700], dict(prefill_chunk=144))])
+def test_gated_state(w, calls, kw, value):
+    _, S = _prompt(BF16, 128, 4, w, True, calls, (50,), value, **kw)
+    assert bool((torch.isnan(S) if math.isnan(value) else S == value).all())
