@@ -28,7 +28,7 @@
 
 #include <algorithm>
 
-#include "glide_device.cuh"
+#include "glide_prefill_rows.cuh"
 
 namespace glide {
 
@@ -276,6 +276,41 @@ struct CallMaps {
 // products of two split operands leave out lo x lo (2^-18 of the result).
 enum : int { kModeShared = 0, kModeSum = 1, kModeLearned = 2, kModeGated = 3 };
 
+// the state at a chunk's start for a single row: the bf16 copies hi and lo (lo of an infinity is not a number) and z
+struct SplitState {
+  const __nv_bfloat16 *hi;
+  size_t lo_half;
+  const float *z0;
+  template <int E>
+  __device__ __forceinline__ void row(int r, int c, float (&x)[E]) const {
+    float lo[E];
+    load_elems<__nv_bfloat16, E>(hi + r * kD + c, x);
+    load_elems<__nv_bfloat16, E>(hi + lo_half + r * kD + c, lo);
+#pragma unroll
+    for (int e = 0; e < E; ++e) x[e] = isfinite(x[e]) ? x[e] + lo[e] : x[e];
+  }
+  __device__ __forceinline__ float z(int r) const { return z0[r]; }
+};
+
+// Gated: the rows of `again` (bit i: row row0 + i of the CTA's 256, whose token 0 is chunk index tok0 of chunk `sub` of unit u)
+// once more, by one warp, from the rows that count for them alone: in the tiles a masked row's weight of zero, and a lo
+// weight of zero or of the other sign, meet whatever V holds.
+template <int G>
+__device__ __noinline__ void recompute_rows(const PrefillParams &p, unsigned again, int row0, int u, int sub, int tok0) {
+  using bf16 = __nv_bfloat16;
+  const int ug = u / p.Hkv, g = u - ug * p.Hkv, lrel = ug / p.B, b = ug - lrel * p.B;
+  const LayerDev ld = p.layers[p.layer_begin + lrel];
+  const size_t uc = size_t(u) * p.nsub + sub;
+  for (; again; again &= again - 1) {
+    const int rw = row0 + __ffs(int(again)) - 1, tl = tok0 + rw / G;
+    const size_t token = (size_t(lrel) * p.B + b) * size_t(p.T) + size_t(p.c0 + sub * p.SC + tl);
+    const size_t at = (token * p.H + p.heads_of[g * G + rw % G]) * kD;
+    const RowJob<bf16, kD> job{Rows<bf16, kD>(p, ld, lrel, b, g), reinterpret_cast<const bf16 *>(p.q) + at, reinterpret_cast<bf16 *>(p.out) + at,
+                               p.gcum + uc * p.SC, p.n0 + p.c0 + sub * p.SC, tl, ld.w, ld.wlin, ld.evicts, ld.merge, p.scale_log2};
+    recompute_row(job, SplitState{reinterpret_cast<const bf16 *>(p.s16) + uc * kD * kD, size_t(p.units_cap) * kD * kD, p.zsnap + uc * kD});
+  }
+}
+
 // bit i: column c + i of a key tile is valid for a row whose valid columns are lo .. hi
 __device__ __forceinline__ uint32_t column_mask(int c, int lo, int hi) {
   const int a = lo - c, b = hi - c;
@@ -303,7 +338,7 @@ __device__ __forceinline__ void split2(float x0, float x1, uint32_t &hi, uint32_
 
 template <int G, int MODE>
 __global__ void __launch_bounds__(kThreads, 1)   // 10 warps = 3 on one scheduler: 168 registers per thread at most
-prefill_attn_tc_kernel(const PrefillParams p, const CUtensorMap *ring_maps, const __grid_constant__ CallMaps cm) {
+prefill_attn_tc_kernel(const __grid_constant__ PrefillParams p, const CUtensorMap *ring_maps, const __grid_constant__ CallMaps cm) {
   using bf16 = __nv_bfloat16;
   constexpr bool SUM = MODE == kModeSum;          // sum of two normalised terms instead of the shared normaliser
   constexpr bool PHI2 = MODE == kModeLearned;
@@ -862,10 +897,15 @@ prefill_attn_tc_kernel(const PrefillParams p, const CUtensorMap *ring_maps, cons
       PF_CLK(5);
       if (ok && (windowed || linear)) {
         const float inv = tok_r < ntokX ? 1.0f / l_sum : 0.f;
+        float chk0 = 0.f, chk1 = 0.f;   // gated: sums of the row's values, finite if all of them are
 #pragma unroll 1
         for (int c0 = 0; c0 < kD; c0 += 32) {
           uint32_t r[32];
           tmem_ld32(tO + c0, r);
+          if (GATED) {
+#pragma unroll
+            for (int i = 0; i < 32; i += 2) add2(chk0, chk1, __uint_as_float(r[i]), __uint_as_float(r[i + 1]));
+          }
 #pragma unroll
           for (int q4 = 0; q4 < 4; ++q4) {
             uint32_t pk[4];
@@ -892,6 +932,11 @@ prefill_attn_tc_kernel(const PrefillParams p, const CUtensorMap *ring_maps, cons
             const int head = __shfl_sync(0xffffffffu, my_head, rr - tk * G);
             if (tk < ntokX) *reinterpret_cast<uint4 *>(obase + (size_t(tk) * p.H + head) * kD) = val[i];
           }
+        }
+        if constexpr (GATED) {
+          __syncwarp();
+          const unsigned again = __ballot_sync(0xffffffffu, !isfinite((chk0 + chk1) * inv) && tok_r < ntokX);
+          if (again) recompute_rows<G>(p, again, X * kRows + (row & ~31), u, sub, tok0);
         }
       }
     }

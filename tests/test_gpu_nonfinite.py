@@ -69,3 +69,13 @@ def test_cuda_core_prefill(dtype, d, G, w, gated, calls, bad, value):
 def test_gated_state(w, calls, kw, value):
     _, S = _prompt(BF16, 128, 4, w, True, calls, (50,), value, **kw)
     assert bool((torch.isnan(S) if math.isnan(value) else S == value).all())
+
+
+# bf16, d = 128 with gates runs on the tcgen05 kernel, whose tiles are 128 rows of keys by 128 of queries: windows inside a tile,
+# over several, longer than a chunk and none; window rows from the ring; a chunk that is carried on its own and in a pass
+@pytest.mark.parametrize("value", [float("nan"), float("inf")])
+@pytest.mark.parametrize("G,w,calls,bad,kw", [
+    (4, 40, [300], (150,), {}), (1, 16, [100, 200], (150, 299), {}), (8, 0, [300], (60,), {}), (2, 600, [700], (300, 690), {}),
+    (4, 64, [257], (256,), {}), (2, 120, [160, 60], (170,), dict(prefill_chunk=64)), (4, 300, [700], (200,), dict(prefill_chunk=144))])
+def test_gated_prefill_on_tcgen05(G, w, calls, bad, kw, value):
+    _check(BF16, 128, G, w, True, calls, bad, value, **kw)
