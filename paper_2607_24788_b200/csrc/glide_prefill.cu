@@ -177,7 +177,10 @@ __global__ void __launch_bounds__(kPrefillThreads) prefill_gcum_kernel(const Pre
     }
 #pragma unroll
     for (int a = 0; a < kAhead; ++a) {
+      // a gate of 0 (a saturated sigmoid) counts as half the smallest positive number: what came before decays to 0 in fp32, and
+      // no difference of two sums is inf - inf
       float s = logf(x[a]);
+      if (s < -104.f) s = -104.f;
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
         const float y = __shfl_up_sync(0xffffffffu, s, o);

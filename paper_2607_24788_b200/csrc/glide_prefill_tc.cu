@@ -863,18 +863,19 @@ prefill_attn_tc_kernel(const __grid_constant__ PrefillParams p, const CUtensorMa
               continue;
             }
             tmem_ld32(tS + c, x);
-            if (!whole) {
+            if (!GATED && !whole) {
 #pragma unroll
               for (int i = 0; i < 32; ++i) x[i] = (m >> i) & 1u ? x[i] : 0u;
             }
 #pragma unroll
             for (int e = 0; e < 16; ++e) {
               if constexpr (GATED) {
-                // a delayed token ii <= i has decayed by exp(g_own - gc[ii]) <= 1 (columns past the row's own are zero:
-                // the limit keeps 0 x inf out)
+                // a delayed token ii <= i has decayed by exp(g_own - gc[ii]) <= 1; the others are left out after the product,
+                // whatever it is (their factor is above 1 and may be infinite, or the gate of a later token not a number)
                 const float g0 = __shfl_sync(0xffffffffu, gl, e * 2), g1 = __shfl_sync(0xffffffffu, gl, e * 2 + 1);
-                const float a0 = __uint_as_float(x[e * 2]) * ex2(fminf(g_own - g0, 0.f) * kLog2e);
-                const float a1 = __uint_as_float(x[e * 2 + 1]) * ex2(fminf(g_own - g1, 0.f) * kLog2e);
+                float a0 = __uint_as_float(x[e * 2]) * ex2((g_own - g0) * kLog2e);
+                float a1 = __uint_as_float(x[e * 2 + 1]) * ex2((g_own - g1) * kLog2e);
+                if (!whole) a0 = (m >> (e * 2)) & 1u ? a0 : 0.f, a1 = (m >> (e * 2 + 1)) & 1u ? a1 : 0.f;
                 add2(sum0, sum1, a0, a1);
                 split2(a0, a1, pk[e], x[e]);
               } else {

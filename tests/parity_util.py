@@ -101,9 +101,10 @@ def gates_for(shape, seed: int, lo: float = 0.6, device="cuda") -> torch.Tensor:
 def run_case(windows: Sequence[int], B: int, H: int, Hkv: int, d: int, dtype: torch.dtype, prompt_calls: Sequence[int],
              n_decode: int, amp: float = 1.0, seed: int = 0, q_to_kv: Optional[Sequence[int]] = None,
              max_tokens: Optional[int] = None, check_prefill_outputs: bool = True, state_checks: bool = True,
-             phi: int = 0, gated: bool = False, **cfg_kw):
+             phi: int = 0, gated: bool = False, gate_lo: float = 0.6, zero_gate_every: int = 0, **cfg_kw):
     """prefill (one call per entry of prompt_calls) then n_decode steps on both sides; asserts parity.
-    phi = 1: the learned feature map with seeded projections; gated: seeded gates with every call."""
+    phi = 1: the learned feature map with seeded projections; gated: seeded gates in (gate_lo, 1) with every call, that of every
+    zero_gate_every-th token 0."""
     dev = "cuda"
     L = len(windows)
     total = sum(prompt_calls) + n_decode
@@ -121,12 +122,21 @@ def run_case(windows: Sequence[int], B: int, H: int, Hkv: int, d: int, dtype: to
     stack = orc.Stack(windows, B, H, Hkv, d, scale, q_to_kv=None if q_to_kv is None else np.asarray(q_to_kv, np.int32),
                       merge=cfg_kw.get("merge", 0), phi=phi, wq=None if wq is None else to_np(wq),
                       wk=None if wk is None else to_np(wk))
+    def gates(shape, pos):
+        if not gated:
+            return None
+        x = gates_for(shape, seed * 131 + pos, gate_lo)
+        if zero_gate_every:   # (prefill [L][B][T][H_kv]; a step: [L][B][H_kv])
+            at = torch.arange(pos, pos + (shape[2] if len(shape) == 4 else 1), device=dev) % zero_gate_every == zero_gate_every - 1
+            x = torch.where(at[:, None] if len(shape) == 4 else at, torch.zeros_like(x), x)
+        return x
+
     pos = 0
     worst = 0.0
     for T in prompt_calls:
         q, k, v = wl.qkv(range(L), range(B), range(pos, pos + T), device=dev)
         out = torch.full_like(q, float("nan")) if check_prefill_outputs else None
-        gate = gates_for((L, B, T, Hkv), seed * 131 + pos) if gated else None
+        gate = gates((L, B, T, Hkv), pos)
         if gated:
             g.glide_prefill_gated(q if check_prefill_outputs else None, k, v, gate, out)
         else:
@@ -141,7 +151,7 @@ def run_case(windows: Sequence[int], B: int, H: int, Hkv: int, d: int, dtype: to
     for s in range(n_decode):
         q, k, v = wl.decode_qkv(pos, device=dev)
         out = torch.full_like(q, float("nan"))
-        gate = gates_for((L, B, Hkv), seed * 131 + pos) if gated else None
+        gate = gates((L, B, Hkv), pos)
         if gated:
             g.glide_decode_step_gated(q, k, v, gate, out)
         else:
