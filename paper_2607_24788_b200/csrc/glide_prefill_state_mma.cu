@@ -98,7 +98,7 @@ __device__ __noinline__ float carry_element(const CarryRows &rows, const float *
 // before the chunk is left as bf16 (z: fp32) for the attention kernel, which runs after this one.
 // MAKE_PHI: phi(K') is made here (parameter-free map); otherwise it is in the scratch.
 template <bool PARTIAL, bool MAKE_PHI, bool GATED>
-__global__ void __launch_bounds__(kThreads) prefill_state_mma_kernel(const PrefillParams p) {
+__global__ void __launch_bounds__(kThreads, GATED ? 3 : 0) prefill_state_mma_kernel(const PrefillParams p) {
   using bf16 = __nv_bfloat16;
   // per stage phi columns (or K' rows, 16 bytes more per row) and V' rows; made phi columns
   constexpr int kInBytes = MAKE_PHI ? kVBytes : kPhiBytes;
@@ -229,29 +229,51 @@ __global__ void __launch_bounds__(kThreads) prefill_state_mma_kernel(const Prefi
     }
     const float *sphi = MAKE_PHI ? made : reinterpret_cast<const float *>(stage[buf]);
     const uint32_t sv = smem_addr(stage[buf]) + kInBytes;
-#pragma unroll
-    for (int kk = 0; kk < kTok / 16; ++kk) {
-      // A = phi(K')^T: element (row r, k i) = phi(k'_i)[r]; fragment registers a0: (gid, 2 tig + {0,1}),
-      // a1: (gid + 8, ..), a2: (gid, 2 tig + 8 + {0,1}), a3: (gid + 8, ..)
+    // A = phi(K')^T: element (row r, k i) = phi(k'_i)[r]; fragment registers a0: (gid, 2 tig + {0,1}),
+    // a1: (gid + 8, ..), a2: (gid, 2 tig + 8 + {0,1}), a3: (gid + 8, ..)
+    auto split_a = [&](int kk, uint32_t (&ah)[4], uint32_t (&am)[4], uint32_t (&al)[4]) {
       const float *base = sphi + (kk * 16 + 2 * tig) * kPhiStride + warp * 16 + gid;
-      uint32_t ah[4], am[4], al[4];
       const float *dk = decay[buf] + kk * 16 + 2 * tig;   // (without gates: exact products with 1)
       split3(base[0] * dk[0], base[kPhiStride] * dk[1], ah[0], am[0], al[0]);
       split3(base[8] * dk[0], base[kPhiStride + 8] * dk[1], ah[1], am[1], al[1]);
       split3(base[8 * kPhiStride] * dk[8], base[9 * kPhiStride] * dk[9], ah[2], am[2], al[2]);
       split3(base[8 * kPhiStride + 8] * dk[8], base[9 * kPhiStride + 8] * dk[9], ah[3], am[3], al[3]);
+    };
+    // 16 tokens by 16 columns on top of d0, d1, smallest terms first
+    auto product = [&](int kk, int dp, const uint32_t (&ah)[4], const uint32_t (&am)[4], const uint32_t (&al)[4], float (&d0)[4], float (&d1)[4]) {
       const int krow = kk * 16 + (lane & 7) + ((lane >> 3) & 1) * 8;
+      uint32_t bfr[4];
+      ldsm_x4_trans(bfr, sv + uint32_t(krow * kVStride + (2 * dp + (lane >> 4)) * 16));
+      mma16816(d0, al, bfr[0], bfr[1]);
+      mma16816(d1, al, bfr[2], bfr[3]);
+      mma16816(d0, am, bfr[0], bfr[1]);
+      mma16816(d1, am, bfr[2], bfr[3]);
+      mma16816(d0, ah, bfr[0], bfr[1]);
+      mma16816(d1, ah, bfr[2], bfr[3]);
+    };
+    if constexpr (GATED) {
+      // The tensor core adds without rounding to nearest, and a gated state is held by other kernels to 2e-7 (S after 1000 tokens,
+      // gates of 0.99 to 1, against fp64; this kernel 5.5e-7 with all sums in the tensor core, 1.5e-7 so): only the 32 tokens of
+      // a stage are summed there, on top of zero, and the stages by the CUDA cores.  (Pass of 1000 tokens, 64 units:
+      // 31.5 us -> 34.)
+      uint32_t ah[kTok / 16][4], am[kTok / 16][4], al[kTok / 16][4];
+#pragma unroll
+      for (int kk = 0; kk < kTok / 16; ++kk) split_a(kk, ah[kk], am[kk], al[kk]);
 #pragma unroll
       for (int dp = 0; dp < kD / 16; ++dp) {
-        uint32_t bfr[4];
-        ldsm_x4_trans(bfr, sv + uint32_t(krow * kVStride + (2 * dp + (lane >> 4)) * 16));
-        // smallest terms first
-        mma16816(acc[2 * dp], al, bfr[0], bfr[1]);
-        mma16816(acc[2 * dp + 1], al, bfr[2], bfr[3]);
-        mma16816(acc[2 * dp], am, bfr[0], bfr[1]);
-        mma16816(acc[2 * dp + 1], am, bfr[2], bfr[3]);
-        mma16816(acc[2 * dp], ah, bfr[0], bfr[1]);
-        mma16816(acc[2 * dp + 1], ah, bfr[2], bfr[3]);
+        float part[2][4] = {};
+#pragma unroll
+        for (int kk = 0; kk < kTok / 16; ++kk) product(kk, dp, ah[kk], am[kk], al[kk], part[0], part[1]);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) acc[2 * dp][e] += part[0][e], acc[2 * dp + 1][e] += part[1][e];
+      }
+    } else {
+#pragma unroll
+      for (int kk = 0; kk < kTok / 16; ++kk) {
+        uint32_t ah[4], am[4], al[4];
+        split_a(kk, ah, am, al);
+#pragma unroll
+        for (int dp = 0; dp < kD / 16; ++dp) product(kk, dp, ah, am, al, acc[2 * dp], acc[2 * dp + 1]);
       }
     }
     if (tid < kRowsPerCta) {

@@ -39,3 +39,29 @@ def test_a_gate_that_is_no_number_shows(dtype, d, kw):
         g.glide_destroy()
     assert torch.equal(outs[1][:, :, :190], outs[0][:, :, :190])
     assert bool(torch.isnan(outs[1][:, :, 190:].float()).all())
+
+
+@pytest.mark.parametrize("w,gate_lo", [(64, 0.95), (64, 0.99), (256, 0.999)])
+def test_precision_of_the_tensor_core_prefill(w, gate_lo):
+    """Outputs and state of 1000 tokens, bf16, against the fp64 oracle, by the tcgen05 kernel and by the CUDA cores.
+    Outputs: what is rounded to bf16 differs from the exact value by the split operands' 2^-17 or so (1e-5), which adds
+    (1e-5 / 1.6e-3)^2 / 2 = 2e-5 of it to the rounding's own 1.6e-3.  State: fp32 sums of up to 1000 terms of one sign, three-way
+    splits of 2^-24; one rounding per 32 tokens and per chunk (measured 2e-7; summed up in the tensor core alone 7.6e-7)."""
+    T, H, Hkv, d = 1000, 8, 2, 128
+    gen = torch.Generator().manual_seed(97)
+    q, k, v = (torch.randn((1, 1, T, h, d), generator=gen).to(BF16).cuda() for h in (H, Hkv, Hkv))
+    gate = (gate_lo + (1 - gate_lo) * torch.rand((1, 1, T, Hkv), generator=gen)).cuda()
+    stack = orc.Stack([w], 1, H, Hkv, d, f32_scale(d))
+    ref = stack.prefill(to_np(q), to_np(k), to_np(v), gate=to_np(gate))
+    oS = stack.cells[0][0].export()[2]
+    err = {}
+    for impl in (glide.GLIDE_PREFILL_AUTO, glide.GLIDE_PREFILL_FMA):
+        g = glide.Glide([w], 1, H, Hkv, d, 1 << 20, dtype=BF16, softmax_scale=f32_scale(d), gated=True, prefill_impl=impl)
+        out = torch.zeros_like(q)
+        g.glide_prefill_gated(q, k, v, gate, out)
+        S = to_np(g.glide_export_state(0)[2][0])
+        err[impl] = (np.linalg.norm(to_np(out) - ref) / np.linalg.norm(ref), np.linalg.norm(S - oS) / np.linalg.norm(oS))
+        g.glide_destroy()
+    print(f"w={w} gates {gate_lo}..1: outputs, S: tcgen05 {err[0]}, CUDA cores {err[3]}")
+    assert err[glide.GLIDE_PREFILL_AUTO][0] <= err[glide.GLIDE_PREFILL_FMA][0] * (1 + 2e-5)
+    assert err[glide.GLIDE_PREFILL_AUTO][1] <= 3e-7
