@@ -667,7 +667,9 @@ prefill_attn_tc_kernel(const __grid_constant__ PrefillParams p, const CUtensorMa
       }
       const bool windowed = te > tf;               // O_X holds a valid accumulation
       if (linear) {
-        if (!windowed) mbar_wait(smem_u32(&sm.bar_q[X]), 0u, failed);   // (a window product implies it)
+        // phi(q) is made from the Q tile, which TMA wrote: its own barrier is what shows these threads the copy (it has completed
+        // long ago if there was a window product, but that the MMA warp waited for it does not count here)
+        mbar_wait(smem_u32(&sm.bar_q[X]), 0u, failed);
         // Any common reference M >= m_ref gives the same quotient O / l.  M = max(m_ref, 0) would rescale O for every
         // row whose window maximum is negative; a floor of -64 keeps 2^-M and everything scaled by it far inside the
         // fp32 / bf16 range (phi <= 1) and makes that rescale a rarity.

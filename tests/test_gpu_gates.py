@@ -65,3 +65,22 @@ def test_precision_of_the_tensor_core_prefill(w, gate_lo):
     print(f"w={w} gates {gate_lo}..1: outputs, S: tcgen05 {err[0]}, CUDA cores {err[3]}")
     assert err[glide.GLIDE_PREFILL_AUTO][0] <= err[glide.GLIDE_PREFILL_FMA][0] * (1 + 2e-5)
     assert err[glide.GLIDE_PREFILL_AUTO][1] <= 3e-7
+
+
+# phi(q) is made from the Q tile that TMA wrote (neighbouring heads of a group) or that its own threads copied (heads of a group
+# apart): the same rows either way, so the same bits
+@pytest.mark.parametrize("G,kw", [(2, {}), (4, dict(merge=1)), (4, dict(gated=True)), (8, {})])
+def test_order_of_heads(G, kw):
+    T, Hkv, d, H = 200, 2, 128, 2 * G
+    gen = torch.Generator(device="cuda").manual_seed(101)
+    q, k, v = (torch.randn((1, 1, T, h, d), generator=gen, device="cuda").to(BF16) for h in (H, Hkv, Hkv))
+    apart = [h % Hkv for h in range(H)]                                   # query head h belongs to KV head h % 2
+    order = sorted(range(H), key=lambda h: (apart[h], h))                 # its heads side by side
+    outs = []
+    for heads, q_to_kv in ((order, None), (list(range(H)), apart)):
+        g = glide.Glide([16], 1, H, Hkv, d, 1 << 20, dtype=BF16, q_to_kv=q_to_kv, **kw)
+        out = torch.zeros_like(q)
+        g.glide_prefill(q[:, :, :, heads].contiguous(), k, v, out)
+        outs.append(out)
+        g.glide_destroy()
+    assert torch.equal(outs[0], outs[1][:, :, :, order])
