@@ -83,3 +83,19 @@ def test_decode_by_unit_or_by_list(dtype, L, B, Hkv, G, d, w, kw):
 def test_decode_many_small_units_take_the_work_list(G, d, kw):
     """More units than SMs with several heads of 64: the list, against the oracle; a range of few of its layers: by unit."""
     run_case([16] * 5, 16, 2 * G, 2, d, F32, [20], 2, amp=4 * d ** -0.5, seed=71 + G, max_tokens=40, **kw)
+
+
+# one CTA per unit, for sure: every merge, the learned map, gates, rings of no, one and a few slots and of the longest there
+@pytest.mark.parametrize("dtype,d,G,windows,kw", [
+    (F32, 128, 2, [320, 7], dict(merge=1)), (F32, 64, 4, [192, 0, 1], dict(merge=2)), (F32, 128, 4, [256, 0, 33], dict(phi=1)),
+    (F32, 64, 8, [128, 5], dict(phi=1, merge=1)), (F32, 64, 2, [384, 0], dict(gated=True)), (F32, 128, 8, [64, 0], dict(phi=1, gated=True)),
+    (BF16, 64, 1, [512, 3], dict(merge=1)), (BF16, 128, 4, [40, 0], dict(phi=1, decode_impl=glide.GLIDE_DECODE_FMA))])
+def test_decode_by_unit_every_kind(dtype, d, G, windows, kw):
+    weights = {}
+    if kw.get("phi"):
+        weights = dict(phi_wq=torch.zeros((len(windows), 2 * G, d, d), device="cuda", dtype=dtype),
+                       phi_wk=torch.zeros((len(windows), 2, d, d), device="cuda", dtype=dtype))
+    g = glide.Glide(windows, 2, 2 * G, 2, d, 600, dtype=dtype, **kw, **weights)
+    assert g.glide_decode_launch_info()["work_items"] == len(windows) * 2 * 2
+    g.glide_destroy()
+    run_case(windows, 2, 2 * G, 2, d, dtype, [70], 3, amp=4 * d ** -0.5, seed=103 + G, max_tokens=600, **kw)

@@ -12,6 +12,17 @@ pytestmark = pytest.mark.gpu
 BF16, F32 = torch.bfloat16, torch.float32
 
 
+# Gates of 0.99 to 1: a chunk of 64 to 256 tokens leaves a quarter to three quarters of the state it started from.  The
+# CUDA-core passes with the sums of the chunks before (four chunks) and with a scan (eleven, five), the tcgen05 kernel with
+# passes of one chunk (prefill_chunk 64) and of several, the learned map, decode of a state that has lasted
+@pytest.mark.parametrize("dtype,d,G,calls,kw", [
+    (F32, 64, 1, [256, 30], dict(prefill_chunk=64)), (F32, 64, 2, [700], {}), (F32, 128, 4, [400, 99], dict(prefill_chunk=80)),
+    (BF16, 64, 2, [500], {}), (BF16, 128, 4, [700, 40], {}), (BF16, 128, 2, [300], dict(prefill_chunk=64)), (BF16, 128, 8, [600], dict(prefill_chunk=144)),
+    (BF16, 128, 1, [300, 1, 30], dict(phi=1)), (F32, 64, 1, [130], dict(phi=1, prefill_chunk=32))])
+def test_states_that_last(dtype, d, G, calls, kw):
+    run_case([0, 40, 200], 2, 2 * G, 2, d, dtype, calls, 6, amp=4 * d ** -0.5, seed=79 + G, gated=True, gate_lo=0.99, **kw)
+
+
 # A gate of 0 empties the state.  (Every 200th token: the running sums of log-gates inside a chunk then stay below 210, where
 # two of them differ by at most 2^-17 from what they should: 8e-6 of a weight.)
 @pytest.mark.parametrize("dtype,d,G,calls,kw", [
