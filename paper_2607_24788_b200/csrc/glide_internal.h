@@ -294,7 +294,7 @@ bool prefill_attn_mma_supported(const glide_ctx *ctx);
 int launch_prefill_attn_mma(glide_ctx *ctx, const PrefillParams &p, cudaStream_t stream);
 bool prefill_state_mma_supported(const glide_ctx *ctx);
 // make_phi: phi(K') (parameter-free map) is made by the carry kernel, which leaves its bf16 rows; otherwise it is in p.phik
-int launch_prefill_state_mma(glide_ctx *ctx, const PrefillParams &p, bool make_phi, cudaStream_t stream);
+int launch_prefill_state_mma(const PrefillParams &p, bool make_phi, cudaStream_t stream);
 // up to four ranges of the workspace (8-byte aligned, sizes multiples of 8) set to zero by one launch
 struct ZeroRanges {
   unsigned char *ptr[4];

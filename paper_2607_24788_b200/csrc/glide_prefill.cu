@@ -18,7 +18,7 @@
 #include <algorithm>
 #include <type_traits>
 
-#include "glide_device.cuh"
+#include "glide_prefill_rows.cuh"
 
 namespace glide {
 
@@ -35,43 +35,22 @@ __device__ __forceinline__ void cp_async16(uint32_t dst, const void *src, bool v
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
 
-template <typename T>
-struct RowSource {
-  const T *ringK, *ringV;   // unit base: [cap][D]
-  const T *callK, *callV;   // (layer, sequence) base: [T][Hkv][D], already offset to KV head g
-  int64_t n0, cap;
-  int64_t call_stride;      // Hkv * D
-  __device__ __forceinline__ const T *k(int64_t j, int D) const {
-    return j >= n0 ? callK + (j - n0) * call_stride : ringK + (j % cap) * D;
+// gate of token j (gated contexts): from the call's gates, or from the ring of gates; 1 when the call has none
+struct Gates {
+  const float *ring, *call;   // unit base [cap]; (layer, sequence) base [T][Hkv], already offset to KV head g
+  int64_t n0, stride;         // Hkv
+  uint32_t cap;
+  __device__ __forceinline__ Gates(const PrefillParams &p, const LayerDev &ld, int lrel, int b, int g) {
+    ring = reinterpret_cast<const float *>(p.ws + ld.ringG) + (size_t(b + p.b0) * p.Hkv + g) * size_t(ld.cap);
+    call = p.gate ? p.gate + (size_t(lrel) * p.B + b) * size_t(p.T) * p.Hkv + g : nullptr;
+    n0 = p.n0;
+    stride = p.Hkv;
+    cap = ld.cap > 0 ? uint32_t(ld.cap) : 1u;
   }
-  __device__ __forceinline__ const T *v(int64_t j, int D) const {
-    return j >= n0 ? callV + (j - n0) * call_stride : ringV + (j % cap) * D;
-  }
-  // gate of token j (gated contexts): from the call's gates, or from the ring of gates; 1 when the call has none
-  const float *ringG, *callG;   // unit base [cap]; (layer, sequence) base [T][Hkv], already offset to KV head g
-  int64_t gate_stride;          // Hkv
-  __device__ __forceinline__ float gate(int64_t j) const {
-    return j >= n0 ? (callG ? callG[(j - n0) * gate_stride] : 1.f) : ringG[j % cap];
+  __device__ __forceinline__ float operator()(int64_t j) const {
+    return j >= n0 ? (call ? call[(j - n0) * stride] : 1.f) : ring[uint32_t(j) % cap];
   }
 };
-
-template <typename T, int D>
-__device__ __forceinline__ RowSource<T> make_source(const PrefillParams &p, const LayerDev &ld, int lrel, int b, int g) {
-  RowSource<T> s;
-  const size_t unit_rows = (size_t(b + p.b0) * p.Hkv + g) * size_t(ld.cap);   // b + b0: the sequence's slot in the context
-  s.ringK = reinterpret_cast<const T *>(p.ws + ld.ringK) + unit_rows * D;
-  s.ringV = reinterpret_cast<const T *>(p.ws + ld.ringV) + unit_rows * D;
-  const size_t seq = (size_t(lrel) * p.B + b) * size_t(p.T) * p.Hkv * D + size_t(g) * D;
-  s.callK = reinterpret_cast<const T *>(p.k) + seq;
-  s.callV = reinterpret_cast<const T *>(p.v) + seq;
-  s.n0 = p.n0;
-  s.cap = ld.cap > 0 ? ld.cap : 1;
-  s.call_stride = int64_t(p.Hkv) * D;
-  s.ringG = p.gated ? reinterpret_cast<const float *>(p.ws + ld.ringG) + unit_rows : nullptr;
-  s.callG = p.gate ? p.gate + (size_t(lrel) * p.B + b) * size_t(p.T) * p.Hkv + g : nullptr;
-  s.gate_stride = p.Hkv;
-  return s;
-}
 
 // 1. phi of the delayed keys of this chunk: one warp per (unit, kTokPerWarp consecutive chunk tokens), the rows'
 // loads issued together (with one row per warp the kernel was bound by the latency of its single load)
@@ -91,14 +70,14 @@ __global__ void __launch_bounds__(kPrefillThreads) prefill_phi_kernel(const Pref
   const int lrel = int(u / (int64_t(p.Hkv) * p.B));
   const LayerDev ld = p.layers[p.layer_begin + lrel];
   if (!ld.evicts) return;
-  const RowSource<T> src = make_source<T, D>(p, ld, lrel, b, g);
+  const Rows<T, D> rows(p, ld, lrel, b, g);
   float x[kTokPerWarp][E];
   bool valid[kTokPerWarp];
 #pragma unroll
   for (int r = 0; r < kTokPerWarp; ++r) {
     const int64_t j = p.n0 + p.c0 + i0 + r - ld.wlin;  // delayed token
     valid[r] = i0 + r < p.C && j >= 0;
-    if (valid[r]) load_elems<T, E>(src.k(j, D) + lane * E, x[r]);
+    if (valid[r]) load_elems<T, E>(rows.k(rows.at(j)) + lane * E, x[r]);
   }
   if constexpr (DP == D) {
 #pragma unroll
@@ -132,15 +111,6 @@ __global__ void __launch_bounds__(kPrefillThreads) prefill_phi_kernel(const Pref
         dst[e] = lo[r][e];
         dst[D + e] = hi[r][e];
       }
-      if (p.phik16) {   // the two halves rounded to bf16, each in its own array, for the tensor-core attention kernel
-        __nv_bfloat16 *d16 = reinterpret_cast<__nv_bfloat16 *>(p.phik16) + (size_t(u) * p.Cmax + i0 + r) * D + lane * E;
-        const size_t half = size_t(p.units_cap) * p.Cmax * D;
-#pragma unroll
-        for (int e = 0; e < E; ++e) {
-          d16[e] = __float2bfloat16_rn(lo[r][e]);
-          d16[half + e] = __float2bfloat16_rn(hi[r][e]);
-        }
-      }
     }
   }
 }
@@ -150,7 +120,6 @@ __global__ void __launch_bounds__(kPrefillThreads) prefill_phi_kernel(const Pref
 // delayed token i has entered the state, exp(gcum[i]) the decay of the state the chunk started from.
 // One warp per (unit, chunk), 32 tokens at a time by a warp scan, all of the chunk's gates asked for first (one thread per
 // unit, token after token, took 92 us for 256 tokens of 256 units: a memory round trip and a logarithm each).
-template <typename T, int D>
 __global__ void __launch_bounds__(kPrefillThreads) prefill_gcum_kernel(const PrefillParams p) {
   const int lane = threadIdx.x & 31;
   const int64_t uc = (int64_t(blockIdx.x) * kPrefillThreads + threadIdx.x) >> 5;
@@ -163,7 +132,7 @@ __global__ void __launch_bounds__(kPrefillThreads) prefill_gcum_kernel(const Pre
   const int lrel = int(u / (int64_t(p.Hkv) * p.B));
   const LayerDev ld = p.layers[p.layer_begin + lrel];
   if (!ld.evicts) return;
-  const RowSource<T> src = make_source<T, D>(p, ld, lrel, b, g);
+  const Gates gate(p, ld, lrel, b, g);
   const int64_t first = p.n0 + p.c0 + chunk_c0 - ld.wlin;   // delayed token of chunk index 0
   float *out = p.gcum + size_t(u) * p.Cmax + chunk_c0;
   constexpr int kAhead = 8;
@@ -173,7 +142,7 @@ __global__ void __launch_bounds__(kPrefillThreads) prefill_gcum_kernel(const Pre
 #pragma unroll
     for (int a = 0; a < kAhead; ++a) {
       const int i = i0 + a * 32 + lane;
-      x[a] = i < chunk_n && first + i >= 0 ? src.gate(first + i) : 1.f;
+      x[a] = i < chunk_n && first + i >= 0 ? gate(first + i) : 1.f;
     }
 #pragma unroll
     for (int a = 0; a < kAhead; ++a) {
@@ -211,7 +180,7 @@ __global__ void __launch_bounds__(kPrefillThreads) prefill_attn_kernel(const Pre
   const int b = int((u / p.Hkv) % p.B);
   const int lrel = int(u / (int64_t(p.Hkv) * p.B));
   const LayerDev ld = p.layers[p.layer_begin + lrel];
-  const RowSource<T> src = make_source<T, D>(p, ld, lrel, b, g);
+  const Rows<T, D> rows(p, ld, lrel, b, g);
   const int64_t tq = p.n0 + p.c0 + i;  // absolute position of the query
   const int ub = (b + p.b0) * p.Hkv + g;
 
@@ -259,11 +228,13 @@ __global__ void __launch_bounds__(kPrefillThreads) prefill_attn_kernel(const Pre
   for (int64_t j = w_lo; j <= tq; j += 2) {
     float kx[2][E], vx[2][E];
     const bool two = j + 1 <= tq;
-    load_elems<T, E>(src.k(j, D) + lane * E, kx[0]);
-    load_elems<T, E>(src.v(j, D) + lane * E, vx[0]);
+    const int64_t off = rows.at(j);
+    load_elems<T, E>(rows.k(off) + lane * E, kx[0]);
+    load_elems<T, E>(rows.v(off) + lane * E, vx[0]);
     if (two) {
-      load_elems<T, E>(src.k(j + 1, D) + lane * E, kx[1]);
-      load_elems<T, E>(src.v(j + 1, D) + lane * E, vx[1]);
+      const int64_t next = rows.at(j + 1);
+      load_elems<T, E>(rows.k(next) + lane * E, kx[1]);
+      load_elems<T, E>(rows.v(next) + lane * E, vx[1]);
     }
     online_row<E, G>(qr, kx[0], vx[0], m, l, acc);
     if (two) online_row<E, G>(qr, kx[1], vx[1], m, l, acc);
@@ -318,7 +289,7 @@ __global__ void __launch_bounds__(kPrefillThreads) prefill_attn_kernel(const Pre
       float fk[NH][E], vx[E];
 #pragma unroll
       for (int nh = 0; nh < NH; ++nh) load_elems<float, E>(pk + size_t(ii) * DP + nh * D + lane * E, fk[nh]);
-      load_elems<T, E>(src.v(j, D) + lane * E, vx);
+      load_elems<T, E>(rows.v(rows.at(j)) + lane * E, vx);
       const float dec = gc ? expf(g_own - gc[ii]) : 1.f;
 #pragma unroll
       for (int h = 0; h < G; ++h) {
@@ -398,7 +369,7 @@ __global__ void __launch_bounds__(kPrefillThreads) prefill_state_kernel(const Pr
   const int64_t first = p.n0 + p.c0 - ld.wlin;    // delayed token of chunk index 0
   const int i_lo = first < 0 ? int(first < -int64_t(p.C) ? p.C : -first) : 0;
   if (i_lo >= p.C) return;
-  const RowSource<T> src = make_source<T, D>(p, ld, lrel, b, g);
+  const Rows<T, D> rows(p, ld, lrel, b, g);
   const int ub = (b + p.b0) * p.Hkv + g;
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
   const float *pk = p.phik + size_t(u) * p.Cmax * dp + rb * kStateRows;
@@ -420,7 +391,7 @@ __global__ void __launch_bounds__(kPrefillThreads) prefill_state_kernel(const Pr
     }
     for (int e = tid; e < kStateTok * kVChunks; e += kPrefillThreads) {
       const int i = e / kVChunks, c = e % kVChunks;
-      const unsigned char *row = reinterpret_cast<const unsigned char *>(src.v(first + i0 + (i < nt ? i : 0), D));
+      const unsigned char *row = reinterpret_cast<const unsigned char *>(rows.v(rows.at(first + i0 + (i < nt ? i : 0))));
       cp_async16(sv + uint32_t(i * kVChunks + c) * 16u, row + c * 16, i < nt);
     }
     cp_async_commit();
@@ -704,11 +675,11 @@ int launch_prefill(glide_ctx *ctx, int layer_begin, int layer_count, int64_t T, 
           prefill_phi_kernel<TT, D, DP><<<warp4_blocks, kPrefillThreads, 0, stream>>>(s);
         }
         if (p.gated)
-          prefill_gcum_kernel<TT, D><<<unsigned((units * s.nsub * 32 + kPrefillThreads - 1) / kPrefillThreads), kPrefillThreads, 0, stream>>>(s);
+          prefill_gcum_kernel<<<unsigned((units * s.nsub * 32 + kPrefillThreads - 1) / kPrefillThreads), kPrefillThreads, 0, stream>>>(s);
         if (out && s.phiq16 && launch_prefill_project(ctx, s, false, stream) != GLIDE_OK) return GLIDE_ERR_CUDA;
         if (out && p.merge != GLIDE_MERGE_SHARED)   // (before the carry: the chunk sums overwrite rows of phi(K'))
           prefill_zcum_kernel<D><<<unsigned((units * s.nsub * D + kPrefillThreads - 1) / kPrefillThreads), kPrefillThreads, 0, stream>>>(s);
-        if (launch_prefill_state_mma(ctx, s, make_phi, stream) != GLIDE_OK) return GLIDE_ERR_CUDA;
+        if (launch_prefill_state_mma(s, make_phi, stream) != GLIDE_OK) return GLIDE_ERR_CUDA;
       }
       if (out && launch_prefill_attn_tc(ctx, s, stream) != GLIDE_OK) return GLIDE_ERR_CUDA;
       prefill_ring_kernel<TT, D><<<warp4_blocks, kPrefillThreads, 0, stream>>>(s);
@@ -726,11 +697,8 @@ int launch_prefill(glide_ctx *ctx, int layer_begin, int layer_count, int64_t T, 
     return for_passes(slots, most, ctx->cfg.head_dim, ctx->elem, [&](const PrefillParams &s) -> int {
       if (p.gated && evicts_in(s.layer_begin, s.layer_count)) {
         const unsigned blocks = unsigned((int64_t(s.layer_count) * units_layer * s.nsub * 32 + kPrefillThreads - 1) / kPrefillThreads);
-        const int rc = dispatch_config(ctx->cfg.io_dtype, ctx->cfg.head_dim, 1, [&](auto tt, auto dd, auto) -> int {
-          prefill_gcum_kernel<typename decltype(tt)::type, decltype(dd)::value><<<blocks, kPrefillThreads, 0, stream>>>(s);
-          return cudaGetLastError() == cudaSuccess ? GLIDE_OK : GLIDE_ERR_CUDA;
-        });
-        if (rc) return rc;
+        prefill_gcum_kernel<<<blocks, kPrefillThreads, 0, stream>>>(s);
+        if (cudaGetLastError() != cudaSuccess) return GLIDE_ERR_CUDA;
       }
       return launch_prefill_fma(ctx, s, stream);
     });
@@ -754,7 +722,7 @@ int launch_prefill(glide_ctx *ctx, int layer_begin, int layer_count, int64_t T, 
         prefill_phi_kernel<TT, D, DP><<<warp4_blocks, kPrefillThreads, 0, stream>>>(p);
       }
       if (any_evicts && p.gated)
-        prefill_gcum_kernel<TT, D><<<unsigned((units * 32 + kPrefillThreads - 1) / kPrefillThreads), kPrefillThreads, 0, stream>>>(p);
+        prefill_gcum_kernel<<<unsigned((units * 32 + kPrefillThreads - 1) / kPrefillThreads), kPrefillThreads, 0, stream>>>(p);
       if (out) {
         if (use_mma) {
           if (launch_prefill_attn_mma(ctx, p, stream) != GLIDE_OK) return GLIDE_ERR_CUDA;
@@ -763,8 +731,8 @@ int launch_prefill(glide_ctx *ctx, int layer_begin, int layer_count, int64_t T, 
         }
       }
       if (any_evicts) {
-        if (state_mma) {
-          if (launch_prefill_state_mma(ctx, p, false, stream) != GLIDE_OK) return GLIDE_ERR_CUDA;
+        if (DP == D || state_mma) {   // (the parameter-free map comes here for bf16 and d = 128 alone)
+          if (launch_prefill_state_mma(p, false, stream) != GLIDE_OK) return GLIDE_ERR_CUDA;
         } else {
           prefill_state_kernel<TT, D><<<unsigned(units * (DP / kStateRows)), kPrefillThreads, 0, stream>>>(p);
         }
@@ -778,8 +746,10 @@ int launch_prefill(glide_ctx *ctx, int layer_begin, int layer_count, int64_t T, 
     constexpr int D = decltype(dd)::value;
     if constexpr (D == 128 && std::is_same<typename decltype(tt)::type, __nv_bfloat16>::value)
       if (passes) return ctx->dp == D ? run_passes(tt, dd, IntTag<D>{}) : run_passes(tt, dd, IntTag<2 * D>{});
-    if (ctx->dp == D) return run_chunks(tt, dd, gg, IntTag<D>{});
-    return run_chunks(tt, dd, gg, IntTag<2 * D>{});
+    if (ctx->dp != D) return run_chunks(tt, dd, gg, IntTag<2 * D>{});
+    // (fp32 and d = 64 with the parameter-free map are the CUDA-core passes')
+    if constexpr (D == 128 && std::is_same<typename decltype(tt)::type, __nv_bfloat16>::value) return run_chunks(tt, dd, gg, IntTag<D>{});
+    else return GLIDE_ERR_UNSUPPORTED;
   });
   return rc;
 }

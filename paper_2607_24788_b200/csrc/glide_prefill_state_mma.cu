@@ -422,8 +422,7 @@ bool prefill_state_mma_supported(const glide_ctx *ctx) {
   return ctx->cfg.io_dtype == GLIDE_BF16 && ctx->cfg.head_dim == kD;
 }
 
-int launch_prefill_state_mma(glide_ctx *ctx, const PrefillParams &p, bool make_phi, cudaStream_t stream) {
-  (void)ctx;
+int launch_prefill_state_mma(const PrefillParams &p, bool make_phi, cudaStream_t stream) {
   const int64_t units = int64_t(p.layer_count) * p.B * p.Hkv;
   const unsigned blocks = unsigned(units * p.nsub * (p.dp / kRowsPerCta));
   auto run = [&](auto partial, auto make, auto gated) {
