@@ -15,6 +15,10 @@
  * attention.  Prefill over T tokens leaves the same state and outputs as T decode steps.
  *
  * Conventions for every call
+ *   - Values.  An infinity or a NaN in a prompt's V reaches the outputs of the tokens that see it and no others on the
+ *     CUDA-core prefill kernels and in gated contexts.  The ungated tensor-core prefill kernels multiply the masked rows of
+ *     a tile of keys by zero: there it makes the outputs of earlier tokens of the same tile NaN as well, so rows that
+ *     are only padding must hold finite values.  Gates lie in [0, 1].
  *   - All pointers named dev_* or documented "device" are device pointers on the
  *     CUDA device that was current at glide_create; "host" pointers are ordinary
  *     host memory.  Device buffers must be contiguous and 16-byte aligned.
@@ -114,15 +118,16 @@ typedef struct {
                               sized for one chunk of every unit.  0: 256, or what suits the call on the CUDA-core prefill
                               kernels with the parameter-free map (64 to 256 in a scratch sized for 256; the order of the
                               fp32 sums then depends on the call's length and on how many sequences it holds) */
-  int32_t decode_chunk;    /* window slots per split-K work item of the decode kernel; 0 selects automatically */
-  int32_t decode_state_splits; /* row blocks the S update/readout of one KV head is split into; 0 selects automatically */
+  int32_t decode_chunk;    /* window slots per split-K work item of the per-item decode kernels; 0 selects automatically (on
+                              the CUDA cores also one thread block per unit, where rings are short) */
+  int32_t decode_state_splits; /* row blocks the S update/readout of one KV head is split into there; 0 selects automatically */
   int32_t decode_impl;     /* glide_decode_impl */
   int32_t prefill_impl;    /* glide_prefill_impl */
   const void *phi_wq;      /* GLIDE_PHI_PROJ_SOFTMAX2: device [n_layers][n_q_heads][d][d] in the I/O dtype, row i column j
                               = W[i][j]; borrowed, must stay alive and unchanged until glide_destroy.  Else NULL. */
   const void *phi_wk;      /* likewise [n_layers][n_kv_heads][d][d] for the keys */
   int32_t gated;           /* 1: gated recurrence (Sec. III-B "GLA-style gating mechanisms"; the paper gives no formula,
-                              the library's reading): every token brings a decay gamma in (0, 1] per KV head, which
+                              the library's reading): every token brings a decay gamma in [0, 1] per KV head, which
                               waits in the ring with its key and value, and the state decays by the gate of the token
                               that enters it: S <- gamma S + phi(k) v^T, z <- gamma z + phi(k).  Gates are passed to
                               glide_prefill_gated / glide_decode_step_gated; the calls without gates use gamma = 1.
@@ -181,7 +186,7 @@ int glide_decode_step(glide_ctx *ctx, const void *dev_q, const void *dev_k, cons
                       void *stream);
 
 /* glide_prefill and glide_decode_step of a context created with gated = 1 (GLIDE_ERR_INVALID_ARG otherwise), with
- * the tokens' gates: dev_gate fp32 [layer_count][B][T][H_kv] (prefill) or [L][B][H_kv] (decode), each in (0, 1];
+ * the tokens' gates: dev_gate fp32 [layer_count][B][T][H_kv] (prefill) or [L][B][H_kv] (decode), each in [0, 1];
  * NULL stands for gates of 1.  The gate of a token decays the state at the step the token enters it (Sec. III-B
  * "GLA-style gating mechanisms", see glide_config.gated). */
 int glide_prefill_gated(glide_ctx *ctx, int32_t layer_begin, int32_t layer_count, int64_t T, const void *dev_q,

@@ -162,8 +162,8 @@ struct PrefillParams {
   void *s16;                 // tcgen05 kernel: bf16 copy of every unit's S as it is at the start of every chunk of the pass,
                              // [halves][units_cap][d][d], index (unit of the pass * nsub + chunk)
   float *zsnap;              // tcgen05 kernel: z at the start of every chunk of the pass, [units_cap][dp], the same index;
-                             // CUDA-core passes: every chunk's sum of phi(K') (their S sums, [unit * nsub + chunk][d][d], are
-                             // in phik)
+                             // CUDA-core passes: every chunk's sum of phi(K') or, after a scan, z at its start (their S sums or
+                             // states, [unit * nsub + chunk][d][d], are in phik)
   void *phiq16;              // tcgen05 kernel, learned map: phi(q) of the chunk's query rows as bf16,
                              // [2 halves][units_cap * SC * G][d], row = (unit * Cmax + token) * G + head of the group
   int64_t units_cap;         // L * B * H_kv of the context: what separates the halves in the three arrays above
@@ -174,10 +174,10 @@ struct PrefillParams {
   int64_t n0;                // tokens absorbed before this call (all layers of the call)
   int64_t T;                 // tokens of this call
   // A pass takes C tokens from call-relative token c0 on, in nsub chunks of SC tokens (the last one may be shorter).  The
-  // CUDA-core and mma.sync attention kernels work on passes of one chunk.
+  // mma.sync attention kernel and prefill_attn_kernel work on passes of one chunk.
   int64_t c0;
   int32_t C;
-  int32_t SC;                // tokens of a chunk (prefill_chunk)
+  int32_t SC;                // tokens of a chunk (prefill_chunk; the CUDA-core passes choose it where the caller did not)
   int32_t nsub;              // chunks of the pass
   int32_t Cmax;              // scratch rows per unit: nsub * SC
   int32_t layer_begin, layer_count;

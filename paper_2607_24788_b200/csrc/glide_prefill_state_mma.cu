@@ -7,7 +7,7 @@
 // 2 C d^2 multiply-adds per KV head leave the CUDA cores (a bf16 or tf32 product of phi(K') itself would miss the
 // 1e-5 state tolerance).  z is summed in fp32 on the CUDA cores from the same staged values.
 //
-// One CTA of 4 warps per (unit, 64 state rows); warp w owns rows 16 w .. 16 w + 15 and all 128 columns
+// One CTA of 4 warps per (unit, chunk of the pass, 64 state rows); warp w owns rows 16 w .. 16 w + 15 and all 128 columns
 // (16 n-tiles of m16n8k16, 64 accumulators per thread).  Tokens are staged 32 at a time through two shared-memory
 // buffers filled by cp.async; row strides are padded (272 bytes) so that the scalar reads of the A fragments and
 // the ldmatrix reads of V' are free of bank conflicts.  With the parameter-free map the kernel makes phi(K') itself from the
