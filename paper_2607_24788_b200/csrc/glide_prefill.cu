@@ -626,9 +626,20 @@ int launch_prefill(glide_ctx *ctx, int layer_begin, int layer_count, int64_t T, 
   // their units, `slots` (unit, chunk) pairs at most (what the scratch holds).
   const int64_t units_layer = int64_t(p.B) * p.Hkv;
   auto for_passes = [&](int64_t slots, int64_t most, int D, size_t elem, auto &&run) -> int {
-    const int nsub_max = int(std::min<int64_t>(most, (T + p.SC - 1) / p.SC));
-    const int fit = int(std::min<int64_t>(layer_count, slots / (units_layer * nsub_max)));
-    const int n_groups = (layer_count + fit - 1) / fit;
+    const int64_t chunks = (T + p.SC - 1) / p.SC;
+    int nsub_max = int(std::min<int64_t>(most, chunks));
+    int fit = nsub_max == 1 ? layer_count : int(std::min<int64_t>(layer_count, slots / (units_layer * nsub_max)));
+    int n_groups = (layer_count + fit - 1) / fit;
+    // One chunk of all layers after the other where that is no more passes and either nothing needs many chunks at a time (no
+    // outputs: the sums go to S directly) or the call is short (two chunks: a pass takes as long as its longest chunk,
+    // and the second one is mostly shorter; with longer windows and calls the layers' attention fills the chip better
+    // with all chunks there); and where slots for few layers would make many more passes (a small prefill_chunk).
+    const int64_t passes = (chunks + nsub_max - 1) / nsub_max * n_groups;
+    if (passes > 2 * chunks || (passes >= chunks && (!out || chunks <= 2))) {
+      nsub_max = 1;
+      fit = layer_count;
+      n_groups = 1;
+    }
     for (int64_t c0 = 0; c0 < T; c0 += int64_t(nsub_max) * p.SC) {
       for (int gi = 0; gi < n_groups; ++gi) {
         const int l0 = int(int64_t(layer_count) * gi / n_groups), l1 = int(int64_t(layer_count) * (gi + 1) / n_groups);

@@ -7,6 +7,7 @@
 //                                  the chunk's start, the scan's or S + the sums of the chunks before it; out
 //   3.  prefill_fma_finish_kernel  S and z move on by the pass if no scan did it, the pass's newest tokens go to the ring,
 //                                  counters advance
+// A pass of one chunk needs no room for sums: 1 comes after 2 and adds to S and z in place.
 // Gated: the running log-gates of the chunks' delayed tokens (gcum) come from a kernel in front; without gates every decay
 // is an exact 1, so that a gated context driven without gates keeps the bits of a plain one.
 // The kernels read K and V rows where they are (ring for tokens older than the call) and make phi in registers; the ring
@@ -93,7 +94,8 @@ __device__ __forceinline__ float chunk_decay(const PrefillParams &p, int64_t u, 
 // are made from K' as they are loaded (all of them in every CTA of a unit: cheaper than a launch in front and a trip
 // through memory), the CTA keeps its 16 columns of them.
 constexpr int kSumTok = 32;    // tokens per tile
-template <typename T, int D>
+// IN_PLACE (passes of one chunk): behind the attention kernel, on top of S and z, so that such passes need no scratch.
+template <typename T, int D, bool IN_PLACE>
 __global__ void __launch_bounds__(2 * kThreads) prefill_fma_sums_kernel(const PrefillParams p) {
   constexpr int LD = kSumTok * D / 4 / kThreads;   // float4 per thread and tile
   constexpr int CG = D / 64;                       // groups of four columns per thread
@@ -184,13 +186,24 @@ __global__ void __launch_bounds__(2 * kThreads) prefill_fma_sums_kernel(const Pr
 #pragma unroll
     for (int c = 0; c < 4 * CG; ++c) acc[r][c] += other[r * kThreads + tid][c];
   if (tid < 16) zacc += ph[1][0][tid];
-  float *dst = p.phik + (size_t(uc) * D + rb * 16 + row) * D + cg * 4;
+  const size_t ub = size_t(id.b + p.b0) * p.Hkv + id.g;
+  float *dst = (IN_PLACE ? reinterpret_cast<float *>(p.ws + ld.S) + ub * D * D : p.phik + size_t(uc) * D * D) + (rb * 16 + row) * D + cg * 4;
+  const float dec = IN_PLACE ? chunk_decay(p, id.u, 0) : 1.f;
 #pragma unroll
   for (int r = 0; r < 2; ++r)
 #pragma unroll
-    for (int q = 0; q < CG; ++q)
-      *reinterpret_cast<float4 *>(dst + r * D + q * 64) = make_float4(acc[r][q * 4], acc[r][q * 4 + 1], acc[r][q * 4 + 2], acc[r][q * 4 + 3]);
-  if (tid < 16) p.zsnap[size_t(uc) * D + rb * 16 + tid] = zacc;
+    for (int q = 0; q < CG; ++q) {
+      float4 x = make_float4(acc[r][q * 4], acc[r][q * 4 + 1], acc[r][q * 4 + 2], acc[r][q * 4 + 3]);
+      if (IN_PLACE) {
+        const float4 s = load4(dst + r * D + q * 64);
+        x = make_float4(fmaf(s.x, dec, x.x), fmaf(s.y, dec, x.y), fmaf(s.z, dec, x.z), fmaf(s.w, dec, x.w));
+      }
+      store4(dst + r * D + q * 64, x);
+    }
+  if (tid < 16) {
+    float *z = (IN_PLACE ? reinterpret_cast<float *>(p.ws + ld.z) + ub * D : p.zsnap + size_t(uc) * D) + rb * 16 + tid;
+    *z = IN_PLACE ? fmaf(*z, dec, zacc) : zacc;
+  }
 }
 
 // 2. Tiles of KT rows: group 0 takes the window's keys, group 1 the chunk's delayed tokens and the rows of the state; group
@@ -580,8 +593,9 @@ int launch_prefill_fma(glide_ctx *ctx, const PrefillParams &p, cudaStream_t stre
     using T = typename decltype(tt)::type;
     constexpr int D = decltype(dd)::value, G = decltype(gg)::value, TOK = kRows / G;
     const unsigned state_ctas = any_evicts ? unsigned(units * (D * D / 4 / kThreads)) : 0u;
-    const bool scan = any_evicts && p.nsub > kDirectChunks<D>;
-    if (any_evicts) prefill_fma_sums_kernel<T, D><<<unsigned(units * p.nsub * (D / 16)), 2 * kThreads, 0, stream>>>(p);
+    const bool in_place = p.nsub == 1, scan = any_evicts && p.nsub > kDirectChunks<D>;
+    const unsigned sum_ctas = unsigned(units * p.nsub * (D / 16));
+    if (any_evicts && !in_place) prefill_fma_sums_kernel<T, D, false><<<sum_ctas, 2 * kThreads, 0, stream>>>(p);
     if (scan) prefill_fma_scan_kernel<D><<<state_ctas, kThreads, 0, stream>>>(p);
     if (p.out) {
       auto kern = prefill_fma_attn_kernel<T, D, G>;
@@ -592,7 +606,8 @@ int launch_prefill_fma(glide_ctx *ctx, const PrefillParams &p, cudaStream_t stre
       const int64_t blocks = units * (int64_t(p.nsub - 1) * ((p.SC + TOK - 1) / TOK) + (p.C - (p.nsub - 1) * p.SC + TOK - 1) / TOK);
       kern<<<unsigned(blocks), 2 * kThreads, sizeof(AttnSmem<D>), stream>>>(p);
     }
-    const unsigned state_blocks = scan ? 0u : state_ctas;
+    if (any_evicts && in_place) prefill_fma_sums_kernel<T, D, true><<<sum_ctas, 2 * kThreads, 0, stream>>>(p);
+    const unsigned state_blocks = scan || in_place ? 0u : state_ctas;
     const unsigned ring_blocks = unsigned((units * p.C * (D / 4) + kThreads - 1) / kThreads);
     prefill_fma_finish_kernel<T, D><<<state_blocks + ring_blocks, kThreads, 0, stream>>>(p, state_blocks);
     return cudaGetLastError() == cudaSuccess ? GLIDE_OK : GLIDE_ERR_CUDA;

@@ -54,3 +54,28 @@ def test_decode_by_unit(dtype, d, G, windows, kw):
     (BF16, 64, 2, 0, [650], True)])
 def test_cuda_core_passes_with_a_scan(dtype, d, G, chunk, calls, gated):
     run_case([0, 64, 300, 630], 2, 2 * G, 2, d, dtype, calls, 2, amp=4 * d ** -0.5, seed=73 + G, gated=gated, prefill_chunk=chunk)
+
+
+# The same prompt with outputs (many chunks of few layers, their sums scanned) and without (one chunk of all layers after the other,
+# sums straight to S), in one call and in calls of two chunks: the same additions, so the same bits.  (Not so for the sum-of-terms
+# merges in bf16, whose phi comes from another kernel when there are outputs.)
+@pytest.mark.parametrize("dtype,d,kw", [
+    (BF16, 128, dict(prefill_chunk=256)), (BF16, 128, dict(prefill_chunk=144, gated=True)),
+    (torch.float32, 64, dict(prefill_chunk=32)), (torch.float32, 128, dict(prefill_chunk=16, merge=2))])
+def test_passes_leave_the_same_state(dtype, d, kw):
+    chunk, L = kw["prefill_chunk"], 5
+    T = 4 * chunk + 9
+    gen = torch.Generator(device="cuda").manual_seed(107)
+    q, k, v = (torch.randn((L, 1, T, h, d), generator=gen, device="cuda").to(dtype) for h in (4, 2, 2))
+    states = []
+    for with_outputs, step in ((True, T), (False, T), (True, 2 * chunk)):
+        g = glide.Glide([0, 16, 100, 300, 1 << 20], 1, 4, 2, d, 1 << 20, dtype=dtype, **kw)
+        for c in range(0, T, step):
+            part = [x[:, :, c:c + step].contiguous() for x in (q, k, v)]
+            g.glide_prefill(part[0] if with_outputs else None, part[1], part[2], torch.empty_like(part[0]) if with_outputs else None)
+        states.append([x.clone() for l in range(4) for x in g.glide_export_state(l)])
+        assert g.glide_device_status() == 0
+        g.glide_destroy()
+    for other in states[1:]:
+        for a, b in zip(states[0], other):
+            assert torch.equal(a, b)
