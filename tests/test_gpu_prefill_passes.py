@@ -73,7 +73,8 @@ def test_passes_leave_the_same_state(dtype, d, kw):
         for c in range(0, T, step):
             part = [x[:, :, c:c + step].contiguous() for x in (q, k, v)]
             g.glide_prefill(part[0] if with_outputs else None, part[1], part[2], torch.empty_like(part[0]) if with_outputs else None)
-        states.append([x.clone() for l in range(4) for x in g.glide_export_state(l)])
+        # (slots that no token has reached hold whatever the workspace held: a ring longer than the prompt is compared up to T)
+        states.append([x[:, :, :T].clone() if i < 2 else x.clone() for l in range(4) for i, x in enumerate(g.glide_export_state(l))])
         assert g.glide_device_status() == 0
         g.glide_destroy()
     for other in states[1:]:
