@@ -1,18 +1,20 @@
 // GLIDE prefill outputs on the 5th-generation tensor cores (tcgen05 + TMEM + TMA), bf16 I/O, head_dim 128.
 //
-// One CTA (10 warps) owns 256 query rows of one (layer, sequence, KV head) unit: two row tiles X = A, B of 128
+// One CTA (19 warps) owns 256 query rows of one (layer, sequence, KV head) unit: two row tiles X = A, B of 128
 // rows each, a row being (token, query head of the group), row = token * G + head.
-//   warps 0-3   softmax of tile A: thread r owns row r = TMEM lane r
-//   warps 4-7   softmax of tile B
-//   warp 8      issues every tcgen05.mma (one elected lane)
-//   warp 9      loads every operand (TMA; row by row where a 16-token group straddles two sources); Q of heads that do not lie
+//   warps 0-3, 8-11    softmax of tile A: two threads per row (TMEM lane), 64 columns each
+//   warps 4-7, 12-15   softmax of tile B
+//   warps 16, 17       issue the tcgen05.mma of A and of B (one elected lane), in turns.  Between two products a warp spends some 1000
+//               cycles on waits, votes and commits, and the tensor core's queue is short: with one warp for both it idled half of
+//               the time
+//   warp 18     loads every operand (TMA; row by row where a 16-token group straddles two sources); Q of heads that do not lie
 //               side by side is copied by the softmax threads
 // Window part, per 128-key tile t (keys are tokens j0 + 0..127, j0 a multiple of 16):
 //   loader    K_t and V_t (ring rows for tokens older than the call, the call's rows otherwise) into a ring of five
 //             32 KiB buffers (kStages), 128-byte swizzle, completion on an mbarrier
 //   MMA       S_X = Q_X K_t^T into TMEM (8 x m128n128k16), committed to an mbarrier the softmax warps wait on
-//   softmax   tcgen05.ld of the own row, mask, row maximum without any shuffle, P = 2^(s - m_ref) as bf16 over the
-//             consumed S columns; the reference m_ref is lazy: O is rescaled in TMEM only when the maximum grows by
+//   softmax   tcgen05.ld of the own half row, mask, row maximum (the other half's by a barrier of two warps, and only when it
+//             grows), P = 2^(s - m_ref) as bf16 over the consumed S columns; the reference m_ref is lazy: O is rescaled in TMEM only when the maximum grows by
 //             more than 2^8
 //   MMA       O_X += P_X V_t (V as the MN-major B operand), then S_X of the next tile: while one row tile is
 //             in its softmax the tensor core works for the other
@@ -20,8 +22,11 @@
 // Linear part (after the window tiles, by the same warps in the same way): with a common reference M = max(m_ref, -64)
 // per row, phi(Q) 2^-M as bf16 times a bf16 copy of the state (inter-chunk), and C = phi(Q) phi(K')^T masked to
 // j' <= i, then C V' (intra-chunk); l accumulates the matching sums.  out = O / l.
-// What bounds it: short windows, the fixed chain of a CTA (Q and K_0 from memory, one softmax, phi, two to three more
-// products, the store); long windows, the softmax threads' exponentials beside the tensor pipe.
+// What bounds it: short windows, the fixed chain of a CTA (24500 cycles: 6800 until Q and K_0 are there and the first product is
+// done, one softmax 3500, phi 2900, two to three more products 8500, the store 2500); long windows, per key tile and row tile the
+// chain softmax (1850) -> P V and the next S (1050 to 1300) -> signals, 3650 cycles in which the two row tiles' products take
+// 2048.  8 layers of 2048 tokens, 32 / 8 heads, windows of 64 / 256 / 1024: 270 / 333 / 525 us; with one softmax thread per row,
+// one MMA warp and phi in one piece 292 / 379 / 576.
 // Every mbarrier wait is bounded; on a time-out the CTA records kDevWaitTimeout, leaves its loops, frees its TMEM
 // columns and returns.
 #include <cuda.h>
@@ -39,9 +44,10 @@ constexpr int kD = 128;
 constexpr int kRows = 128;            // rows per row tile
 constexpr int kKT = 128;              // keys per tile
 constexpr int kGroup = 16;            // tokens per TMA box
-constexpr int kSoftmaxThreads = 256;
-constexpr int kThreads = 320;
-constexpr int kMmaWarp = 8, kLoadWarp = 9;
+constexpr int kHalf = kD / 2;         // columns of a softmax thread: two threads per row
+constexpr int kSoftmaxThreads = 512;
+constexpr int kThreads = 608;
+constexpr int kMmaWarp = 16, kLoadWarp = 18;   // (MMA warps: one per row tile)
 constexpr uint32_t kTileBytes = 32768;   // [2 boxes][128 rows][64 bf16]
 constexpr uint32_t kBoxBytes = 16384;
 constexpr uint32_t kGroupBytes = kGroup * 128;   // one 16-token box of 64 columns
@@ -103,7 +109,8 @@ __device__ __forceinline__ void issue_mma(bool leader, uint32_t tmem_d, uint32_t
   }
 }
 // the same product with the A operand in TMEM: lane = row, 32-bit column c = elements 2c (low half) and 2c+1 of
-// the row, 8 columns per k16 step (PAIRS: two steps, then a gap of 16 columns); B MN-major in shared memory
+// the row, 8 columns per k16 step, elements 64 .. 127 from column 64 on (PAIRS: two steps, then a gap of 16 columns); B
+// MN-major in shared memory
 template <bool PAIRS>
 __device__ __forceinline__ void issue_mma_ts(bool leader, uint32_t tmem_d, uint32_t tmem_a, uint32_t b_tile, bool accumulate) {
   const uint32_t idesc = make_idesc(true);
@@ -114,7 +121,7 @@ __device__ __forceinline__ void issue_mma_ts(bool leader, uint32_t tmem_d, uint3
       asm volatile(
           "{\n\t.reg .pred p;\n\t.reg .b64 b;\n\tsetp.ne.b32 p, %4, 0;\n\tmov.b64 b, {%2, %5};\n\t"
           "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], b, %3, p;\n\t}" ::"r"(tmem_d),
-          "r"(tmem_a + (PAIRS ? (ks >> 1) * 32 + (ks & 1) * 8 : ks * 8)), "r"(b0 + uint32_t(ks * 2048 >> 4)), "r"(idesc), "r"((accumulate || ks > 0) ? 1u : 0u), "r"(kDescHi)
+          "r"(tmem_a + (PAIRS ? (ks >> 1) * 32 + (ks & 1) * 8 : (ks >> 2) * 64 + (ks & 3) * 8)), "r"(b0 + uint32_t(ks * 2048 >> 4)), "r"(idesc), "r"((accumulate || ks > 0) ? 1u : 0u), "r"(kDescHi)
           : "memory");
   }
 }
@@ -251,10 +258,11 @@ struct Smem {
   unsigned char kv[kStages][kTileBytes]; // K and V tiles in turn; linear part: state, phi(K') and V' tiles
   float z[2 * kD];                       // z of the unit (both halves with the learned map)
   uint64_t bar_full[kStages];            // the buffer's K or V tile has landed
-  uint64_t bar_free[kStages];            // the MMAs that read the buffer have completed
-  uint64_t bar_q[2];                     // Q_X staged (TMA, or the 128 threads that copied it)
+  uint64_t bar_free[kStages];            // the MMAs that read the buffer have completed (one arrival per row tile)
+  uint64_t bar_q[2];                     // Q_X staged (TMA, or the 256 threads that copied it)
   uint64_t bar_s[2];                     // MMA -> softmax threads of X: the products issued for X so far have completed
-  uint64_t bar_p[2];                     // softmax threads of X -> MMA: the A operand of X's next products is ready (128)
+  uint64_t bar_p[2];                     // softmax threads of X -> MMA: the A operand of X's next products is ready (one arrival per warp)
+  uint64_t bar_turn[2];                  // window part: the other row tile's batch of products has been issued
   uint64_t bar_done;                     // every window MMA has completed
   uint64_t bar_state;                    // the bf16 state and z of the unit have landed (learned map: phi(Q) as well)
   uint64_t bar_pk[2];                    // the phi(K') tile of an intra-chunk step has landed (even / odd steps)
@@ -262,8 +270,9 @@ struct Smem {
   uint64_t bar_lfree[2];                 // the MMAs that read an intra-chunk step's buffers have completed
   uint32_t tmem_base;
   int failed;
+  float exch[kSoftmaxThreads / 2];       // a value of each row on its way between the row's two threads
 };
-static_assert(sizeof(Smem) + 1024 <= 232448, "shared memory of one CTA");
+static_assert(sizeof(Smem) <= 232448, "shared memory of one CTA");
 
 // the call's K (or V) rows as a 4-D tensor {d, Hkv, T, layers x sequences}: boxes of 16 tokens x 64 columns of one KV head
 struct CallMaps {
@@ -328,6 +337,29 @@ __device__ __forceinline__ void fma2(float &a0, float &a1, float x0, float x1, f
       : "=f"(a0), "=f"(a1)
       : "f"(x0), "f"(x1), "f"(s), "f"(c));
 }
+__device__ __forceinline__ void dot2(float &a0, float &a1, float x0, float x1, float y0, float y1) {   // a += x * y
+  asm("{\n\t.reg .b64 a, x, y;\n\tmov.b64 a, {%0, %1};\n\tmov.b64 x, {%2, %3};\n\tmov.b64 y, {%4, %5};\n\t"
+      "fma.rn.f32x2 a, x, y, a;\n\tmov.b64 {%0, %1}, a;\n\t}"
+      : "+f"(a0), "+f"(a1)
+      : "f"(x0), "f"(x1), "f"(y0), "f"(y1));
+}
+__device__ __forceinline__ float lg2(float x) {
+  float y;
+  asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+__device__ __forceinline__ float max3(float a, float b, float c) {
+  float r;
+  asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+  return r;
+}
+__device__ __forceinline__ uint32_t max_bf16x2(uint32_t a, uint32_t b) {
+  uint32_t r;
+  asm("max.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
+  return r;
+}
+__device__ __forceinline__ float bf16_lo(uint32_t x) { return __uint_as_float(x << 16); }
+__device__ __forceinline__ float bf16_hi(uint32_t x) { return __uint_as_float(x & 0xffff0000u); }
 __device__ __forceinline__ void add2(float &a0, float &a1, float x0, float x1) {
   asm("{\n\t.reg .b64 a, x;\n\tmov.b64 a, {%0, %1};\n\tmov.b64 x, {%2, %3};\n\tadd.rn.f32x2 a, a, x;\n\tmov.b64 {%0, %1}, a;\n\t}"
       : "+f"(a0), "+f"(a1)
@@ -340,7 +372,7 @@ __device__ __forceinline__ void split2(float x0, float x1, uint32_t &hi, uint32_
 }
 
 template <int G, int MODE>
-__global__ void __launch_bounds__(kThreads, 1)   // 10 warps = 3 on one scheduler: 168 registers per thread at most
+__global__ void __launch_bounds__(kThreads, 1)   // 19 warps = 5 on one scheduler: 96 registers per thread at most
 prefill_attn_tc_kernel(const __grid_constant__ PrefillParams p, const CUtensorMap *ring_maps, const __grid_constant__ CallMaps cm) {
   using bf16 = __nv_bfloat16;
   constexpr bool SUM = MODE == kModeSum;          // sum of two normalised terms instead of the shared normaliser
@@ -350,7 +382,7 @@ prefill_attn_tc_kernel(const __grid_constant__ PrefillParams p, const CUtensorMa
   constexpr int TOKT = kRows / G;    // tokens per row tile
   constexpr int TOKC = 2 * TOKT;     // tokens per CTA
   extern __shared__ __align__(1024) unsigned char smem_raw[];
-  Smem &sm = *reinterpret_cast<Smem *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  Smem &sm = *reinterpret_cast<Smem *>(smem_raw);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   // CTAs of a unit: those of its full chunks, then those of the last one, the last tokens first (their windows are the
   // longest of a new prompt); from here on "the chunk" is the CTA's own
@@ -365,77 +397,93 @@ prefill_attn_tc_kernel(const __grid_constant__ PrefillParams p, const CUtensorMa
   const int64_t uc = int64_t(u) * p.nsub + sub;                        // (unit, chunk): index into the scratch arrays
   const int ug = u / p.Hkv, g = u - ug * p.Hkv, lrel = ug / p.B, b = ug - lrel * p.B;
   const int layer = p.layer_begin + lrel;
-  const LayerDev ld = p.layers[layer];
   const int ntok = min(TOKC, chunk_n - tok0);
   const int ntokA = min(TOKT, ntok), ntokB = ntok - ntokA;
   const bool hasB = ntokB > 0;
-  const int64_t tq0 = p.n0 + chunk_c0 + tok0;
-  const int64_t tq_last = tq0 + ntok - 1;
-  const int64_t w = ld.w;
-  const int64_t wl = ld.wlin;                      // delay of the linear stream: w, or 0 when the state holds every token
+  volatile int *failed = &sm.failed;
+  const LayerDev ld = p.layers[layer];
+  // The loader warp sets up the barriers and asks for Q before anything that waits for the layer table.
+  const bool aligned = (smem_u32(smem_raw) & 1023u) == 0;   // (the swizzled tiles have to start on a multiple of 1024)
+  const bool q_by_tma = p.q_tma && aligned;
+  int status = 0;
+  if (warp == kLoadWarp && lane == 0) {
+    status = *reinterpret_cast<volatile int32_t *>(&p.ctl->status);
+    const int n_rows = hasB ? 2 : 1;              // row tiles: each one frees a buffer
+    for (int s = 0; s < kStages; ++s) {
+      mbar_init(smem_u32(&sm.bar_full[s]), 2);
+      mbar_init(smem_u32(&sm.bar_free[s]), n_rows);
+    }
+    for (int x = 0; x < 2; ++x) {
+      mbar_init(smem_u32(&sm.bar_q[x]), p.q_tma ? 1 : 2 * kRows);
+      mbar_init(smem_u32(&sm.bar_s[x]), 1);
+      mbar_init(smem_u32(&sm.bar_turn[x]), 1);
+      mbar_init(smem_u32(&sm.bar_p[x]), kSoftmaxThreads / 32 / 2);
+      mbar_init(smem_u32(&sm.bar_pk[x]), 1);
+      mbar_init(smem_u32(&sm.bar_vp[x]), 2);
+      mbar_init(smem_u32(&sm.bar_lfree[x]), n_rows);
+    }
+    mbar_init(smem_u32(&sm.bar_done), n_rows);
+    mbar_init(smem_u32(&sm.bar_state), 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    // Q_X, when the group's heads lie side by side.  (Tokens past the tile's last one are zeros or the next tile's rows:
+    // their results are not stored.)
+    for (int x = 0; q_by_tma && x < n_rows; ++x) {
+      const uint32_t bar = smem_u32(&sm.bar_q[x]), dst = smem_u32(sm.q[x]);
+      mbar_expect_tx(bar, kTileBytes);
+      tma_load_4d(dst, &cm.q, 0, g * G, chunk_c0 + tok0 + x * TOKT, lrel * p.B + b, bar);
+      tma_load_4d(dst + kBoxBytes, &cm.q, 64, g * G, chunk_c0 + tok0 + x * TOKT, lrel * p.B + b, bar);
+    }
+  }
+  // (positions stay below 2^30, the most tokens a context may hold; a longer window is no other than that)
+  constexpr int64_t kMost = int64_t(1) << 30;
+  const int n0 = int(p.n0);
+  const int tq0 = n0 + chunk_c0 + tok0;
+  const int tq_last = tq0 + ntok - 1;
+  const int w = int(ld.w < kMost ? ld.w : kMost);
+  const int wl = int(ld.wlin < kMost ? ld.wlin : kMost);   // delay of the linear stream: w, or 0 when the state holds every token
   const uint32_t cap = ld.cap > 0 ? uint32_t(ld.cap) : 1u;
   const size_t unit_rows = (size_t(b + p.b0) * p.Hkv + g) * size_t(ld.cap);   // b + b0: the sequence's slot in the context
   const size_t seq = (size_t(lrel) * p.B + b) * size_t(p.T);
-  volatile int *failed = &sm.failed;
 #ifdef GLIDE_PF_CLOCKS
   long long pf_t_ = clock64();
   if (threadIdx.x == 0) atomicAdd(&g_pf_clk[8], 1ull);
 #endif
 
-  // a time-out recorded by an earlier CTA ends the launch quickly
-  if (*reinterpret_cast<volatile int32_t *>(&p.ctl->status) == kDevWaitTimeout) return;
-
-  int64_t j_lo = tq0 - w + 1;
+  int j_lo = tq0 - w + 1;
   if (j_lo < 0) j_lo = 0;
-  j_lo &= ~int64_t(kGroup - 1);   // key tiles start at a multiple of the TMA box
-  const int n_tiles = w > 0 ? int((tq_last - j_lo) / kKT) + 1 : 0;
+  j_lo &= ~(kGroup - 1);   // key tiles start at a multiple of the TMA box
+  const int n_tiles = w > 0 ? (tq_last - j_lo) / kKT + 1 : 0;
   // key tiles that row tile X has valid keys in: [t_first(X), t_end(X)) (A may end, B begin one tile off the CTA's range)
   auto t_first = [&](int x) {
-    const int64_t lo = tq0 + x * TOKT - w + 1;
-    return lo <= j_lo ? 0 : int((lo - j_lo) / kKT);
+    const int lo = tq0 + x * TOKT - w + 1;
+    return lo <= j_lo ? 0 : (lo - j_lo) / kKT;
   };
-  auto t_end = [&](int x) { return n_tiles == 0 ? 0 : int((tq0 + x * TOKT + (x ? ntokB : ntokA) - 1 - j_lo) / kKT) + 1; };
+  auto t_end = [&](int x) { return n_tiles == 0 ? 0 : (tq0 + x * TOKT + (x ? ntokB : ntokA) - 1 - j_lo) / kKT + 1; };
 
   if (warp == kMmaWarp) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(smem_u32(&sm.tmem_base)) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
-  // The loader warp sets up the barriers and is the first to go on: Q and the first K tile are on their way before the CTA
-  // meets for the first time (it needs nothing from the other warps: it zeroes what has to be zero itself).
   if (warp == kLoadWarp) {
-    if (lane == 0) {
-      for (int s = 0; s < kStages; ++s) {
-        mbar_init(smem_u32(&sm.bar_full[s]), 2);
-        mbar_init(smem_u32(&sm.bar_free[s]), 1);
-      }
-      for (int x = 0; x < 2; ++x) {
-        mbar_init(smem_u32(&sm.bar_q[x]), p.q_tma ? 1 : kRows);
-        mbar_init(smem_u32(&sm.bar_s[x]), 1);
-        mbar_init(smem_u32(&sm.bar_p[x]), kRows);
-        mbar_init(smem_u32(&sm.bar_pk[x]), 1);
-        mbar_init(smem_u32(&sm.bar_vp[x]), 2);
-        mbar_init(smem_u32(&sm.bar_lfree[x]), 1);
-      }
-      mbar_init(smem_u32(&sm.bar_done), 1);
-      mbar_init(smem_u32(&sm.bar_state), 1);
-      asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-      sm.failed = 0;
-      // Q_X, when the group's heads lie side by side.  (Tokens past the tile's last one are zeros or the next tile's rows:
-      // their results are not stored.)
-      for (int x = 0; p.q_tma && x < (hasB ? 2 : 1); ++x) {
-        const uint32_t bar = smem_u32(&sm.bar_q[x]), dst = smem_u32(sm.q[x]);
-        mbar_expect_tx(bar, kTileBytes);
-        tma_load_4d(dst, &cm.q, 0, g * G, chunk_c0 + tok0 + x * TOKT, lrel * p.B + b, bar);
-        tma_load_4d(dst + kBoxBytes, &cm.q, 64, g * G, chunk_c0 + tok0 + x * TOKT, lrel * p.B + b, bar);
-      }
+    // a time-out recorded by an earlier CTA ends the launch quickly
+    if (lane == 0) sm.failed = status == kDevWaitTimeout || !aligned;
+    // The others may go on; this warp does not wait for them: it touches no TMEM and zeroes what has to be zero itself.  (A
+    // barrier of its own: the one at the end of the CTA may be reached by this warp before the others have met here.)
+    __syncwarp();
+    asm volatile("barrier.cta.arrive 9, %0;" ::"n"(kThreads) : "memory");
+    if (*failed) {   // (set before the meeting: the same for all)
+      int alone = 0;
+      for (int x = 0; q_by_tma && x < (hasB ? 2 : 1); ++x) mbar_wait(smem_u32(&sm.bar_q[x]), 0u, &alone);   // no copy outlives the CTA
+      if (lane == 0 && !aligned) atomicExch(&p.ctl->status, kDevWaitTimeout);
+      return;
     }
     // Token groups past the CTA's last token are never loaded (only the last tile has such groups), and what a
     // masked key's V row holds is multiplied by a zero weight, so it has to be finite: those rows of the buffer that
     // will hold the last V tile start at zero (earlier tiles that pass through the buffer leave real rows behind).
     if (n_tiles > 0) {
       const int last_slot = (2 * (n_tiles - 1) + 1) % kStages;
-      const int64_t j0_last = j_lo + int64_t(n_tiles - 1) * kKT;
-      const int first_skipped = int((tq_last - j0_last) / kGroup) + 1;   // groups [first_skipped, 8) are not loaded
+      const int j0_last = j_lo + (n_tiles - 1) * kKT;
+      const int first_skipped = (tq_last - j0_last) / kGroup + 1;   // groups [first_skipped, 8) are not loaded
       const int n16 = (kKT / kGroup - first_skipped) * int(kGroupBytes / 16);
       for (int half = 0; half < 2; ++half) {
         uint4 *dst = reinterpret_cast<uint4 *>(&sm.kv[last_slot][half * kBoxBytes + first_skipped * kGroupBytes]);
@@ -443,49 +491,53 @@ prefill_attn_tc_kernel(const __grid_constant__ PrefillParams p, const CUtensorMa
       }
       fence_async_smem();
     }
-    __syncwarp();   // (the barriers are set up for every lane)
+    __syncwarp();
   }
-  // Q_X otherwise: 128 rows x 16 chunks by the 128 threads of each row tile, asked for before the set-up's barrier so that the copy
+  // Q_X otherwise: 128 rows x 16 chunks by the 256 threads of each row tile, asked for before the set-up's barrier so that the copy
   // runs while the other warps finish setting up (it needs nothing of that; nothing else writes these tiles).  A thread's
-  // rows are 8 apart, so all of them belong to one head of the group (G divides 8).
-  const int X = (tid >> 7) & 1;                   // row tile of this thread (softmax warps only)
+  // rows are 16 apart, so all of them belong to one head of the group (G divides 16).
+  const int X = (warp >> 2) & 1, H = warp >> 3;   // row tile and column half of this thread (softmax warps only)
   const int row = tid & 127;
   const int ntokX = X ? ntokB : ntokA;
   const bool activeX = tid < kSoftmaxThreads && ntokX > 0;
   if (activeX && !p.q_tma) {
-    const int c = row & 15, r0 = row >> 4, h2 = r0 % G;
+    const int c = row & 15, r0 = (row >> 4) + 8 * H, h2 = r0 % G;
     const bf16 *src = reinterpret_cast<const bf16 *>(p.q) +
                       ((seq + size_t(chunk_c0 + tok0 + X * TOKT)) * p.H + p.heads_of[g * G + h2]) * kD + c * 8;
     const uint32_t dst = smem_u32(sm.q[X]) + sw128(r0, c);   // (r & 7 is the same for all rows of the thread)
 #pragma unroll 4
-    for (int i = 0; i < 16; ++i) {
-      const int tk = (r0 + 8 * i) / G;
+    for (int i = 0; i < 8; ++i) {
+      const int tk = (r0 + 16 * i) / G;
       const bool valid = tk < ntokX;
-      cp_async16(dst + uint32_t(i) * 8u * 128u, src + (valid ? size_t(tk) * p.H * kD : 0), valid);
+      cp_async16(dst + uint32_t(i) * 16u * 128u, src + (valid ? size_t(tk) * p.H * kD : 0), valid);
     }
     cp_async_commit();
   }
-  // the CTA's first meeting: barriers and TMEM are set up (the loader comes to it with its second tile)
+  // the CTA's first meeting: barriers and TMEM are set up
   uint32_t tmem = 0;
-  auto meet = [&]() {
+  if (warp != kLoadWarp) {
     fence_async_smem();
     tc_fence_before();
-    __syncthreads();
+    asm volatile("barrier.cta.sync 9, %0;" ::"n"(kThreads) : "memory");
     tc_fence_after();
     tmem = sm.tmem_base;
     PF_CLK(0);
-  };
-  if (warp != kLoadWarp) meet();
+    if (*failed) {
+      cp_async_wait_all();
+      if (warp == kMmaWarp) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem) : "memory");
+      return;
+    }
+  }
   const uint32_t sQ0 = smem_u32(sm.q[0]);
   const uint32_t sKV0 = smem_u32(sm.kv[0]);
   auto q_addr = [&](int x) { return sQ0 + uint32_t(x) * kTileBytes; };
   auto kv_addr = [&](int slot) { return sKV0 + uint32_t(slot) * kTileBytes; };
   // Linear part: what it needs is known now, so that the loader can fetch it behind the last key tiles.
   const bool linear = ld.evicts && tq_last >= wl;
-  const int64_t folded = p.n0 + chunk_c0 - wl;   // tokens below this index are in S, z at the start of the chunk
+  const int folded = n0 + chunk_c0 - wl;   // tokens below this index are in S, z at the start of the chunk
   const bool need_state = linear && folded > 0;
   // intra-chunk steps: delayed tokens of this chunk up to the CTA's last token, 128 at a time
-  const int i_lo = folded < 0 ? int(-folded < int64_t(chunk_n) ? -folded : int64_t(chunk_n)) : 0;
+  const int i_lo = folded < 0 ? min(-folded, chunk_n) : 0;
   const int i_hi = tok0 + ntok - 1;
   const int it0 = i_lo & ~(kKT - 1);
   const int n_itiles = (linear && it0 <= i_hi) ? (i_hi - it0) / kKT + 1 : 0;   // (linear without a state: at least one)
@@ -504,27 +556,63 @@ prefill_attn_tc_kernel(const __grid_constant__ PrefillParams p, const CUtensorMa
   auto slot_vp = [&](int t) { return TWO ? 4 : late_slot(3 + (t & 1)); };
 
   if (tid < kSoftmaxThreads) {
-    // =========================== softmax threads: one row each ===========================
+    // =========================== softmax threads: half a row each ===========================
+    // Two threads per row, in warps that share a scheduler: thread (X, H, row) has columns 64 H .. 64 H + 63 of every 128-column
+    // operand of the row.  One warp per scheduler and row tile waited on its own chain of loads, maxima, exponentials and stores (a
+    // CTA took some 5000 issue slots of 29500 cycles); a pair of warps fills each other's gaps.  What the row has in common goes
+    // through sm.exch behind barriers of the two warps, which every thread of a pair passes equally often: after a time-out the
+    // waits return at once and the loops run on, storing nothing.
     // Every hand-over of row tile X is its own: the threads of A and of B meet only at the end of the CTA, so that one
     // tile's arithmetic runs beside the other's products.  bar_s completes once per batch of products of X, bar_p once
     // per operand that X's threads have written; both sides count in the same order.
     const int tok_r = row / G;
     const int tl = tok0 + X * TOKT + tok_r;         // chunk-relative token of this row
-    const int64_t tok_abs = p.n0 + chunk_c0 + tl;
-    const uint32_t tS = tmem + (uint32_t((warp & 3) * 32) << 16) + uint32_t(X) * 128u;
+    const int tok_abs = n0 + chunk_c0 + tl;
+    const uint32_t tS = tmem + (uint32_t((warp & 3) * 32) << 16) + uint32_t(X) * 128u + uint32_t(H) * 64u;
     const uint32_t tO = tS + 256u;
-    float m_ref = -CUDART_INF_F, l_sum = 0.f;
+    float m_ref = -CUDART_INF_F, l_sum = 0.f;       // l: of this thread's columns
     uint32_t n_s = 0;                               // batches of products waited for
+    bool ok = true;
+    const int my_head = p.heads_of[g * G + lane % G];   // (head of group member h: lane h has it)
     auto wait_s = [&]() {
-      const bool got = mbar_wait(smem_u32(&sm.bar_s[X]), n_s & 1u, failed);
+      if (ok) ok = mbar_wait(smem_u32(&sm.bar_s[X]), n_s & 1u, failed);
       ++n_s;
       tc_fence_after();
-      return bool(__all_sync(0xffffffffu, got));    // warp-uniform: the TMEM accesses need every lane
+      ok = __all_sync(0xffffffffu, ok);             // warp-uniform
     };
-    // multiply this thread's O row by f (warp-collective TMEM read-modify-write)
+    auto wait_once = [&](uint64_t &bar) { ok = ok && mbar_wait(smem_u32(&bar), 0u, failed); };
+    // the operand that the MMA warp waits for is complete as far as this warp goes
+    auto hand_over = [&]() {
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(smem_u32(&sm.bar_p[X]));
+    };
+    const int pair_bar = 1 + (warp & 7);            // named barrier of warps w and w + 8
+    auto pair_sync = [&]() { asm volatile("barrier.cta.sync %0, 64;" ::"r"(pair_bar) : "memory"); };
+    auto pair_any = [&](bool x) {
+      uint32_t r;
+      asm volatile(
+          "{\n\t.reg .pred p, q;\n\tsetp.ne.u32 q, %1, 0;\n\tbarrier.cta.red.or.pred p, %2, 64, q;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+          : "=r"(r)
+          : "r"(uint32_t(x)), "r"(pair_bar)
+          : "memory");
+      return r != 0;
+    };
+    // f(first thread's value, second thread's value) in both threads of a row
+    auto combine = [&](float v, auto &&f) {
+      float *slot = &sm.exch[tid & (kSoftmaxThreads / 2 - 1)];
+      if (H == 0) *slot = v;
+      pair_sync();
+      if (H == 1) *slot = v = f(*slot, v);
+      pair_sync();
+      return H == 0 ? *slot : v;
+    };
+    auto row_sum_of = [&](float v) { return combine(v, [](float a, float b) { return a + b; }); };
+    auto row_max_of = [&](float v) { return combine(v, [](float a, float b) { return fmaxf(a, b); }); };
+    // multiply this thread's part of the O row by f (warp-collective TMEM read-modify-write)
     auto scale_o = [&](float f) {
 #pragma unroll 1
-      for (int c0 = 0; c0 < kD; c0 += 32) {
+      for (int c0 = 0; c0 < kHalf; c0 += 32) {
         uint32_t r[32];
         tmem_ld32(tO + c0, r);
 #pragma unroll
@@ -532,8 +620,8 @@ prefill_attn_tc_kernel(const __grid_constant__ PrefillParams p, const CUtensorMa
         tmem_st32(tO + c0, r);
       }
     };
-    // weights of columns c .. c + 31 over columns c / 2 .. c / 2 + 15; gated: hi over c .. c + 15, lo (first half of x)
-    // over c + 16 .. c + 31
+    // weights of columns c .. c + 31 over columns c / 2 .. c / 2 + 15 (of the half); gated: hi over c .. c + 15, lo (first half
+    // of x) over c + 16 .. c + 31
     auto store_p = [&](int c, const uint32_t (&pk)[16], const uint32_t (&x)[32]) {
       if constexpr (GATED) {
         uint32_t lo[16];
@@ -545,24 +633,31 @@ prefill_attn_tc_kernel(const __grid_constant__ PrefillParams p, const CUtensorMa
         tmem_st16(tS + (c >> 1), pk);
       }
     };
-    // the lazy reference for a tile whose row maximum (raw) is mx: it moves, and O and l are rescaled, only when the maximum
-    // grows by more than 2^kLazy; returns what the weights are taken against
+    // the lazy reference for a tile whose maximum over this thread's columns (raw) is mx: it moves, and O and l are rescaled, only
+    // when the row's maximum grows by more than 2^kLazy; returns what the weights are taken against
     auto move_ref = [&](float mx, bool first) {
-      mx *= p.scale_log2;   // (the scale is positive: it is applied to the maximum)
-      float f = 1.f;
-      if (mx > m_ref + kLazy || (m_ref == -CUDART_INF_F && mx > -CUDART_INF_F)) {
-        f = m_ref == -CUDART_INF_F ? 0.f : ex2(m_ref - mx);
-        m_ref = mx;
+      auto grows = [&]() {
+        const float ms = mx * p.scale_log2;   // (the scale is positive: it is applied to the maximum)
+        return ms > m_ref + kLazy || (m_ref == -CUDART_INF_F && ms > -CUDART_INF_F);
+      };
+      if (pair_any(grows())) {
+        mx = row_max_of(mx);
+        float f = 1.f;
+        if (grows()) {
+          mx *= p.scale_log2;
+          f = m_ref == -CUDART_INF_F ? 0.f : ex2(m_ref - mx);
+          m_ref = mx;
+        }
+        if (!first && __any_sync(0xffffffffu, f != 1.f)) scale_o(f);
+        l_sum *= f;
       }
-      if (!first && __any_sync(0xffffffffu, f != 1.f)) scale_o(f);
-      l_sum *= f;
       return m_ref == -CUDART_INF_F ? 0.f : m_ref;
     };
     auto row_max = [&](const uint32_t (&x)[32], float mx) {
       float m4[4] = {mx, -CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F};
 #pragma unroll
-      for (int i = 0; i < 32; ++i) m4[i & 3] = fmaxf(m4[i & 3], __uint_as_float(x[i]));
-      return fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3]));
+      for (int i = 0; i < 32; i += 2) m4[(i >> 1) & 3] = max3(m4[(i >> 1) & 3], __uint_as_float(x[i]), __uint_as_float(x[i + 1]));
+      return fmaxf(max3(m4[0], m4[1], m4[2]), m4[3]);
     };
     // weights of columns c .. c + 31 (scores x) over the S columns this thread has already consumed (columns c / 2 ..
     // c / 2 + 15); the sum uses the weights as the tensor core sees them
@@ -578,42 +673,34 @@ prefill_attn_tc_kernel(const __grid_constant__ PrefillParams p, const CUtensorMa
           split2(a0, a1, pk[e], x[e]);   // (x[e] has been read: element e comes from x[2 e] and x[2 e + 1])
         } else {
           pk[e] = pack_bf16x2(ex2(a0), ex2(a1));
-          add2(sum0, sum1, __uint_as_float(pk[e] << 16), __uint_as_float(pk[e] & 0xffff0000u));
+          add2(sum0, sum1, bf16_lo(pk[e]), bf16_hi(pk[e]));
         }
       }
       store_p(c, pk, x);
     };
-    // One key tile without a masked key: two passes over its columns, the next 32 on their way while some are used.
+    // One key tile without a masked key: two passes over the thread's columns (all 64 scores held between their maximum and their
+    // weights leave too few registers: 96 a thread).
     auto soft_tile = [&](bool first) {
-      float mx = -CUDART_INF_F, sum0 = 0.f, sum1 = 0.f;
-      uint32_t r[2][32];
-      tmem_ld32_nowait(tS, r[0]);
-#pragma unroll
-      for (int c = 0; c < kKT; c += 32) {
-        uint32_t (&x)[32] = r[(c >> 5) & 1];
-        tmem_wait_ld(x);
-        tmem_ld32_nowait(tS + ((c + 32) & (kKT - 1)), r[((c >> 5) & 1) ^ 1]);   // (after the last columns: the first of pass 2)
-        mx = row_max(x, mx);
-      }
-      tmem_wait_ld(r[0]);
+      float sum0 = 0.f, sum1 = 0.f;
+      uint32_t x[32];
+      tmem_ld32(tS + 32, x);
+      float mx = row_max(x, -CUDART_INF_F);
+      tmem_ld32(tS, x);
+      mx = row_max(x, mx);
       const float mr = move_ref(mx, first);
-#pragma unroll
-      for (int c = 0; c < kKT; c += 32) {
-        uint32_t (&x)[32] = r[(c >> 5) & 1];
-        tmem_wait_ld(x);
-        if (c + 32 < kKT) tmem_ld32_nowait(tS + c + 32, r[((c >> 5) & 1) ^ 1]);
-        weights(c, x, mr, sum0, sum1);
-      }
+      weights(0, x, mr, sum0, sum1);   // (over columns that have been read)
+      tmem_ld32(tS + 32, x);
+      weights(32, x, mr, sum0, sum1);
       tmem_wait_st();
       l_sum += sum0 + sum1;
     };
-    // One key tile with masked keys (valid columns lo .. hi of this row).  32 columns at a time, those in which no row of the
-    // warp has a valid one left out; the loops stay rolled: with everything unrolled the kernel was 210 KB of code that a CTA
+    // One key tile with masked keys (valid columns lo .. hi of this row's half).  32 columns at a time, those in which no row of
+    // the warp has a valid one left out; the loops stay rolled: with everything unrolled the kernel was 210 KB of code that a CTA
     // fetched once per phase (a CTA's first key tile took 12000 cycles, a later one 2500).
     auto soft_tile_masked = [&](int lo, int hi, bool first) {
       float mx = -CUDART_INF_F, sum0 = 0.f, sum1 = 0.f;
 #pragma unroll 1
-      for (int c = 0; c < kKT; c += 32) {
+      for (int c = 0; c < kHalf; c += 32) {
         const uint32_t m = column_mask(c, lo, hi);
         if (!__any_sync(0xffffffffu, m)) continue;
         uint32_t x[32];
@@ -624,7 +711,7 @@ prefill_attn_tc_kernel(const __grid_constant__ PrefillParams p, const CUtensorMa
       }
       const float mr = move_ref(mx, first);
 #pragma unroll 1
-      for (int c = 0; c < kKT; c += 32) {
+      for (int c = 0; c < kHalf; c += 32) {
         const uint32_t m = column_mask(c, lo, hi);
         uint32_t x[32];
         if (!__any_sync(0xffffffffu, m)) {
@@ -648,31 +735,56 @@ prefill_attn_tc_kernel(const __grid_constant__ PrefillParams p, const CUtensorMa
         fence_async_smem();
         mbar_arrive(smem_u32(&sm.bar_q[X]));
       }
-      const int64_t tqX0 = tq0 + X * TOKT, tqX_last = tqX0 + ntokX - 1;
+      // phi(q) of the parameter-free map is e^(q - max) / sum; both numbers come from the Q tile while the first product runs, the
+      // values later (the tile is the products' operand until then)
+      float q_mxl = 0.f, q_sum = 1.f;                // max log2(e); sum (over the row)
+      auto load_q = [&](uint32_t (&v)[32]) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          const uint4 v4 = *reinterpret_cast<const uint4 *>(sm.q[X] + sw128(row, H * 8 + i));
+          v[i * 4] = v4.x, v[i * 4 + 1] = v4.y, v[i * 4 + 2] = v4.z, v[i * 4 + 3] = v4.w;
+        }
+      };
+      if (linear && !PHI2) {
+        wait_once(sm.bar_q[X]);
+        uint32_t v[32];
+        load_q(v);
+        uint32_t m2 = v[0];
+#pragma unroll
+        for (int i = 1; i < 32; ++i) m2 = max_bf16x2(m2, v[i]);
+        q_mxl = row_max_of(fmaxf(bf16_lo(m2), bf16_hi(m2))) * kLog2e;
+        if (!SUM) {
+          float sum0 = 0.f, sum1 = 0.f;
+#pragma unroll
+          for (int i = 0; i < 32; ++i) {
+            float a0, a1;
+            fma2(a0, a1, bf16_lo(v[i]), bf16_hi(v[i]), kLog2e, -q_mxl);
+            add2(sum0, sum1, ex2(a0), ex2(a1));
+          }
+          q_sum = row_sum_of(sum0 + sum1);
+        }
+      }
+      const int tqX0 = tq0 + X * TOKT, tqX_last = tqX0 + ntokX - 1;
       const int tf = t_first(X), te = t_end(X);
-      bool ok = true;
       for (int t = tf; t < te; ++t) {
-        ok = wait_s();
-        if (!ok) break;
+        wait_s();
+        if (tid == X * kRows) {   // S of the tile and P V of the tile before have completed
+          mbar_arrive(smem_u32(&sm.bar_free[2 * t % kStages]));
+          if (t > tf) mbar_arrive(smem_u32(&sm.bar_free[(2 * t - 1) % kStages]));
+        }
         if (t == tf) PF_CLK(11); else PF_CLK(12);
-        const int64_t j0 = j_lo + int64_t(t) * kKT;
+        const int j0 = j_lo + t * kKT;
         if (j0 + kKT - 1 <= tqX0 && j0 > tqX_last - w) {
           soft_tile(t == tf);
         } else {
-          // valid columns of this row: lo <= c <= hi
-          const int64_t lo64 = tok_abs - w + 1 - j0, hi64 = tok_abs - j0;
-          soft_tile_masked(int(lo64 < 0 ? 0 : (lo64 > kKT ? kKT : lo64)), int(hi64 < -1 ? -1 : (hi64 > kKT - 1 ? kKT - 1 : hi64)),
-                           t == tf);
+          // valid columns of this row: lo <= c <= hi (a token more than 2^30 - 1 before another is none)
+          soft_tile_masked(max(tok_abs - w + 1 - j0, 0) - H * kHalf, min(tok_abs - j0, kKT - 1) - H * kHalf, t == tf);
         }
-        tc_fence_before();      // this thread's TMEM accesses precede the MMAs that read P and overwrite S
-        mbar_arrive(smem_u32(&sm.bar_p[X]));
+        hand_over();            // this thread's TMEM accesses precede the MMAs that read P and overwrite S
         if (t == tf) PF_CLK(13); else PF_CLK(14);
       }
       const bool windowed = te > tf;               // O_X holds a valid accumulation
       if (linear) {
-        // phi(q) is made from the Q tile, which TMA wrote: its own barrier is what shows these threads the copy (it has completed
-        // long ago if there was a window product, but that the MMA warp waited for it does not count here)
-        mbar_wait(smem_u32(&sm.bar_q[X]), 0u, failed);
         // Any common reference M >= m_ref gives the same quotient O / l.  M = max(m_ref, 0) would rescale O for every
         // row whose window maximum is negative; a floor of -64 keeps 2^-M and everything scaled by it far inside the
         // fp32 / bf16 range (phi <= 1) and makes that rescale a rarity.
@@ -685,133 +797,94 @@ prefill_attn_tc_kernel(const __grid_constant__ PrefillParams p, const CUtensorMa
         const float M = has_lin ? fmaxf(m_ref, -64.f) : m_ref;
         float fw = m_ref == -CUDART_INF_F ? 0.f : ex2(m_ref - M);
         const float fl = has_lin ? ex2(-M) : 0.f;
-        if (SUM) fw = l_sum > 0.f ? 1.0f / l_sum : 0.f;
-        l_sum = SUM ? 1.f : l_sum * fw;
-        if (PHI2 || (SUM && need_state)) mbar_wait(smem_u32(&sm.bar_state), 0u, failed);   // phi(Q); z
+        if (SUM) {
+          const float l = row_sum_of(l_sum);
+          fw = l > 0.f ? 1.0f / l : 0.f;
+          l_sum = 0.5f;                             // (of each half: the final division is by 1)
+        } else {
+          l_sum *= fw;
+        }
+        if (PHI2 || (SUM && need_state)) wait_once(sm.bar_state);   // phi(Q); z
         unsigned char *tileX = sm.q[X];
         float dot = 0.f;
         const float g_own = GATED ? p.gcum[size_t(uc) * p.SC + min(tl, chunk_n - 1)] : 0.f;
         const float dec0 = GATED ? ex2(g_own * kLog2e) : 1.f;   // what the chunk-start state has decayed to
         if constexpr (!PHI2) {
-          // this row of Q is still in the shared tile, and every S product of X has completed: phi(q) takes its place,
-          // eight values at a time: maximum, then exponentials (left as bf16) and their sum, then the scaled values
-          // (four chunks are loaded before any of them is used: a store to the tile in between would hold the loads back)
-          float mx = -CUDART_INF_F;
-          uint4 v4[4];
-          auto load_chunks = [&](int c0) {
-#pragma unroll
-            for (int i = 0; i < 4; ++i) v4[i] = *reinterpret_cast<const uint4 *>(tileX + sw128(row, c0 + i));
-          };
-#pragma unroll 1
-          for (int c0 = 0; c0 < 16; c0 += 4) {
-            load_chunks(c0);
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-              const uint32_t w4[4] = {v4[i].x, v4[i].y, v4[i].z, v4[i].w};
-#pragma unroll
-              for (int e = 0; e < 4; ++e) mx = fmaxf(mx, fmaxf(__uint_as_float(w4[e] << 16), __uint_as_float(w4[e] & 0xffff0000u)));
-            }
-          }
-          float sum0 = 0.f, sum1 = 0.f, dz0 = 0.f, dz1 = 0.f;
-          const float mxl = mx * kLog2e;
-          const float2 *zrow = reinterpret_cast<const float2 *>(p.zcum + (size_t(uc) * p.SC + size_t(tok_r < ntokX ? tl : tok0)) * kD);
-#pragma unroll 1
-          for (int c0 = 0; c0 < 16; c0 += 4) {
-            load_chunks(c0);
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-              const int c = c0 + i;
-              uint32_t w4[4] = {v4[i].x, v4[i].y, v4[i].z, v4[i].w};
-#pragma unroll
-              for (int e = 0; e < 4; ++e) {
-                float a0, a1;
-                fma2(a0, a1, __uint_as_float(w4[e] << 16), __uint_as_float(w4[e] & 0xffff0000u), kLog2e, -mxl);
-                const float e0 = ex2(a0), e1 = ex2(a1);
-                add2(sum0, sum1, e0, e1);
-                if (SUM) {
-                  const float2 zc = __ldg(zrow + c * 4 + e);
-                  dz0 = fmaf(e0, zc.x + (need_state ? sm.z[c * 8 + e * 2] : 0.f), dz0);
-                  dz1 = fmaf(e1, zc.y + (need_state ? sm.z[c * 8 + e * 2 + 1] : 0.f), dz1);
-                }
-                w4[e] = pack_bf16x2(e0, e1);
-              }
-              if (!GATED) v4[i] = make_uint4(w4[0], w4[1], w4[2], w4[3]);
-            }
-            if (!GATED)
-#pragma unroll
-              for (int i = 0; i < 4; ++i) *reinterpret_cast<uint4 *>(tileX + sw128(row, c0 + i)) = v4[i];
-          }
-          // shared normaliser: phi(q) 2^-M;  sum of terms: phi(q) / (phi(q) . z_row) = e / (e . z_row)
-          const float dz = dz0 + dz1;
-          const float sc = SUM ? ((has_lin && dz > 0.f) ? 1.0f / dz : 0.f) : fl * __frcp_rn(sum0 + sum1);
+          // this half row of Q is still in the shared tile, and every S product of X has completed: phi(q) takes its place
+          uint32_t v[32];
+          load_q(v);
           const bool with_z = !SUM && need_state;
-          if (with_z) mbar_wait(smem_u32(&sm.bar_state), 0u, failed);   // z has landed
+          const float *zh = sm.z + H * kHalf;
           float dot1 = 0.f;
+          if (SUM) {
+            // sum of terms: phi(q) / (phi(q) . z_row) = e / (e . z_row)
+            const float2 *zrow =
+                reinterpret_cast<const float2 *>(p.zcum + (size_t(uc) * p.SC + size_t(tok_r < ntokX ? tl : tok0)) * kD + H * kHalf);
+            float dz0 = 0.f, dz1 = 0.f;
+#pragma unroll
+            for (int i = 0; i < 32; ++i) {
+              float a0, a1;
+              fma2(a0, a1, bf16_lo(v[i]), bf16_hi(v[i]), kLog2e, -q_mxl);
+              const float2 zc = __ldg(zrow + i);
+              dot2(dz0, dz1, ex2(a0), ex2(a1), zc.x + (need_state ? zh[i * 2] : 0.f), zc.y + (need_state ? zh[i * 2 + 1] : 0.f));
+            }
+            q_sum = row_sum_of(dz0 + dz1);
+          }
+          if (with_z) wait_once(sm.bar_state);     // z has landed
           if constexpr (GATED) {
-            // the values in fp32 (the exponentials once more), hi in place, lo in a buffer of the finished window part
-            mbar_wait(smem_u32(&sm.bar_done), 0u, failed);
-#pragma unroll 2
-            for (int c = 0; c < 16; ++c) {
-              uint4 *at = reinterpret_cast<uint4 *>(tileX + sw128(row, c));
-              const uint4 v = *at;
-              uint32_t w4[4] = {v.x, v.y, v.z, v.w}, lo4[4];
+            // fp32 values, hi in place, lo in a buffer of the finished window part
+            const float sc = fl * __frcp_rn(q_sum);
+            wait_once(sm.bar_done);
+#pragma unroll
+            for (int c = 0; c < 8; ++c) {
+              uint32_t hi4[4], lo4[4];
 #pragma unroll
               for (int e = 0; e < 4; ++e) {
+                const uint32_t x = v[c * 4 + e];
                 float a0, a1;
-                fma2(a0, a1, __uint_as_float(w4[e] << 16), __uint_as_float(w4[e] & 0xffff0000u), kLog2e, -mxl);
+                fma2(a0, a1, bf16_lo(x), bf16_hi(x), kLog2e, -q_mxl);
                 a0 = ex2(a0) * sc, a1 = ex2(a1) * sc;
-                split2(a0, a1, w4[e], lo4[e]);
-                if (with_z) {
-                  const float2 zz = *reinterpret_cast<const float2 *>(&sm.z[c * 8 + e * 2]);
-                  dot = fmaf(a0, zz.x, dot);
-                  dot1 = fmaf(a1, zz.y, dot1);
-                }
+                split2(a0, a1, hi4[e], lo4[e]);
+                if (with_z) dot2(dot, dot1, a0, a1, zh[c * 8 + e * 2], zh[c * 8 + e * 2 + 1]);
               }
-              *at = make_uint4(w4[0], w4[1], w4[2], w4[3]);
-              *reinterpret_cast<uint4 *>(sm.kv[X] + sw128(row, c)) = make_uint4(lo4[0], lo4[1], lo4[2], lo4[3]);
+              *reinterpret_cast<uint4 *>(tileX + sw128(row, H * 8 + c)) = make_uint4(hi4[0], hi4[1], hi4[2], hi4[3]);
+              *reinterpret_cast<uint4 *>(sm.kv[X] + sw128(row, H * 8 + c)) = make_uint4(lo4[0], lo4[1], lo4[2], lo4[3]);
             }
             dot = (dot + dot1) * dec0;
-            dot1 = 0.f;
           } else {
-#pragma unroll 1
-            for (int c0 = 0; c0 < 16; c0 += 4) {
-              load_chunks(c0);
+            // shared normaliser: phi(q) 2^-M.  The factor goes into the exponent, so that a value is rounded once.
+            const bool some = has_lin && (!SUM || q_sum > 0.f);
+            const float shift = some ? q_mxl + lg2(q_sum) + (SUM ? 0.f : M) : CUDART_INF_F;
 #pragma unroll
-              for (int i = 0; i < 4; ++i) {
-                uint32_t w4[4] = {v4[i].x, v4[i].y, v4[i].z, v4[i].w};
+            for (int c = 0; c < 8; ++c) {
+              uint32_t o4[4];
 #pragma unroll
-                for (int e = 0; e < 4; ++e) w4[e] = pack_bf16x2(__uint_as_float(w4[e] << 16) * sc, __uint_as_float(w4[e] & 0xffff0000u) * sc);
-                v4[i] = make_uint4(w4[0], w4[1], w4[2], w4[3]);
-                if (with_z) {
-#pragma unroll
-                  for (int e = 0; e < 4; ++e) {
-                    const float2 zz = *reinterpret_cast<const float2 *>(&sm.z[(c0 + i) * 8 + e * 2]);
-                    dot = fmaf(__uint_as_float(w4[e] << 16), zz.x, dot);
-                    dot1 = fmaf(__uint_as_float(w4[e] & 0xffff0000u), zz.y, dot1);
-                  }
-                }
+              for (int e = 0; e < 4; ++e) {
+                const uint32_t x = v[c * 4 + e];
+                float a0, a1;
+                fma2(a0, a1, bf16_lo(x), bf16_hi(x), kLog2e, -shift);
+                o4[e] = pack_bf16x2(ex2(a0), ex2(a1));
+                if (with_z) dot2(dot, dot1, bf16_lo(o4[e]), bf16_hi(o4[e]), zh[c * 8 + e * 2], zh[c * 8 + e * 2 + 1]);
               }
-#pragma unroll
-              for (int i = 0; i < 4; ++i) *reinterpret_cast<uint4 *>(tileX + sw128(row, c0 + i)) = v4[i];
+              *reinterpret_cast<uint4 *>(tileX + sw128(row, H * 8 + c)) = make_uint4(o4[0], o4[1], o4[2], o4[3]);
             }
+            dot += dot1;
           }
-          dot += dot1;
         } else {
-          // this thread's row of phi+ and of phi-: times 2^-M, back as bf16; the dot with z uses the rounded values
+          // this thread's part of phi+ and of phi-: times 2^-M, back as bf16; the dot with z uses the rounded values
 #pragma unroll 1
           for (int hf = 0; hf < 2; ++hf) {
             unsigned char *tile = hf == 0 ? tileX : sm.kv[X];
 #pragma unroll 4
-            for (int c = 0; c < 16; ++c) {
+            for (int c = H * 8; c < H * 8 + 8; ++c) {
               uint4 *at = reinterpret_cast<uint4 *>(tile + sw128(row, c));
               const uint4 v4 = *at;
               uint32_t w4[4] = {v4.x, v4.y, v4.z, v4.w};
 #pragma unroll
               for (int e = 0; e < 4; ++e) {
-                w4[e] = pack_bf16x2(__uint_as_float(w4[e] << 16) * fl, __uint_as_float(w4[e] & 0xffff0000u) * fl);
+                w4[e] = pack_bf16x2(bf16_lo(w4[e]) * fl, bf16_hi(w4[e]) * fl);
                 if (need_state)
-                  dot += __uint_as_float(w4[e] << 16) * sm.z[hf * kD + c * 8 + e * 2] +
-                         __uint_as_float(w4[e] & 0xffff0000u) * sm.z[hf * kD + c * 8 + e * 2 + 1];
+                  dot += bf16_lo(w4[e]) * sm.z[hf * kD + c * 8 + e * 2] + bf16_hi(w4[e]) * sm.z[hf * kD + c * 8 + e * 2 + 1];
               }
               *at = make_uint4(w4[0], w4[1], w4[2], w4[3]);
             }
@@ -819,18 +892,17 @@ prefill_attn_tc_kernel(const __grid_constant__ PrefillParams p, const CUtensorMa
         }
         l_sum += dot;
         if (windowed) {
-          ok = wait_s() && ok;                     // the last P V has completed
-          if (ok && __any_sync(0xffffffffu, fw != 1.f)) scale_o(fw);
+          wait_s();                                // the last P V has completed
+          if (__any_sync(0xffffffffu, fw != 1.f)) scale_o(fw);
         }
         fence_async_smem();
-        tc_fence_before();
-        mbar_arrive(smem_u32(&sm.bar_p[X]));
+        hand_over();
         PF_CLK(10);
-        if (GATED && need_state && ok) {
+        if (GATED && need_state) {
           // phi(q) S is in the S columns: it has decayed by dec0 since the chunk began, row by row, so it is added here
-          ok = wait_s();
+          wait_s();
 #pragma unroll 1
-          for (int c0 = 0; c0 < kD && ok; c0 += 32) {
+          for (int c0 = 0; c0 < kHalf; c0 += 32) {
             uint32_t o[32], x[32];
             tmem_ld32_nowait(tS + c0, x);
             if (windowed) tmem_ld32_nowait(tO + c0, o);
@@ -841,26 +913,24 @@ prefill_attn_tc_kernel(const __grid_constant__ PrefillParams p, const CUtensorMa
               o[i] = __float_as_uint(fmaf(__uint_as_float(x[i]), dec0, windowed ? __uint_as_float(o[i]) : 0.f));
             tmem_st32(tO + c0, o);
           }
-          tc_fence_before();
-          mbar_arrive(smem_u32(&sm.bar_p[X]));
+          hand_over();
         }
         // C row -> bf16 over the same TMEM columns, masked to the delayed tokens j' <= i of the row (the values already
         // carry 2^-M); the row's weight sum goes to l
-        for (int t = 0; t < n_itiles && ok; ++t) {
-          ok = wait_s();
-          if (!ok) break;
+        for (int t = 0; t < n_itiles; ++t) {
+          wait_s();
           PF_CLK(3);
           const int i0 = it0 + t * kKT;
           float sum0 = 0.f, sum1 = 0.f;
-          const int lo = i_lo - i0, hi = tl - i0;
+          const int lo = i_lo - i0 - H * kHalf, hi = tl - i0 - H * kHalf;
           // a tile that lies wholly before the row tile's first token (and after the first delayed token) needs no mask
           const bool whole = i0 + kKT - 1 <= tok0 + X * TOKT && i0 >= i_lo;
 #pragma unroll 1
-          for (int c = 0; c < kKT; c += 32) {
+          for (int c = 0; c < kHalf; c += 32) {
             uint32_t pk[16], x[32];
             const uint32_t m = whole ? ~0u : column_mask(c, lo, hi);
             // the running log-gates of the 32 columns' tokens, one per lane
-            const float gl = GATED ? __ldg(p.gcum + size_t(uc) * p.SC + min(i0 + c + lane, chunk_n - 1)) : 0.f;
+            const float gl = GATED ? __ldg(p.gcum + size_t(uc) * p.SC + min(i0 + H * kHalf + c + lane, chunk_n - 1)) : 0.f;
             if (!__any_sync(0xffffffffu, m)) {   // no row of the warp has a delayed token here
 #pragma unroll
               for (int e = 0; e < 16; ++e) pk[e] = x[e] = 0u;
@@ -885,27 +955,27 @@ prefill_attn_tc_kernel(const __grid_constant__ PrefillParams p, const CUtensorMa
                 split2(a0, a1, pk[e], x[e]);
               } else {
                 pk[e] = pack_bf16x2(__uint_as_float(x[e * 2]), __uint_as_float(x[e * 2 + 1]));
-                add2(sum0, sum1, __uint_as_float(pk[e] << 16), __uint_as_float(pk[e] & 0xffff0000u));
+                add2(sum0, sum1, bf16_lo(pk[e]), bf16_hi(pk[e]));
               }
             }
             store_p(c, pk, x);
           }
           tmem_wait_st();
           if (!SUM) l_sum += sum0 + sum1;
-          tc_fence_before();
-          mbar_arrive(smem_u32(&sm.bar_p[X]));
+          hand_over();
           PF_CLK(4);
         }
       }
       // ---- normalise and store: through the Q tile (every product that read it has completed), so that a warp's stores
-      // are whole rows ----
-      if (ok && (windowed || linear)) ok = wait_s();   // every product of X has completed
-      PF_CLK(5);
-      if (ok && (windowed || linear)) {
-        const float inv = tok_r < ntokX ? 1.0f / l_sum : 0.f;
+      // are whole lines ----
+      if (windowed || linear) {
+        const float l_row = row_sum_of(l_sum);
+        wait_s();                                  // every product of X has completed
+        PF_CLK(5);
+        const float inv = tok_r < ntokX ? 1.0f / l_row : 0.f;
         float chk0 = 0.f, chk1 = 0.f;   // gated: sums of the row's values, finite if all of them are
 #pragma unroll 1
-        for (int c0 = 0; c0 < kD; c0 += 32) {
+        for (int c0 = 0; c0 < kHalf; c0 += 32) {
           uint32_t r[32];
           tmem_ld32(tO + c0, r);
           if (GATED) {
@@ -918,67 +988,68 @@ prefill_attn_tc_kernel(const __grid_constant__ PrefillParams p, const CUtensorMa
 #pragma unroll
             for (int e = 0; e < 4; ++e)
               pk[e] = pack_bf16x2(__uint_as_float(r[q4 * 8 + e * 2]) * inv, __uint_as_float(r[q4 * 8 + e * 2 + 1]) * inv);
-            *reinterpret_cast<uint4 *>(sm.q[X] + sw128(row, (c0 >> 3) + q4)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+            *reinterpret_cast<uint4 *>(sm.q[X] + sw128(row, H * 8 + (c0 >> 3) + q4)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
           }
         }
-        // a warp stores the 32 rows its own threads have written (lanes 0-15 one row, lanes 16-31 the next); a lane's rows
-        // are 2 apart
+        // a warp stores the 32 half rows its own threads have written, eight lanes to each; a lane's rows are 4 apart
         __syncwarp();
-        const int c = lane & 15, r0 = (row & ~31) + (lane >> 4);
-        const int my_head = p.heads_of[g * G + lane % G];   // (head of group member h: lane h has it)
+        const int c = H * 8 + (lane & 7), r0 = (row & ~31) + (lane >> 3);
         bf16 *obase = reinterpret_cast<bf16 *>(p.out) + (seq + size_t(chunk_c0 + tok0 + X * TOKT)) * p.H * kD + c * 8;
 #pragma unroll 1
-        for (int i0 = 0; i0 < 16; i0 += 4) {
+        for (int i0 = 0; i0 < 8; i0 += 4) {
           uint4 val[4];
 #pragma unroll
-          for (int i = 0; i < 4; ++i) val[i] = *reinterpret_cast<const uint4 *>(sm.q[X] + sw128(r0 + 2 * (i0 + i), c));
+          for (int i = 0; i < 4; ++i) val[i] = *reinterpret_cast<const uint4 *>(sm.q[X] + sw128(r0 + 4 * (i0 + i), c));
 #pragma unroll
           for (int i = 0; i < 4; ++i) {
-            const int rr = r0 + 2 * (i0 + i), tk = rr / G;
+            const int rr = r0 + 4 * (i0 + i), tk = rr / G;
             const int head = __shfl_sync(0xffffffffu, my_head, rr - tk * G);
-            if (tk < ntokX) *reinterpret_cast<uint4 *>(obase + (size_t(tk) * p.H + head) * kD) = val[i];
+            if (ok && tk < ntokX) *reinterpret_cast<uint4 *>(obase + (size_t(tk) * p.H + head) * kD) = val[i];
           }
         }
         if constexpr (GATED) {
-          __syncwarp();
-          const unsigned again = __ballot_sync(0xffffffffu, !isfinite((chk0 + chk1) * inv) && tok_r < ntokX);
-          if (again) recompute_rows<G>(p, again, X * kRows + (row & ~31), u, sub, tok0);
+          // rows of which either half is not finite, by the first warp of the pair when both have stored
+          const bool bad = !isfinite((chk0 + chk1) * inv) && tok_r < ntokX;
+          const unsigned again = __ballot_sync(0xffffffffu, row_sum_of(bad ? 1.f : 0.f) > 0.f);
+          if (H == 0 && again && ok) recompute_rows<G>(p, again, X * kRows + (row & ~31), u, sub, tok0);
         }
       }
     }
-  } else if (warp == kMmaWarp) {
-    // =========================== MMA warp ===========================
-    // The warp stays together (every wait ends in a vote), one elected lane issues.
+  } else if (warp < kLoadWarp) {
+    // =========================== MMA warps ===========================
+    // A warp stays together (every wait ends in a vote), one elected lane issues.
     const bool leader = elect_one();
     const uint32_t tm = __shfl_sync(0xffffffffu, tmem, 0);
-    const int nx = hasB ? 2 : 1;
-    const int tf0 = t_first(0), tf1 = t_first(1), te0 = t_end(0), te1 = hasB ? t_end(1) : 0;
-    uint32_t p_phase = 0;                          // bit x: parity of the next operand of X
-    bool ok = true;
+    const int x = __shfl_sync(0xffffffffu, warp, 0) - kMmaWarp;   // the row tile
+    const uint32_t tS = tm + uint32_t(x) * 128u, tO = tS + 256u;
+    const int tf = t_first(x), te = t_end(x);
+    uint32_t p_phase = 0;                          // parity of the next operand
+    bool ok = x == 0 || hasB;
     auto wait = [&](uint64_t &bar, uint32_t parity) {
       ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&bar), parity, failed));
-      tc_fence_after();
       return ok;
     };
-    auto wait_p = [&](int x) {
-      const uint32_t par = (p_phase >> x) & 1u;
-      p_phase ^= 1u << x;
-      return wait(sm.bar_p[x], par);
+    auto wait_p = [&]() {
+      const uint32_t par = p_phase;
+      p_phase ^= 1u;
+      wait(sm.bar_p[x], par);
+      tc_fence_after();
+      return ok;
     };
     auto commit = [&](uint64_t &bar) {
       if (leader) mma_commit(smem_u32(&bar));
     };
-    // O_X (+)= A_X B with A_X in the S columns of X: packed bf16 behind one another, or hi and lo in turn every 32 columns
-    auto issue_ts = [&](int x, uint32_t b_tile, bool accumulate) {
+    // O (+)= A B with A in the S columns: packed bf16, or hi and lo in turn every 32 columns
+    auto issue_ts = [&](uint32_t b_tile, bool accumulate) {
       if (!GATED) {
-        issue_mma_ts<false>(leader, tm + 256 + x * 128, tm + x * 128, b_tile, accumulate);
+        issue_mma_ts<false>(leader, tO, tS, b_tile, accumulate);
       } else {
-        issue_mma_ts<true>(leader, tm + 256 + x * 128, tm + x * 128, b_tile, accumulate);
-        issue_mma_ts<true>(leader, tm + 256 + x * 128, tm + x * 128 + 16, b_tile, true);
+        issue_mma_ts<true>(leader, tO, tS, b_tile, accumulate);
+        issue_mma_ts<true>(leader, tO, tS + 16, b_tile, true);
       }
     };
     // D (+)= [Q tile of X | buffer X] . [buffer 2 | buffer 3], the map's halves or hi and lo
-    auto issue_two = [&](int x, uint32_t d, bool b_mn, bool accumulate) {
+    auto issue_two = [&](uint32_t d, bool b_mn, bool accumulate) {
       issue_mma(leader, d, q_addr(x), kv_addr(2), b_mn, accumulate);
       if (GATED) {
         issue_mma(leader, d, kv_addr(x), kv_addr(2), b_mn, true);
@@ -988,38 +1059,41 @@ prefill_attn_tc_kernel(const __grid_constant__ PrefillParams p, const CUtensorMa
       }
     };
     PF_LAP_INIT();
-    // t = -1: the first S products; then per key tile P V of the tile and S of the next one
+    // t = -1: the first S product; then per key tile P V of the tile and S of the next one.  The two warps take turns: products of
+    // A and B that run mixed end together, and then both tiles' softmax runs beside nothing (5000 cycles per key tile against
+    // 3700).  Buffers are freed by the softmax threads when they see the next product's completion, and only those that no
+    // later product follows here: a commit takes a place in the tensor core's queue.
     for (int t = -1; t < n_tiles && ok; ++t) {
       const int seqV = 2 * t + 1, seqK = 2 * t + 2;
       const bool more = t + 1 < n_tiles;
+      const bool pv = t >= tf && t < te, qk = t + 1 >= tf && t + 1 < te;
       PF_LAP(18);
       if (t >= 0) wait(sm.bar_full[seqV % kStages], uint32_t(seqV / kStages) & 1u);
-      PF_LAP(16);
       if (ok && more) wait(sm.bar_full[seqK % kStages], uint32_t(seqK / kStages) & 1u);
+      PF_LAP(16);
+      if (ok && qk && t + 1 == tf) wait(sm.bar_q[x], 0u);
+      if (ok && hasB && (x == 1 || t >= 0)) wait(sm.bar_turn[x], uint32_t(x == 1 ? t + 1 : t) & 1u);
       PF_LAP(17);
-#pragma unroll 1
-      for (int x = 0; x < nx && ok; ++x) {
-        const int tf = x ? tf1 : tf0, te = x ? te1 : te0;
-        if (t >= tf && t < te) {
-          PF_LAP(18);
-          if (!wait_p(x)) break;
-          PF_LAP(19);
-          issue_ts(x, kv_addr(seqV % kStages), t > tf);
-          if (t + 1 == te) commit(sm.bar_s[x]);   // the window part of O_X
-        }
-        if (t + 1 >= tf && t + 1 < te) {
-          if (t + 1 == tf && !wait(sm.bar_q[x], 0u)) break;
-          issue_mma(leader, tm + x * 128, q_addr(x), kv_addr(seqK % kStages), false, false);
-          commit(sm.bar_s[x]);
-        }
+      if (ok && pv) wait_p();
+      if (!ok) break;
+      PF_LAP(19);
+      if (pv) {
+        issue_ts(kv_addr(seqV % kStages), t > tf);
+        if (t + 1 == te) commit(sm.bar_s[x]);      // the window part of O
       }
-      if (ok) {
-        if (t >= 0) commit(sm.bar_free[seqV % kStages]);
-        if (more) commit(sm.bar_free[seqK % kStages]);
+      if (qk) {
+        issue_mma(leader, tS, q_addr(x), kv_addr(seqK % kStages), false, false);
+        commit(sm.bar_s[x]);
+      }
+      if (leader) {
+        if (hasB) mbar_arrive(smem_u32(&sm.bar_turn[x ^ 1]));
+        if (pv && t + 1 == te) mma_commit(smem_u32(&sm.bar_free[seqV % kStages]));
+        if (!pv && t >= 0) mbar_arrive(smem_u32(&sm.bar_free[seqV % kStages]));   // (a tile without a valid key for this row tile)
+        if (!qk && more) mbar_arrive(smem_u32(&sm.bar_free[seqK % kStages]));
       }
       // The query rows of the CTA that will take this place one wave later are asked into L2 (line by line: bulk prefetches of
       // the rows took the memory pipe 12000 cycles; before the first products the address arithmetic held them up by 1900).
-      if (t < 0 && blockIdx.x + unsigned(p.sm_count) < gridDim.x) {
+      if (t < 0 && x == (hasB ? 1 : 0) && blockIdx.x + unsigned(p.sm_count) < gridDim.x) {
         const unsigned nb = blockIdx.x + unsigned(p.sm_count), nu = nb / unsigned(ctas_per_unit);
         const int ncta = ctas_per_unit - 1 - int(nb - nu * unsigned(ctas_per_unit)), nsub = ncta / ctas_per_chunk;
         const int ncol = (ncta - nsub * ctas_per_chunk) * TOKC, ntok0 = nsub * p.SC + ncol;   // relative to the pass
@@ -1033,30 +1107,23 @@ prefill_attn_tc_kernel(const __grid_constant__ PrefillParams p, const CUtensorMa
       }
     }
     if (ok) commit(sm.bar_done);
+    const bool windowed = te > tf;
     if (ok && linear && !TWO) {
-      // the first C = phi(Q) phi(K')^T of each row tile, then phi(Q) S (inter-chunk): the softmax threads convert C while the
-      // state's products run (their completion shows in the next batch)
-#pragma unroll 1
-      for (int x = 0; x < nx && ok; ++x) {
-        if (!wait_p(x) || !wait(sm.bar_pk[0], 0u)) break;
-        issue_mma(leader, tm + x * 128, q_addr(x), kv_addr(slot_pk(0)), false, false);
+      // the first C = phi(Q) phi(K')^T, then phi(Q) S (inter-chunk): the softmax threads convert C while the state's product
+      // runs (its completion shows in the next batch)
+      if (wait_p() && wait(sm.bar_pk[0], 0u)) {
+        issue_mma(leader, tS, q_addr(x), kv_addr(slot_pk(0)), false, false);
         commit(sm.bar_s[x]);
       }
-      if (ok && need_state && wait(sm.bar_state, 0u))
-#pragma unroll 1
-        for (int x = 0; x < nx; ++x)
-          issue_mma(leader, tm + 256 + x * 128, q_addr(x), kv_addr(slot_state()), true, x ? te1 > tf1 : te0 > tf0);
+      if (ok && need_state && wait(sm.bar_state, 0u)) issue_mma(leader, tO, q_addr(x), kv_addr(slot_state()), true, windowed);
       for (int t = 0; t < n_itiles && ok; ++t) {
         wait(sm.bar_vp[t & 1], uint32_t(t >> 1) & 1u);
         if (ok && t + 1 < n_itiles) wait(sm.bar_pk[(t + 1) & 1], uint32_t((t + 1) >> 1) & 1u);
-#pragma unroll 1
-        for (int x = 0; x < nx && ok; ++x) {
-          if (!wait_p(x)) break;
-          issue_ts(x, kv_addr(slot_vp(t)), (x ? te1 > tf1 : te0 > tf0) || need_state || t > 0);
-          if (t + 1 < n_itiles) issue_mma(leader, tm + x * 128, q_addr(x), kv_addr(slot_pk(t + 1)), false, false);
-          commit(sm.bar_s[x]);
-        }
-        if (ok) commit(sm.bar_lfree[t & 1]);   // V'(t) has been read, and phi(K')(t) before it
+        if (!ok || !wait_p()) break;
+        issue_ts(kv_addr(slot_vp(t)), windowed || need_state || t > 0);
+        if (t + 1 < n_itiles) issue_mma(leader, tS, q_addr(x), kv_addr(slot_pk(t + 1)), false, false);
+        commit(sm.bar_s[x]);
+        commit(sm.bar_lfree[t & 1]);   // V'(t) has been read, and phi(K')(t) before it
       }
     }
     if (ok && linear && TWO) {
@@ -1064,30 +1131,20 @@ prefill_attn_tc_kernel(const __grid_constant__ PrefillParams p, const CUtensorMa
       // and C V'; the phi(K') halves of a step take the buffers of the state, or of the step before.  Gated: phi(Q) S goes
       // to the S columns, from where the softmax threads add it to O with the row's decay.
       if (GATED && need_state) wait(sm.bar_state, 0u);
-#pragma unroll 1
-      for (int x = 0; x < nx && ok; ++x) {
-        if (!wait_p(x)) break;
-        if (need_state) issue_two(x, GATED ? tm + x * 128 : tm + 256 + x * 128, true, !GATED && (x ? te1 > tf1 : te0 > tf0));
+      if (ok && wait_p()) {
+        if (need_state) issue_two(GATED ? tS : tO, true, !GATED && windowed);
         if (GATED && need_state) commit(sm.bar_s[x]);
+        commit(sm.bar_lfree[0]);
       }
-      if (ok) commit(sm.bar_lfree[0]);
-#pragma unroll 1
-      for (int x = 0; GATED && need_state && x < nx && ok; ++x) wait_p(x);   // the state's part has left the S columns
+      if (GATED && need_state && ok) wait_p();   // the state's part has left the S columns
       for (int t = 0; t < n_itiles && ok; ++t) {
-        wait(sm.bar_pk[0], uint32_t(t) & 1u);
-#pragma unroll 1
-        for (int x = 0; x < nx && ok; ++x) {
-          issue_two(x, tm + x * 128, false, false);
-          commit(sm.bar_s[x]);
-        }
-        if (ok) wait(sm.bar_vp[0], uint32_t(t) & 1u);
-#pragma unroll 1
-        for (int x = 0; x < nx && ok; ++x) {
-          if (!wait_p(x)) break;
-          issue_ts(x, kv_addr(4), (x ? te1 > tf1 : te0 > tf0) || need_state || t > 0);
-          if (t + 1 == n_itiles) commit(sm.bar_s[x]);
-        }
-        if (ok) commit(sm.bar_lfree[0]);
+        if (!wait(sm.bar_pk[0], uint32_t(t) & 1u)) break;
+        issue_two(tS, false, false);
+        commit(sm.bar_s[x]);
+        if (!wait(sm.bar_vp[0], uint32_t(t) & 1u) || !wait_p()) break;
+        issue_ts(kv_addr(4), windowed || need_state || t > 0);
+        if (t + 1 == n_itiles) commit(sm.bar_s[x]);
+        commit(sm.bar_lfree[0]);
       }
     }
   } else {
@@ -1115,11 +1172,8 @@ prefill_attn_tc_kernel(const __grid_constant__ PrefillParams p, const CUtensorMa
     // that one thread fetches, then the V' tiles of the intra-chunk steps (with the phi(K') tiles of later steps).
     const int n_window = 2 * n_tiles;
     const int n_jobs = n_window + (linear ? 1 + n_itiles : 0);
-    const int meet_job = n_window > 0 ? 1 : 0;   // (a CTA has no job or at least two; only a window's first tile waits for nobody)
-    if (n_jobs == 0) meet();
 #pragma unroll 1
     for (int job = 0; job < n_jobs; ++job) {
-      if (job == meet_job) meet();
       if (job == n_window) {
         if (lane == 0 && !TWO) {
           // the bf16 state (with z), then the phi(K') tiles of the first two intra-chunk steps
@@ -1172,7 +1226,7 @@ prefill_attn_tc_kernel(const __grid_constant__ PrefillParams p, const CUtensorMa
       const bool is_v = late || (job & 1);
       const int slot = late ? slot_vp(ts) : job % kStages;
       const uint32_t bar = late ? smem_u32(&sm.bar_vp[TWO ? 0 : ts & 1]) : smem_u32(&sm.bar_full[slot]);
-      const int64_t j0 = late ? folded + it0 + int64_t(ts) * kKT : j_lo + int64_t(ts) * kKT;
+      const int j0 = late ? folded + it0 + ts * kKT : j_lo + ts * kKT;
       if (!late) {
         PF_LAP_INIT();
         if (job >= kStages) ok = mbar_wait(smem_u32(&sm.bar_free[slot]), uint32_t(job / kStages - 1) & 1u, failed);
@@ -1201,16 +1255,16 @@ prefill_attn_tc_kernel(const __grid_constant__ PrefillParams p, const CUtensorMa
       }
       ok = __all_sync(0xffffffffu, ok);
       if (!ok) break;
-      const int64_t left = tq_last - j0;                         // >= 0: the tile holds at least one valid token
-      const int ngroups = left >= kKT - 1 ? kKT / kGroup : int(left / kGroup) + 1;
+      const int left = tq_last - j0;                         // >= 0: the tile holds at least one valid token
+      const int ngroups = left >= kKT - 1 ? kKT / kGroup : left / kGroup + 1;
       // A full tile that lies in one source without a wrap takes two boxes of 128 rows (the layout in shared memory
       // is that of eight 16-row boxes).  Tiles that reach past the last token keep the 16-row path, which never
       // loads a later token's row.  (left >= kKT - 1: every row of the tile is a token up to the last one; eight groups
       // alone would also admit a last group that is only partly valid)
       if (j0 >= 0 && left >= kKT - 1) {
-        const uint32_t slot_row0 = (j0 >> 32) == 0 ? uint32_t(j0) % cap : uint32_t(uint64_t(j0) % cap);
-        const bool all_call = j0 >= p.n0;
-        if (all_call || (j0 + kKT <= p.n0 && slot_row0 + kKT <= cap)) {
+        const uint32_t slot_row0 = uint32_t(j0) % cap;
+        const bool all_call = j0 >= n0;
+        if (all_call || (j0 + kKT <= n0 && slot_row0 + kKT <= cap)) {
           if (lane == 0) {
             mbar_expect_tx(bar, kTileBytes);
             const uint32_t dst = kv_addr(slot);
@@ -1220,11 +1274,11 @@ prefill_attn_tc_kernel(const __grid_constant__ PrefillParams p, const CUtensorMa
             const bool ahead = !late && ts + kAhead < n_tiles;
             if (all_call) {
               const CUtensorMap *m = is_v ? &cm.v128 : &cm.k128;
-              tma_load_4d(dst, m, 0, g, int(j0 - p.n0), lrel * p.B + b, bar);
-              tma_load_4d(dst + kBoxBytes, m, 64, g, int(j0 - p.n0), lrel * p.B + b, bar);
+              tma_load_4d(dst, m, 0, g, j0 - n0, lrel * p.B + b, bar);
+              tma_load_4d(dst + kBoxBytes, m, 64, g, j0 - n0, lrel * p.B + b, bar);
               if (ahead) {
-                tma_prefetch_4d(m, 0, g, int(j0 - p.n0) + kAhead * kKT, lrel * p.B + b);
-                tma_prefetch_4d(m, 64, g, int(j0 - p.n0) + kAhead * kKT, lrel * p.B + b);
+                tma_prefetch_4d(m, 0, g, j0 - n0 + kAhead * kKT, lrel * p.B + b);
+                tma_prefetch_4d(m, 64, g, j0 - n0 + kAhead * kKT, lrel * p.B + b);
               }
             } else {
               const CUtensorMap *m = is_v ? ringV128 : ringK128;
@@ -1241,11 +1295,11 @@ prefill_attn_tc_kernel(const __grid_constant__ PrefillParams p, const CUtensorMa
         }
       }
       // this lane's group: where it comes from and whether one box covers it
-      const int64_t j = j0 + gi * kGroup;
+      const int j = j0 + gi * kGroup;
       const bool mine = gi < kKT / kGroup && (late || gi < ngroups);
-      const bool from_call = j >= p.n0;
-      const uint32_t slot_row = j < 0 ? 0u : ((j >> 32) == 0 ? uint32_t(j) % cap : uint32_t(uint64_t(j) % cap));
-      const bool boxed = mine && gi < ngroups && j >= 0 && (from_call || (j + kGroup <= p.n0 && slot_row + kGroup <= cap));
+      const bool from_call = j >= n0;
+      const uint32_t slot_row = j < 0 ? 0u : uint32_t(j) % cap;
+      const bool boxed = mine && gi < ngroups && j >= 0 && (from_call || (j + kGroup <= n0 && slot_row + kGroup <= cap));
       const unsigned boxed_mask = __ballot_sync(0xffffffffu, boxed);
       const unsigned manual_mask = __ballot_sync(0xffffffffu, mine && !boxed);
       if (lane == 0) mbar_expect_tx(bar, uint32_t(__popc(boxed_mask)) * 2u * kGroupBytes);
@@ -1254,8 +1308,8 @@ prefill_attn_tc_kernel(const __grid_constant__ PrefillParams p, const CUtensorMa
         const uint32_t dst = kv_addr(slot) + uint32_t(gi) * kGroupBytes;
         if (from_call) {
           const CUtensorMap *m = is_v ? &cm.v : &cm.k;
-          tma_load_4d(dst, m, 0, g, int(j - p.n0), lrel * p.B + b, bar);
-          tma_load_4d(dst + kBoxBytes, m, 64, g, int(j - p.n0), lrel * p.B + b, bar);
+          tma_load_4d(dst, m, 0, g, j - n0, lrel * p.B + b, bar);
+          tma_load_4d(dst + kBoxBytes, m, 64, g, j - n0, lrel * p.B + b, bar);
         } else {
           tma_tile(dst, is_v ? ringV : ringK, int(unit_rows + slot_row), bar);
         }
@@ -1268,11 +1322,11 @@ prefill_attn_tc_kernel(const __grid_constant__ PrefillParams p, const CUtensorMa
         for (int i = 0; i < kGroup * 16 / 32; ++i) {
           const int id = lane + 32 * i;
           const int r = id >> 4, c = id & 15;
-          const int64_t jj = j0 + gm * kGroup + r;
+          const int jj = j0 + gm * kGroup + r;
           uint4 val = make_uint4(0u, 0u, 0u, 0u);
           if (jj >= 0 && jj <= tq_last) {
-            const uint32_t sr = (jj >> 32) == 0 ? uint32_t(jj) % cap : uint32_t(uint64_t(jj) % cap);
-            const bf16 *src = jj >= p.n0 ? (is_v ? callVp : callKp) + size_t(jj - p.n0) * call_stride
+            const uint32_t sr = uint32_t(jj) % cap;
+            const bf16 *src = jj >= n0 ? (is_v ? callVp : callKp) + size_t(jj - n0) * call_stride
                                          : (is_v ? ringVp : ringKp) + size_t(sr) * kD;
             val = *reinterpret_cast<const uint4 *>(src + c * 8);
           }
@@ -1369,7 +1423,7 @@ int launch_prefill_attn_tc(glide_ctx *ctx, const PrefillParams &pass, cudaStream
   auto launch = [&](auto gg) -> int {
     constexpr int G = decltype(gg)::value;
     constexpr int TOKC = 2 * kRows / G;
-    const size_t smem = sizeof(Smem) + 1024;
+    const size_t smem = sizeof(Smem);
     const int64_t blocks = units * (int64_t(p.nsub - 1) * ((p.SC + TOKC - 1) / TOKC) + (p.C - (p.nsub - 1) * p.SC + TOKC - 1) / TOKC);
     auto run = [&](auto kern) -> int {
       if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)) != cudaSuccess) {
