@@ -191,6 +191,7 @@ struct PrefillParams {
   int64_t *n_dev;            // [L] position counters
   int32_t sm_count;
   int32_t q_tma;             // tcgen05 kernel: the query rows come by TMA (every group's heads lie side by side)
+  int32_t sums_by_row;       // tensor-core pipeline: a chunk's sum lies row by row in its scratch rows (else by halves, see the carry kernels)
   int64_t advance;           // the pass's last kernel adds this to its layers' counters (0: none)
   float *gcum;               // gated: running sums of log(gate) of the chunk's delayed tokens, [units][Cmax]
 };
@@ -295,6 +296,7 @@ int launch_prefill_attn_mma(glide_ctx *ctx, const PrefillParams &p, cudaStream_t
 bool prefill_state_mma_supported(const glide_ctx *ctx);
 // make_phi: phi(K') (parameter-free map) is made by the carry kernel, which leaves its bf16 rows; otherwise it is in p.phik
 int launch_prefill_state_mma(const PrefillParams &p, bool make_phi, cudaStream_t stream);
+int launch_prefill_carry_tc(const PrefillParams &p, cudaStream_t stream);
 // up to four ranges of the workspace (8-byte aligned, sizes multiples of 8) set to zero by one launch
 struct ZeroRanges {
   unsigned char *ptr[4];

@@ -1,5 +1,6 @@
 // Chunk-scan carry of the prefill for bf16 I/O and d = 128 on the tensor cores, at fp32 accuracy:
 //   S += phi(K')^T V',  z += sum phi(K')      over the chunk's delayed tokens (k'_i = k_{i-w}).
+// (phi from the scratch, or gates; the parameter-free map without gates is the kernel of glide_prefill_carry_tc.cu.)
 // V' is bf16 already.  phi(K') is fp32 in the chunk scratch; every value is split into three bf16 terms
 // (x = hi + mid + lo, each the bf16 rounding of what the previous ones left: an error-free split of the 24-bit
 // significand), so the three products phi_term^T V' are exact in fp32 and only the fp32 accumulation of the tensor
@@ -10,10 +11,9 @@
 // One CTA of 4 warps per (unit, chunk of the pass, 64 state rows); warp w owns rows 16 w .. 16 w + 15 and all 128 columns
 // (16 n-tiles of m16n8k16, 64 accumulators per thread).  Tokens are staged 32 at a time through two shared-memory
 // buffers filled by cp.async; row strides are padded (272 bytes) so that the scalar reads of the A fragments and
-// the ldmatrix reads of V' are free of bank conflicts.  With the parameter-free map the kernel makes phi(K') itself from the
-// staged K' rows (both CTAs of a unit's chunk the whole row, for its normaliser, each keeping its 64 columns) and leaves
-// the bf16 rows for the attention kernel: as a kernel in front, phi cost a trip of 512 bytes per token through memory.
-// 8 x 2048 tokens, 4 layers: 107 us for phi and 126 for the carry, 188 together.
+// the ldmatrix reads of V' are free of bank conflicts.  In gated contexts with the parameter-free map the kernel makes phi(K')
+// itself from the staged K' rows (both CTAs of a unit's chunk the whole row, for its normaliser, each keeping its 64 columns) and
+// leaves the bf16 rows for the attention kernel: as a kernel in front, phi cost a trip of 512 bytes per token through memory.
 #include <algorithm>
 #include <type_traits>
 
@@ -96,7 +96,7 @@ __device__ __noinline__ float carry_element(const CarryRows &rows, const float *
 // of S (64 state rows x 128 values = 128 scratch rows x the CTA's 64 columns, z in row 128: chunks of more than 128
 // tokens), and prefill_scan_kernel adds the sums up in chunk order.  Otherwise S is updated in place, and its value
 // before the chunk is left as bf16 (z: fp32) for the attention kernel, which runs after this one.
-// MAKE_PHI: phi(K') is made here (parameter-free map); otherwise it is in the scratch.
+// MAKE_PHI: phi(K') is made here (parameter-free map, gated); otherwise it is in the scratch.
 template <bool PARTIAL, bool MAKE_PHI, bool GATED>
 __global__ void __launch_bounds__(kThreads, GATED ? 3 : 0) prefill_state_mma_kernel(const PrefillParams p) {
   using bf16 = __nv_bfloat16;
@@ -371,7 +371,8 @@ __global__ void __launch_bounds__(kThreads) prefill_scan_kernel(const PrefillPar
   const int k0 = first < 0 ? int(-first / p.SC) : 0;
   const int ub = (b + p.b0) * p.Hkv + g;
   const int r = j * 4 + (tid >> 5), col = (tid & 31) * 4;
-  const float *part = p.phik + (size_t(u) * p.Cmax + 2 * (r & 63) + (col >> 6)) * p.dp + (r >> 6) * 64 + (col & 63);
+  const float *part = p.sums_by_row ? p.phik + size_t(u) * p.Cmax * kD + r * kD + col
+                                    : p.phik + (size_t(u) * p.Cmax + 2 * (r & 63) + (col >> 6)) * p.dp + (r >> 6) * 64 + (col & 63);
   const size_t step = size_t(p.SC) * p.dp;
   float4 *Sp = reinterpret_cast<float4 *>(reinterpret_cast<float *>(p.ws + ld.S) + (size_t(ub) * p.dp + r) * kD + col);
   const int half = r / kD;
@@ -422,8 +423,18 @@ bool prefill_state_mma_supported(const glide_ctx *ctx) {
   return ctx->cfg.io_dtype == GLIDE_BF16 && ctx->cfg.head_dim == kD;
 }
 
-int launch_prefill_state_mma(const PrefillParams &p, bool make_phi, cudaStream_t stream) {
+int launch_prefill_state_mma(const PrefillParams &pass, bool make_phi, cudaStream_t stream) {
+  PrefillParams p = pass;
+  p.sums_by_row = make_phi && !p.gated;
   const int64_t units = int64_t(p.layer_count) * p.B * p.Hkv;
+  auto scan = [&]() -> int {
+    if (p.nsub > 1) prefill_scan_kernel<<<unsigned(units * (p.dp / 4)), kThreads, 0, stream>>>(p);
+    return cudaGetLastError() == cudaSuccess ? GLIDE_OK : GLIDE_ERR_CUDA;
+  };
+  if (p.sums_by_row) {
+    const int rc = launch_prefill_carry_tc(p, stream);
+    return rc ? rc : scan();
+  }
   const unsigned blocks = unsigned(units * p.nsub * (p.dp / kRowsPerCta));
   auto run = [&](auto partial, auto make, auto gated) {
     prefill_state_mma_kernel<decltype(partial)::value, decltype(make)::value, decltype(gated)::value><<<blocks, kThreads, 0, stream>>>(p);
@@ -434,15 +445,11 @@ int launch_prefill_state_mma(const PrefillParams &p, bool make_phi, cudaStream_t
     if (p.nsub > 1) run(yes, yes, yes);
     else if (make_phi) run(no, yes, yes);
     else run(no, no, yes);
-  } else if (make_phi) {
-    if (p.nsub > 1) run(yes, yes, no);
-    else run(no, yes, no);
   } else {
     if (p.nsub > 1) run(yes, no, no);
     else run(no, no, no);
   }
-  if (p.nsub > 1) prefill_scan_kernel<<<unsigned(units * (p.dp / 4)), kThreads, 0, stream>>>(p);
-  return cudaGetLastError() == cudaSuccess ? GLIDE_OK : GLIDE_ERR_CUDA;
+  return scan();
 }
 
 }  // namespace glide

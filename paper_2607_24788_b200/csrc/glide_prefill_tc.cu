@@ -35,6 +35,7 @@
 #include <algorithm>
 
 #include "glide_prefill_rows.cuh"
+#include "glide_tc.cuh"
 
 namespace glide {
 
@@ -51,44 +52,17 @@ constexpr int kMmaWarp = 16, kLoadWarp = 18;   // (MMA warps: one per row tile)
 constexpr uint32_t kTileBytes = 32768;   // [2 boxes][128 rows][64 bf16]
 constexpr uint32_t kBoxBytes = 16384;
 constexpr uint32_t kGroupBytes = kGroup * 128;   // one 16-token box of 64 columns
-constexpr uint32_t kWaitLimit = 1u << 20;
 constexpr float kLazy = 8.0f;         // rescale O only when the row maximum grows by more than 2^8
 constexpr int kStages = 5;
 
-__device__ __forceinline__ uint32_t smem_u32(const void *p) { return uint32_t(__cvta_generic_to_shared(p)); }
 // byte offset of 16-byte chunk c16 (0..15) of row `row` inside a [2][128][64] bf16 tile with 128-byte swizzle
 __device__ __forceinline__ uint32_t sw128(int row, int c16) {
   return uint32_t((c16 >> 3) * kBoxBytes + row * 128 + (((c16 & 7) ^ (row & 7)) << 4));
-}
-__device__ __forceinline__ void cp_async16(uint32_t dst, const void *src, bool valid) {
-  const int bytes = valid ? 16 : 0;
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
-__device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
-__device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ float ex2(float x) {
-  float y;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
-__device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
-  uint32_t r;
-  asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
-  return r;
 }
 // instruction descriptor: fp32 accumulate, bf16 A and B, M = N = 128; b_mn: B operand is MN-major
 __device__ __forceinline__ uint32_t make_idesc(bool b_mn) {
   return (1u << 4) | (1u << 7) | (1u << 10) | (b_mn ? (1u << 16) : 0u) | ((128u >> 3) << 17) | ((128u >> 4) << 24);
 }
-// Shared-memory matrix descriptor, 128-byte swizzle, as its two words: address and leading offset in the low one, the rest
-// constant.  The steps of a product differ by constants in the address field (16-byte units; no tile crosses its range).
-__device__ __forceinline__ uint32_t desc_lo(uint32_t saddr, uint32_t lbo_bytes) {
-  return ((saddr & 0x3FFFF) >> 4) | ((lbo_bytes >> 4) << 16);
-}
-constexpr uint32_t kDescHi = (1024u >> 4) | (1u << 14) | (2u << 29);
 // 8 MMAs of one 128 x 128 x 128 product; B K-major (D = A B^T) or MN-major (D (+)= A B).  Called by the MMA warp as a
 // whole, with operands that are the same in all lanes: the instruction takes them from uniform registers, and in code of
 // one diverged lane every step moved them there anew (3400 cycles to issue the 32 MMAs of a key tile, which run in 2048).
@@ -124,37 +98,6 @@ __device__ __forceinline__ void issue_mma_ts(bool leader, uint32_t tmem_d, uint3
           "r"(tmem_a + (PAIRS ? (ks >> 1) * 32 + (ks & 1) * 8 : (ks >> 2) * 64 + (ks & 3) * 8)), "r"(b0 + uint32_t(ks * 2048 >> 4)), "r"(idesc), "r"((accumulate || ks > 0) ? 1u : 0u), "r"(kDescHi)
           : "memory");
   }
-}
-__device__ __forceinline__ bool elect_one() {
-  uint32_t p;
-  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
-  return p != 0;
-}
-__device__ __forceinline__ void mma_commit(uint32_t bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
-}
-__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
-}
-__device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-}
-// Bounded wait; gives up early when another thread of the CTA has already timed out.
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int *failed) {
-  for (uint32_t spin = 0; spin < kWaitLimit; ++spin) {
-    uint32_t ok;
-    asm volatile("{.reg .pred p; mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2; selp.u32 %0, 1, 0, p;}"
-                 : "=r"(ok)
-                 : "r"(bar), "r"(parity)
-                 : "memory");
-    if (ok) return true;
-    if ((spin & 1023u) == 1023u && *failed) return false;
-  }
-  *failed = 1;
-  return false;
 }
 __device__ __forceinline__ void bulk_load(uint32_t dst, const void *src, uint32_t bytes, uint32_t bar) {
   asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
@@ -205,7 +148,6 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
   tmem_ld32_nowait(taddr, r);
   tmem_wait_ld(r);
 }
-__device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&r)[32]) {
   asm volatile(
       "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], "

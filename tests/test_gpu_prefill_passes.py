@@ -80,3 +80,26 @@ def test_passes_leave_the_same_state(dtype, d, kw):
     for other in states[1:]:
         for a, b in zip(states[0], other):
             assert torch.equal(a, b)
+
+
+# Chunk sums on tcgen05: stages of 32 tokens with every kind of remainder, the first delayed token inside a stage, chunks from one
+# stage to the largest (passes of one chunk update S in place), rings that wrap, no ring at all.  Against fp64; bound: the tensor core
+# adds 3 chunk / 16 products to a running sum without rounding to nearest (2^-23 of it each at most), the scan one sum per chunk.
+@pytest.mark.parametrize("chunk,w,calls", [(64, 16, [97]), (144, 0, [145, 31]), (160, 33, [481, 1]), (256, 300, [513, 40, 700]), (1024, 31, [1055]),
+                                           (0, 100, [101, 1000])])
+def test_chunk_sums_on_tcgen05(chunk, w, calls):
+    T = sum(calls)
+    gen = torch.Generator(device="cuda").manual_seed(chunk + w)
+    q, k, v = (torch.randn((1, 2, T, h, 128), generator=gen, device="cuda").to(BF16) for h in (4, 2, 2))
+    g = glide.Glide([w], 2, 4, 2, 128, 1 << 20, prefill_chunk=chunk)
+    at = 0
+    for n in calls:
+        part = [x[:, :, at:at + n].contiguous() for x in (q, k, v)]
+        g.glide_prefill(*part, torch.empty_like(part[0]))
+        at += n
+    S, z = g.glide_export_state(0)[2:]
+    phi = torch.softmax(k[0].double(), -1)[:, :T - w].transpose(1, 2)
+    for got, want in ((S, phi.transpose(-1, -2) @ v[0, :, :T - w].double().transpose(1, 2)), (z, phi.sum(2))):
+        bound = (3 * (chunk or 256) / 16 + T / (chunk or 256) + 2) * 2.0 ** -23
+        assert ((got - want).norm() / want.norm()).item() <= bound
+    assert g.glide_device_status() == 0
