@@ -482,59 +482,60 @@ __global__ void __launch_bounds__(kPrefillThreads) prefill_zcum_kernel(const Pre
   }
 }
 
-// 4. ring fill: the pass's newest min(C, cap) tokens, and the layers' counters on the last pass; one warp per (unit, kTokPerWarp consecutive chunk tokens)
+// 4. ring fill: the pass's newest min(C, cap) tokens, and the layers' counters on the last pass.  A CTA takes kRingTok of a unit's
+// tokens, a thread 16 bytes of a row; all of a thread's rows of K and V are asked for before any is stored.  (A warp per four
+// tokens with 8 bytes a lane, warps for the tokens that are not kept among them, and 64-bit remainders: 75.6 us for 8 x 2048 tokens
+// of 4 layers, 210 MB.)
+constexpr int kRingTok = 64, kRingThreads = 256;
 template <typename T, int D>
-__global__ void __launch_bounds__(kPrefillThreads) prefill_ring_kernel(const PrefillParams p) {
-  constexpr int E = D / 32;
-  const int lane = threadIdx.x & 31;
-  const int64_t wid = (int64_t(blockIdx.x) * kPrefillThreads + threadIdx.x) >> 5;
-  const int64_t units = int64_t(p.layer_count) * p.B * p.Hkv;
-  const int groups = (p.C + kTokPerWarp - 1) / kTokPerWarp;
+__global__ void __launch_bounds__(kRingThreads) prefill_ring_kernel(const PrefillParams p, int groups) {
+  constexpr int kChunks = D * int(sizeof(T)) / 16;               // 16-byte chunks of a row
+  constexpr int kRows = kRingThreads / kChunks;                  // rows that the CTA moves at a time
+  constexpr int kPer = (kRingTok + kRows - 1) / kRows;
   if (blockIdx.x == 0 && p.advance)
-    for (int l = threadIdx.x; l < p.layer_count; l += kPrefillThreads) p.n_dev[p.layer_begin + l] += p.advance;
-  if (wid >= units * groups) return;
-  const int i0 = int(wid % groups) * kTokPerWarp;
-  const int64_t u = wid / groups;
-  const int g = int(u % p.Hkv);
-  const int b = int((u / p.Hkv) % p.B);
-  const int lrel = int(u / (int64_t(p.Hkv) * p.B));
-  const LayerDev ld = p.layers[p.layer_begin + lrel];
-  if (ld.cap == 0) return;
-  T kx[kTokPerWarp][E], vx[kTokPerWarp][E];
-  bool valid[kTokPerWarp];
+    for (int l = threadIdx.x; l < p.layer_count; l += kRingThreads) p.n_dev[p.layer_begin + l] += p.advance;
+  const unsigned u = blockIdx.x / unsigned(groups), grp = blockIdx.x - u * unsigned(groups);
+  const unsigned ug = u / unsigned(p.Hkv), g = u - ug * unsigned(p.Hkv), lrel = ug / unsigned(p.B), b = ug - lrel * unsigned(p.B);
+  const LayerDev &ld = p.layers[p.layer_begin + int(lrel)];
+  const uint32_t cap = uint32_t(ld.cap);
+  const int kept = int(uint32_t(p.C) < cap ? uint32_t(p.C) : cap);   // (older tokens of the pass would be overwritten anyway)
+  const int i0 = p.C - kept + int(grp) * kRingTok;
+  if (i0 >= p.C) return;
+  const int c = threadIdx.x % kChunks, r0 = threadIdx.x / kChunks;
+  const size_t seq = (size_t(lrel) * p.B + b) * size_t(p.T) + size_t(p.c0);
+  const size_t unit = (size_t(b + p.b0) * p.Hkv + g) * size_t(cap);
+  const uint4 *ks = reinterpret_cast<const uint4 *>(p.k) + c, *vs = reinterpret_cast<const uint4 *>(p.v) + c;
+  uint4 *kd = reinterpret_cast<uint4 *>(p.ws + ld.ringK) + c, *vd = reinterpret_cast<uint4 *>(p.ws + ld.ringV) + c;
+  uint4 kx[kPer], vx[kPer];
 #pragma unroll
-  for (int r = 0; r < kTokPerWarp; ++r) {
-    const int i = i0 + r;
-    valid[r] = i < p.C && int64_t(i) >= int64_t(p.C) - ld.cap;   // older tokens of the chunk are overwritten anyway
-    if (valid[r]) {
-      const size_t src = (((size_t(lrel) * p.B + b) * size_t(p.T) + size_t(p.c0 + i)) * p.Hkv + g) * D + lane * E;
-      const T *ks = reinterpret_cast<const T *>(p.k) + src;
-      const T *vs = reinterpret_cast<const T *>(p.v) + src;
-#pragma unroll
-      for (int e = 0; e < E; ++e) {
-        kx[r][e] = ks[e];
-        vx[r][e] = vs[e];
-      }
+  for (int r = 0; r < kPer; ++r) {
+    const int i = i0 + r0 + r * kRows;
+    if (r0 + r * kRows < kRingTok && i < p.C) {
+      const size_t src = ((seq + size_t(i)) * p.Hkv + g) * kChunks;
+      kx[r] = ks[src];
+      vx[r] = vs[src];
     }
   }
 #pragma unroll
-  for (int r = 0; r < kTokPerWarp; ++r) {
-    if (!valid[r]) continue;
-    const int64_t j = p.n0 + p.c0 + i0 + r;
-    const size_t dst = ((size_t(b + p.b0) * p.Hkv + g) * size_t(ld.cap) + size_t(j % ld.cap)) * D + lane * E;
-    T *kd = reinterpret_cast<T *>(p.ws + ld.ringK) + dst;
-    T *vd = reinterpret_cast<T *>(p.ws + ld.ringV) + dst;
-#pragma unroll
-    for (int e = 0; e < E; ++e) {
-      kd[e] = kx[r][e];
-      vd[e] = vx[r][e];
-    }
-    if (p.gated && lane == 0) {   // the token's gate waits in the ring with it
-      const size_t slot = (size_t(b + p.b0) * p.Hkv + g) * size_t(ld.cap) + size_t(j % ld.cap);
-      reinterpret_cast<float *>(p.ws + ld.ringG)[slot] =
-          p.gate ? p.gate[((size_t(lrel) * p.B + b) * size_t(p.T) + size_t(p.c0 + i0 + r)) * p.Hkv + g] : 1.f;
+  for (int r = 0; r < kPer; ++r) {
+    const int i = i0 + r0 + r * kRows;
+    if (r0 + r * kRows < kRingTok && i < p.C) {
+      const size_t slot = unit + uint32_t(p.n0 + p.c0 + i) % cap;   // (positions stay below 2^30)
+      kd[slot * kChunks] = kx[r];
+      vd[slot * kChunks] = vx[r];
+      if (p.gated && c == 0)   // the token's gate waits in the ring with it
+        reinterpret_cast<float *>(p.ws + ld.ringG)[slot] = p.gate ? p.gate[(seq + size_t(i)) * p.Hkv + g] : 1.f;
     }
   }
+}
+// (host) the ring kernel over a pass: as many groups of tokens per unit as the longest ring of its layers keeps
+template <typename T, int D>
+void launch_ring(const glide_ctx *ctx, const PrefillParams &p, cudaStream_t stream) {
+  int64_t kept = 1;
+  for (int l = p.layer_begin; l < p.layer_begin + p.layer_count; ++l) kept = std::max(kept, std::min<int64_t>(p.C, ctx->layers[size_t(l)].cap));
+  const int groups = int((kept + kRingTok - 1) / kRingTok);
+  const int64_t units = int64_t(p.layer_count) * p.B * p.Hkv;
+  prefill_ring_kernel<T, D><<<unsigned(units * groups), kRingThreads, 0, stream>>>(p, groups);
 }
 
 // The ranges one after the other, 16 bytes per store where the address allows (S and z start on a 2 MiB multiple).  One
@@ -693,7 +694,7 @@ int launch_prefill(glide_ctx *ctx, int layer_begin, int layer_count, int64_t T, 
         if (launch_prefill_state_mma(s, make_phi, stream) != GLIDE_OK) return GLIDE_ERR_CUDA;
       }
       if (out && launch_prefill_attn_tc(ctx, s, stream) != GLIDE_OK) return GLIDE_ERR_CUDA;
-      prefill_ring_kernel<TT, D><<<warp4_blocks, kPrefillThreads, 0, stream>>>(s);
+      launch_ring<TT, D>(ctx, s, stream);
       return cudaGetLastError() == cudaSuccess ? GLIDE_OK : GLIDE_ERR_CUDA;
     });
   };
@@ -748,7 +749,7 @@ int launch_prefill(glide_ctx *ctx, int layer_begin, int layer_count, int64_t T, 
           prefill_state_kernel<TT, D><<<unsigned(units * (DP / kStateRows)), kPrefillThreads, 0, stream>>>(p);
         }
       }
-      prefill_ring_kernel<TT, D><<<warp4_blocks, kPrefillThreads, 0, stream>>>(p);
+      launch_ring<TT, D>(ctx, p, stream);
       if (cudaGetLastError() != cudaSuccess) return GLIDE_ERR_CUDA;
     }
     return GLIDE_OK;
