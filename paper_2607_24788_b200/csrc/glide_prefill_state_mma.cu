@@ -352,69 +352,86 @@ __global__ void __launch_bounds__(kThreads, GATED ? 3 : 0) prefill_state_mma_ker
 }
 
 // The chunk sums of a pass added up in chunk order: S and z of the context move on by the whole pass, and their values at
-// the start of every chunk are left for the attention kernel (bf16 copy of S, fp32 z) when there are outputs.  One CTA per
-// (unit, 4 rows of S), a thread owns four columns of a row; the sums of four chunks are loaded together, so that the
-// chain over the chunks is one of additions and not of memory round trips.
-__global__ void __launch_bounds__(kThreads) prefill_scan_kernel(const PrefillParams p) {
+// the start of every chunk are left for the attention kernel (bf16 copy of S, fp32 z) when there are outputs (SNAP).  One CTA per
+// (unit, 4 rows of S): four warps with four columns of a row per thread, and a fifth for z, whose four chains of one value per chunk
+// would hold up a warp that has its own.  The sums of the next four chunks are on their way while four are added.
+template <bool GATED, bool SNAP>
+__global__ void __launch_bounds__(kThreads + 32) prefill_scan_kernel(const PrefillParams p) {
   using bf16 = __nv_bfloat16;
-  const int ctas_per_unit = p.dp / 4;
-  const int64_t u = blockIdx.x / ctas_per_unit;
-  const int j = int(blockIdx.x % ctas_per_unit), tid = threadIdx.x;
-  const int g = int(u % p.Hkv);
-  const int b = int((u / p.Hkv) % p.B);
-  const int lrel = int(u / (int64_t(p.Hkv) * p.B));
-  const LayerDev ld = p.layers[p.layer_begin + lrel];
+  const unsigned ctas_per_unit = unsigned(p.dp) / 4;
+  const int u = int(blockIdx.x / ctas_per_unit);
+  const int j = int(blockIdx.x - unsigned(u) * ctas_per_unit), tid = threadIdx.x;
+  const int ug = u / p.Hkv, g = u - ug * p.Hkv, lrel = ug / p.B, b = ug - lrel * p.B;
+  const LayerDev &ld = p.layers[p.layer_begin + lrel];
   if (!ld.evicts) return;
   // chunks before the first delayed token add nothing (and have left no sum): k0 is the first that does
   const int64_t first = p.n0 + p.c0 - ld.wlin;
   if (first + p.C <= 0) return;
-  const int k0 = first < 0 ? int(-first / p.SC) : 0;
+  const int k0 = first < 0 ? int(-first) / p.SC : 0;
   const int ub = (b + p.b0) * p.Hkv + g;
-  const int r = j * 4 + (tid >> 5), col = (tid & 31) * 4;
-  const float *part = p.sums_by_row ? p.phik + size_t(u) * p.Cmax * kD + r * kD + col
-                                    : p.phik + (size_t(u) * p.Cmax + 2 * (r & 63) + (col >> 6)) * p.dp + (r >> 6) * 64 + (col & 63);
   const size_t step = size_t(p.SC) * p.dp;
-  float4 *Sp = reinterpret_cast<float4 *>(reinterpret_cast<float *>(p.ws + ld.S) + (size_t(ub) * p.dp + r) * kD + col);
-  const int half = r / kD;
-  bf16 *snap = p.s16 ? reinterpret_cast<bf16 *>(p.s16) + ((size_t(half) * p.units_cap + u * p.nsub) * kD + (r - half * kD)) * kD + col
-                     : nullptr;
-  float4 s = *Sp;
-  const size_t lo_half = p.gated ? size_t(p.units_cap) * kD * kD : 0;
   // gated: what the state has decayed by over chunk k (tokens before the first delayed one count as gates of 1)
-  const float *gc = p.gated ? p.gcum + size_t(u) * p.Cmax - 1 : nullptr;
-  auto chunk_decay = [&](int k) { return gc ? expf(gc[min((k + 1) * p.SC, p.C)]) : 1.f; };
-  constexpr int kAhead = 4;
-  for (int k = k0; k < p.nsub; k += kAhead) {
-    float4 x[kAhead];
+  const float *gc = GATED ? p.gcum + size_t(u) * p.Cmax - 1 : nullptr;
+  // f(k, value of the sum of chunk k) for every chunk, kAhead loads together
+  auto over_chunks = [&](auto ahead, auto load, auto &&f) {
+    constexpr int kAhead = decltype(ahead)::value;
+    using Value = decltype(load(0));
+    const int n = p.nsub;
+    Value x[kAhead], y[kAhead];
+#pragma unroll
+    for (int a = 0; a < kAhead; ++a) x[a] = load(min(k0 + a, n - 1));
+    int k = k0;
+    for (; k + kAhead <= n; k += kAhead) {
+#pragma unroll
+      for (int a = 0; a < kAhead; ++a) y[a] = load(min(k + kAhead + a, n - 1));
+#pragma unroll
+      for (int a = 0; a < kAhead; ++a) f(k + a, GATED ? expf(gc[min((k + a + 1) * p.SC, p.C)]) : 1.f, x[a]);
+#pragma unroll
+      for (int a = 0; a < kAhead; ++a) x[a] = y[a];
+    }
 #pragma unroll
     for (int a = 0; a < kAhead; ++a)
-      if (k + a < p.nsub) x[a] = *reinterpret_cast<const float4 *>(part + size_t(k + a) * step);
-#pragma unroll
-    for (int a = 0; a < kAhead; ++a) {
-      if (k + a >= p.nsub) break;
-      if (snap) {
-        store_s16(snap + size_t(k + a) * kD * kD, lo_half, s.x, s.y);
-        store_s16(snap + size_t(k + a) * kD * kD + 2, lo_half, s.z, s.w);
-      }
-      const float dec = chunk_decay(k + a);
-      s.x = fmaf(s.x, dec, x[a].x);
-      s.y = fmaf(s.y, dec, x[a].y);
-      s.z = fmaf(s.z, dec, x[a].z);
-      s.w = fmaf(s.w, dec, x[a].w);
-    }
-  }
-  *Sp = s;
-  if (tid < 4) {   // z of the CTA's four rows
-    const int rz = j * 4 + tid;
+      if (k + a < n) f(k + a, GATED ? expf(gc[min((k + a + 1) * p.SC, p.C)]) : 1.f, x[a]);
+  };
+  if (tid >= kThreads) {   // z of the CTA's four rows
+    if (tid >= kThreads + 4) return;
+    const int rz = j * 4 + tid - kThreads;
     const float *pz = p.phik + (size_t(u) * p.Cmax + kD) * p.dp + rz;
     float *zp = reinterpret_cast<float *>(p.ws + ld.z) + size_t(ub) * p.dp + rz;
     float z = *zp;
-    for (int k = k0; k < p.nsub; ++k) {
-      if (snap) p.zsnap[(size_t(u) * p.nsub + k) * p.dp + rz] = z;
-      z = fmaf(z, chunk_decay(k), pz[size_t(k) * step]);
-    }
+    over_chunks(IntTag<8>{}, [&](int k) { return pz[size_t(k) * step]; }, [&](int k, float dec, float x) {
+      if (SNAP) p.zsnap[(size_t(u) * p.nsub + k) * p.dp + rz] = z;
+      z = fmaf(z, dec, x);
+    });
     *zp = z;
+    return;
   }
+  const int r = j * 4 + (tid >> 5), col = (tid & 31) * 4;
+  const float *part = p.sums_by_row ? p.phik + size_t(u) * p.Cmax * kD + r * kD + col
+                                    : p.phik + (size_t(u) * p.Cmax + 2 * (r & 63) + (col >> 6)) * p.dp + (r >> 6) * 64 + (col & 63);
+  float4 *Sp = reinterpret_cast<float4 *>(reinterpret_cast<float *>(p.ws + ld.S) + (size_t(ub) * p.dp + r) * kD + col);
+  const int half = r / kD;
+  bf16 *snap = SNAP ? reinterpret_cast<bf16 *>(p.s16) + ((size_t(half) * p.units_cap + size_t(u) * p.nsub) * kD + (r - half * kD)) * kD + col
+                    : nullptr;
+  const size_t lo_half = size_t(p.units_cap) * kD * kD;
+  float4 s = *Sp;
+  over_chunks(IntTag<4>{}, [&](int k) { return *reinterpret_cast<const float4 *>(part + size_t(k) * step); }, [&](int k, float dec, const float4 &x) {
+    if (SNAP) {
+      bf16 *at = snap + size_t(k) * kD * kD;
+      const __nv_bfloat162 h0 = __floats2bfloat162_rn(s.x, s.y), h1 = __floats2bfloat162_rn(s.z, s.w);
+      *reinterpret_cast<uint2 *>(at) = make_uint2(*reinterpret_cast<const uint32_t *>(&h0), *reinterpret_cast<const uint32_t *>(&h1));
+      if (GATED) {
+        const __nv_bfloat162 l0 = __floats2bfloat162_rn(s.x - __low2float(h0), s.y - __high2float(h0));
+        const __nv_bfloat162 l1 = __floats2bfloat162_rn(s.z - __low2float(h1), s.w - __high2float(h1));
+        *reinterpret_cast<uint2 *>(at + lo_half) = make_uint2(*reinterpret_cast<const uint32_t *>(&l0), *reinterpret_cast<const uint32_t *>(&l1));
+      }
+    }
+    s.x = fmaf(s.x, dec, x.x);
+    s.y = fmaf(s.y, dec, x.y);
+    s.z = fmaf(s.z, dec, x.z);
+    s.w = fmaf(s.w, dec, x.w);
+  });
+  *Sp = s;
 }
 
 }  // namespace
@@ -428,7 +445,14 @@ int launch_prefill_state_mma(const PrefillParams &pass, bool make_phi, cudaStrea
   p.sums_by_row = make_phi && !p.gated;
   const int64_t units = int64_t(p.layer_count) * p.B * p.Hkv;
   auto scan = [&]() -> int {
-    if (p.nsub > 1) prefill_scan_kernel<<<unsigned(units * (p.dp / 4)), kThreads, 0, stream>>>(p);
+    if (p.nsub > 1) {
+      const unsigned ctas = unsigned(units * (p.dp / 4));
+      auto run = [&](auto gated, auto snap) { prefill_scan_kernel<decltype(gated)::value, decltype(snap)::value><<<ctas, kThreads + 32, 0, stream>>>(p); };
+      const std::true_type yes{};
+      const std::false_type no{};
+      if (p.gated) p.s16 ? run(yes, yes) : run(yes, no);
+      else p.s16 ? run(no, yes) : run(no, no);
+    }
     return cudaGetLastError() == cudaSuccess ? GLIDE_OK : GLIDE_ERR_CUDA;
   };
   if (p.sums_by_row) {
