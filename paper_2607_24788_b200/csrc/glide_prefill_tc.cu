@@ -33,6 +33,7 @@
 #include <cstring>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "glide_prefill_rows.cuh"
 #include "glide_tc.cuh"
@@ -620,25 +621,47 @@ prefill_attn_tc_kernel(const __grid_constant__ PrefillParams p, const CUtensorMa
       }
       store_p(c, pk, x);
     };
-    // One key tile without a masked key: two passes over the thread's columns (all 64 scores held between their maximum and their
-    // weights leave too few registers: 96 a thread).
-    auto soft_tile = [&](bool first) {
+    // One key tile against the reference as it is (0 for a row's first tile), in one pass: no maximum is looked for.  The largest
+    // weight says afterwards whether that was right: up to 2^32, and for a first tile not below 2^-32, fp32 sums and bf16 weights are
+    // as precise as against the maximum itself.  Otherwise (false, to both threads of all rows of the pair) nothing has
+    // happened, the scores are still there, and the tile goes through soft_tile_masked.  (Two passes: 1850 cycles a tile.)
+    auto soft_tile = [&](auto masked, int lo, int hi, bool first) {
       float sum0 = 0.f, sum1 = 0.f;
-      uint32_t x[32];
-      tmem_ld32(tS + 32, x);
-      float mx = row_max(x, -CUDART_INF_F);
-      tmem_ld32(tS, x);
-      mx = row_max(x, mx);
-      const float mr = move_ref(mx, first);
-      weights(0, x, mr, sum0, sum1);   // (over columns that have been read)
-      tmem_ld32(tS + 32, x);
-      weights(32, x, mr, sum0, sum1);
-      tmem_wait_st();
+      const float mr = first ? 0.f : m_ref;
+      uint32_t pk[32], mx2 = 0u;
+      bool some = false;
+#pragma unroll
+      for (int c = 0; c < kHalf; c += 32) {
+        uint32_t x[32];
+        tmem_ld32(tS + c, x);
+        if (decltype(masked)::value) {
+          const uint32_t m = column_mask(c, lo, hi);
+          some = some || m != 0;
+#pragma unroll
+          for (int i = 0; i < 32; ++i) x[i] = (m >> i) & 1u ? x[i] : 0xff800000u;
+        }
+#pragma unroll
+        for (int e = 0; e < 16; ++e) {
+          float a0, a1;
+          fma2(a0, a1, __uint_as_float(x[e * 2]), __uint_as_float(x[e * 2 + 1]), p.scale_log2, -mr);
+          const uint32_t w2 = pack_bf16x2(ex2(a0), ex2(a1));
+          mx2 = max_bf16x2(mx2, w2);
+          add2(sum0, sum1, bf16_lo(w2), bf16_hi(w2));   // the sum uses the weights as the tensor core sees them
+          pk[(c >> 1) + e] = w2;
+        }
+      }
+      const float mx = fmaxf(bf16_lo(mx2), bf16_hi(mx2));
+      const bool low = first && (some || !decltype(masked)::value) && mx < 0x1p-32f;
+      if (pair_any(!(mx <= 0x1p32f) || low)) return false;
+      tmem_st32(tS, pk);
       l_sum += sum0 + sum1;
+      if (first) m_ref = 0.f;
+      return true;
     };
     // One key tile with masked keys (valid columns lo .. hi of this row's half).  32 columns at a time, those in which no row of
     // the warp has a valid one left out; the loops stay rolled: with everything unrolled the kernel was 210 KB of code that a CTA
-    // fetched once per phase (a CTA's first key tile took 12000 cycles, a later one 2500).
+    // fetched once per phase (a CTA's first key tile took 12000 cycles, a later one 2500).  For gated contexts, rows that have no
+    // reference yet, and tiles that soft_tile leaves alone.
     auto soft_tile_masked = [&](int lo, int hi, bool first) {
       float mx = -CUDART_INF_F, sum0 = 0.f, sum1 = 0.f;
 #pragma unroll 1
@@ -716,12 +739,18 @@ prefill_attn_tc_kernel(const __grid_constant__ PrefillParams p, const CUtensorMa
         }
         if (t == tf) PF_CLK(11); else PF_CLK(12);
         const int j0 = j_lo + t * kKT;
-        if (j0 + kKT - 1 <= tqX0 && j0 > tqX_last - w) {
-          soft_tile(t == tf);
-        } else {
-          // valid columns of this row: lo <= c <= hi (a token more than 2^30 - 1 before another is none)
-          soft_tile_masked(max(tok_abs - w + 1 - j0, 0) - H * kHalf, min(tok_abs - j0, kKT - 1) - H * kHalf, t == tf);
+        const bool whole = j0 + kKT - 1 <= tqX0 && j0 > tqX_last - w;
+        // valid columns of this row: lo <= c <= hi (a token more than 2^30 - 1 before another is none)
+        const int lo = max(tok_abs - w + 1 - j0, 0), hi = min(tok_abs - j0, kKT - 1);
+        bool done = false;
+        if constexpr (!GATED) {
+          // (what is asked here is the same in both warps of a pair: their threads share the rows)
+          if (t == tf ? !__any_sync(0xffffffffu, lo > hi) : !__any_sync(0xffffffffu, m_ref == -CUDART_INF_F)) {
+            if (whole) done = soft_tile(std::false_type{}, 0, kHalf - 1, t == tf);
+            else done = soft_tile(std::true_type{}, lo - H * kHalf, hi - H * kHalf, t == tf);
+          }
         }
+        if (!done) soft_tile_masked(lo - H * kHalf, hi - H * kHalf, t == tf);
         hand_over();            // this thread's TMEM accesses precede the MMAs that read P and overwrite S
         if (t == tf) PF_CLK(13); else PF_CLK(14);
       }
