@@ -428,6 +428,8 @@ __global__ void __launch_bounds__(kUnitThreads<D, G>) glide_decode_unit_kernel(c
   __shared__ __align__(16) float lin[RPI][G][D];
   __shared__ __align__(16) float phiq[G][DP], phik[DP], ve_s[D];
   __shared__ float lin_b[G];
+  dependents_may_start();
+  wait_for_predecessor();
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int unit_rel = blockIdx.x, per_layer = p.B * p.Hkv;
   const int layer = p.layer_begin + unit_rel / per_layer, ub = unit_rel % per_layer;
@@ -900,7 +902,7 @@ int launch_decode(glide_ctx *ctx, int layer_begin, int layer_count, const void *
     using T = typename decltype(tt)::type;
     constexpr int D = decltype(dd)::value, G = decltype(gg)::value, DP = decltype(pp)::value;
     if (decode_by_unit(ctx, layer_begin, layer_count))
-      glide_decode_unit_kernel<T, D, G, DP><<<unsigned(layer_count * p.B * p.Hkv), kUnitThreads<D, G>, 0, stream>>>(p);
+      launch_chained(glide_decode_unit_kernel<T, D, G, DP>, unsigned(layer_count * p.B * p.Hkv), kUnitThreads<D, G>, 0, stream, p);
     else
       glide_decode_kernel<T, D, G, DP><<<ctx->decode_grid, kDecodeThreads, 0, stream>>>(p);
     if (cudaGetLastError() != cudaSuccess) return GLIDE_ERR_CUDA;

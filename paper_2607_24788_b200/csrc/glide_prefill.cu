@@ -121,6 +121,8 @@ __global__ void __launch_bounds__(kPrefillThreads) prefill_phi_kernel(const Pref
 // One warp per (unit, chunk), 32 tokens at a time by a warp scan, all of the chunk's gates asked for first (one thread per
 // unit, token after token, took 92 us for 256 tokens of 256 units: a memory round trip and a logarithm each).
 __global__ void __launch_bounds__(kPrefillThreads) prefill_gcum_kernel(const PrefillParams p) {
+  dependents_may_start();
+  wait_for_predecessor();
   const int lane = threadIdx.x & 31;
   const int64_t uc = (int64_t(blockIdx.x) * kPrefillThreads + threadIdx.x) >> 5;
   const int64_t units = int64_t(p.layer_count) * p.B * p.Hkv;
@@ -492,6 +494,8 @@ __global__ void __launch_bounds__(kRingThreads) prefill_ring_kernel(const Prefil
   constexpr int kChunks = D * int(sizeof(T)) / 16;               // 16-byte chunks of a row
   constexpr int kRows = kRingThreads / kChunks;                  // rows that the CTA moves at a time
   constexpr int kPer = (kRingTok + kRows - 1) / kRows;
+  dependents_may_start();
+  wait_for_predecessor();   // (the attention kernel reads the rings as they were)
   if (blockIdx.x == 0 && p.advance)
     for (int l = threadIdx.x; l < p.layer_count; l += kRingThreads) p.n_dev[p.layer_begin + l] += p.advance;
   const unsigned u = blockIdx.x / unsigned(groups), grp = blockIdx.x - u * unsigned(groups);
@@ -535,12 +539,14 @@ void launch_ring(const glide_ctx *ctx, const PrefillParams &p, cudaStream_t stre
   for (int l = p.layer_begin; l < p.layer_begin + p.layer_count; ++l) kept = std::max(kept, std::min<int64_t>(p.C, ctx->layers[size_t(l)].cap));
   const int groups = int((kept + kRingTok - 1) / kRingTok);
   const int64_t units = int64_t(p.layer_count) * p.B * p.Hkv;
-  prefill_ring_kernel<T, D><<<unsigned(units * groups), kRingThreads, 0, stream>>>(p, groups);
+  launch_chained(prefill_ring_kernel<T, D>, unsigned(units * groups), kRingThreads, 0, stream, p, groups);
 }
 
 // The ranges one after the other, 16 bytes per store where the address allows (S and z start on a 2 MiB multiple).  One
 // launch: as four memsets a reset of a small context took four launches of 1.6 us and the gaps between them.
 __global__ void __launch_bounds__(256) zero_kernel(const ZeroRanges z) {
+  dependents_may_start();
+  wait_for_predecessor();
   const size_t first = size_t(blockIdx.x) * 256 + threadIdx.x, step = size_t(gridDim.x) * 256;
 #pragma unroll
   for (int r = 0; r < 4; ++r) {
@@ -558,7 +564,7 @@ int launch_zero(const glide_ctx *ctx, const ZeroRanges &z, cudaStream_t stream) 
   for (size_t n : z.bytes) most = std::max(most, n);
   // 16 bytes a thread up to a full chip, more rounds per thread above
   const size_t blocks = std::min<size_t>((most / 16 + 255) / 256 + 1, size_t(ctx->sm_count) * 8);
-  zero_kernel<<<unsigned(blocks), 256, 0, stream>>>(z);
+  launch_chained(zero_kernel, unsigned(blocks), 256, 0, stream, z);
   if (cudaGetLastError() != cudaSuccess) return GLIDE_ERR_CUDA;
   return GLIDE_OK;
 }
@@ -687,7 +693,7 @@ int launch_prefill(glide_ctx *ctx, int layer_begin, int layer_count, int64_t T, 
           prefill_phi_kernel<TT, D, DP><<<warp4_blocks, kPrefillThreads, 0, stream>>>(s);
         }
         if (p.gated)
-          prefill_gcum_kernel<<<unsigned((units * s.nsub * 32 + kPrefillThreads - 1) / kPrefillThreads), kPrefillThreads, 0, stream>>>(s);
+          launch_chained(prefill_gcum_kernel, unsigned((units * s.nsub * 32 + kPrefillThreads - 1) / kPrefillThreads), kPrefillThreads, 0, stream, s);
         if (out && s.phiq16 && launch_prefill_project(ctx, s, false, stream) != GLIDE_OK) return GLIDE_ERR_CUDA;
         if (out && p.merge != GLIDE_MERGE_SHARED)   // (before the carry: the chunk sums overwrite rows of phi(K'))
           prefill_zcum_kernel<D><<<unsigned((units * s.nsub * D + kPrefillThreads - 1) / kPrefillThreads), kPrefillThreads, 0, stream>>>(s);
@@ -709,7 +715,7 @@ int launch_prefill(glide_ctx *ctx, int layer_begin, int layer_count, int64_t T, 
     return for_passes(slots, most, ctx->cfg.head_dim, ctx->elem, [&](const PrefillParams &s) -> int {
       if (p.gated && evicts_in(s.layer_begin, s.layer_count)) {
         const unsigned blocks = unsigned((int64_t(s.layer_count) * units_layer * s.nsub * 32 + kPrefillThreads - 1) / kPrefillThreads);
-        prefill_gcum_kernel<<<blocks, kPrefillThreads, 0, stream>>>(s);
+        launch_chained(prefill_gcum_kernel, blocks, kPrefillThreads, 0, stream, s);
         if (cudaGetLastError() != cudaSuccess) return GLIDE_ERR_CUDA;
       }
       return launch_prefill_fma(ctx, s, stream);

@@ -102,6 +102,8 @@ __global__ void __launch_bounds__(2 * kThreads) prefill_fma_sums_kernel(const Pr
   static_assert(2 * kThreads * (4 * CG + 1) <= kSumTok * D, "the second group's sums fit its tile");
   __shared__ __align__(16) float ph[2][kSumTok][16];   // [group]
   __shared__ __align__(16) float vt[2][kSumTok][D];
+  dependents_may_start();
+  wait_for_predecessor();
   const int grp = threadIdx.x / kThreads, tid = threadIdx.x % kThreads;
   const int rb = int(blockIdx.x % (D / 16));
   const int64_t uc = blockIdx.x / (D / 16);
@@ -252,6 +254,8 @@ __global__ void __launch_bounds__(2 * kThreads, 1) prefill_fma_attn_kernel(const
   constexpr int CG = D / 64;
   constexpr int TOK = kRows / G;                   // tokens per CTA
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  dependents_may_start();
+  wait_for_predecessor();
   const int grp = threadIdx.x / kThreads, tid = threadIdx.x % kThreads;
   auto &all = *reinterpret_cast<AttnSmem<D> *>(smem_raw);
   typename AttnSmem<D>::Group &sm = all.grp[grp];
@@ -551,6 +555,8 @@ __device__ __forceinline__ void add_sums(const PrefillParams &p, int64_t e) {
 // slot then holds the state at its start
 template <int D>
 __global__ void __launch_bounds__(kThreads) prefill_fma_scan_kernel(const PrefillParams p) {
+  dependents_may_start();
+  wait_for_predecessor();
   add_sums<D, true>(p, int64_t(blockIdx.x) * kThreads + threadIdx.x);
 }
 
@@ -558,6 +564,8 @@ __global__ void __launch_bounds__(kThreads) prefill_fma_scan_kernel(const Prefil
 // to slot (position mod cap), one thread per four entries of a K and a V row.
 template <typename T, int D>
 __global__ void __launch_bounds__(kThreads) prefill_fma_finish_kernel(const PrefillParams p, unsigned state_blocks) {
+  dependents_may_start();
+  wait_for_predecessor();
   const int tid = threadIdx.x;
   if (blockIdx.x == 0 && p.advance)
     for (int l = tid; l < p.layer_count; l += kThreads) p.n_dev[p.layer_begin + l] += p.advance;
@@ -595,8 +603,8 @@ int launch_prefill_fma(glide_ctx *ctx, const PrefillParams &p, cudaStream_t stre
     const unsigned state_ctas = any_evicts ? unsigned(units * (D * D / 4 / kThreads)) : 0u;
     const bool in_place = p.nsub == 1, scan = any_evicts && p.nsub > kDirectChunks<D>;
     const unsigned sum_ctas = unsigned(units * p.nsub * (D / 16));
-    if (any_evicts && !in_place) prefill_fma_sums_kernel<T, D, false><<<sum_ctas, 2 * kThreads, 0, stream>>>(p);
-    if (scan) prefill_fma_scan_kernel<D><<<state_ctas, kThreads, 0, stream>>>(p);
+    if (any_evicts && !in_place) launch_chained(prefill_fma_sums_kernel<T, D, false>, sum_ctas, 2 * kThreads, 0, stream, p);
+    if (scan) launch_chained(prefill_fma_scan_kernel<D>, state_ctas, kThreads, 0, stream, p);
     if (p.out) {
       auto kern = prefill_fma_attn_kernel<T, D, G>;
       if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(sizeof(AttnSmem<D>))) != cudaSuccess) {
@@ -604,12 +612,12 @@ int launch_prefill_fma(glide_ctx *ctx, const PrefillParams &p, cudaStream_t stre
         return GLIDE_ERR_CUDA;
       }
       const int64_t blocks = units * (int64_t(p.nsub - 1) * ((p.SC + TOK - 1) / TOK) + (p.C - (p.nsub - 1) * p.SC + TOK - 1) / TOK);
-      kern<<<unsigned(blocks), 2 * kThreads, sizeof(AttnSmem<D>), stream>>>(p);
+      launch_chained(kern, unsigned(blocks), 2 * kThreads, sizeof(AttnSmem<D>), stream, p);
     }
-    if (any_evicts && in_place) prefill_fma_sums_kernel<T, D, true><<<sum_ctas, 2 * kThreads, 0, stream>>>(p);
+    if (any_evicts && in_place) launch_chained(prefill_fma_sums_kernel<T, D, true>, sum_ctas, 2 * kThreads, 0, stream, p);
     const unsigned state_blocks = scan || in_place ? 0u : state_ctas;
     const unsigned ring_blocks = unsigned((units * p.C * (D / 4) + kThreads - 1) / kThreads);
-    prefill_fma_finish_kernel<T, D><<<state_blocks + ring_blocks, kThreads, 0, stream>>>(p, state_blocks);
+    launch_chained(prefill_fma_finish_kernel<T, D>, state_blocks + ring_blocks, kThreads, 0, stream, p, state_blocks);
     return cudaGetLastError() == cudaSuccess ? GLIDE_OK : GLIDE_ERR_CUDA;
   });
 }

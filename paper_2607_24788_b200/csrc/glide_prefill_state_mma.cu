@@ -99,6 +99,8 @@ __device__ __noinline__ float carry_element(const CarryRows &rows, const float *
 // MAKE_PHI: phi(K') is made here (parameter-free map, gated); otherwise it is in the scratch.
 template <bool PARTIAL, bool MAKE_PHI, bool GATED>
 __global__ void __launch_bounds__(kThreads, GATED ? 3 : 0) prefill_state_mma_kernel(const PrefillParams p) {
+  dependents_may_start();
+  wait_for_predecessor();
   using bf16 = __nv_bfloat16;
   // per stage phi columns (or K' rows, 16 bytes more per row) and V' rows; made phi columns
   constexpr int kInBytes = MAKE_PHI ? kVBytes : kPhiBytes;
@@ -358,6 +360,8 @@ __global__ void __launch_bounds__(kThreads, GATED ? 3 : 0) prefill_state_mma_ker
 template <bool GATED, bool SNAP>
 __global__ void __launch_bounds__(kThreads + 32) prefill_scan_kernel(const PrefillParams p) {
   using bf16 = __nv_bfloat16;
+  dependents_may_start();
+  wait_for_predecessor();
   const unsigned ctas_per_unit = unsigned(p.dp) / 4;
   const int u = int(blockIdx.x / ctas_per_unit);
   const int j = int(blockIdx.x - unsigned(u) * ctas_per_unit), tid = threadIdx.x;
@@ -447,7 +451,9 @@ int launch_prefill_state_mma(const PrefillParams &pass, bool make_phi, cudaStrea
   auto scan = [&]() -> int {
     if (p.nsub > 1) {
       const unsigned ctas = unsigned(units * (p.dp / 4));
-      auto run = [&](auto gated, auto snap) { prefill_scan_kernel<decltype(gated)::value, decltype(snap)::value><<<ctas, kThreads + 32, 0, stream>>>(p); };
+      auto run = [&](auto gated, auto snap) {
+        launch_chained(prefill_scan_kernel<decltype(gated)::value, decltype(snap)::value>, ctas, kThreads + 32, 0, stream, p);
+      };
       const std::true_type yes{};
       const std::false_type no{};
       if (p.gated) p.s16 ? run(yes, yes) : run(yes, no);
@@ -461,7 +467,7 @@ int launch_prefill_state_mma(const PrefillParams &pass, bool make_phi, cudaStrea
   }
   const unsigned blocks = unsigned(units * p.nsub * (p.dp / kRowsPerCta));
   auto run = [&](auto partial, auto make, auto gated) {
-    prefill_state_mma_kernel<decltype(partial)::value, decltype(make)::value, decltype(gated)::value><<<blocks, kThreads, 0, stream>>>(p);
+    launch_chained(prefill_state_mma_kernel<decltype(partial)::value, decltype(make)::value, decltype(gated)::value>, blocks, kThreads, 0, stream, p);
   };
   const std::true_type yes{};
   const std::false_type no{};
