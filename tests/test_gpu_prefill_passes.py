@@ -103,3 +103,33 @@ def test_chunk_sums_on_tcgen05(chunk, w, calls):
         bound = (3 * (chunk or 256) / 16 + T / (chunk or 256) + 2) * 2.0 ** -23
         assert ((got - want).norm() / want.norm()).item() <= bound
     assert g.glide_device_status() == 0
+
+
+# Launches that start while the one before them runs out (programmatic dependent launch): reset, prompt of several passes and decode
+# steps issued back to back leave the bits that they leave with the device idle between any two calls.
+@pytest.mark.parametrize("dtype,d,heads,windows,kw", [
+    (torch.float32, 64, 2, [64], dict()), (torch.float32, 64, 2, [0, 16, 100], dict(gated=True)), (torch.float32, 128, 8, [40, 0], dict(prefill_chunk=16)),
+    (BF16, 128, 8, [0, 16, 100, 300], dict(prefill_chunk=144)), (BF16, 128, 8, [16, 600, 100], dict(gated=True)), (BF16, 128, 4, [33, 0], dict(merge=1))])
+def test_calls_back_to_back(dtype, d, heads, windows, kw):
+    L, T, steps = len(windows), 700, 4
+    gen = torch.Generator(device="cuda").manual_seed(109)
+    q, k, v = (torch.randn((L, 2, T + steps, h, d), generator=gen, device="cuda").to(dtype) for h in (heads, 2, 2))
+    prompt, tokens = [x[:, :, :T].contiguous() for x in (q, k, v)], [[x[:, :, T + i].contiguous() for x in (q, k, v)] for i in range(steps)]
+    results = []
+    for idle in (True, False, False):
+        g = glide.Glide(windows, 2, heads, 2, d, 1 << 20, dtype=dtype, **kw)
+        outs = [torch.empty_like(prompt[0])] + [torch.empty_like(t[0]) for t in tokens]
+        torch.cuda.synchronize()
+        for _ in range(2):   # (the second prompt begins in what the first has left)
+            decode = [lambda t=t, o=o: g.glide_decode_step(*t, o) for t, o in zip(tokens, outs[1:])]
+            for call in [g.glide_reset, lambda: g.glide_prefill(*prompt, outs[0])] + decode:
+                call()
+                if idle:
+                    torch.cuda.synchronize()
+        state = [x for l, w in enumerate(windows) for x in g.glide_export_state(l)[(0 if w else 2):]]
+        assert g.glide_device_status() == 0
+        results.append(outs + state)
+        g.glide_destroy()
+    for other in results[1:]:
+        for a, b in zip(results[0], other):
+            assert torch.equal(a, b)
