@@ -24,7 +24,7 @@
 // j' <= i, then C V' (intra-chunk); l accumulates the matching sums.  out = O / l.
 // What bounds it: short windows, the fixed chain of a CTA (24500 cycles: 6800 until Q and K_0 are there and the first product is
 // done, one softmax 3500, phi 2900, two to three more products 8500, the store 2500); long windows, per key tile and row tile the
-// chain softmax (1850) -> P V and the next S (1050 to 1300) -> signals, 3650 cycles in which the two row tiles' products take
+// chain softmax (1770) -> P V and the next S (1050 to 1300) -> signals, 3570 cycles in which the two row tiles' products take
 // 2048.  8 layers of 2048 tokens, 32 / 8 heads, windows of 64 / 256 / 1024: 270 / 333 / 525 us; with one softmax thread per row,
 // one MMA warp and phi in one piece 292 / 379 / 576.
 // Every mbarrier wait is bounded; on a time-out the CTA records kDevWaitTimeout, leaves its loops, frees its TMEM
@@ -348,6 +348,14 @@ prefill_attn_tc_kernel(const __grid_constant__ PrefillParams p, const CUtensorMa
   // The loader warp sets up the barriers and asks for Q before anything that waits for the layer table.
   const bool aligned = (smem_u32(smem_raw) & 1023u) == 0;   // (the swizzled tiles have to start on a multiple of 1024)
   const bool q_by_tma = p.q_tma && aligned;
+  // one lane: Q_X, when the group's heads lie side by side.  (Tokens past the tile's last one are zeros or the next tile's rows:
+  // their results are not stored.)
+  auto ask_q = [&](int x) {
+    const uint32_t bar = smem_u32(&sm.bar_q[x]), dst = smem_u32(sm.q[x]);
+    mbar_expect_tx(bar, kTileBytes);
+    tma_load_4d(dst, &cm.q, 0, g * G, chunk_c0 + tok0 + x * TOKT, lrel * p.B + b, bar);
+    tma_load_4d(dst + kBoxBytes, &cm.q, 64, g * G, chunk_c0 + tok0 + x * TOKT, lrel * p.B + b, bar);
+  };
   int status = 0;
   if (warp == kLoadWarp && lane == 0) {
     status = *reinterpret_cast<volatile int32_t *>(&p.ctl->status);
@@ -368,14 +376,8 @@ prefill_attn_tc_kernel(const __grid_constant__ PrefillParams p, const CUtensorMa
     mbar_init(smem_u32(&sm.bar_done), n_rows);
     mbar_init(smem_u32(&sm.bar_state), 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    // Q_X, when the group's heads lie side by side.  (Tokens past the tile's last one are zeros or the next tile's rows:
-    // their results are not stored.)
-    for (int x = 0; q_by_tma && x < n_rows; ++x) {
-      const uint32_t bar = smem_u32(&sm.bar_q[x]), dst = smem_u32(sm.q[x]);
-      mbar_expect_tx(bar, kTileBytes);
-      tma_load_4d(dst, &cm.q, 0, g * G, chunk_c0 + tok0 + x * TOKT, lrel * p.B + b, bar);
-      tma_load_4d(dst + kBoxBytes, &cm.q, 64, g * G, chunk_c0 + tok0 + x * TOKT, lrel * p.B + b, bar);
-    }
+    // (Q_B behind K_0, which the first product needs before it: 8001 tokens layer by layer 7.09 -> 6.94 ms, 8 x 2048 10.2 -> 10.1)
+    if (q_by_tma) ask_q(0);
   }
   // (positions stay below 2^30, the most tokens a context may hold; a longer window is no other than that)
   constexpr int64_t kMost = int64_t(1) << 30;
@@ -416,7 +418,7 @@ prefill_attn_tc_kernel(const __grid_constant__ PrefillParams p, const CUtensorMa
     asm volatile("barrier.cta.arrive 9, %0;" ::"n"(kThreads) : "memory");
     if (*failed) {   // (set before the meeting: the same for all)
       int alone = 0;
-      for (int x = 0; q_by_tma && x < (hasB ? 2 : 1); ++x) mbar_wait(smem_u32(&sm.bar_q[x]), 0u, &alone);   // no copy outlives the CTA
+      if (q_by_tma) mbar_wait(smem_u32(&sm.bar_q[0]), 0u, &alone);   // no copy outlives the CTA
       if (lane == 0 && !aligned) atomicExch(&p.ctl->status, kDevWaitTimeout);
       return;
     }
@@ -1143,8 +1145,10 @@ prefill_attn_tc_kernel(const __grid_constant__ PrefillParams p, const CUtensorMa
     // that one thread fetches, then the V' tiles of the intra-chunk steps (with the phi(K') tiles of later steps).
     const int n_window = 2 * n_tiles;
     const int n_jobs = n_window + (linear ? 1 + n_itiles : 0);
+    const int job_qb = q_by_tma && hasB ? min(n_window, 1) : -1;   // the job before which Q_B is asked for
 #pragma unroll 1
     for (int job = 0; job < n_jobs; ++job) {
+      if (job == job_qb && lane == 0) ask_q(1);
       if (job == n_window) {
         if (lane == 0 && !TWO) {
           // the bf16 state (with z), then the phi(K') tiles of the first two intra-chunk steps
