@@ -215,6 +215,7 @@ struct Smem {
   int failed;
   float exch[kSoftmaxThreads / 2];       // a value of each row on its way between the row's two threads
 };
+static_assert(kLazy == 8.0f, "soft_tile's bound is 2^kLazy");
 static_assert(sizeof(Smem) <= 232448, "shared memory of one CTA");
 
 // the call's K (or V) rows as a 4-D tensor {d, Hkv, T, layers x sequences}: boxes of 16 tokens x 64 columns of one KV head
@@ -623,22 +624,21 @@ prefill_attn_tc_kernel(const __grid_constant__ PrefillParams p, const CUtensorMa
       }
       store_p(c, pk, x);
     };
-    // One key tile against the reference as it is (0 for a row's first tile), in one pass: no maximum is looked for.  The largest
-    // weight says afterwards whether that was right: up to 2^32, and for a first tile not below 2^-32, fp32 sums and bf16 weights are
-    // as precise as against the maximum itself.  Otherwise (false, to both threads of all rows of the pair) nothing has
-    // happened, the scores are still there, and the tile goes through soft_tile_masked.  (Two passes: 1850 cycles a tile.)
-    auto soft_tile = [&](auto masked, int lo, int hi, bool first) {
+    // A later key tile against the reference as it is, in one pass: no maximum is looked for.  The largest weight says afterwards whether
+    // that was right: below 2^kLazy the reference stays, as it does in soft_tile_masked.  Otherwise (false, to both threads of all
+    // rows of the pair) nothing has happened, the scores are still there, and the tile goes through soft_tile_masked.  (Two passes: 1840
+    // cycles a tile, one 1770.  A row's first tile is taken against its maximum: against 0 a short window's tile took 2400 cycles
+    // instead of 3500, but the rounding of the largest weights, which are 1 against the maximum, cost 6 % in precision.)
+    auto soft_tile = [&](auto masked, int lo, int hi) {
       float sum0 = 0.f, sum1 = 0.f;
-      const float mr = first ? 0.f : m_ref;
+      const float mr = m_ref;
       uint32_t pk[32], mx2 = 0u;
-      bool some = false;
 #pragma unroll
       for (int c = 0; c < kHalf; c += 32) {
         uint32_t x[32];
         tmem_ld32(tS + c, x);
         if (decltype(masked)::value) {
           const uint32_t m = column_mask(c, lo, hi);
-          some = some || m != 0;
 #pragma unroll
           for (int i = 0; i < 32; ++i) x[i] = (m >> i) & 1u ? x[i] : 0xff800000u;
         }
@@ -653,11 +653,9 @@ prefill_attn_tc_kernel(const __grid_constant__ PrefillParams p, const CUtensorMa
         }
       }
       const float mx = fmaxf(bf16_lo(mx2), bf16_hi(mx2));
-      const bool low = first && (some || !decltype(masked)::value) && mx < 0x1p-32f;
-      if (pair_any(!(mx <= 0x1p32f) || low)) return false;
+      if (pair_any(!(mx < 0x1p8f))) return false;
       tmem_st32(tS, pk);
       l_sum += sum0 + sum1;
-      if (first) m_ref = 0.f;
       return true;
     };
     // One key tile with masked keys (valid columns lo .. hi of this row's half).  32 columns at a time, those in which no row of
@@ -747,9 +745,9 @@ prefill_attn_tc_kernel(const __grid_constant__ PrefillParams p, const CUtensorMa
         bool done = false;
         if constexpr (!GATED) {
           // (what is asked here is the same in both warps of a pair: their threads share the rows)
-          if (t == tf ? !__any_sync(0xffffffffu, lo > hi) : !__any_sync(0xffffffffu, m_ref == -CUDART_INF_F)) {
-            if (whole) done = soft_tile(std::false_type{}, 0, kHalf - 1, t == tf);
-            else done = soft_tile(std::true_type{}, lo - H * kHalf, hi - H * kHalf, t == tf);
+          if (t > tf && !__any_sync(0xffffffffu, m_ref == -CUDART_INF_F)) {
+            if (whole) done = soft_tile(std::false_type{}, 0, kHalf - 1);
+            else done = soft_tile(std::true_type{}, lo - H * kHalf, hi - H * kHalf);
           }
         }
         if (!done) soft_tile_masked(lo - H * kHalf, hi - H * kHalf, t == tf);
