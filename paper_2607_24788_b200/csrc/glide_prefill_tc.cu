@@ -660,8 +660,8 @@ prefill_attn_tc_kernel(const __grid_constant__ PrefillParams p, const CUtensorMa
     };
     // One key tile with masked keys (valid columns lo .. hi of this row's half).  32 columns at a time, those in which no row of
     // the warp has a valid one left out; the loops stay rolled: with everything unrolled the kernel was 210 KB of code that a CTA
-    // fetched once per phase (a CTA's first key tile took 12000 cycles, a later one 2500).  For gated contexts, rows that have no
-    // reference yet, and tiles that soft_tile leaves alone.
+    // fetched once per phase (a CTA's first key tile took 12000 cycles, a later one 2500).  For the masked tiles of gated contexts, rows
+    // that have no reference yet, and tiles that soft_tile leaves alone.
     auto soft_tile_masked = [&](int lo, int hi, bool first) {
       float mx = -CUDART_INF_F, sum0 = 0.f, sum1 = 0.f;
 #pragma unroll 1
@@ -689,6 +689,26 @@ prefill_attn_tc_kernel(const __grid_constant__ PrefillParams p, const CUtensorMa
         tmem_ld32(tS + c, x);
 #pragma unroll
         for (int i = 0; i < 32; ++i) x[i] = (m >> i) & 1u ? x[i] : 0xff800000u;
+        weights(c, x, mr, sum0, sum1);
+      }
+      tmem_wait_st();
+      l_sum += sum0 + sum1;
+    };
+    // Gated: a key tile without a masked key, in the two passes of soft_tile_masked without its masks and votes.  4 layers, 4000 tokens
+    // on windows of 1024 / 4096 / 16384: 1.61 / 2.55 / 5.03 ms; through soft_tile_masked 1.69 / 2.91 / 6.35, which was more than with
+    // one thread per row (1.65 / 2.71 / 5.63).  (In one pass as soft_tile, hi and lo kept in 64 registers: 1.61 / 2.51 / 4.88, but with
+    // 64 bytes more of spills 1.5 % longer at windows of 64.)
+    auto soft_tile_gated = [&](bool first) {
+      float mx = -CUDART_INF_F, sum0 = 0.f, sum1 = 0.f;
+      uint32_t x[32];
+      tmem_ld32(tS, x);
+      mx = row_max(x, mx);
+      tmem_ld32(tS + 32, x);
+      mx = row_max(x, mx);
+      const float mr = move_ref(mx, first);
+#pragma unroll 1
+      for (int c = 0; c < kHalf; c += 32) {
+        tmem_ld32(tS + c, x);
         weights(c, x, mr, sum0, sum1);
       }
       tmem_wait_st();
@@ -743,7 +763,10 @@ prefill_attn_tc_kernel(const __grid_constant__ PrefillParams p, const CUtensorMa
         // valid columns of this row: lo <= c <= hi (a token more than 2^30 - 1 before another is none)
         const int lo = max(tok_abs - w + 1 - j0, 0), hi = min(tok_abs - j0, kKT - 1);
         bool done = false;
-        if constexpr (!GATED) {
+        if constexpr (GATED) {
+          if (whole) soft_tile_gated(t == tf);
+          done = whole;
+        } else {
           // (what is asked here is the same in both warps of a pair: their threads share the rows)
           if (t > tf && !__any_sync(0xffffffffu, m_ref == -CUDART_INF_F)) {
             if (whole) done = soft_tile(std::false_type{}, 0, kHalf - 1);

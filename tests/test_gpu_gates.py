@@ -95,3 +95,69 @@ def test_order_of_heads(G, kw):
         outs.append(out)
         g.glide_destroy()
     assert torch.equal(outs[0], outs[1][:, :, :, order])
+
+
+def _gated_outputs_f64(q, k, v, gate, w, n0):
+    """Outputs of tokens n0 .. of one sequence, shared normaliser, in fp64: q [T][H][d] from token n0 on, k, v, gate of all tokens."""
+    N, Hkv, d = k.shape
+    G, j = q.shape[1] // Hkv, torch.arange(N, device=q.device)
+    t = j[n0:, None]
+    outs = []
+    for h in range(q.shape[1]):
+        qq, kk, vv, log_g = q[:, h].double(), k[:, h // G].double(), v[:, h // G].double(), gate[:, h // G].double().log().cumsum(0)
+        s = torch.where((j <= t) & (j > t - w), qq @ kk.T * f32_scale(d), -torch.inf)
+        m = s.amax(-1, keepdim=True)
+        phi = torch.softmax(qq, -1) @ torch.softmax(kk, -1).T * (log_g[(t - w).clamp(min=0)] - log_g[None]).clamp(max=0).exp()
+        p = (s - m).exp() + torch.where(j <= t - w, phi * (-m).exp(), 0.)
+        outs.append(p @ vv / p.sum(-1, keepdim=True))
+    return torch.stack(outs, 1)
+
+
+# Key tiles without a masked key on the tcgen05 kernel: rows of every group size, a window whose first whole tile is also the row's
+# first (a turn behind a long context), scores that grow from tile to tile, so that the reference moves in each, and scores that stay.
+# Bound: an output is within 2^-9 of itself when it is rounded to bf16; two split terms of the weights and V in bf16 add 2^-17.
+@pytest.mark.parametrize("G,w,n0,T,growing", [(1, 700, 900, 300, True), (2, 1 << 20, 0, 700, True), (4, 512, 1024, 200, False), (4, 385, 640, 129, True),
+                                              (8, 300, 513, 97, False), (8, 1 << 20, 1000, 33, True)])
+def test_gated_key_tiles_without_a_masked_key(G, w, n0, T, growing):
+    N, Hkv, d = n0 + T, 2, 128
+    gen = torch.Generator(device="cuda").manual_seed(113 + G)
+    q, k, v = (torch.randn((1, 1, N, h, d), generator=gen, device="cuda") for h in (Hkv * G, Hkv, Hkv))
+    if growing:   # (the largest of 128 scores grows by more than 2^8 per tile)
+        k *= (1 + torch.arange(N, device="cuda") / 32).view(1, 1, N, 1, 1)
+    q, k, v = (x.to(BF16) for x in (q, k, v))
+    gate = 0.99 + 0.01 * torch.rand((1, 1, N, Hkv), generator=gen, device="cuda")
+    g = glide.Glide([w], 1, Hkv * G, Hkv, d, 1 << 20, dtype=BF16, softmax_scale=f32_scale(d), gated=True)
+    if n0:
+        g.glide_prefill_gated(None, *(x[:, :, :n0].contiguous() for x in (k, v, gate)), None)
+    new = [x[:, :, n0:].clone() for x in (q, k, v, gate)]   # (a slice of one sequence is contiguous, but not on a multiple of 16 bytes)
+    out = torch.full_like(new[0], float("nan"))
+    g.glide_prefill_gated(*new, out)
+    assert g.glide_device_status() == 0
+    want = _gated_outputs_f64(new[0][0, 0], k[0, 0], v[0, 0], gate[0, 0], w, n0)
+    assert ((out[0, 0] - want).norm() / want.norm()).item() <= 2.0 ** -9 + 2.0 ** -17
+
+
+def test_a_gated_long_window_takes_its_products_time():
+    """A gated key tile has three products where one without gates has two (K, and V with the weights' two terms): on long windows
+    the call takes no longer than that by more than a fifteenth (1.33 times as long; 1.68 when whole tiles went through the masked
+    tiles' code)."""
+    T, H, Hkv, d, w, n = 2048, 32, 8, 128, 16384, 3
+    gen = torch.Generator(device="cuda").manual_seed(127)
+    q, k, v = (torch.randn((2, 1, T, h, d), generator=gen, device="cuda").to(BF16) for h in (H, Hkv, Hkv))
+    out, took = torch.empty_like(q), {}
+    for gated in (False, True):
+        g = glide.Glide([w, w], 1, H, Hkv, d, 1 << 20, dtype=BF16, gated=gated)
+        for _ in range(w // T):
+            g.glide_prefill(None, k, v, None)
+        times = []
+        for _ in range(1 + n):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            g.glide_prefill(q, k, v, out)
+            b.record()
+            b.synchronize()
+            times.append(a.elapsed_time(b))
+        took[gated] = min(times[1:])
+        g.glide_destroy()
+    print(f"without gates {took[False]:.3f} ms, gated {took[True]:.3f}")
+    assert took[True] <= 1.6 * took[False]
