@@ -11,16 +11,18 @@ namespace glide {
 
 constexpr float kLog2e = 1.4426950408889634f;
 
-// Programmatic dependent launch: the launch behind this one may take SMs as soon as every CTA of this grid has started ...
+// Programmatic dependent launch: the launch behind this one may take SMs as soon as every CTA of this grid has called this or ended.
+// Its CTAs then hold their places while they wait, and those of the launch after it, which nothing but this call holds back, get what
+// places are left.  Grids of less than half the SMs' number lost more by that than the launches cost, so a kernel calls it as late as
+// still hides the launch, behind its own wait at the earliest.  At the top it stands in the scan, ring and reset kernels: behind
+// them comes an ordinary launch, or one with a CTA for every SM, or (after a reset) a single call.
 __device__ __forceinline__ void dependents_may_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 // ... and waits here until the one before has completed.  Every CTA of a kernel that is launched by launch_chained passes this,
 // also one that has nothing to do: so a grid that has completed means that all before it have.
 __device__ __forceinline__ void wait_for_predecessor() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 // (host) a launch that may start while the one before it in the stream runs out.  Nothing is read before the wait, so what the launch
-// before is does not matter.  What it gives: one fp32 layer of 4 heads, decode step 8.2 -> 5.9 us, prompt of 512 tokens with reset and
-// step 46.7 -> 41.9; scan and ring of the tensor-core prefill (8001 tokens layer by layer) 7.31 -> 7.14 ms, its gates and mma.sync carry
-// too (1000 gated tokens) 1.011 -> 0.975.  The tcgen05 kernels are launched in the ordinary way: with the carry chained the 8001 tokens
-// took 7.24 ms, with the attention kernel as well 7.22 (7.30 when it asked for Q before the wait), 8 x 2048 tokens 10.1 -> 10.2.
+// before is does not matter.  It hides the launch of calls that follow one another; a call after idle is no faster.  The tcgen05
+// kernels are launched in the ordinary way: chained, they took as long or longer (carry and attention of 8001 tokens layer by layer).
 template <typename... KernelArgs, typename... Args>
 cudaError_t launch_chained(void (*kernel)(KernelArgs...), unsigned blocks, unsigned threads, size_t smem, cudaStream_t stream, Args &&...args) {
   cudaLaunchAttribute attr[1];

@@ -133,3 +133,59 @@ def test_calls_back_to_back(dtype, d, heads, windows, kw):
     for other in results[1:]:
         for a, b in zip(results[0], other):
             assert torch.equal(a, b)
+
+
+def _time_ms(run, repeats=6):
+    """The shortest of some runs (the first one left out), by events around it; all of a run is queued before the device begins it."""
+    times = []
+    for _ in range(repeats + 1):
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        torch.cuda._sleep(8_000_000)   # (4 ms and more)
+        a.record()
+        run()
+        b.record()
+        b.synchronize()
+        times.append(a.elapsed_time(b))
+    return min(times[1:])
+
+
+# The thread blocks of a launch that has started early keep their places while they wait, and what is launched behind them gets the
+# places that are left.  Each case is one that this made slower than launches that do not overlap (thread blocks for less than half of
+# the SMs, long chains of launches): back to back against the same tokens with an event, which nothing overlaps, between any two calls.
+# The bounds lie between the ratios with the next launch let go as late as is useful (0.74, 0.40, 0.89) and at a kernel's beginning
+# (0.82, 0.50, 1.03).
+@pytest.mark.parametrize("what,bound", [("decode", 0.79)])
+def test_overlapping_launches_hold_nothing_up(what, bound):
+    gen = torch.Generator(device="cuda").manual_seed(131)
+    rows = lambda L, n, h, d, dtype: torch.randn((L, 1, n, h, d), generator=gen, device="cuda").to(dtype)
+    if what == "decode":
+        g = glide.Glide([512] * 8, 1, 8, 8, 64, 1 << 20, dtype=torch.float32)
+        q, k, v, out = (rows(8, 600, 8, 64, torch.float32) for _ in range(4))
+        g.glide_prefill(None, k, v, None)
+        step = [x[:, :, 0].contiguous() for x in (q, k, v, out)]
+        together = lambda: [g.glide_decode_step(*step) for _ in range(32)]
+        calls = [lambda: g.glide_decode_step(*step)] * 32
+    elif what == "cuda-core prefill":
+        g = glide.Glide([64, 300], 1, 4, 4, 128, 1 << 20, dtype=torch.float32, prefill_chunk=256)
+        k, v = (rows(2, 8192, 4, 128, torch.float32) for _ in range(2))
+        together = lambda: g.glide_prefill(None, k, v, None)
+        parts = [[x[:, :, c:c + 256].contiguous() for x in (k, v)] for c in range(0, 8192, 256)]
+        calls = [lambda p=p: g.glide_prefill(None, *p, None) for p in parts]
+    else:
+        g = glide.Glide([4096, 1024, 256, 64], 1, 32, 8, 128, 1 << 20, dtype=BF16, gated=True)
+        k, v = (rows(4, 4096, 8, 128, BF16) for _ in range(2))
+        together = lambda: g.glide_prefill_gated(None, k, v, None, None)
+        parts = [[x[:, :, c:c + 256].contiguous() for x in (k, v)] for c in range(0, 4096, 256)]
+        calls = [lambda p=p: g.glide_prefill_gated(None, *p, None, None) for p in parts]
+    between = torch.cuda.Event(enable_timing=True)
+
+    def apart():
+        for call in calls:
+            call()
+            between.record()
+
+    t_together, t_apart = _time_ms(together), _time_ms(apart)
+    assert g.glide_device_status() == 0
+    g.glide_destroy()
+    print(f"{what}: {t_together * 1e3:.1f} us, with events between {t_apart * 1e3:.1f}")
+    assert t_together <= bound * t_apart
