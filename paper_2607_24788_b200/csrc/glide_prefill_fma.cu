@@ -102,7 +102,6 @@ __global__ void __launch_bounds__(2 * kThreads) prefill_fma_sums_kernel(const Pr
   static_assert(2 * kThreads * (4 * CG + 1) <= kSumTok * D, "the second group's sums fit its tile");
   __shared__ __align__(16) float ph[2][kSumTok][16];   // [group]
   __shared__ __align__(16) float vt[2][kSumTok][D];
-  dependents_may_start();
   wait_for_predecessor();
   const int grp = threadIdx.x / kThreads, tid = threadIdx.x % kThreads;
   const int rb = int(blockIdx.x % (D / 16));
@@ -172,6 +171,7 @@ __global__ void __launch_bounds__(2 * kThreads) prefill_fma_sums_kernel(const Pr
     }
     group_sync(grp);
   }
+  dependents_may_start();   // (8192 tokens of one fp32 layer, state only, d = 64 / 128 x 2 layers: 141 / 448 us; at every kernel's top 191 / 562, not at all 167 / 496)
   // the second group's sums on top of the first's, through the second group's tile
   float (*other)[4 * CG + 1] = reinterpret_cast<float (*)[4 * CG + 1]>(&vt[1][0][0]);   // [2 * kThreads]
   if (grp == 1) {
@@ -254,7 +254,6 @@ __global__ void __launch_bounds__(2 * kThreads, 1) prefill_fma_attn_kernel(const
   constexpr int CG = D / 64;
   constexpr int TOK = kRows / G;                   // tokens per CTA
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  dependents_may_start();
   wait_for_predecessor();
   const int grp = threadIdx.x / kThreads, tid = threadIdx.x % kThreads;
   auto &all = *reinterpret_cast<AttnSmem<D> *>(smem_raw);
@@ -454,6 +453,7 @@ __global__ void __launch_bounds__(2 * kThreads, 1) prefill_fma_attn_kernel(const
     }
     group_sync(grp);
   }
+  dependents_may_start();   // (512 tokens of 4 units, d = 64: 30 us with all; at the top 35, not at all 39)
 #pragma unroll
   for (int r = 0; r < 2; ++r) l[r] = lanes_sum<16>(l[r]);
   // group 1 hands its part over in its V tile (16 x d floats) and the row sums in its weights
@@ -555,8 +555,7 @@ __device__ __forceinline__ void add_sums(const PrefillParams &p, int64_t e) {
 // slot then holds the state at its start
 template <int D>
 __global__ void __launch_bounds__(kThreads) prefill_fma_scan_kernel(const PrefillParams p) {
-  dependents_may_start();
-  wait_for_predecessor();
+  wait_for_predecessor();   // (the launch behind this one is let go as its CTAs end: they are short)
   add_sums<D, true>(p, int64_t(blockIdx.x) * kThreads + threadIdx.x);
 }
 
@@ -564,7 +563,6 @@ __global__ void __launch_bounds__(kThreads) prefill_fma_scan_kernel(const Prefil
 // to slot (position mod cap), one thread per four entries of a K and a V row.
 template <typename T, int D>
 __global__ void __launch_bounds__(kThreads) prefill_fma_finish_kernel(const PrefillParams p, unsigned state_blocks) {
-  dependents_may_start();
   wait_for_predecessor();
   const int tid = threadIdx.x;
   if (blockIdx.x == 0 && p.advance)
