@@ -121,7 +121,6 @@ __global__ void __launch_bounds__(kPrefillThreads) prefill_phi_kernel(const Pref
 // One warp per (unit, chunk), 32 tokens at a time by a warp scan, all of the chunk's gates asked for first (one thread per
 // unit, token after token, took 92 us for 256 tokens of 256 units: a memory round trip and a logarithm each).
 __global__ void __launch_bounds__(kPrefillThreads) prefill_gcum_kernel(const PrefillParams p) {
-  dependents_may_start();
   wait_for_predecessor();
   const int lane = threadIdx.x & 31;
   const int64_t uc = (int64_t(blockIdx.x) * kPrefillThreads + threadIdx.x) >> 5;

@@ -99,7 +99,7 @@ __device__ __noinline__ float carry_element(const CarryRows &rows, const float *
 // MAKE_PHI: phi(K') is made here (parameter-free map, gated); otherwise it is in the scratch.
 template <bool PARTIAL, bool MAKE_PHI, bool GATED>
 __global__ void __launch_bounds__(kThreads, GATED ? 3 : 0) prefill_state_mma_kernel(const PrefillParams p) {
-  dependents_may_start();
+  if (!GATED) dependents_may_start();
   wait_for_predecessor();
   using bf16 = __nv_bfloat16;
   // per stage phi columns (or K' rows, 16 bytes more per row) and V' rows; made phi columns
@@ -313,6 +313,7 @@ __global__ void __launch_bounds__(kThreads, GATED ? 3 : 0) prefill_state_mma_ker
       __syncthreads();   // (PARTIAL: the sums go over the scratch that was read)
     }
   }
+  if (GATED) dependents_may_start();   // (8 layers of 8000 tokens, state only: 1.18 ms; at the kernel's top, and in the gcum kernel, 1.44, not at all 1.48)
   // accumulator fragment: c0, c1 -> (row gid, cols 2 tig + {0,1}); c2, c3 -> row gid + 8
   if (PARTIAL) {   // (every read of these scratch columns lies before the loop's last barrier)
 #pragma unroll
