@@ -189,3 +189,120 @@ def test_overlapping_launches_hold_nothing_up(what, bound):
     g.glide_destroy()
     print(f"{what}: {t_together * 1e3:.1f} us, with events between {t_apart * 1e3:.1f}")
     assert t_together <= bound * t_apart
+
+
+# A chunk's sum in passes of several chunks (their sums by row in the scratch, added up by the scan): six layers, a call with outputs of
+# three chunks or more, so that a pass holds three at least.  The layer with w = T - 1 has one delayed token, of the pass's last chunk,
+# w = T - 3 three.  Chunk 144: stages with a remainder.
+def _states_after(windows, chunk, calls, B=2):
+    T = sum(calls)
+    gen = torch.Generator(device="cuda").manual_seed(chunk + T)
+    q, k, v = (torch.randn((len(windows), B, T, h, 128), generator=gen, device="cuda").to(BF16) for h in (4, 2, 2))
+    g = glide.Glide(windows, B, 4, 2, 128, 1 << 20, prefill_chunk=chunk)
+    at = 0
+    for n in calls:
+        part = [x[:, :, at:at + n].contiguous() for x in (q, k, v)]
+        g.glide_prefill(*part, torch.empty_like(part[0]))
+        at += n
+    states = [g.glide_export_state(l)[2:] for l in range(len(windows))]
+    assert g.glide_device_status() == 0
+    g.glide_destroy()
+    return k, v, states
+
+
+# Bound: the tensor core adds without rounding to nearest, so the error grows with the number of products added to a running sum, 3 of
+# 16 tokens each; 8.2e-7 was measured with chunks of 256 tokens, random keys and values.  Not twice that, and in proportion for
+# longer chunks.  (A phi of two terms instead of three is 2.3e-6 to 2.6e-6 off by itself.)
+@pytest.mark.parametrize("chunk,calls", [(144, [1000]), (256, [700, 900]), (1024, [3100])])
+def test_sums_of_several_chunks_against_fp64(chunk, calls):
+    windows, T, bound = [0, 16, 100, 304, 31, 1 << 20], sum(calls), 1.5e-6 * max(1, chunk / 256)
+    k, v, states = _states_after(windows, chunk, calls)
+    for l, w in enumerate(windows[:-1]):
+        S, z = states[l]
+        phi = torch.softmax(k[l].double(), -1)[:, :T - w].transpose(1, 2)
+        want = phi.transpose(-1, -2) @ v[l][:, :T - w].double().transpose(1, 2)
+        err, errz = ((S - want).norm() / want.norm()).item(), ((z - phi.sum(2)).norm() / phi.sum(2).norm()).item()
+        print(f"chunk {chunk}, w = {w}: S {err:.2e}, z {errz:.2e}")
+        assert err <= bound and errz <= bound
+
+
+# One delayed token: z is its phi(k) in fp32 and S the products of the three terms of that with V, exact but for two sums of the tensor
+# core, each operand of which loses less than 2^-23 of the result.  (Without the third term 2^-18 at most, 2e-6 on average.)  A pass of
+# one chunk and passes of several; three tokens: three such sums each.
+@pytest.mark.parametrize("layers,chunk", [(1, 64), (1, 256), (6, 144), (6, 256)])
+def test_terms_of_phi_in_the_carry(layers, chunk):
+    T = 3 * chunk + 17
+    k, v, states = _states_after([T - 1, T - 3, 16, 100, 304, 0][:layers], chunk, [T])
+    S, z = (x.double() for x in states[0])
+    exact = z[..., None] * v[0][:, 0].double()[:, :, None, :]
+    assert ((S - exact).abs() <= 4 * 2.0 ** -23 * exact.abs()).all()
+    if layers > 1:
+        S, z = (x.double() for x in states[1])
+        phi = torch.softmax(k[1].double(), -1)[:, :3].transpose(1, 2)
+        want = phi.transpose(-1, -2) @ v[1][:, :3].double().transpose(1, 2)
+        # (phi itself: the exponent is rounded at up to 2^3, the sum and the quotient: 8 2^-24 ln 2 and a few 2^-24)
+        assert ((S - want).norm() / want.norm()).item() <= (8 + 8) * 2.0 ** -24
+
+
+# As test_calls_back_to_back, for calls that it leaves out: slots of different lengths, reset, parked and filled again between steps (the
+# streaming decode kernel reads their offsets before it waits for what is in front), and layer by layer, with the learned map (its
+# feature kernel asks for its matrices before it waits) and without.
+@pytest.mark.parametrize("kind,dtype,d,heads,kw", [
+    ("slots", BF16, 128, 8, dict()), ("slots", torch.float32, 64, 4, dict()), ("slots", BF16, 128, 8, dict(gated=True)), ("layers", BF16, 128, 8, dict(phi=1)),
+    ("layers", BF16, 128, 8, dict()), ("layers", torch.float32, 64, 2, dict()), ("layers", torch.float32, 128, 4, dict(phi=1))])
+def test_slots_and_layers_back_to_back(kind, dtype, d, heads, kw):
+    windows, B, T, steps = [0, 16, 300], 3, 400, 4
+    L, kw = len(windows), dict(kw)
+    gen = torch.Generator(device="cuda").manual_seed(137)
+    rand = lambda *shape: torch.randn(shape, generator=gen, device="cuda").to(dtype)
+    if kw.get("phi"):
+        kw.update(phi_wq=(rand(L, heads, d, d) * d ** -0.5).contiguous(), phi_wk=(rand(L, 2, d, d) * d ** -0.5).contiguous())
+    prompts = [[rand(L, T - 90 * b, h, d) for h in (heads, 2, 2)] for b in range(B)]
+    level = [rand(L, B, T, h, d) for h in (heads, 2, 2)]
+    tokens = [[rand(L, B, h, d) for h in (heads, 2, 2)] for _ in range(steps)]
+    results = []
+    for idle in (True, False, False):
+        g = glide.Glide(windows, B, heads, 2, d, 1 << 20, dtype=dtype, **kw)
+        outs, calls = [], []
+
+        def step(t, l=None):
+            s = slice(0, L) if l is None else slice(l, l + 1)
+            outs.append(torch.zeros_like(t[0][s]))
+            calls.append(lambda o=outs[-1]: g.glide_decode_step(*t, o) if l is None else g.glide_decode_step_layers(*(x[s] for x in t), o, l, 1))
+
+        def fill(b):
+            outs.append(torch.zeros_like(prompts[b][0]))
+            calls.extend([lambda: g.glide_reset_seq(b), lambda o=outs[-1]: g.glide_prefill_seq(b, *prompts[b], o)])
+
+        for _ in range(2):
+            if kind == "slots":
+                for b in range(B):
+                    fill(b)
+                calls.append(lambda: g.glide_park_seq(1))
+                step(tokens[0])
+                step(tokens[1])
+                fill(0)
+                step(tokens[2])
+                fill(1)
+                step(tokens[3])
+            else:
+                calls.append(g.glide_reset)
+                for l in range(L):
+                    outs.append(torch.zeros_like(level[0][l:l + 1]))
+                    calls.append(lambda o=outs[-1], l=l: g.glide_prefill(*(x[l:l + 1] for x in level), o, layer_begin=l, layer_count=1))
+                for t in tokens[:3]:
+                    for l in range(L):
+                        step(t, l)
+                step(tokens[3])
+        torch.cuda.synchronize()
+        for call in calls:
+            call()
+            if idle:
+                torch.cuda.synchronize()
+        torch.cuda.synchronize()
+        assert g.glide_device_status() == 0
+        results.append(outs + [x for l, w in enumerate(windows) for x in g.glide_export_state(l)[2:]])
+        g.glide_destroy()
+    for other in results[1:]:
+        for a, b in zip(results[0], other):
+            assert torch.equal(a, b)
