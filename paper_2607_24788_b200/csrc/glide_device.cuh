@@ -14,8 +14,9 @@ constexpr float kLog2e = 1.4426950408889634f;
 // Programmatic dependent launch: the launch behind this one may take SMs as soon as every CTA of this grid has called this or ended.
 // Its CTAs then hold their places while they wait, and those of the launch after it, which nothing but this call holds back, get what
 // places are left.  Grids of less than half the SMs' number lost more by that than the launches cost, so a kernel calls it as late as
-// still hides the launch, behind its own wait at the earliest.  At the top it stands in the scan, ring and reset kernels: behind
-// them comes an ordinary launch, or one with a CTA for every SM, or (after a reset) a single call.
+// still hides the launch, behind its own wait at the earliest (a kernel that never does lets it go as its CTAs end).  At the top it
+// stands in the scan, ring and reset kernels and the ungated carry: behind them comes an ordinary launch, one with a CTA for
+// every SM, the ring fill or (after a reset) a single call.
 __device__ __forceinline__ void dependents_may_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 // ... and waits here until the one before has completed.  Every CTA of a kernel that is launched by launch_chained passes this,
 // also one that has nothing to do: so a grid that has completed means that all before it have.

@@ -9,10 +9,13 @@
 // as the MN-major A operand (a token's row as it is) and its rounding for the attention kernel, and sum z on the way; warp 8 issues
 // six m128n128k16 per stage with V' as the MN-major B operand.  K' and V' rows come by cp.async two stages ahead (rings of three and
 // four buffers: V' is read until the products of its stage have completed), the terms are double-buffered.
-// What bounds it: memory where there are many chunks (8 x 2048 tokens, 4 layers: 524 MB of rows, rounded phi and sums in 93 us, 5.6
-// TB/s), the chain of a CTA where there are few (8001 tokens of one layer, 256 CTAs: 20 us).  The mma.sync form before it, two CTAs
-// of 64 rows that both staged K' and made phi, took 185 and 43 us; it remains for the learned map and for gates.  Against fp64 S is as
-// far off as with it (8.2e-7 after 4096 tokens, both), z less (6.4e-8, 8.0e-8).
+// What bounds it: the chain of a CTA's stages.  8 x 2048 tokens of 4 layers take eight launches of 256 CTAs, 93 us (11.6 a launch), in
+// which 268 MB of rows come from HBM and 256 MB of rounded phi and sums go to L2; 8001 tokens of one layer 20 us.  (ncu, one launch of
+// 256 CTAs with cold caches: 23.6 us, 31 MB read, 0.7 written, 103 MB of L2 traffic, tensor pipe 12 %.)  The mma.sync form before it,
+// two CTAs of 64 rows that both staged K' and made phi, took 185 and 43 us; it remains where phi comes from another kernel (the learned
+// map, sum-of-terms merges with outputs, outputs by the mma.sync or CUDA-core kernel) and for gates.  Against fp64 S is as far
+// off as with it (chunks of 256 tokens 7.9e-7, both; the tensor core adds without rounding to nearest, so with the chunk's length: 144 tokens
+// 4.7e-7, 1024 2.5e-6 to 3.4e-6), z less (5.6e-8, 8.0e-8).
 // Every mbarrier wait is bounded; after a time-out the CTA runs its loop out without waiting, stores nothing, records
 // kDevWaitTimeout, frees its TMEM columns and returns.
 #include <type_traits>

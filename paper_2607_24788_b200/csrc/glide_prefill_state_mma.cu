@@ -1,6 +1,7 @@
 // Chunk-scan carry of the prefill for bf16 I/O and d = 128 on the tensor cores, at fp32 accuracy:
 //   S += phi(K')^T V',  z += sum phi(K')      over the chunk's delayed tokens (k'_i = k_{i-w}).
-// (phi from the scratch, or gates; the parameter-free map without gates is the kernel of glide_prefill_carry_tc.cu.)
+// For gates, and where another kernel makes phi (the learned map, sum-of-terms merges with outputs, outputs by the mma.sync or the
+// CUDA-core kernel); all else is the kernel of glide_prefill_carry_tc.cu.
 // V' is bf16 already.  phi(K') is fp32 in the chunk scratch; every value is split into three bf16 terms
 // (x = hi + mid + lo, each the bf16 rounding of what the previous ones left: an error-free split of the 24-bit
 // significand), so the three products phi_term^T V' are exact in fp32 and only the fp32 accumulation of the tensor
@@ -96,12 +97,13 @@ __device__ __noinline__ float carry_element(const CarryRows &rows, const float *
 // of S (64 state rows x 128 values = 128 scratch rows x the CTA's 64 columns, z in row 128: chunks of more than 128
 // tokens), and prefill_scan_kernel adds the sums up in chunk order.  Otherwise S is updated in place, and its value
 // before the chunk is left as bf16 (z: fp32) for the attention kernel, which runs after this one.
-// MAKE_PHI: phi(K') is made here (parameter-free map, gated); otherwise it is in the scratch.
+// MAKE_PHI: phi(K') is made here (parameter-free map, gated, no sum-of-terms merge); otherwise it is in the scratch.
 template <bool PARTIAL, bool MAKE_PHI, bool GATED>
 __global__ void __launch_bounds__(kThreads, GATED ? 3 : 0) prefill_state_mma_kernel(const PrefillParams p) {
   if (!GATED) dependents_may_start();
   wait_for_predecessor();
   using bf16 = __nv_bfloat16;
+  static_assert(!MAKE_PHI || GATED, "without gates glide_prefill_carry_tc.cu makes phi");
   // per stage phi columns (or K' rows, 16 bytes more per row) and V' rows; made phi columns
   constexpr int kInBytes = MAKE_PHI ? kVBytes : kPhiBytes;
   __shared__ __align__(16) unsigned char stage[2][kInBytes + kVBytes];
@@ -210,8 +212,7 @@ __global__ void __launch_bounds__(kThreads, GATED ? 3 : 0) prefill_state_mma_ker
         if (p16 && there) {
           bf16 *out = p16 + size_t(i0 + tok) * kD + (part & 1) * 32;
 #pragma unroll
-          for (int hl = 0; hl < 2; ++hl) {   // gated: what the rounding left, in the second half of the array
-            if (hl == 1 && !GATED) break;
+          for (int hl = 0; hl < 2; ++hl) {   // (what the rounding left in the second half of the array)
 #pragma unroll
             for (int i = 0; i < 32; i += 8) {
               uint32_t o[4];

@@ -22,11 +22,11 @@
 // Linear part (after the window tiles, by the same warps in the same way): with a common reference M = max(m_ref, -64)
 // per row, phi(Q) 2^-M as bf16 times a bf16 copy of the state (inter-chunk), and C = phi(Q) phi(K')^T masked to
 // j' <= i, then C V' (intra-chunk); l accumulates the matching sums.  out = O / l.
-// What bounds it: short windows, the fixed chain of a CTA (24500 cycles: 6800 until Q and K_0 are there and the first product is
-// done, one softmax 3500, phi 2900, two to three more products 8500, the store 2500); long windows, per key tile and row tile the
-// chain softmax (1770) -> P V and the next S (1050 to 1300) -> signals, 3570 cycles in which the two row tiles' products take
-// 2048.  8 layers of 2048 tokens, 32 / 8 heads, windows of 64 / 256 / 1024: 270 / 333 / 525 us; with one softmax thread per row,
-// one MMA warp and phi in one piece 292 / 379 / 576.
+// What bounds it: short windows, the fixed chain of a CTA (windows of 64, 23100 cycles: set-up 740, 6500 until Q and K_0 are there
+// and the first product is done, one softmax 3600, phi 2700, its products 3000, C 2000, the last products 1300, the store 3200); long
+// windows, per key tile and row tile the chain softmax (1770) -> P V and the next S (1050 to 1300) -> signals, 3500 cycles in which the
+// two row tiles' products take 2048.  8 layers of 2048 tokens, 32 / 8 heads, windows of 64 / 256 / 1024: 255 / 316 / 479 us for all; with
+// one softmax thread per row, one MMA warp and phi in one piece 292 / 379 / 576.
 // Every mbarrier wait is bounded; on a time-out the CTA records kDevWaitTimeout, leaves its loops, frees its TMEM
 // columns and returns.
 #include <cuda.h>
@@ -377,7 +377,7 @@ prefill_attn_tc_kernel(const __grid_constant__ PrefillParams p, const CUtensorMa
     mbar_init(smem_u32(&sm.bar_done), n_rows);
     mbar_init(smem_u32(&sm.bar_state), 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    // (Q_B behind K_0, which the first product needs before it: 8001 tokens layer by layer 7.09 -> 6.94 ms, 8 x 2048 10.2 -> 10.1)
+    // (Q_B behind K_0, which the first product needs before it: 8001 tokens layer by layer 2 %, 8 x 2048 1 % less, at commit 1790120)
     if (q_by_tma) ask_q(0);
   }
   // (positions stay below 2^30, the most tokens a context may hold; a longer window is no other than that)
